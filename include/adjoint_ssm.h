@@ -87,8 +87,9 @@ typedef struct {          /* parameters of one layer (device pointers) */
   const void  *W_C;       /* [N,P] io dtype */
   const float *A_log;     /* [P,N] fp32 (AS_A_SCALAR: [P]), A = -exp(A_log) */
   const void  *Wcat;      /* optional, may be NULL: [P+32, P] io dtype, the rows of W_delta, W_B, W_C stacked, as written
-                             by as_pack_weights.  Only the bf16 tensor-core contractions read it (bf16 io, P % 32 == 0);
-                             when NULL they pack a copy into the scratch on every call (one more small kernel). */
+                             by as_pack_weights.  Only the bf16 tensor-core contractions read it (bf16 io; the
+                             gradient calls only where P % 32 == 0); when NULL, or in a gradient call at another width,
+                             they pack a copy into the scratch on every call (one more small kernel). */
 } as_params_t;
 
 typedef struct {          /* gradient outputs (device pointers); parameter gradients are fp32, summed over the batch */

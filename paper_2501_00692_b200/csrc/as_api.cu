@@ -51,18 +51,22 @@ int check_params(const as_params_t* pr) {
     if (e__ != 0) return AS_ERR_CUDA;     \
   } while (0)
 
-// Wcat of the call: the caller's packed copy if it gave one, else packed here into the scratch
-int wcat_of(const Plan& pl, const as_params_t* pr, char* ws, cudaStream_t st, const void** wcat) {
-  if (pr->Wcat) { *wcat = pr->Wcat; return AS_OK; }
-  AS_TRY(tc_pack_wcat(pl.P, pl.KL, pr, ws + pl.off_wcat, st));
-  *wcat = ws + pl.off_wcat;
+// Wcat of the call and how often it holds W_B and W_C: the caller's packed copy if it gave one, else packed here into the
+// scratch.  The gradient of a width that is not a multiple of 32 needs them once per term of the dB, dC split.
+struct Wcat { const void* p; int reps; };
+int wcat_of(const Plan& pl, const as_params_t* pr, bool grad, char* ws, cudaStream_t st, Wcat* wcat) {
+  wcat->reps = grad ? pl.gsplit : 1;
+  if (pr->Wcat && wcat->reps == 1) { wcat->p = pr->Wcat; return AS_OK; }
+  char* at = ws + (grad ? pl.off_wcatx : pl.off_wcat);
+  AS_TRY(tc_pack_wcat(pl.P, pl.KL, wcat->reps, pr, at, st));
+  wcat->p = at;
   return AS_OK;
 }
 
 // steps 1-3 of SSM(.): Delta = softplus(x W_delta^T + b), B = x W_B^T, C = x W_C^T  (every layer of the call)
-int projections(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, char* ws, cudaStream_t st) {
+int projections(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const void* x, char* ws, cudaStream_t st) {
   if (pl.tc) {
-    AS_TRY(tc_projections(pl, pr, wcat, x, ws, st));
+    AS_TRY(tc_projections(pl, pr, wcat.p, wcat.reps, x, ws, st));
     return AS_OK;
   }
   const int bf = pl.io == AS_BF16;
@@ -97,7 +101,7 @@ int pick_splitk(int64_t tiles, int64_t K) {
 }
 
 // the net-VJPs: weight gradients (contractions over all tokens) and the input gradient, for every layer of the call
-int contractions(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws,
+int contractions(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const void* x, const as_grads_t* out, char* ws,
                  cudaStream_t st) {
   const int bf = pl.io == AS_BF16;
   const size_t e = bf ? 2 : 4;
@@ -106,7 +110,7 @@ int contractions(const Plan& pl, const as_params_t* pr, const void* wcat, const 
   if (pl.tc) {
     AS_TRY(tc_weight_grads(pl, x, out, ws, st));
     mark(5, st);
-    if (out->dx) AS_TRY(tc_input_grad(pl, wcat, out->dx, ws, st));
+    if (out->dx) AS_TRY(tc_input_grad(pl, wcat.p, out->dx, ws, st));
     mark(6, st);
     return AS_OK;
   }
@@ -246,8 +250,8 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
   AS_TRY((int)cudaMemsetAsync(w + pl.off_status, 0, 256, st));
-  const void* wcat = nullptr;
-  if (pl.tc) { e = wcat_of(pl, params, w, st, &wcat); if (e) return e; }
+  Wcat wcat{};
+  if (pl.tc) { e = wcat_of(pl, params, false, w, st, &wcat); if (e) return e; }
   e = projections(pl, params, wcat, x, w, st);
   if (e) return e;
   ScanPtrs sp{x, nullptr, params->A_log, w};
@@ -292,7 +296,7 @@ int as_pack_weights(const as_shape_t* shape, int32_t layers, const as_params_t* 
   if (!aligned16(wcat)) return AS_ERR_ALIGN;
   if (layers < 1) return AS_ERR_SHAPE;
   if (shape->io != AS_BF16) return AS_ERR_DTYPE;   // only the bf16 tensor-core contractions read a packed copy
-  AS_TRY(tc_pack_wcat(shape->d_model, layers, params, wcat, reinterpret_cast<cudaStream_t>(stream)));
+  AS_TRY(tc_pack_wcat(shape->d_model, layers, 1, params, wcat, reinterpret_cast<cudaStream_t>(stream)));
   return AS_OK;
 }
 
@@ -313,8 +317,8 @@ int as_adjoint_grad_layers(const as_shape_t* shape, int32_t layers, const as_par
   mark(0, st);
   e = zero_outputs(pl, flags, out, w, st);
   if (e) return e;
-  const void* wcat = nullptr;
-  if (pl.tc) { e = wcat_of(pl, params, w, st, &wcat); if (e) return e; }
+  Wcat wcat{};
+  if (pl.tc) { e = wcat_of(pl, params, true, w, st, &wcat); if (e) return e; }
   e = projections(pl, params, wcat, x, w, st);
   if (e) return e;
   mark(1, st);
@@ -342,8 +346,8 @@ int as_full_bptt_grad(const as_shape_t* shape, const as_params_t* params, const 
   char* w = reinterpret_cast<char*>(ws);
   e = zero_outputs(pl, flags, out, w, st);
   if (e) return e;
-  const void* wcat = nullptr;
-  if (pl.tc) { e = wcat_of(pl, params, w, st, &wcat); if (e) return e; }
+  Wcat wcat{};
+  if (pl.tc) { e = wcat_of(pl, params, true, w, st, &wcat); if (e) return e; }
   e = projections(pl, params, wcat, x, w, st);
   if (e) return e;
   ScanPtrs sp{x, dy, params->A_log, w};

@@ -8,6 +8,9 @@
 //   DW   : dWcat = Gcat^T X  over all tokens     (A MN-major, B MN-major; split-K, fp32 reduction)
 //   DX   : dx = dx_dir + Gcat Wcat               (A K-major, B MN-major; add + bf16 store)
 // with Wcat = [W_delta; W_B; W_C] ([P+32, P]) and Gcat = [du | dB | dC] ([tokens, P+32]), both bf16.
+// Widths that are not a multiple of 32 keep all 24 bits of dB and dC: Gcat then ends in three such pairs (the fp32 sums
+// split into three bf16 terms, which is exact) and the Wcat of the input gradient repeats W_B and W_C three times
+// (Plan.gsplit), so the contraction of the split equals the contraction of the fp32 values.
 // No cluster multicast is used anywhere.  Every mbarrier wait is bounded; on timeout the kernel records
 // AS_ERR_TIMEOUT in the status word, stops issuing work, frees its TMEM and returns.
 #include <cuda.h>
@@ -39,9 +42,12 @@ struct TcArgs {
   int kblocks;          // number of BK-blocks along K (DW: per layer)
   int splitk;
   int P;                // d_model
+  int wrows;            // rows of one layer's Wcat as stored (P + 32, or P + 96 with the three-term split)
+  int grp;              // DW: rows per reduce-add (16, or 8 where P is not a multiple of 16: no group straddles two outputs)
   int layers;           // independent problems stacked along the leading dimension of every tensor
   int64_t rows_layer;   // token rows per layer (a multiple of BM when layers > 1)
   const float* bias;    // PROJ: b_delta [layers, P]
+  float* bc;            // PROJ: [B | C] rows, for the plain stores where P is not a multiple of 16
   int* status;
 };
 
@@ -181,7 +187,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
   const int mt = (int)((a.M + BM - 1) / BM), nt = (a.N + BN - 1) / BN;
   const int ntiles = mt * nt * a.splitk * ((ML && EPI == TC_DW) ? a.layers : 1);
   const int kper = (a.kblocks + a.splitk - 1) / a.splitk;
-  const int NWc = a.P + NBC;                       // rows of one layer's Wcat
+  const int NWc = a.wrows;                         // rows of one layer's Wcat
   volatile int* abortp = &abort_s;
 
   if (threadIdx.x == 0) {
@@ -364,7 +370,25 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
             tmem_ld16(tcol, r);
             if (lane == 0) bulk_wait_read<1>();         // the operation that last used this buffer has read it
             __syncwarp();
-            if (EPI == TC_PROJ && nb < a.P) {
+            if (EPI == TC_PROJ && nb + CW > a.P && (a.P & 15)) {
+              // the chunk that holds the border between Delta and [B | C], and those after it, where that border is no
+              // multiple of 16: a TMA store would have to start left of the [B | C] rows, so those columns go out as
+              // plain 16-byte stores of the lane's row
+              const int64_t row = mrow + lane;
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int col = nb + 4 * q;
+                float4 v = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]),
+                                       __uint_as_float(r[4 * q + 3]));
+                if (col < a.P) {
+                  const float4 bv = __ldg(reinterpret_cast<const float4*>(bias_l + col));
+                  v = make_float4(softplus_f(v.x + bv.x), softplus_f(v.y + bv.y), softplus_f(v.z + bv.z), softplus_f(v.w + bv.w));
+                } else if (col < a.P + NBC && row < a.M) {
+                  *reinterpret_cast<float4*>(a.bc + row * NBC + col - a.P) = v;
+                }
+                *reinterpret_cast<float4*>(buf + swz64(lane, q)) = v;   // Delta columns go out below, clipped at P
+              }
+            } else if (EPI == TC_PROJ && nb < a.P) {
               const float4* b4 = reinterpret_cast<const float4*>(bias_l + nb);
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
@@ -383,17 +407,18 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
             if (lane == 0) {
               if (EPI == TC_PROJ) {
                 if (nb < a.P) tma_store_2d(&tmO0, buf, nb, mrow);       // Delta
-                else tma_store_2d(&tmO1, buf, nb - a.P, mrow);          // [B | C]
+                else if (!(a.P & 15)) tma_store_2d(&tmO1, buf, nb - a.P, mrow);   // [B | C]
               } else {
-                // rows of Wcat space: [0, P) dW_delta, [P, P+16) dW_B, [P+16, P+32) dW_C; 16-row groups never straddle
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                  const int mr = mrow + 16 * hh;
-                  const void* src = buf + hh * 1024;
+                // rows of Gcat space: [0, P) dW_delta, then 16 rows dW_B and 16 rows dW_C (three such pairs with the
+                // split: their sums add up in the output); a group of grp rows never straddles two outputs
+#pragma unroll 1
+                for (int r0 = 0; r0 < 32; r0 += a.grp) {
+                  const int mr = mrow + r0, e = mr - a.P;
+                  const void* src = buf + r0 * 64;
                   const int l1 = ML ? lay * a.P : 0, l2 = ML ? lay * NS : 0;   // this layer's rows of the stacked outputs
-                  if (mr < a.P) tma_reduce_add_2d(&tmO0, src, nb, l1 + mr);
-                  else if (mr < a.P + NS) tma_reduce_add_2d(&tmO1, src, nb, l2 + mr - a.P);
-                  else if (mr < a.P + 2 * NS) tma_reduce_add_2d(&tmO2, src, nb, l2 + mr - a.P - NS);
+                  if (e < 0) tma_reduce_add_2d(&tmO0, src, nb, l1 + mr);
+                  else if (mr < a.M && (e & 16) == 0) tma_reduce_add_2d(&tmO1, src, nb, l2 + (e & 15));
+                  else if (mr < a.M) tma_reduce_add_2d(&tmO2, src, nb, l2 + (e & 15));
                 }
               }
               bulk_commit();
@@ -419,20 +444,22 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
 }
 
 // ---- small helpers -------------------------------------------------------------------------------
-// Wcat[l] = [W_delta[l]; W_B[l]; W_C[l]] for every layer l (blockIdx.y)
-__global__ void pack_wcat_kernel(int P, const __nv_bfloat16* __restrict__ Wd, const __nv_bfloat16* __restrict__ WB,
+// Wcat[l] = [W_delta[l]; W_B[l]; W_C[l]] for every layer l (blockIdx.y), W_B and W_C `reps` times over
+__global__ void pack_wcat_kernel(int P, int reps, const __nv_bfloat16* __restrict__ Wd, const __nv_bfloat16* __restrict__ WB,
                                  const __nv_bfloat16* __restrict__ WC, __nv_bfloat16* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n = (int64_t)(P + NBC) * P;
+  const int64_t n = (int64_t)(P + reps * NBC) * P;
   if (i >= n) return;
   const int64_t l = blockIdx.y;
   Wd += l * P * P; WB += l * NS * P; WC += l * NS * P; out += l * n;
   const int64_t row = i / P, col = i % P;
-  out[i] = row < P ? Wd[i] : (row < P + NS ? WB[(row - P) * P + col] : WC[(row - P - NS) * P + col]);
+  const int64_t e = (row - P) & (NBC - 1);
+  out[i] = row < P ? Wd[i] : (e < NS ? WB[e * P + col] : WC[(e - NS) * P + col]);
 }
 
-// [dB | dC] fp32 sums -> the last 32 bf16 columns of Gcat; eight values per thread (P and the row pitch are multiples
-// of 32 elements on this path, so every access is 16-byte aligned)
+// [dB | dC] fp32 sums -> the last bf16 columns of Gcat; eight values per thread (P and the row pitch are multiples of 8
+// elements, so every access is 16-byte aligned).  SPLIT: as three bf16 terms, 32 columns each, that add up to the fp32 value.
+template <int SPLIT>
 __global__ void cvt_dbc_kernel(int64_t rows, int ldg, int P, const float* __restrict__ dbc, __nv_bfloat16* __restrict__ gcat) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // one group of 8 columns
   if (i >= rows * (NBC / 8)) return;
@@ -440,11 +467,19 @@ __global__ void cvt_dbc_kernel(int64_t rows, int ldg, int P, const float* __rest
   const int c = (int)(i % (NBC / 8)) * 8;
   const float4 a = __ldg(reinterpret_cast<const float4*>(dbc + row * NBC + c));
   const float4 b = __ldg(reinterpret_cast<const float4*>(dbc + row * NBC + c + 4));
-  uint4 o;
-  __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o);
-  o2[0] = __floats2bfloat162_rn(a.x, a.y); o2[1] = __floats2bfloat162_rn(a.z, a.w);
-  o2[2] = __floats2bfloat162_rn(b.x, b.y); o2[3] = __floats2bfloat162_rn(b.z, b.w);
-  *reinterpret_cast<uint4*>(gcat + row * ldg + P + c) = o;
+  float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int t = 0; t < SPLIT; ++t) {
+    uint4 o;
+    __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      o2[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+      const float2 f = __bfloat1622float2(o2[k]);
+      v[2 * k] -= f.x; v[2 * k + 1] -= f.y;
+    }
+    *reinterpret_cast<uint4*>(gcat + row * ldg + P + t * NBC + c) = o;
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -512,10 +547,10 @@ int launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap 
 constexpr int TBN = 256;   // tile width of the weight-gradient and input-gradient contractions
 constexpr int PBN = 208;   // projections: N = P + 32; for P = 768 four 208-wide tiles waste 4 % where 256 wastes 22 %
 
-int tc_pack_wcat(int P, int layers, const as_params_t* pr, void* wcat, cudaStream_t st) {
-  const int64_t n = (int64_t)(P + NBC) * P;
+int tc_pack_wcat(int P, int layers, int reps, const as_params_t* pr, void* wcat, cudaStream_t st) {
+  const int64_t n = (int64_t)(P + reps * NBC) * P;
   pack_wcat_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)layers), 256, 0, st>>>(
-      P, (const __nv_bfloat16*)pr->W_delta, (const __nv_bfloat16*)pr->W_B, (const __nv_bfloat16*)pr->W_C,
+      P, reps, (const __nv_bfloat16*)pr->W_delta, (const __nv_bfloat16*)pr->W_B, (const __nv_bfloat16*)pr->W_C,
       (__nv_bfloat16*)wcat);
   count_launch();
   return (int)cudaGetLastError();
@@ -530,9 +565,9 @@ static inline int layer_groups(const Plan& pl, LayerLoop* g) {
   return 0;   // the caller loops over single layers
 }
 
-int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, char* ws, cudaStream_t st) {
+int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x, char* ws, cudaStream_t st) {
   const int64_t rows = (int64_t)pl.Bg * pl.T;
-  const int P = pl.P, NW = P + NBC;
+  const int P = pl.P, NW = P + wreps * NBC;
   LayerLoop one;
   const bool batched = layer_groups(pl, &one) == 1;
   for (int l0 = 0; l0 < pl.KL; l0 += batched ? pl.KL : 1) {
@@ -542,8 +577,9 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, cons
     if (make_map(&tmA, (const char*)x + (size_t)l0 * rows * P * 2, M, P, P, BM)) return 1;
     if (make_map(&tmB, (const char*)wcat + (size_t)l0 * NW * P * 2, (uint64_t)NW * nl, P, P, PBN)) return 1;
     TcArgs a{};
-    a.M = M; a.N = NW; a.kblocks = (P + BK - 1) / BK; a.splitk = 1; a.P = P; a.layers = nl; a.rows_layer = rows;
+    a.M = M; a.N = P + NBC; a.kblocks = (P + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.grp = 16; a.layers = nl; a.rows_layer = rows;
     a.bias = pr->b_delta + (size_t)l0 * P;
+    a.bc = (float*)(ws + pl.off_bc) + (size_t)l0 * rows * NBC;
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
     if (make_map_out_f32(&tmO[0], ws + pl.off_delta + (size_t)l0 * rows * P * 4, M, P, 32)) return 1;
@@ -558,8 +594,9 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, cons
 int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* ws, cudaStream_t st) {
   const int64_t rows = (int64_t)pl.Bg * pl.T;
   const int64_t Mall = rows * pl.KL;
-  const int P = pl.P, NW = P + NBC;
-  cvt_dbc_kernel<<<(unsigned)((Mall * (NBC / 8) + 255) / 256), 256, 0, st>>>(Mall, NW, P, (const float*)(ws + pl.off_dbc),
+  const int P = pl.P, NW = pl.du_ld;
+  auto cvt = pl.gsplit == 3 ? cvt_dbc_kernel<3> : cvt_dbc_kernel<1>;
+  cvt<<<(unsigned)((Mall * (NBC / 8) + 255) / 256), 256, 0, st>>>(Mall, NW, P, (const float*)(ws + pl.off_dbc),
                                                                        (__nv_bfloat16*)(ws + pl.off_du));
   count_launch();
   if (cudaGetLastError() != cudaSuccess) return 1;
@@ -568,10 +605,11 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
   for (int l0 = 0; l0 < pl.KL; l0 += batched ? pl.KL : 1) {
     const int nl = batched ? pl.KL : 1;
     CUtensorMap tmA, tmB;
-    if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, rows * nl, NW, NW, 64)) return 1;   // Gcat as [K=tokens, M=P+32]
+    if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, rows * nl, NW, NW, 64)) return 1;   // Gcat as [K=tokens, M]
     if (make_map(&tmB, (const char*)x + (size_t)l0 * rows * P * 2, rows * nl, P, P, 64)) return 1;       // X as [K=tokens, N=P]
     TcArgs a{};
-    a.M = NW; a.N = P; a.kblocks = (int)((rows + BK - 1) / BK); a.P = P; a.layers = nl; a.rows_layer = rows;
+    a.M = NW; a.N = P; a.kblocks = (int)((rows + BK - 1) / BK); a.P = P; a.wrows = NW; a.grp = P % 16 ? 8 : 16;
+    a.layers = nl; a.rows_layer = rows;
     const int tiles = ((NW + BM - 1) / BM) * ((P + TBN - 1) / TBN) * nl;
     int sk = sm_count() / tiles;   // about one tile per persistent CTA (two measured 3 % slower at C3: more reduce-adds)
     if (sk > a.kblocks) sk = a.kblocks;
@@ -580,9 +618,9 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
     a.splitk = (a.kblocks + kper - 1) / kper;   // no empty split: every tile has at least one K block
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
-    if (make_map_out_f32(&tmO[0], out->dW_delta + (size_t)l0 * P * P, (uint64_t)P * nl, P, 16)) return 1;
-    if (make_map_out_f32(&tmO[1], out->dW_B + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, 16)) return 1;
-    if (make_map_out_f32(&tmO[2], out->dW_C + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, 16)) return 1;
+    if (make_map_out_f32(&tmO[0], out->dW_delta + (size_t)l0 * P * P, (uint64_t)P * nl, P, (uint32_t)a.grp)) return 1;
+    if (make_map_out_f32(&tmO[1], out->dW_B + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, (uint32_t)a.grp)) return 1;
+    if (make_map_out_f32(&tmO[2], out->dW_C + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, (uint32_t)a.grp)) return 1;
     const int e = launch_tc<MAJ_MN, MAJ_MN, TC_DW, TBN>(tmA, tmB, tmO, a, st);
     if (e) return e;
   }
@@ -591,17 +629,17 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
 
 int tc_input_grad(const Plan& pl, const void* wcat, void* dx, char* ws, cudaStream_t st) {
   const int64_t rows = (int64_t)pl.Bg * pl.T;
-  const int P = pl.P, NW = P + NBC;
+  const int P = pl.P, NW = pl.du_ld;   // K of the contraction: the columns of Gcat, the rows of Wcat
   LayerLoop one;
   const bool batched = layer_groups(pl, &one) == 1;
   for (int l0 = 0; l0 < pl.KL; l0 += batched ? pl.KL : 1) {
     const int nl = batched ? pl.KL : 1;
     const int64_t M = rows * nl;
     CUtensorMap tmA, tmB;
-    if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, M, NW, NW, BM)) return 1;            // Gcat as [M=tokens, K=P+32]
-    if (make_map(&tmB, (const char*)wcat + (size_t)l0 * NW * P * 2, (uint64_t)NW * nl, P, P, 64)) return 1;   // Wcat as [K=P+32, N=P]
+    if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, M, NW, NW, BM)) return 1;            // Gcat as [M=tokens, K]
+    if (make_map(&tmB, (const char*)wcat + (size_t)l0 * NW * P * 2, (uint64_t)NW * nl, P, P, 64)) return 1;   // Wcat as [K, N=P]
     TcArgs a{};
-    a.M = M; a.N = P; a.kblocks = (NW + BK - 1) / BK; a.splitk = 1; a.P = P; a.layers = nl; a.rows_layer = rows;
+    a.M = M; a.N = P; a.kblocks = (NW + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.grp = 16; a.layers = nl; a.rows_layer = rows;
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
     if (make_map_out_bf16(&tmO[0], (char*)dx + (size_t)l0 * rows * P * 2, M, P)) return 1;

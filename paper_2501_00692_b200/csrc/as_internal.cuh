@@ -94,12 +94,13 @@ struct Plan {
   int scalar;       // 1: one decay rate per channel (A_log is [P]), 0: one per (channel, state)
   int tiles;        // ceil(P / CH) channel tiles
   int bw;           // channels per staged row: min(CH, P)
-  int tc;           // 1: bf16 tensor-core contractions (bf16 I/O and d_model % 32 == 0), 0: FP32-pipe GEMMs
-  int du_ld;        // row pitch (elements) of the du buffer: P, or P+32 when it is the left part of Gcat = [du|dB|dC]
+  int tc;           // 1: bf16 tensor-core contractions (bf16 I/O), 0: FP32-pipe GEMMs
+  int gsplit;       // bf16 terms per value of dB, dC in Gcat: 1, or 3 (exact) where d_model % 32 != 0
+  int du_ld;        // row pitch (elements) of the du buffer: P, or P + 32 gsplit when it is the left part of Gcat = [du|dB|dC..]
   // byte offsets into the workspace
   size_t off_status, off_delta, off_bc, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
       off_partd, off_hstart, off_carry, off_swin, off_du, off_dxdir, off_dbc, off_dxacc,
-      off_bptt_ckpt, off_wcat, total_fwd, total_grad;
+      off_bptt_ckpt, off_wcat, off_wcatx, total_fwd, total_grad;
 };
 
 int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl);
@@ -137,8 +138,9 @@ int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st);
 int launch_finish_dx(const Plan& pl, const float* dxacc, const void* dxdir, void* dx, cudaStream_t st);
 
 // bf16 tensor-core path (as_gemm_tc.cu)
-int tc_pack_wcat(int P, int layers, const as_params_t* pr, void* wcat, cudaStream_t st);
-int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, char* ws, cudaStream_t st);
+int tc_pack_wcat(int P, int layers, int reps, const as_params_t* pr, void* wcat, cudaStream_t st);
+int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x, char* ws,
+                   cudaStream_t st);
 int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* ws, cudaStream_t st);
 int tc_input_grad(const Plan& pl, const void* wcat, void* dx, char* ws, cudaStream_t st);
 

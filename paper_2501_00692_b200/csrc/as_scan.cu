@@ -30,8 +30,9 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.KL = layers < 1 ? 1 : layers; p.Bg = sh->batch;
   p.B = p.KL * p.Bg; p.P = sh->d_model; p.T = sh->seqlen; p.io = sh->io;
   p.scalar = sh->a_structure == AS_A_SCALAR ? 1 : 0;
-  p.tc = (sh->io == AS_BF16 && sh->d_model % 32 == 0) ? 1 : 0;
-  p.du_ld = p.tc ? p.P + NBC : p.P;
+  p.tc = sh->io == AS_BF16 ? 1 : 0;
+  p.gsplit = p.P % 32 == 0 ? 1 : 3;
+  p.du_ld = p.tc ? p.P + p.gsplit * NBC : p.P;
   p.full = tbar >= p.T;
   p.tbar = p.full ? p.T : tbar;
   p.tiles = (p.P + CH - 1) / CH;
@@ -67,6 +68,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.off_hstart = take(BSB * 4);
   p.off_wcat = take((size_t)p.KL * (p.P + NBC) * p.P * 2);
   p.total_fwd = o;
+  p.off_wcatx = p.tc && p.gsplit > 1 ? take((size_t)p.KL * p.du_ld * p.P * 2) : p.off_wcat;
   p.off_ckpt = take((size_t)p.B * p.NC * p.tiles * TILE_FLOATS * 4);
   p.off_cs = take((size_t)p.B * p.NC * p.P * 4);
   p.off_muloc = take(BSB * 4);

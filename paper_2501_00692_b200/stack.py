@@ -32,7 +32,7 @@ class Stack:
         self.yhat = torch.empty(batch, seqlen, d_model, dtype=dtype, device=device)
         self.ytilde = torch.empty_like(self.yhat)
         # the bf16 tensor-core contractions read [W_delta; W_B; W_C] as one matrix: packed once here, per layer
-        if io == B.AS_BF16 and d_model % 32 == 0:
+        if io == B.AS_BF16:
             for th in self.thetas:
                 if th.get("Wcat") is None:
                     th["Wcat"] = torch.empty(B.as_wcat_bytes(self.shape), dtype=torch.uint8, device=device)
