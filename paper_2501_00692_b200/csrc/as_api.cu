@@ -69,44 +69,13 @@ int projections(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const v
     AS_TRY(tc_projections(pl, pr, wcat.p, wcat.reps, x, ws, st));
     return AS_OK;
   }
-  const int bf = pl.io == AS_BF16;
-  const size_t e = bf ? 2 : 4;
-  const int64_t M = (int64_t)pl.Bg * pl.T;
-  const size_t P = pl.P;
-  for (int l = 0; l < pl.KL; ++l) {
-    GemmArgs g{};
-    g.A = (const char*)x + l * M * P * e; g.a_bf16 = bf; g.a_sm = pl.P; g.a_sk = 1;
-    g.b_bf16 = bf; g.b_sn = pl.P; g.b_sk = 1;
-    g.M = M; g.K = pl.P; g.splitk = 1;
-    g.Bm = (const char*)pr->W_delta + l * P * P * e; g.N = pl.P;
-    g.C = reinterpret_cast<float*>(ws + pl.off_delta) + l * M * P; g.ldc = pl.P; g.coff = 0;
-    g.bias = pr->b_delta + l * P; g.epi = EPI_SOFTPLUS_BIAS;
-    AS_TRY(launch_gemm_simt(g, st));
-    g.epi = EPI_STORE; g.bias = nullptr; g.N = NS; g.C = reinterpret_cast<float*>(ws + pl.off_bc) + l * M * NBC; g.ldc = NBC;
-    g.Bm = (const char*)pr->W_B + l * NS * P * e; g.coff = 0;
-    AS_TRY(launch_gemm_simt(g, st));
-    g.Bm = (const char*)pr->W_C + l * NS * P * e; g.coff = NS;
-    AS_TRY(launch_gemm_simt(g, st));
-  }
+  AS_TRY(simt_projections(pl, pr, x, ws, st));
   return AS_OK;
-}
-
-int pick_splitk(int64_t tiles, int64_t K) {
-  int64_t s = ((int64_t)sm_count() * 4 + tiles - 1) / tiles;
-  const int64_t maxs = (K + 255) / 256;
-  if (s > maxs) s = maxs;
-  if (s < 1) s = 1;
-  if (s > 1024) s = 1024;
-  return (int)s;
 }
 
 // the net-VJPs: weight gradients (contractions over all tokens) and the input gradient, for every layer of the call
 int contractions(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const void* x, const as_grads_t* out, char* ws,
                  cudaStream_t st) {
-  const int bf = pl.io == AS_BF16;
-  const size_t e = bf ? 2 : 4;
-  const int64_t M = (int64_t)pl.Bg * pl.T;
-  const int P = pl.P;
   if (pl.tc) {
     AS_TRY(tc_weight_grads(pl, x, out, ws, st));
     mark(5, st);
@@ -114,44 +83,8 @@ int contractions(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const 
     mark(6, st);
     return AS_OK;
   }
-  for (int l = 0; l < pl.KL; ++l) {
-    const void* du = ws + pl.off_du + (size_t)l * M * pl.du_ld * e;
-    const float* dbc = reinterpret_cast<const float*>(ws + pl.off_dbc) + (size_t)l * M * NBC;
-    const void* xl = (const char*)x + (size_t)l * M * P * e;
-    // dW_delta[i,j] = sum_m du[m,i] x[m,j]
-    GemmArgs g{};
-    g.A = du; g.a_bf16 = bf; g.a_sm = 1; g.a_sk = P;
-    g.Bm = xl; g.b_bf16 = bf; g.b_sn = 1; g.b_sk = P;
-    g.C = out->dW_delta + (size_t)l * P * P; g.ldc = P; g.coff = 0; g.M = P; g.N = P; g.K = M; g.epi = EPI_ATOMIC;
-    g.splitk = pick_splitk((int64_t)((P + 63) / 64) * ((P + 63) / 64), M);
-    AS_TRY(launch_gemm_simt(g, st));
-    // dW_B, dW_C
-    g.A = dbc; g.a_bf16 = 0; g.a_sm = 1; g.a_sk = NBC; g.M = NS;
-    g.splitk = pick_splitk((P + 63) / 64, M);
-    g.C = out->dW_B + (size_t)l * NS * P;
-    AS_TRY(launch_gemm_simt(g, st));
-    g.A = dbc + NS; g.C = out->dW_C + (size_t)l * NS * P;
-    AS_TRY(launch_gemm_simt(g, st));
-  }
+  AS_TRY(simt_gradients(pl, pr, x, out, ws, st));   // both contractions in one launch: the second phase reads zero
   mark(5, st);
-  if (out->dx) {  // dx = dx_dir + du W_delta + dB W_B + dC W_C
-    for (int l = 0; l < pl.KL; ++l) {
-      const void* du = ws + pl.off_du + (size_t)l * M * pl.du_ld * e;
-      const float* dbc = reinterpret_cast<const float*>(ws + pl.off_dbc) + (size_t)l * M * NBC;
-      float* acc = reinterpret_cast<float*>(ws + pl.off_dxacc) + (size_t)l * M * P;
-      GemmArgs g{};
-      g.A = du; g.a_bf16 = bf; g.a_sm = P; g.a_sk = 1;
-      g.Bm = (const char*)pr->W_delta + (size_t)l * P * P * e; g.b_bf16 = bf; g.b_sn = 1; g.b_sk = P;
-      g.C = acc; g.ldc = P; g.coff = 0; g.M = M; g.N = P; g.K = P; g.epi = EPI_STORE; g.splitk = 1;
-      AS_TRY(launch_gemm_simt(g, st));
-      g.A = dbc; g.a_bf16 = 0; g.a_sm = NBC; g.a_sk = 1; g.K = NS; g.epi = EPI_ACCUM;
-      g.Bm = (const char*)pr->W_B + (size_t)l * NS * P * e;
-      AS_TRY(launch_gemm_simt(g, st));
-      g.A = dbc + NS; g.Bm = (const char*)pr->W_C + (size_t)l * NS * P * e;
-      AS_TRY(launch_gemm_simt(g, st));
-    }
-    AS_TRY(launch_finish_dx(pl, reinterpret_cast<const float*>(ws + pl.off_dxacc), ws + pl.off_dxdir, out->dx, st));
-  }
   mark(6, st);
   return AS_OK;
 }

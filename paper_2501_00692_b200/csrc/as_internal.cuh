@@ -99,7 +99,7 @@ struct Plan {
   int du_ld;        // row pitch (elements) of the du buffer: P, or P + 32 gsplit when it is the left part of Gcat = [du|dB|dC..]
   // byte offsets into the workspace
   size_t off_status, off_delta, off_bc, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
-      off_partd, off_hstart, off_carry, off_swin, off_du, off_dxdir, off_dbc, off_dxacc,
+      off_partd, off_hstart, off_carry, off_swin, off_du, off_dxdir, off_dbc,
       off_bptt_ckpt, off_wcat, off_wcatx, total_fwd, total_grad;
 };
 
@@ -108,18 +108,9 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl);
 inline int64_t a_stride(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }
 
 // ---- launchers (each returns a cudaError_t as int) ------------------------------------------
-// C[m, coff + n] (ldc) = epi( sum_k A(m,k) B(n,k) ), fp32 accumulation on the FP32 pipe.
-enum { EPI_STORE = 0, EPI_SOFTPLUS_BIAS = 1, EPI_ATOMIC = 2, EPI_ACCUM = 3 };
-struct GemmArgs {
-  const void* A; int a_bf16; int64_t a_sm, a_sk;   // element strides of A(m,k)
-  const void* Bm; int b_bf16; int64_t b_sn, b_sk;  // element strides of B(n,k)
-  float* C; int64_t ldc; int64_t coff;
-  const float* bias;
-  int64_t M; int N; int64_t K;
-  int epi;
-  int splitk;                                      // >1 only with EPI_ATOMIC
-};
-int launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
+// FP32-pipe contractions of fp32 I/O (as_gemm_simt.cu): projections, and the weight and input gradients in one launch
+int simt_projections(const Plan& pl, const as_params_t* pr, const void* x, char* ws, cudaStream_t st);
+int simt_gradients(const Plan& pl, const as_params_t* pr, const void* x, const as_grads_t* out, char* ws, cudaStream_t st);
 
 struct ScanPtrs {
   const void *x, *dy;
@@ -135,7 +126,6 @@ int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_
 int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st);   // the segment pass in the same form
 int launch_adjoint_main(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st);
 int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st);
-int launch_finish_dx(const Plan& pl, const float* dxacc, const void* dxdir, void* dx, cudaStream_t st);
 
 // bf16 tensor-core path (as_gemm_tc.cu)
 int tc_pack_wcat(int P, int layers, int reps, const as_params_t* pr, void* wcat, cudaStream_t st);

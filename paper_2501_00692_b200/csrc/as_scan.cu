@@ -79,7 +79,6 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.off_du = take(BT * (size_t)p.du_ld * e);
   p.off_dxdir = take(BTP * e);
   p.off_dbc = take(BT * NBC * 4);
-  p.off_dxacc = take(p.tc ? 256 : BTP * 4);
   p.off_bptt_ckpt = take((size_t)p.B * ((p.T + 63) / 64) * p.P * NS * 4);
   p.total_grad = o;
   *pl = p;
@@ -1176,13 +1175,6 @@ __global__ void wait_selftest_kernel(int* status, uint32_t limit) {
   if (bad && threadIdx.x == 0) atomicExch(status, AS_ERR_TIMEOUT);
 }
 
-template <typename IO>
-__global__ void finish_dx_kernel(int64_t n, const float* __restrict__ acc, const IO* __restrict__ dxdir,
-                                 IO* __restrict__ dx) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) st_io<IO>(dx + i, acc[i] + ld_io<IO>(dxdir + i));
-}
-
 // ---- tensor maps for the [B*T, P] activation tiles (box = CK tokens x bw channels, no swizzle) --------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1292,17 +1284,6 @@ int launch_adjoint_main(const Plan& pl, const ScanPtrs& sp, float* dA_log, float
 
 int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st) {
   wait_selftest_kernel<<<1, 32, 0, st>>>(status, limit);
-  count_launch();
-  return (int)cudaGetLastError();
-}
-
-int launch_finish_dx(const Plan& pl, const float* dxacc, const void* dxdir, void* dx, cudaStream_t st) {
-  const int64_t n = (int64_t)pl.B * pl.T * pl.P;
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  if (pl.io == AS_BF16)
-    finish_dx_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(n, dxacc, (const __nv_bfloat16*)dxdir, (__nv_bfloat16*)dx);
-  else
-    finish_dx_kernel<float><<<blocks, 256, 0, st>>>(n, dxacc, (const float*)dxdir, (float*)dx);
   count_launch();
   return (int)cudaGetLastError();
 }
