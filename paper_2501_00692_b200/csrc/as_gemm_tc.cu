@@ -43,7 +43,6 @@ struct TcArgs {
   int splitk;
   int P;                // d_model
   int wrows;            // rows of one layer's Wcat as stored (P + 32, or P + 96 with the three-term split)
-  int grp;              // DW: rows per reduce-add (16, or 8 where P is not a multiple of 16: no group straddles two outputs)
   int layers;           // independent problems stacked along the leading dimension of every tensor
   int64_t rows_layer;   // token rows per layer (a multiple of BM when layers > 1)
   const float* bias;    // PROJ: b_delta [layers, P]
@@ -166,7 +165,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 //                      buffer a while the issuer already fills buffer a^1 for the next tile
 // Tile order: n fastest, then m, then the K split, so concurrently running CTAs share A rows through L2.
 // ML: several layers stacked along the leading dimension of every tensor (false compiles the single-layer code).
-template <int AMAJ, int BMAJ, int EPI, int BN, bool ML>
+// OFF: P is not a multiple of 16 (the code for it costs the projections 10 % wherever it is compiled in).
+template <int AMAJ, int BMAJ, int EPI, int BN, bool ML, bool OFF>
 __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA,
                                                            const __grid_constant__ CUtensorMap tmB,
                                                            const __grid_constant__ CUtensorMap tmO0,
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
             tmem_ld16(tcol, r);
             if (lane == 0) bulk_wait_read<1>();         // the operation that last used this buffer has read it
             __syncwarp();
-            if (EPI == TC_PROJ && nb + CW > a.P && (a.P & 15)) {
+            if (EPI == TC_PROJ && OFF && nb + CW > a.P) {
               // the chunk that holds the border between Delta and [B | C], and those after it, where that border is no
               // multiple of 16: a TMA store would have to start left of the [B | C] rows, so those columns go out as
               // plain 16-byte stores of the lane's row
@@ -407,12 +407,12 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
             if (lane == 0) {
               if (EPI == TC_PROJ) {
                 if (nb < a.P) tma_store_2d(&tmO0, buf, nb, mrow);       // Delta
-                else if (!(a.P & 15)) tma_store_2d(&tmO1, buf, nb - a.P, mrow);   // [B | C]
+                else if (!OFF) tma_store_2d(&tmO1, buf, nb - a.P, mrow);   // [B | C]
               } else {
                 // rows of Gcat space: [0, P) dW_delta, then 16 rows dW_B and 16 rows dW_C (three such pairs with the
-                // split: their sums add up in the output); a group of grp rows never straddles two outputs
-#pragma unroll 1
-                for (int r0 = 0; r0 < 32; r0 += a.grp) {
+                // split: their sums add up in the output); a group of 16 (OFF: 8) rows never straddles two outputs
+#pragma unroll
+                for (int r0 = 0; r0 < 32; r0 += OFF ? 8 : 16) {
                   const int mr = mrow + r0, e = mr - a.P;
                   const void* src = buf + r0 * 64;
                   const int l1 = ML ? lay * a.P : 0, l2 = ML ? lay * NS : 0;   // this layer's rows of the stacked outputs
@@ -523,9 +523,9 @@ int make_map_out_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t
   return make_map_t(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, CU_TENSOR_MAP_SWIZZLE_64B, base, rows, cols, cols, 32, 32);
 }
 
-template <int AMAJ, int BMAJ, int EPI, int BN, bool ML>
+template <int AMAJ, int BMAJ, int EPI, int BN, bool ML, bool OFF>
 int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const TcArgs& a, cudaStream_t st) {
-  auto kern = gemm_tc_kernel<AMAJ, BMAJ, EPI, BN, ML>;
+  auto kern = gemm_tc_kernel<AMAJ, BMAJ, EPI, BN, ML, OFF>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, Cfg<BN>::SMEM_DYN, done)) return 1;
   const int64_t ntiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * (EPI == TC_DW ? a.layers : 1);
@@ -538,8 +538,11 @@ int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorM
 
 template <int AMAJ, int BMAJ, int EPI, int BN>
 int launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const TcArgs& a, cudaStream_t st) {
-  return a.layers > 1 ? launch_tc_ml<AMAJ, BMAJ, EPI, BN, true>(tmA, tmB, tmO, a, st)
-                      : launch_tc_ml<AMAJ, BMAJ, EPI, BN, false>(tmA, tmB, tmO, a, st);
+  if (EPI != TC_DX && a.P % 16)   // the input gradient has no border inside a chunk
+    return a.layers > 1 ? launch_tc_ml<AMAJ, BMAJ, EPI, BN, true, EPI != TC_DX>(tmA, tmB, tmO, a, st)
+                        : launch_tc_ml<AMAJ, BMAJ, EPI, BN, false, EPI != TC_DX>(tmA, tmB, tmO, a, st);
+  return a.layers > 1 ? launch_tc_ml<AMAJ, BMAJ, EPI, BN, true, false>(tmA, tmB, tmO, a, st)
+                      : launch_tc_ml<AMAJ, BMAJ, EPI, BN, false, false>(tmA, tmB, tmO, a, st);
 }
 
 }  // namespace
@@ -577,7 +580,7 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int 
     if (make_map(&tmA, (const char*)x + (size_t)l0 * rows * P * 2, M, P, P, BM)) return 1;
     if (make_map(&tmB, (const char*)wcat + (size_t)l0 * NW * P * 2, (uint64_t)NW * nl, P, P, PBN)) return 1;
     TcArgs a{};
-    a.M = M; a.N = P + NBC; a.kblocks = (P + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.grp = 16; a.layers = nl; a.rows_layer = rows;
+    a.M = M; a.N = P + NBC; a.kblocks = (P + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.layers = nl; a.rows_layer = rows;
     a.bias = pr->b_delta + (size_t)l0 * P;
     a.bc = (float*)(ws + pl.off_bc) + (size_t)l0 * rows * NBC;
     a.status = (int*)(ws + pl.off_status);
@@ -608,7 +611,7 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
     if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, rows * nl, NW, NW, 64)) return 1;   // Gcat as [K=tokens, M]
     if (make_map(&tmB, (const char*)x + (size_t)l0 * rows * P * 2, rows * nl, P, P, 64)) return 1;       // X as [K=tokens, N=P]
     TcArgs a{};
-    a.M = NW; a.N = P; a.kblocks = (int)((rows + BK - 1) / BK); a.P = P; a.wrows = NW; a.grp = P % 16 ? 8 : 16;
+    a.M = NW; a.N = P; a.kblocks = (int)((rows + BK - 1) / BK); a.P = P; a.wrows = NW;
     a.layers = nl; a.rows_layer = rows;
     const int tiles = ((NW + BM - 1) / BM) * ((P + TBN - 1) / TBN) * nl;
     int sk = sm_count() / tiles;   // about one tile per persistent CTA (two measured 3 % slower at C3: more reduce-adds)
@@ -618,9 +621,9 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
     a.splitk = (a.kblocks + kper - 1) / kper;   // no empty split: every tile has at least one K block
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
-    if (make_map_out_f32(&tmO[0], out->dW_delta + (size_t)l0 * P * P, (uint64_t)P * nl, P, (uint32_t)a.grp)) return 1;
-    if (make_map_out_f32(&tmO[1], out->dW_B + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, (uint32_t)a.grp)) return 1;
-    if (make_map_out_f32(&tmO[2], out->dW_C + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, (uint32_t)a.grp)) return 1;
+    if (make_map_out_f32(&tmO[0], out->dW_delta + (size_t)l0 * P * P, (uint64_t)P * nl, P, P % 16 ? 8 : 16)) return 1;
+    if (make_map_out_f32(&tmO[1], out->dW_B + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, P % 16 ? 8 : 16)) return 1;
+    if (make_map_out_f32(&tmO[2], out->dW_C + (size_t)l0 * NS * P, (uint64_t)NS * nl, P, P % 16 ? 8 : 16)) return 1;
     const int e = launch_tc<MAJ_MN, MAJ_MN, TC_DW, TBN>(tmA, tmB, tmO, a, st);
     if (e) return e;
   }
@@ -639,7 +642,7 @@ int tc_input_grad(const Plan& pl, const void* wcat, void* dx, char* ws, cudaStre
     if (make_map(&tmA, ws + pl.off_du + (size_t)l0 * rows * NW * 2, M, NW, NW, BM)) return 1;            // Gcat as [M=tokens, K]
     if (make_map(&tmB, (const char*)wcat + (size_t)l0 * NW * P * 2, (uint64_t)NW * nl, P, P, 64)) return 1;   // Wcat as [K, N=P]
     TcArgs a{};
-    a.M = M; a.N = P; a.kblocks = (NW + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.grp = 16; a.layers = nl; a.rows_layer = rows;
+    a.M = M; a.N = P; a.kblocks = (NW + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.layers = nl; a.rows_layer = rows;
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
     if (make_map_out_bf16(&tmO[0], (char*)dx + (size_t)l0 * rows * P * 2, M, P)) return 1;
