@@ -1,0 +1,690 @@
+// Main adjoint kernel: per segment, the reverse cotangent recurrence with the exact window exit, the per-token
+// vector-Jacobian products and their sums.
+//
+// Thread mapping: as in the ascending kernels a thread owns two channels (pair k) and eight of their 16 states (lane parity
+// `half`), but here the two CHANNELS of a state share a packed register pair.  The staged Delta, x and dy rows then are
+// packed operands as they lie, sums over states end with both channels' sums in one pair, and only B_t and C_t, which all
+// channels share, are needed twice: the pre-pass leaves them doubled, (B_n, B_n), in a buffer of their own.
+//
+// Bound: dispatch of the arithmetic pipes, with MUFU.EX2 next (3 warps per scheduler; each token costs a warp about 320
+// instructions for 512 state-steps).  Measured at C3 sizes (2 x 65,536 tokens, 768 channels): full form 1.50 -> 1.39 ms
+// against packing the states of a channel, whose (Delta, Delta), (x, x), (dy, dy) pairs, finalisation of every token by
+// both lanes and separate abar h product cost more.  Tried on the way and slower: sums over channels by a shuffle
+// butterfly with lane-dependent state order (1.56 against 1.43 ms), warps that meet only at mbarriers (+4 %: in step, the
+// four schedulers share the instruction cache), the token loop unrolled 4 and 8 times (+3 %, +12 %).
+#include "as_scan.cuh"
+
+namespace as {
+namespace {
+
+constexpr int MAIN_CTAS = 3;     // resident CTAs per SM the kernel is compiled for (up to 168 registers per thread)
+constexpr int WRED_Q = 32 * 4 + 8;   // floats per quarter-block of the per-warp reduction scratch (512 B + 32 B skew)
+constexpr int NSU = 8;           // states (slots) of a thread: one (channel 0, channel 1) pair each
+
+// ---- tensor memory as a per-thread scratchpad ------------------------------------------------------
+// The kernel runs no MMA, so the SM's tensor memory is free.  Each CTA allocates 128 of the 512 columns of its SM (three
+// CTAs are resident) and every thread parks the state before each of the chunk's eight tokens in its own TMEM lane:
+// warp w of the 4-warp CTA owns lanes [32w, 32w+32), a 32x32b access moves 16 registers of each lane to or from 16
+// consecutive columns.  The state after the last token stays in registers.
+constexpr int TM_TOK = 16;             // columns per token
+constexpr int TM_COLS = CK * TM_TOK;   // columns [16 j, 16 j + 16): state before token j of the current chunk
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const u64 (&v)[NSU]) {
+  uint32_t r[16];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) asm("mov.b64 {%0, %1}, %2;" : "=r"(r[2 * u]), "=r"(r[2 * u + 1]) : "l"(v[u]));
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// asynchronous load; the registers may be read after tmem_wait_ld on the same array, which passes them through
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16], u64 (&v)[NSU]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+#pragma unroll
+  for (int u = 0; u < 8; ++u) asm("mov.b64 %0, {%1, %2};" : "=l"(v[u]) : "r"(r[2 * u]), "r"(r[2 * u + 1]));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// lo * lo + hi * hi: two scalar operations take as long as one packed one, and save the addition
+__device__ __forceinline__ float dot2(u64 a, u64 b) {
+  float al, ah, bl, bh;
+  upk(a, al, ah);
+  upk(b, bl, bh);
+  return fmaf(ah, bh, al * bl);
+}
+// the channel pair of a staged row, from a pointer that already addresses it
+template <typename IO> __device__ __forceinline__ u64 lds_pair(const uint8_t* p);
+template <> __device__ __forceinline__ u64 lds_pair<float>(const uint8_t* p) { return *reinterpret_cast<const u64*>(p); }
+template <> __device__ __forceinline__ u64 lds_pair<__nv_bfloat16>(const uint8_t* p) {
+  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
+  return pk(t.x, t.y);
+}
+// The thread's 16 values inside a tile block of the scan kernels, regrouped: slot u is state u (of the thread's eight) of
+// both channels.  Block order: pair iu = 2 q + e of scan thread tid at ((q * NTHR + tid) * 2 + e), pair 4 ch + m holding
+// states 2m, 2m+1 of channel ch.
+__device__ __forceinline__ void load_slots(const u64* blk, int tid, u64 (&v)[NSU]) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int at = ((m >> 1) * NTHR + tid) * 2 + (m & 1);
+    float a0, a1, b0, b1;
+    upk(blk[at], a0, a1);
+    upk(blk[at + 2 * NTHR * 2], b0, b1);
+    v[2 * m] = pk(a0, b0);
+    v[2 * m + 1] = pk(a1, b1);
+  }
+}
+// sigmoid(u) = 1 - exp(-Delta).  bf16 outputs: the direct form (absolute error 2e-7) above Delta = 1/32, three series terms
+// below (relative error < 2e-6; written so that no operation needs two constants, each of which would cost a move);
+// fp32 outputs use the longer cancellation-free form.
+template <int ESZ> __device__ __forceinline__ float sigmoid_of(float d) {
+  if (ESZ == 4) return sig_from_delta(d);
+  const float small = d * fmaf(d, __fadd_rn(__fmul_rn(d, 1.f / 6.f), -0.5f), 1.f);
+  return d < 0.03125f ? small : 1.f - ex2_approx(-d * LOG2E);
+}
+template <typename IO> __device__ __forceinline__ void st_pair(uint8_t* p, float a, float b);
+template <> __device__ __forceinline__ void st_pair<float>(uint8_t* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+template <> __device__ __forceinline__ void st_pair<__nv_bfloat16>(uint8_t* p, float a, float b) {
+  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
+}
+// abar for the slots from the channel pair's exponent scales.  With a scalar rate the states of a channel share one factor.
+template <bool SC>
+__device__ __forceinline__ void decay_slots(u64 e2, const u64 (&A2)[NSU], u64 (&a)[NSU]) {
+  if (SC) {
+    const u64 ac = ex2_2(mul2(e2, A2[0]));
+#pragma unroll
+    for (int u = 0; u < NSU; ++u) a[u] = ac;
+  } else {
+#pragma unroll
+    for (int u = 0; u < NSU; ++u) a[u] = ex2_2(mul2(e2, A2[u]));
+  }
+}
+
+// shared memory: staged chunk (TMA / bulk copies), two stages
+constexpr int DBC_ROW = 2 * NS * 4;   // one token's (B_n, B_n) x 16 or (C_n, C_n) x 16
+template <int ESZ, bool WIN>
+struct StageM {
+  // a chunk takes thousands of cycles: one chunk of look-ahead suffices, and with fp32 rows and window rows even that would
+  // leave room for two CTAs per SM instead of three, which hide the copies better (C2: 94 -> 71 us)
+  static constexpr int N = WIN && ESZ == 4 ? 1 : 2;
+  static constexpr int X = 0;
+  static constexpr int D = X + CK * CH * ESZ;
+  static constexpr int G = D + CK * CH * 4;
+  static constexpr int BC = G + CK * CH * ESZ;
+  static constexpr int CC = BC + CK * DBC_ROW;
+  static constexpr int CS = CC + CK * DBC_ROW;
+  static constexpr int G2 = CS + CH * 4;
+  static constexpr int D2 = G2 + (WIN ? CK * CH * ESZ : 0);
+  static constexpr int CC2 = D2 + (WIN ? CK * CH * 4 : 0);
+  static constexpr int BYTES = CC2 + (WIN ? CK * DBC_ROW : 0);
+};
+struct WinS { double sw[NCH]; float2 a2max; };   // window bookkeeping of a thread, out of the walk's registers
+// behind the stages: the chunk checkpoint, the output tiles [warp][du, dx_dir][CK][32 channels], the per-token [dB | dC] sums of
+// each warp (two chunks in flight), the per-warp scratch of the channel reduction, the true segment-start state, the window
+// bookkeeping, mbarriers.  All of it dynamic: the walk is compiled as a function of its own (see adjoint_main_kernel).
+template <int ESZ, bool WIN> struct MainCfg {
+  static constexpr int CKP = StageM<ESZ, WIN>::N * StageM<ESZ, WIN>::BYTES;
+  static constexpr int OUT = CKP + TILE_FLOATS * 4;
+  static constexpr int OUT_TILE = CK * 32 * ESZ;
+  static constexpr int RED = OUT + (NTHR / 32) * 2 * OUT_TILE;
+  static constexpr int WRED = RED + 2 * (NTHR / 32) * CK * NBC * 4;
+  static constexpr int HST = WRED + (NTHR / 32) * 4 * WRED_Q * 4;
+  static constexpr int WINS = HST + NSU / 2 * NTHR * 16;
+  static constexpr int BARS = WINS + (WIN ? NTHR * (int)sizeof(WinS) : 0);
+  static constexpr int SMEM_DYN = BARS + 64 + 128;
+};
+
+// ------------------------------------------------------------------------------------------------
+// One CTA per (channel tile, segment, batch element), chunks walked last to first.  Per chunk: rebuild the states from the
+// chunk checkpoint and park them in tensor memory, then walk the tokens backwards: mu recurrence (with the exact window
+// exit), the per-token vector-Jacobian products, the channel sums dB_t / dC_t, and the per-channel outputs du_t and dx_dir_t
+// (collected in shared memory, stored by TMA once per chunk).
+// FULL: full form.  WIN: with the window-exit terms (truncated form, segments where they can matter).
+// ------------------------------------------------------------------------------------------------
+template <typename IO, bool FULL, bool WIN, bool SC>
+__device__ __forceinline__ void adjoint_segment(const CUtensorMap& tmX, const CUtensorMap& tmD, const CUtensorMap& tmG,
+                                                const CUtensorMap& tmDu, const CUtensorMap& tmDx, const Plan& pl,
+                                                const float* __restrict__ A_log, char* __restrict__ ws,
+                                                float* __restrict__ dA_log, float* __restrict__ db_delta) {
+  static_assert(NCH == 2 && NTHR == 128, "tensor-memory parking assumes 4 warps and 16 state registers per thread");
+  constexpr int ESZ = IoSz<IO>::v;
+  using St = StageM<ESZ, !FULL>;
+  using Cf = MainCfg<ESZ, !FULL>;
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);   // stays a shared-space pointer
+  constexpr int NST = St::N;
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + Cf::BARS);   // [NST]: the stage's copies have landed
+  uint64_t* ckp_bar = full_bar + NST;                          // the checkpoint tile has landed
+  uint64_t* ckp_free = ckp_bar + 1;                                    // every warp has read it
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(ckp_free + 1);
+  typedef float Red[NTHR / 32][CK][NBC];
+  Red* red = reinterpret_cast<Red*>(smem + Cf::RED);
+  ulonglong2* hst_s = reinterpret_cast<ulonglong2*>(smem + Cf::HST) + threadIdx.x;   // [NSU / 2], NTHR apart
+  WinS* win_s = reinterpret_cast<WinS*>(smem + Cf::WINS) + threadIdx.x;
+
+  const int tile = blockIdx.x, s = blockIdx.y, b = blockIdx.z;
+  const int P = pl.P;
+  const Who w = who(tile, P);
+  const int lane = w.tid & 31, warp = w.tid >> 5;
+  const int64_t T = pl.T, tbar = pl.tbar;
+  const int64_t t0 = (int64_t)s * pl.L;
+  const int64_t t1 = min(T, t0 + pl.L);
+  const int nchunk = (int)((t1 - t0 + CK - 1) / CK);
+  const float* bcd = reinterpret_cast<const float*>(ws + pl.off_bcd);   // doubled B rows, then doubled C rows
+  const int64_t cplane = ((int64_t)pl.B * pl.T + CK) * NBC;
+  const float* ckpt = reinterpret_cast<const float*>(ws + pl.off_ckpt);
+  const float* cs = reinterpret_cast<const float*>(ws + pl.off_cs);
+  float* dbc = reinterpret_cast<float*>(ws + pl.off_dbc);
+  int* status = reinterpret_cast<int*>(ws + pl.off_status);
+  const int ncs = min(CH, P - tile * CH);   // channels of this tile that exist
+  const int64_t BT = (int64_t)pl.B * T;
+  const int64_t grow0 = (int64_t)(b % pl.Bg) * T - (int64_t)b * T;   // added to an x / Delta row to get the dy row
+  const int chf = w.half;
+
+  // rates: slot u is state 8 half + u
+  u64 A2[NSU];
+  {
+    float mx[NCH] = {-3.0e38f, -3.0e38f};   // least negative exponent scale of each channel over all 16 states
+#pragma unroll
+    for (int u = 0; u < NSU; ++u) {
+      float a[NCH] = {0.f, 0.f};
+      if (w.act) {
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+          a[c] = -__expf(__ldg(A_log + (pl.scalar ? (int64_t)(w.pa + c) : (int64_t)(w.pa + c) * NS + 8 * w.half + u))) * LOG2E;
+          mx[c] = fmaxf(mx[c], a[c]);
+        }
+      }
+      A2[u] = pk(a[0], a[1]);
+    }
+    if (WIN) {
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) mx[c] = fmaxf(mx[c], __shfl_xor_sync(0xffffffffu, mx[c], 1));
+      win_s->a2max = make_float2(mx[0], mx[1]);
+    }
+  }
+
+  if (w.tid == 0) {
+    for (int i = 0; i < NST; ++i) mbar_init(&full_bar[i], 1);
+    mbar_init(ckp_bar, 1);
+    mbar_init(ckp_free, NTHR / 32);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)), "n"(TM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tm = *tmem_base_s + ((uint32_t)(32 * warp) << 16);   // this warp's lanes, column 0 of the allocation
+
+  const uint32_t tx_base = (uint32_t)(CK * CH * ESZ * 2 + CK * CH * 4 + 2 * CK * DBC_ROW + ncs * 4 +
+                                      (WIN ? CK * CH * ESZ + CK * CH * 4 : 0));
+  // chunks are visited last to first: the i-th visited chunk is c = nchunk-1-i
+  auto chunk_t = [&](int i) { return t0 + (int64_t)(nchunk - 1 - i) * CK; };
+  auto issue = [&](int i) {
+    const int st = i % NST;
+    uint8_t* sm = smem + st * St::BYTES;
+    const int64_t tc = chunk_t(i);
+    const int64_t row = (int64_t)b * T + tc;
+    const int64_t cc = (int64_t)b * pl.NC + tc / CK;
+    const int64_t row2 = row + tbar;             // first token leaving the window of this chunk's tokens
+    const bool win_rows = WIN && row2 < BT;      // its C rows exist (else no token of the chunk has t + Tbar < T)
+    mbar_expect_tx(&full_bar[st], tx_base + (win_rows ? CK * DBC_ROW : 0));
+    tma_2d(sm + St::X, &tmX, tile * CH, row, &full_bar[st]);
+    tma_2d(sm + St::D, &tmD, tile * CH, row, &full_bar[st]);
+    tma_2d(sm + St::G, &tmG, tile * CH, row + grow0, &full_bar[st]);
+    bulk_1d(sm + St::BC, bcd + row * NBC, CK * DBC_ROW, &full_bar[st]);
+    bulk_1d(sm + St::CC, bcd + cplane + row * NBC, CK * DBC_ROW, &full_bar[st]);
+    bulk_1d(sm + St::CS, cs + cc * P + tile * CH, ncs * 4, &full_bar[st]);
+    if (WIN) {
+      // rows of the tokens leaving the window; rows past the sequence end (t + Tbar >= T) are not looked at below
+      tma_2d(sm + St::G2, &tmG, tile * CH, row2 + grow0, &full_bar[st]);
+      tma_2d(sm + St::D2, &tmD, tile * CH, row2, &full_bar[st]);
+      if (win_rows) bulk_1d(sm + St::CC2, bcd + cplane + row2 * NBC, CK * DBC_ROW, &full_bar[st]);
+    }
+  };
+  auto issue_ckp = [&](int i) {   // checkpoint tile of the i-th visited chunk (single buffer)
+    const int64_t cc = (int64_t)b * pl.NC + chunk_t(i) / CK;
+    mbar_expect_tx(ckp_bar, TILE_FLOATS * 4);
+    bulk_1d(smem + Cf::CKP, ckpt + (cc * pl.tiles + tile) * TILE_FLOATS, TILE_FLOATS * 4, ckp_bar);
+  };
+  if (w.tid == 0) {
+    for (int i = 0; i < NST && i < nchunk; ++i) issue(i);
+    issue_ckp(0);
+  }
+  if (t1 == T && T % CK != 0) {   // CTA-uniform: the first visited chunk sticks out past the sequence end: its rows there become zeros
+    const bool ok = mbar_wait(&full_bar[0], 0);
+    if (ok) {
+      const int nt = (int)(T % CK);
+      zero_rows(smem + St::D, CH * 4, nt, w.tid);
+      zero_rows(smem + St::G, CH * ESZ, nt, w.tid);
+      zero_rows(smem + St::BC, DBC_ROW, nt, w.tid);
+      zero_rows(smem + St::CC, DBC_ROW, nt, w.tid);
+    }
+    __syncthreads();
+  }
+
+  u64 mu[NSU], dAacc[NSU];
+  const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
+#pragma unroll
+  for (int u = 0; u < NSU; ++u) { mu[u] = 0ull; dAacc[u] = 0ull; }
+  if (s + 1 < pl.S) {
+    // what the segment's reverse recurrence starts from: suffix of the block that holds segment s + 1, prefix of the next
+    // block up to segment s + m, and the first r tokens of segment s + m + 1 (see the carry kernel); for windows of a few
+    // segments their Horner sum right here
+    const int s1 = s + 1, m = pl.m, last = min(s + m, pl.S - 1);
+    const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd) + (int64_t)b * pl.S * P + w.pa;
+    const double* tot = reinterpret_cast<const double*>(ws + pl.off_total) + (int64_t)b * pl.S * P + w.pa;
+    double sw[NCH] = {0.0, 0.0};   // Delta sum of the window that starts after the segment's last token
+    auto block = [&](size_t off, int sg) {
+      return reinterpret_cast<const u64*>(ws + off) + (((int64_t)b * pl.S + sg) * pl.tiles + tile) * (TILE_FLOATS / 2);
+    };
+    if (FULL) {
+      load_slots(block(pl.off_suf, s1), w.tid, mu);
+    } else {
+      const float* partd = reinterpret_cast<const float*>(ws + pl.off_partd) + ((int64_t)b * pl.S + s1 + m) * P + w.pa;
+      const bool part = s1 + m < pl.S;
+      if (pl.direct) {
+        if (part) load_slots(block(pl.off_mupart, s1 + m), w.tid, mu);
+        for (int sg = last; sg > s; --sg) {
+          float d[NCH];
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) {
+            d[c] = w.act ? __ldg(segd + (int64_t)sg * P + c) : 0.f;
+            sw[c] += (double)d[c];
+          }
+          u64 dec[NSU], v[NSU];
+          decay_slots<SC>(pk(d[0], d[1]), A2, dec);
+          load_slots(block(pl.off_muloc, sg), w.tid, v);
+#pragma unroll
+          for (int u = 0; u < NSU; ++u) mu[u] = fma2(dec[u], mu[u], v[u]);
+        }
+      } else {
+        auto add = [&](size_t off, int sg, int upto) {   // mu += exp(A * Delta of segments s+1 .. upto) * block
+          float d[NCH] = {0.f, 0.f};
+          if (w.act)
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) d[c] = (float)(tot[(int64_t)upto * P + c] - tot[(int64_t)s * P + c]);
+          u64 dec[NSU], v[NSU];
+          decay_slots<SC>(pk(d[0], d[1]), A2, dec);
+          load_slots(block(off, sg), w.tid, v);
+#pragma unroll
+          for (int u = 0; u < NSU; ++u) mu[u] = fma2(dec[u], v[u], mu[u]);
+        };
+        const int be = (s1 / m + 1) * m - 1;
+        load_slots(block(pl.off_suf, s1), w.tid, mu);
+        if (last > be) add(pl.off_pre, last, be);
+        if (part) add(pl.off_mupart, s1 + m, last);
+        if (w.act)
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) sw[c] = tot[(int64_t)last * P + c] - tot[(int64_t)s * P + c];
+      }
+      if (part && w.act)
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) sw[c] += (double)__ldg(partd + c);
+    }
+    if (WIN)
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) win_s->sw[c] = sw[c];
+  } else if (WIN) {
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) win_s->sw[c] = 0.0;
+  }
+  {   // true segment-start state: parked in shared memory, read back once per chunk
+    u64 hst[NSU];
+    load_slots(reinterpret_cast<const u64*>(ws + pl.off_hstart) + sb * (TILE_FLOATS / 2), w.tid, hst);
+#pragma unroll
+    for (int q = 0; q < NSU / 2; ++q) hst_s[q * NTHR] = make_ulonglong2(hst[2 * q], hst[2 * q + 1]);
+  }
+  float dbacc0 = 0.f, dbacc1 = 0.f;   // db_delta of the two channels over this lane's tokens
+  bool failed = false;
+  int fail_i = 0, ckp_issued = 0;     // thread 0: where the walk stopped, last checkpoint copy issued
+
+  for (int i = 0; i < nchunk; ++i) {
+    const int rb = i & 1;
+    uint8_t* sm = smem + (i % NST) * St::BYTES;
+    bool ok = mbar_wait(&full_bar[i % NST], (i / NST) & 1);
+    ok = mbar_wait(ckp_bar, i & 1) && ok;
+    ok = __all_sync(0xffffffffu, ok);   // warp-uniform: the tensor-memory accesses below are warp-collective
+    const int64_t tc = chunk_t(i);
+    const int nt = (int)min((int64_t)CK, t1 - tc);
+    const int nwin = WIN ? (int)max((int64_t)0, min((int64_t)CK, T - tbar - tc)) : 0;   // tokens j < nwin have t + Tbar < T
+    // window Delta sum: fp64 value at the chunk's last token + an fp32 running offset inside the chunk
+    u64 swl = 0ull, swc = 0ull;
+    bool chunk_live = false;   // warp-uniform: does any exit factor W of this chunk reach 2^-64 ?
+    uint8_t* const out = smem + Cf::OUT + warp * 2 * Cf::OUT_TILE;   // du; dx_dir one tile on
+    if (ok) {
+      // state at the chunk start: local checkpoint + decayed true segment-start state
+      u64 h[NSU];
+      load_slots(reinterpret_cast<const u64*>(smem + Cf::CKP), w.tid, h);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ckp_free);   // this warp is done with the checkpoint buffer
+      {
+        const u64 csv = w.act ? *reinterpret_cast<const u64*>(sm + St::CS + 8 * w.k) : 0ull;   // the 1D copy covers existing channels
+        u64 dec[NSU];
+        decay_slots<SC>(csv, A2, dec);
+#pragma unroll
+        for (int q = 0; q < NSU / 2; ++q) {
+          const ulonglong2 hq = hst_s[q * NTHR];
+          h[2 * q] = fma2(dec[2 * q], hq.x, h[2 * q]);
+          h[2 * q + 1] = fma2(dec[2 * q + 1], hq.y, h[2 * q + 1]);
+        }
+      }
+      if (WIN) {
+        // Delta of the tokens leaving the window during this chunk.  Inside the chunk the window sum never drops
+        // below (sum at the chunk's last token) - (their total), so if even that bound gives W < 2^-64 for every
+        // state of every lane, the exit terms of the whole chunk are skipped: they are far below one rounding unit
+        // of mu.  The decision is taken once per chunk and per warp.
+        u64 sd = 0ull, sd2 = 0ull;
+#pragma unroll
+        for (int j = 0; j < CK; ++j) {
+          sd = add2(sd, lds_pair<float>(sm + St::D + j * CH * 4 + 8 * w.k));
+          const u64 d2v = lds_pair<float>(sm + St::D2 + j * CH * 4 + 8 * w.k);
+          if (j < nwin) sd2 = add2(sd2, d2v);
+        }
+        float d0, d1, e0, e1;
+        upk(sd, d0, d1);
+        upk(sd2, e0, e1);
+        const double s0 = win_s->sw[0], s1 = win_s->sw[1];
+        const float2 am = win_s->a2max;
+        swc = pk((float)s0, (float)s1);
+        win_s->sw[0] = s0 + (double)(d0 - e0);   // window sum at the previous chunk's last token
+        win_s->sw[1] = s1 + (double)(d1 - e1);
+        const bool live = ((float)s0 - e0) * am.x > -64.f || ((float)s1 - e1) * am.y > -64.f;
+        chunk_live = __any_sync(0xffffffffu, live && w.act && nwin > 0);
+      }
+      const uint8_t* pB = sm + St::BC + 64 * w.half;   // this thread's slots in the doubled B row of the chunk's first token
+      // forward rebuild: the states before the chunk's tokens go to tensor memory, the one after the last stays
+#pragma unroll
+      for (int j = 0; j < CK; ++j) {
+        tmem_st16(tm + TM_TOK * j, h);
+        const u64 d2 = lds_pair<float>(sm + St::D + j * CH * 4 + 8 * w.k);
+        const u64 dx2 = mul2(d2, lds_pair<IO>(sm + St::X + j * CH * ESZ + 2 * ESZ * w.k));
+        u64 af = 0ull;
+        if (SC) af = ex2_2(mul2(d2, A2[0]));   // scalar rate: one factor for the channel's states
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const ulonglong2 bq = *reinterpret_cast<const ulonglong2*>(pB + j * DBC_ROW + 16 * m);
+          h[2 * m] = fma2(SC ? af : ex2_2(mul2(d2, A2[2 * m])), h[2 * m], mul2(dx2, bq.x));
+          h[2 * m + 1] = fma2(SC ? af : ex2_2(mul2(d2, A2[2 * m + 1])), h[2 * m + 1], mul2(dx2, bq.y));
+        }
+      }
+      tmem_wait_st();
+      if (w.tid == 0 && i + 1 < nchunk) {   // every warp has the checkpoint in registers by now: fetch the next chunk's
+        if (mbar_wait(ckp_free, i & 1)) { issue_ckp(i + 1); ckp_issued = i + 1; }
+        else ok = false;
+      }
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the last chunk's stores have read the tile
+      __syncwarp();
+      // backward walk; row pointers walk down with the tokens, two at a time: lane `half` of a channel pair finalises token
+      // 2 jp + 1 - half for both channels
+      const uint8_t* pD = sm + St::D + (CK - 1) * CH * 4 + 8 * w.k;               // Delta row (fp32)
+      const uint8_t* pX = sm + St::X + (CK - 1) * CH * ESZ + 2 * ESZ * w.k;       // x row; dy row at + (St::G - St::X)
+      pB += (CK - 1) * DBC_ROW;
+      uint8_t* pO = out + (CK - 1 - w.half) * 32 * ESZ + 2 * ESZ * (lane >> 1);
+      const uint8_t* pDo = pD - w.half * CH * 4;
+      const uint8_t* pXo = pX - w.half * CH * ESZ;
+      float* pR = &red[rb][warp][CK - 1][((lane >> 1) & 8) * 2 + 8 * w.half + ((lane >> 1) & 7)];
+      float* wred = reinterpret_cast<float*>(smem + Cf::WRED) + warp * 4 * WRED_Q;
+      const float* rd = wred + (lane >> 3) * WRED_Q + w.half * 4 + ((lane >> 1) & 3);
+      uint32_t tmj = tm + TM_TOK * (CK - 1);
+#pragma unroll 1
+      for (int jp = CK / 2 - 1; jp >= 0; --jp) {
+        u64 sk[2], dk[2];   // state sums of the two tokens
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+          const int j = 2 * jp + 1 - o;
+          const u64 d2 = lds_pair<float>(pD - o * CH * 4);
+          const u64 x2 = lds_pair<IO>(pX - o * CH * ESZ);
+          const u64 g2 = lds_pair<IO>(pX + (St::G - St::X) - o * CH * ESZ);
+          const u64 dx2 = mul2(d2, x2);
+          float vB[NSU], vC[NSU];
+          // dC: h is the state after this token
+#pragma unroll
+          for (int u = 0; u < NSU; ++u) vC[u] = dot2(g2, h[u]);
+          uint32_t hr[16];
+          tmem_ld16(tmj - o * TM_TOK, hr);   // the state before it, needed at the end of the token
+          // mu_i += g_i C_i   (mu already carries abar_{i+1} mu_{i+1})
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const ulonglong2 cq = *reinterpret_cast<const ulonglong2*>(pB + (St::CC - St::BC) + 16 * m - o * DBC_ROW);
+            mu[2 * m] = fma2(g2, cq.x, mu[2 * m]);
+            mu[2 * m + 1] = fma2(g2, cq.y, mu[2 * m + 1]);
+          }
+          if (WIN && chunk_live && j >= nwin) swl = add2(swl, d2);   // no token leaves: the window only grows towards t-1
+          if (WIN && chunk_live && j < nwin) {
+            // exact exit of token t2 = t + Tbar from the window: subtract W_i gC_{t2}, W_i = exp(A * sum_{j=i+1..t2} Delta_j)
+            const u64 d2v = lds_pair<float>(pD + (St::D2 - St::D) - o * CH * 4);
+            const u64 ng2 = mul2(lds_pair<IO>(pX + (St::G2 - St::X) - o * CH * ESZ), pk(-1.f, -1.f));
+            const u64 sw2 = add2(swc, swl);
+            swl = add2(swl, fma2(d2v, pk(-1.f, -1.f), d2));   // window of token t-1: (t-1, t-1+Tbar]
+            u64 wf[NSU];
+            decay_slots<SC>(sw2, A2, wf);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const ulonglong2 cq = *reinterpret_cast<const ulonglong2*>(pB + (St::CC2 - St::BC) + 16 * m - o * DBC_ROW);
+              mu[2 * m] = fma2(wf[2 * m], mul2(ng2, cq.x), mu[2 * m]);
+              mu[2 * m + 1] = fma2(wf[2 * m + 1], mul2(ng2, cq.y), mu[2 * m + 1]);
+            }
+          }
+          u64 sacc = 0ull, dacc = 0ull;
+          {
+            u64 af = 0ull;
+            if (SC) af = ex2_2(mul2(d2, A2[0]));
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const ulonglong2 bq = *reinterpret_cast<const ulonglong2*>(pB + 16 * m - o * DBC_ROW);
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const int u = 2 * m + e;
+                vB[u] = dot2(mu[u], dx2);                                            // dB partial (two channels)
+                sacc = u == 0 ? mul2(mu[u], bq.x) : fma2(mu[u], e ? bq.y : bq.x, sacc);
+                mu[u] = mul2(mu[u], SC ? af : ex2_2(mul2(d2, A2[u])));               // ready for token i-1
+              }
+            }
+          }
+          tmem_wait_ld(hr, h);   // h_{i-1}
+#pragma unroll
+          for (int u = 0; u < NSU; ++u) {
+            const u64 q = mul2(mu[u], h[u]);            // (abar_i mu_i) h_{i-1}
+            dacc = u == 0 ? mul2(q, A2[u]) : fma2(q, A2[u], dacc);
+            dAacc[u] = fma2(q, d2, dAacc[u]);
+          }
+          sk[o] = sacc; dk[o] = dacc;
+          // sum over the warp's 16 channel pairs: every lane parks its 16 partials (dB[8*half+0..7], dC[8*half+0..7])
+          // in shared memory, then lane l adds up value (l >> 1) over the 16 lanes of its parity.  Quarter-blocks
+          // of 4 values are 544 bytes apart so that both the 16-byte stores and the 4-byte loads are conflict-free.
+          {
+            __syncwarp();   // the previous token's loads from wred are done
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              *reinterpret_cast<float4*>(wred + q * WRED_Q + lane * 4) = make_float4(vB[4 * q], vB[4 * q + 1], vB[4 * q + 2], vB[4 * q + 3]);
+              *reinterpret_cast<float4*>(wred + (2 + q) * WRED_Q + lane * 4) = make_float4(vC[4 * q], vC[4 * q + 1], vC[4 * q + 2], vC[4 * q + 3]);
+            }
+            __syncwarp();
+            float part[16];
+#pragma unroll
+            for (int i2 = 0; i2 < 16; ++i2) part[i2] = rd[i2 * 8];
+#pragma unroll
+            for (int wdt = 8; wdt >= 1; wdt >>= 1)   // pairwise tree: 4 dependent adds instead of 16
+#pragma unroll
+              for (int i2 = 0; i2 < wdt; ++i2) part[i2] += part[i2 + wdt];
+            *(pR - o * NBC) = part[0];   // this warp's slot
+          }
+        }
+        {
+          // the lanes of a channel pair trade the halves of the state sums: each keeps one token
+          float a0, a1, b0, b1;
+          upk(sk[0], a0, a1); upk(sk[1], b0, b1);
+          const float s0 = (chf ? b0 : a0) + __shfl_xor_sync(0xffffffffu, chf ? a0 : b0, 1);
+          const float s1 = (chf ? b1 : a1) + __shfl_xor_sync(0xffffffffu, chf ? a1 : b1, 1);
+          upk(dk[0], a0, a1); upk(dk[1], b0, b1);
+          const float q0 = (chf ? b0 : a0) + __shfl_xor_sync(0xffffffffu, chf ? a0 : b0, 1);
+          const float q1 = (chf ? b1 : a1) + __shfl_xor_sync(0xffffffffu, chf ? a1 : b1, 1);
+          const float2 d = *reinterpret_cast<const float2*>(pDo);
+          float x0, x1;
+          upk(lds_pair<IO>(pXo), x0, x1);
+          const float u0 = fmaf(q0, LN2, x0 * s0) * sigmoid_of<ESZ>(d.x), u1 = fmaf(q1, LN2, x1 * s1) * sigmoid_of<ESZ>(d.y);
+          dbacc0 += u0; dbacc1 += u1;
+          st_pair<IO>(pO, u0, u1);
+          st_pair<IO>(pO + Cf::OUT_TILE, d.x * s0, d.y * s1);
+        }
+        pD -= 2 * CH * 4; pX -= 2 * CH * ESZ; pDo -= 2 * CH * 4; pXo -= 2 * CH * ESZ; pO -= 2 * 32 * ESZ; pR -= 2 * NBC;
+        tmj -= 2 * TM_TOK; pB -= 2 * DBC_ROW;
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the output tile is read by TMA
+    }
+    if (__syncthreads_or(ok ? 0 : 1)) { failed = true; fail_i = i; break; }
+    const int64_t row = (int64_t)b * T + tc;
+    if (nt == CK) {
+      if (lane == 0 && 32 * warp < ncs) {
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                     ::"l"(&tmDu), "r"(tile * CH + 32 * warp), "r"((int)row), "r"(smem_u32(out)) : "memory");
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                     ::"l"(&tmDx), "r"(tile * CH + 32 * warp), "r"((int)row), "r"(smem_u32(out + Cf::OUT_TILE)) : "memory");
+      }
+    } else if (w.tid < ncs) {   // rows past the sequence end belong to the next batch element: only those that exist
+      const IO* o = reinterpret_cast<const IO*>(out) + lane;
+      IO* du = reinterpret_cast<IO*>(ws + pl.off_du) + row * pl.du_ld + tile * CH + w.tid;
+      IO* dx = reinterpret_cast<IO*>(ws + pl.off_dxdir) + row * P + tile * CH + w.tid;
+      for (int j = 0; j < nt; ++j) { du[(int64_t)j * pl.du_ld] = o[j * 32]; dx[(int64_t)j * P] = o[(CK + j) * 32]; }
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    if (w.tid == 0 && i + NST < nchunk) issue(i + NST);
+    {   // channel sums of the chunk over the four warps, two per thread
+      const int j = w.tid >> 4, q = 2 * (w.tid & 15);
+      float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int w2 = 0; w2 < NTHR / 32; ++w2) {
+        const float2 v = *reinterpret_cast<const float2*>(&red[rb][w2][j][q]);
+        sum.x += v.x; sum.y += v.y;
+      }
+      if (j < nt) atomicAdd(reinterpret_cast<float2*>(dbc + (row + j) * NBC + q), sum);
+    }
+  }
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the output tiles outlive their stores
+  if (failed) {
+    if (w.tid == 0) {
+      // copies already issued still target this CTA's shared memory: one more bounded wait for each before leaving
+      for (int i2 = fail_i; i2 < nchunk && i2 < fail_i + NST; ++i2)
+        mbar_wait(&full_bar[i2 % NST], (i2 / NST) & 1);
+      mbar_wait(ckp_bar, ckp_issued & 1);
+      atomicExch(status, AS_ERR_TIMEOUT);
+    }
+  } else {
+    if (!pl.scalar) {
+      if (w.act)
+#pragma unroll
+        for (int u = 0; u < NSU; ++u) {
+          float alo, ahi, vlo, vhi;
+          upk(A2[u], alo, ahi);
+          upk(dAacc[u], vlo, vhi);
+          float* dst = dA_log + (int64_t)w.pa * NS + 8 * w.half + u;
+          atomicAdd(dst, vlo * (alo * LN2));
+          atomicAdd(dst + NS, vhi * (ahi * LN2));
+        }
+    } else {   // tied rate: the channel's gradient is the sum over its 16 states (8 here, 8 in the pair lane)
+      u64 tsum = 0ull;
+#pragma unroll
+      for (int u = 0; u < NSU; ++u) tsum = fma2(dAacc[u], A2[u], tsum);
+      float tlo, thi;
+      upk(tsum, tlo, thi);
+      tlo += __shfl_xor_sync(0xffffffffu, tlo, 1);
+      thi += __shfl_xor_sync(0xffffffffu, thi, 1);
+      if (w.act) atomicAdd(dA_log + w.pa + chf, (chf ? thi : tlo) * LN2);
+    }
+    dbacc0 += __shfl_xor_sync(0xffffffffu, dbacc0, 1);
+    dbacc1 += __shfl_xor_sync(0xffffffffu, dbacc1, 1);
+    if (w.act) atomicAdd(db_delta + w.pa + chf, chf ? dbacc1 : dbacc0);
+  }
+  // give the tensor memory back (every exit path comes through here)
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_base_s), "n"(TM_COLS) : "memory");
+  }
+}
+
+template <typename IO, bool WIN, bool SC>
+__device__ __noinline__ void adjoint_segment_truncated(const CUtensorMap& tmX, const CUtensorMap& tmD, const CUtensorMap& tmG,
+                                                       const CUtensorMap& tmDu, const CUtensorMap& tmDx, const Plan& pl,
+                                                       const float* __restrict__ A_log, char* __restrict__ ws,
+                                                       float* __restrict__ dA_log, float* __restrict__ db_delta) {
+  adjoint_segment<IO, false, WIN, SC>(tmX, tmD, tmG, tmDu, tmDx, pl, A_log, ws, dA_log, db_delta);
+}
+
+// The truncated form chooses per CTA between the walks with and without window-exit terms (the carry kernel has found out
+// where they can matter).  They are functions of their own so that each gets its own register allocation.
+template <typename IO, bool FULL, bool SC>
+__global__ void __launch_bounds__(NTHR, MAIN_CTAS)
+adjoint_main_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
+                    const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmDu,
+                    const __grid_constant__ CUtensorMap tmDx, const __grid_constant__ Plan pl, const float* __restrict__ A_log,
+                    char* __restrict__ ws, float* __restrict__ dA_log, float* __restrict__ db_delta) {
+  const int lay = (int)blockIdx.z / pl.Bg;   // this layer's rates and parameter-gradient rows; dy is shared by the layers
+  A_log += (int64_t)lay * a_stride_dev(pl);
+  dA_log += (int64_t)lay * a_stride_dev(pl);
+  db_delta += (int64_t)lay * pl.P;
+  if (FULL) adjoint_segment<IO, true, false, SC>(tmX, tmD, tmG, tmDu, tmDx, pl, A_log, ws, dA_log, db_delta);
+  else if (__ldg(reinterpret_cast<const int*>(ws + pl.off_live) + ((int64_t)blockIdx.z * pl.S + blockIdx.y) * pl.tiles + blockIdx.x))
+    adjoint_segment_truncated<IO, true, SC>(tmX, tmD, tmG, tmDu, tmDx, pl, A_log, ws, dA_log, db_delta);
+  else
+    adjoint_segment_truncated<IO, false, SC>(tmX, tmD, tmG, tmDu, tmDx, pl, A_log, ws, dA_log, db_delta);
+}
+
+template <typename IO, bool FULL, bool SC>
+int launch_main_t(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
+  Maps m;
+  if (make_maps(pl, sp, &m)) return 1;
+  constexpr bool BF = sizeof(IO) == 2;
+  CUtensorMap mdu, mdx;
+  if (act_map(&mdu, sp.ws + pl.off_du, pl, pl.B, sizeof(IO), BF, pl.du_ld, 32)) return 1;
+  if (act_map(&mdx, sp.ws + pl.off_dxdir, pl, pl.B, sizeof(IO), BF, pl.P, 32)) return 1;
+  constexpr int bytes = MainCfg<sizeof(IO), !FULL>::SMEM_DYN;
+  auto kern = adjoint_main_kernel<IO, FULL, SC>;
+  static bool done[AS_MAX_DEVICES] = {};
+  if (ensure_dynamic_smem(kern, bytes, done)) return 1;
+  kern<<<dim3(pl.tiles, pl.S, pl.B), NTHR, bytes, st>>>(m.x, m.d, m.g, mdu, mdx, pl, sp.A_log, sp.ws, dA_log, db_delta);
+  count_launch();
+  return (int)cudaGetLastError();
+}
+template <typename IO, bool SC>
+int launch_main_s(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
+  return pl.full ? launch_main_t<IO, true, SC>(pl, sp, dA_log, db_delta, st)
+                 : launch_main_t<IO, false, SC>(pl, sp, dA_log, db_delta, st);
+}
+
+}  // namespace
+
+int launch_adjoint_main(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
+  if (pl.io == AS_BF16)
+    return pl.scalar ? launch_main_s<__nv_bfloat16, true>(pl, sp, dA_log, db_delta, st)
+                     : launch_main_s<__nv_bfloat16, false>(pl, sp, dA_log, db_delta, st);
+  return pl.scalar ? launch_main_s<float, true>(pl, sp, dA_log, db_delta, st)
+                   : launch_main_s<float, false>(pl, sp, dA_log, db_delta, st);
+}
+
+}  // namespace as

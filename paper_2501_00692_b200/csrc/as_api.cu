@@ -150,7 +150,12 @@ int as_workspace_bytes(const as_shape_t* shape, int64_t tbar, size_t* fwd_bytes,
   e = make_plan(shape, tbar, 1, &pl);
   if (e) return e;
   if (fwd_bytes) *fwd_bytes = pl.total_fwd;
-  if (grad_bytes) *grad_bytes = pl.total_grad;
+  if (grad_bytes) {
+    *grad_bytes = pl.total_grad;
+    e = make_plan(shape, shape->seqlen, 1, &pl);   // as_full_bptt_grad and the full form cut the time differently
+    if (e) return e;
+    if (pl.total_grad > *grad_bytes) *grad_bytes = pl.total_grad;
+  }
   return AS_OK;
 }
 
@@ -212,6 +217,7 @@ int as_workspace_bytes_layers(const as_shape_t* shape, int32_t layers, int64_t t
   e = make_plan(shape, tbar, layers, &pl);
   if (e) return e;
   if (grad_bytes) *grad_bytes = pl.total_grad;
+  if (layers == 1) return as_workspace_bytes(shape, tbar, nullptr, grad_bytes);
   return AS_OK;
 }
 

@@ -89,6 +89,7 @@ struct Plan {
   int S;            // number of segments
   int64_t NC;       // number of CK-token chunks = ceil(T/CK)
   int m;            // tbar / L   (whole segments inside a window that starts on a segment boundary)
+  int direct;       // windows of at most four whole segments: the main kernel sums them from mu_loc, no block sums
   int r;            // tbar % L   (tokens of the following partial segment)
   int io;           // as_dtype_t
   int scalar;       // 1: one decay rate per channel (A_log is [P]), 0: one per (channel, state)
@@ -98,8 +99,8 @@ struct Plan {
   int gsplit;       // bf16 terms per value of dB, dC in Gcat: 1, or 3 (exact) where d_model % 32 != 0
   int du_ld;        // row pitch (elements) of the du buffer: P, or P + 32 gsplit when it is the left part of Gcat = [du|dB|dC..]
   // byte offsets into the workspace
-  size_t off_status, off_delta, off_bc, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
-      off_partd, off_hstart, off_carry, off_swin, off_du, off_dxdir, off_dbc,
+  size_t off_status, off_delta, off_bc, off_bcd, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
+      off_partd, off_hstart, off_suf, off_pre, off_total, off_live, off_du, off_dxdir, off_dbc,
       off_bptt_ckpt, off_wcat, off_wcatx, total_fwd, total_grad;
 };
 

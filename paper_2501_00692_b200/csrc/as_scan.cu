@@ -9,14 +9,9 @@
 // Arithmetic on the two states (2m, 2m+1) of a channel is packed into f32x2 instructions, which halves
 // the issue slots the FP32 pipe needs and leaves room for MUFU.EX2, shuffles and shared-memory loads.
 // Inputs of a chunk (x, Delta, dy tiles by 2D TMA; B/C rows, the chunk checkpoint and its cumulative
-// Delta by 1D bulk copies) land in a shared-memory ring guarded by mbarriers with bounded waits.  The main
-// adjoint kernel parks the rebuilt per-token states of a chunk in tensor memory (tcgen05.st / tcgen05.ld)
-// instead of registers or shared memory.
-#include <cuda.h>
-
-#include <type_traits>
-
-#include "as_internal.cuh"
+// Delta by 1D bulk copies) land in a shared-memory ring guarded by mbarriers with bounded waits.
+// This file: the plan, the ascending kernels and the carries across segments; the main adjoint kernel is in as_adjoint.cu.
+#include "as_scan.cuh"
 
 namespace as {
 
@@ -37,22 +32,35 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.tbar = p.full ? p.T : tbar;
   p.tiles = (p.P + CH - 1) / CH;
   p.bw = p.P < CH ? p.P : CH;
-  const int64_t ctas = (int64_t)p.tiles * p.B;
-  // full waves of the main kernel's resident CTAs (SMs x CTAs per SM)
+  // Full waves of the main kernel's resident CTAs (SMs x CTAs per SM).  A partly filled wave costs as much as a full one
+  // (T = 30,000, P = 256: 147 us at two waves, 155 at one and a half), and a CTA has a fixed cost of some 20 tokens' time.
+  // So: three waves (two in the full form) while segments stay at 160 tokens or more, which balances the tail of long
+  // runs; else two, else one; and where not even one wave can be filled, segments as short as two chunks (one chunk for
+  // short sequences, whose full-form carries are cheap): latency counts there, and it is the tokens of a segment.
   const int64_t slots = (int64_t)sm_count() * 3;   // resident CTAs of the main kernel
-  // three waves in the truncated form (shorter segments balance the tail better than they cost in carries); the
-  // full form's reverse carry is sequential over the segments, which favours fewer of them
-  int64_t s_target = ((p.full ? 2 : 3) * slots) / ctas;
-  if (s_target < 1) s_target = 1;
-  int64_t L = (p.T + s_target - 1) / s_target;
-  L = (L + CK - 1) / CK * CK;
-  if (L < 64) L = 64;
+  auto segment = [&](int64_t ctas) {
+    int64_t l = 0;
+    for (int waves = p.full ? 2 : 3; waves >= 1; --waves) {
+      int64_t s_target = waves * slots / ctas;
+      if (s_target < 1) s_target = 1;
+      l = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;
+      if (l >= 160) break;
+    }
+    return l;
+  };
+  // Several layers fill the chip with longer segments; short runs keep the segments that each layer alone would get (then
+  // a layer's results do not depend on how many it is computed with).
+  int64_t L = segment((int64_t)p.tiles * p.B);
+  if (L < 160) L = segment((int64_t)p.tiles * p.Bg);
+  const int64_t lmin = p.full && p.T <= 1024 ? CK : 2 * CK;
+  if (L < lmin) L = lmin;
   if (L > 2048) L = 2048;
   p.L = (int)L;
   p.S = (int)((p.T + L - 1) / L);
   p.NC = (p.T + CK - 1) / CK;
   p.m = (int)(p.tbar / L);
   p.r = (int)(p.tbar % L);
+  p.direct = !p.full && p.m <= 4;
   const size_t e = sh->io == AS_BF16 ? 2 : 4;
   const size_t BTP = (size_t)p.B * p.T * p.P;
   const size_t BT = (size_t)p.B * p.T;
@@ -69,218 +77,27 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.off_wcat = take((size_t)p.KL * (p.P + NBC) * p.P * 2);
   p.total_fwd = o;
   p.off_wcatx = p.tc && p.gsplit > 1 ? take((size_t)p.KL * p.du_ld * p.P * 2) : p.off_wcat;
+  p.off_bcd = take((BT + CK) * 2 * NBC * 4);   // doubled B rows, then doubled C rows
   p.off_ckpt = take((size_t)p.B * p.NC * p.tiles * TILE_FLOATS * 4);
   p.off_cs = take((size_t)p.B * p.NC * p.P * 4);
   p.off_muloc = take(BSB * 4);
   p.off_mupart = take(BSB * 4);
   p.off_partd = take(BSP * 4);
-  p.off_carry = take(BSB * 4);
-  p.off_swin = take(BSP * 8);
+  p.off_suf = take(BSB * 4);
+  p.off_pre = take(BSB * 4);
+  p.off_total = take(BSP * 8);
+  p.off_live = take((size_t)p.B * p.S * p.tiles * 4);
   p.off_du = take(BT * (size_t)p.du_ld * e);
   p.off_dxdir = take(BTP * e);
   p.off_dbc = take(BT * NBC * 4);
   p.off_bptt_ckpt = take((size_t)p.B * ((p.T + 63) / 64) * p.P * NS * 4);
   p.total_grad = o;
   *pl = p;
-  // segments (plus the NU blocks of the forward carry) fill gridDim.y, (layer, batch) gridDim.z
+  // segments fill gridDim.y, (layer, batch) gridDim.z
   return (p.S > 65535 - NU || p.B > 65535) ? AS_ERR_LIMIT : AS_OK;
 }
 
 namespace {
-
-typedef unsigned long long u64;   // two packed fp32 values (lo = even state, hi = odd state)
-
-__device__ __forceinline__ int64_t a_stride_dev(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }
-
-__device__ __forceinline__ u64 pk(float lo, float hi) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk(u64 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 ex2_2(u64 e) {
-  float lo, hi;
-  upk(e, lo, hi);
-  return pk(ex2_approx(lo), ex2_approx(hi));
-}
-__device__ __forceinline__ float hsum(u64 v) {
-  float lo, hi;
-  upk(v, lo, hi);
-  return lo + hi;
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-constexpr uint32_t WAIT_LIMIT = 1u << 22;
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = WAIT_LIMIT) {
-  const uint32_t addr = smem_u32(bar);
-  for (uint32_t it = 0; it < limit; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-__device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* tm, int c0, int64_t c1, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(tm), "r"(c0), "r"((int)c1), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-
-template <typename IO> struct IoSz { static constexpr int v = sizeof(IO); };
-
-// shared-memory stage of one chunk of the ascending kernels: x, Delta, [B | C] rows and (pre-pass) dy
-template <int ESZ, bool WITH_G>
-struct Stage {
-  static constexpr int X = 0;
-  static constexpr int D = X + CK * CH * ESZ;
-  static constexpr int BC = D + CK * CH * 4;
-  static constexpr int G = BC + CK * NBC * 4;
-  static constexpr int BYTES = G + (WITH_G ? CK * CH * ESZ : 0);
-};
-constexpr int NSTAGE = 3;        // ascending kernels
-constexpr int WRED_Q = 32 * 4 + 8;   // floats per quarter-block of the per-warp reduction scratch (512 B + 32 B skew)
-constexpr int MAIN_CTAS = 3;    // resident CTAs per SM the main kernel is compiled for (up to 168 registers per thread)
-constexpr int FW_UNROLL = 8;     // unroll factor of the main adjoint kernel's forward rebuild loop (the whole chunk)
-constexpr int BW_UNROLL = 2;     // unroll factor of the main adjoint kernel's backward token loop
-constexpr int NSTAGE_MAIN = 2;   // main adjoint kernel: a chunk takes thousands of cycles, one chunk of lookahead suffices
-
-// per-thread values of its NCH channels
-struct ChV { float v[NCH]; };
-__device__ __forceinline__ ChV ch_zero() { ChV r; for (int c = 0; c < NCH; ++c) r.v[c] = 0.f; return r; }
-
-// row j of a staged [CK x CH] tile, channels NCH*k .. NCH*k + NCH-1
-template <typename IO> __device__ __forceinline__ ChV lds_ch(const uint8_t* tile, int j, int k);
-template <> __device__ __forceinline__ ChV lds_ch<float>(const uint8_t* tile, int j, int k) {
-  ChV r;
-  if (NCH == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(tile + (j * CH + 2 * k) * 4);
-    r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  } else {
-    r.v[0] = *reinterpret_cast<const float*>(tile + (j * CH + k) * 4);
-  }
-  return r;
-}
-template <> __device__ __forceinline__ ChV lds_ch<__nv_bfloat16>(const uint8_t* tile, int j, int k) {
-  ChV r;
-  if (NCH == 2) {
-    const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + (j * CH + 2 * k) * 2));
-    r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  } else {
-    r.v[0] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + (j * CH + k) * 2));
-  }
-  return r;
-}
-// the same from a pointer that already addresses this thread's channels in the row
-template <typename IO> __device__ __forceinline__ ChV lds_chp(const uint8_t* p);
-template <> __device__ __forceinline__ ChV lds_chp<float>(const uint8_t* p) {
-  ChV r;
-  const float2 t = *reinterpret_cast<const float2*>(p);
-  r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  return r;
-}
-template <> __device__ __forceinline__ ChV lds_chp<__nv_bfloat16>(const uint8_t* p) {
-  ChV r;
-  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-  r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  return r;
-}
-// NCH consecutive floats of a global per-channel array
-__device__ __forceinline__ ChV ldg_ch(const float* p) {
-  ChV r;
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) r.v[c] = __ldg(p + c);
-  return r;
-}
-__device__ __forceinline__ void stg_ch(float* p, const float (&v)[NCH]) {
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) p[c] = v[c];
-}
-
-struct Who {          // what this thread owns
-  int tid, k, half;   // pair index, state half
-  int pa;             // first of its NCH channels
-  bool act;           // the channels exist (P is a multiple of 8, so all or none)
-};
-__device__ __forceinline__ Who who(int tile, int P) {
-  Who w;
-  w.tid = threadIdx.x; w.k = w.tid >> 1; w.half = w.tid & 1;
-  w.pa = tile * CH + NCH * w.k;
-  w.act = w.pa < P;
-  return w;
-}
-// A2[u] = -exp(A_log) * log2(e) for unit u = ch*4 + m  ->  states (8*half + 2m, +1) of channel pa + ch
-// (scalar structure: the channel's single rate for every state)
-__device__ __forceinline__ void load_A2(const float* A_log, const Who& w, u64 (&A2)[NU], int scalar) {
-#pragma unroll
-  for (int u = 0; u < NU; ++u) {
-    float2 v = make_float2(0.f, 0.f);
-    if (w.act) {
-      if (scalar) { const float a = __ldg(A_log + w.pa + u / 4); v = make_float2(a, a); }
-      else v = __ldg(reinterpret_cast<const float2*>(A_log + (int64_t)(w.pa + u / 4) * NS + 8 * w.half + 2 * (u % 4)));
-    }
-    A2[u] = pk(-__expf(v.x) * LOG2E, -__expf(v.y) * LOG2E);
-  }
-}
-// 16 values of this thread inside a 2048-float tile block: float4 q of thread tid at (q*128 + tid)
-__device__ __forceinline__ void load_block(const float* blk, int tid, u64 (&v)[NU]) {
-  const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
-#pragma unroll
-  for (int q = 0; q < 2 * NCH; ++q) {
-    const ulonglong2 t = b2[q * NTHR + tid];
-    v[2 * q] = t.x; v[2 * q + 1] = t.y;
-  }
-}
-__device__ __forceinline__ void load_block_g(const float* blk, int tid, u64 (&v)[NU]) {
-  const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
-#pragma unroll
-  for (int q = 0; q < 2 * NCH; ++q) {
-    const ulonglong2 t = __ldg(b2 + q * NTHR + tid);
-    v[2 * q] = t.x; v[2 * q + 1] = t.y;
-  }
-}
-__device__ __forceinline__ void store_block(float* blk, int tid, const u64 (&v)[NU]) {
-  ulonglong2* b2 = reinterpret_cast<ulonglong2*>(blk);
-#pragma unroll
-  for (int q = 0; q < 2 * NCH; ++q) b2[q * NTHR + tid] = make_ulonglong2(v[2 * q], v[2 * q + 1]);
-}
-
-// sigmoid(u) from Delta = softplus(u): 1 - exp(-Delta), without cancellation for small Delta
-__device__ __forceinline__ float sig_from_delta(float d) {
-  const float big = 1.f - ex2_approx(-d * LOG2E);
-  float s = fmaf(-d, 1.f / 7.f, 1.f);
-  s = fmaf(-d * (1.f / 6.f), s, 1.f);
-  s = fmaf(-d * (1.f / 5.f), s, 1.f);
-  s = fmaf(-d * (1.f / 4.f), s, 1.f);
-  s = fmaf(-d * (1.f / 3.f), s, 1.f);
-  s = fmaf(-d * (1.f / 2.f), s, 1.f);
-  return d < 0.125f ? d * s : big;
-}
 
 // ------------------------------------------------------------------------------------------------
 // ascending pass over one segment.
@@ -292,14 +109,18 @@ __device__ __forceinline__ float sig_from_delta(float d) {
 // Tokens past the end of the sequence inside the last chunk are neutralised by zeroing their staged
 // Delta, dy and B/C rows (Delta = 0 gives abar = 1 and a zero input term), so the token code has no branches.
 // ------------------------------------------------------------------------------------------------
-enum { PRE_FWD = 0, PRE_ADJ = 1, PRE_Y = 2 };
+// shared-memory stage of one chunk of the ascending kernels: x, Delta, [B | C] rows and (pre-pass) dy
+template <int ESZ, bool WITH_G>
+struct Stage {
+  static constexpr int X = 0;
+  static constexpr int D = X + CK * CH * ESZ;
+  static constexpr int BC = D + CK * CH * 4;
+  static constexpr int G = BC + CK * NBC * 4;
+  static constexpr int BYTES = G + (WITH_G ? CK * CH * ESZ : 0);
+};
+constexpr int NSTAGE = 3;        // ascending kernels
 
-// zero the staged rows [nt, CK) of a [CK x CH] tile (row_bytes per token) - all threads of the CTA
-__device__ __forceinline__ void zero_rows(uint8_t* tile, int row_bytes, int nt, int tid) {
-  uint4* p = reinterpret_cast<uint4*>(tile + nt * row_bytes);
-  const int n16 = (CK - nt) * row_bytes / 16;
-  for (int i = tid; i < n16; i += NTHR) p[i] = make_uint4(0u, 0u, 0u, 0u);
-}
+enum { PRE_FWD = 0, PRE_ADJ = 1, PRE_Y = 2 };
 
 template <typename IO, int MODE, bool SC>
 __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__ CUtensorMap tmX,
@@ -372,6 +193,14 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
       store_block(reinterpret_cast<float*>(ws + pl.off_ckpt) + (cc * pl.tiles + tile) * TILE_FLOATS, w.tid, h);
       if (w.half == 0 && w.act)
         stg_ch(reinterpret_cast<float*>(ws + pl.off_cs) + cc * P + w.pa, cum);
+    }
+    if (MODE == PRE_ADJ && tile == 0 && ok) {   // the rows once more, doubled, for the main kernel's packed channel pairs
+      const int j = w.tid >> 4, q = w.tid & 15;
+      const float2 v = *reinterpret_cast<const float2*>(sm + St::BC + j * NBC * 4 + 8 * q);
+      if (j < nt) {   // B rows, then C rows
+        float* dst = reinterpret_cast<float*>(ws + pl.off_bcd) + (q < 8 ? 0 : ((int64_t)pl.B * pl.T + CK) * NBC);
+        *reinterpret_cast<float4*>(dst + ((int64_t)b * pl.T + tc + j) * NBC + 4 * (q & 7)) = make_float4(v.x, v.x, v.y, v.y);
+      }
     }
     if (nt < CK) {   // only the last chunk of a sequence
       if (ok) {
@@ -483,682 +312,271 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
 }
 
 // ------------------------------------------------------------------------------------------------
-// carries across segments.  Thread (b, tile, tid) owns the same 16 (channel, state) slots as in the scans.
+// carries across segments.  The segment decays are exp(A * sum of Delta), so each carry is a linear recurrence over the
+// segments; a chain of S dependent steps would leave the kernel waiting for latency (full form, T = 50,000, P = 80,
+// S = 1250: 200 us).  So a CTA takes 32 state pairs (one per lane: 256 contiguous bytes of a tile block) and its warps cut
+// the segments into ranges: scan each range from zero, combine the ranges' (end value, decay) in shared memory, scan
+// again from the true start.  Every pass reads CARRY_UB segments' values at once.
 // ------------------------------------------------------------------------------------------------
-// hstart[s]: true state entering segment s (sequential in s).  The recurrence over segments is a chain of dependent
-// steps, so the kernel is latency-bound: one thread per state pair (u = the unit of the scan kernels'
-// thread), and the loads of a batch of 16 segments are issued together, one batch ahead of the one being applied.
-__device__ __forceinline__ void fixup_h_block(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws,
-                                              int tile, int b, int u) {
-  const Who w = who(tile, pl.P);
+constexpr int CARRY_UB = 8;
+constexpr int CARRY_WARPS = 32;                  // most warps of a CTA
+constexpr int CARRY_SLICES = TILE_FLOATS / 64;   // CTAs per (tile, batch element): 64 floats each
+
+struct Slot {           // the state pair of a lane: pair `iu` of its tile block
+  int lane, warp, nw;
+  int iu, p;            // index in units of u64, channel
+  bool act, first;      // the channel exists; this lane speaks for the channel
+  u64 A2;
+};
+__device__ __forceinline__ Slot slot(const Plan& pl, const float* A_log, int tile, int b, int sl) {
+  Slot t;
+  t.lane = threadIdx.x & 31; t.warp = threadIdx.x >> 5; t.nw = blockDim.x >> 5;
+  t.iu = sl * 32 + t.lane;
+  // pair iu: half (iu & 1) of float4 q of scan thread tid, i.e. its unit u = 2 q + (iu & 1)
+  const int q = (t.iu >> 1) / NTHR, tid = (t.iu >> 1) % NTHR, u = 2 * q + (t.iu & 1);
+  t.p = tile * CH + NCH * (tid >> 1) + u / 4;
+  t.act = t.p < pl.P;
+  t.first = t.act && (tid & 1) == 0 && (u & 3) == 0;
   A_log += (int64_t)(b / pl.Bg) * a_stride_dev(pl);
-  u64 A2all[NU];
-  load_A2(A_log, w, A2all, pl.scalar);
-  u64 A2u = 0ull;
-#pragma unroll
-  for (int i = 0; i < NU; ++i) A2u = i == u ? A2all[i] : A2u;
-  const int ch = u / 4;                                  // which of the thread's channels the unit belongs to
+  float2 v = make_float2(0.f, 0.f);
+  if (t.act) {
+    if (pl.scalar) { const float a = __ldg(A_log + t.p); v = make_float2(a, a); }
+    else v = __ldg(reinterpret_cast<const float2*>(A_log + (int64_t)t.p * NS + 8 * (tid & 1) + 2 * (u & 3)));
+  }
+  t.A2 = pk(-__expf(v.x) * LOG2E, -__expf(v.y) * LOG2E);
+  return t;
+}
+__device__ __forceinline__ u64 decay_of(u64 A2, float d) { return ex2_2(mul2(pk(d, d), A2)); }
+
+struct CarrySmem {      // one entry per warp and lane
+  u64 val[CARRY_WARPS][32], dec[CARRY_WARPS][32];
+  float sum[CARRY_WARPS][32];
+  double tot[CARRY_WARPS][32];
+};
+
+// hstart[s]: true state entering segment s
+__device__ __forceinline__ void carry_h(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws, int tile,
+                                        int b, int sl, CarrySmem& sm) {
+  const Slot t = slot(pl, A_log, tile, b, sl);
   const u64* hend = reinterpret_cast<const u64*>(ws + pl.off_hend);
   const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd);
   u64* hstart = reinterpret_cast<u64*>(ws + pl.off_hstart);
-  // unit u of thread tid inside a tile block: float4 q = u / 2 at (q * NTHR + tid), its low or high half
-  const int64_t in_blk = ((int64_t)(u >> 1) * NTHR + w.tid) * 2 + (u & 1);   // in u64 units
-  constexpr int UN = 16;
-  u64 he[2][UN];
-  float sd[2][UN];
-  auto fetch = [&](int s0, int buf) {
+  const int n = (pl.S + t.nw - 1) / t.nw, sA = min(pl.S, t.warp * n), sB = min(pl.S, sA + n);
+  const int64_t stride = (int64_t)pl.tiles * (TILE_FLOATS / 2);
+  const int64_t at0 = ((int64_t)b * pl.S * pl.tiles + tile) * (TILE_FLOATS / 2) + t.iu, ch0 = (int64_t)b * pl.S * pl.P + t.p;
+  u64 he[CARRY_UB];
+  float sd[CARRY_UB];
+  auto fetch = [&](int s0) {   // slots past the range: decay 1, add 0
 #pragma unroll
-    for (int i = 0; i < UN; ++i) {
-      const int s = min(s0 + i, pl.S - 1);
-      const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
-      he[buf][i] = __ldg(hend + sb * (TILE_FLOATS / 2) + in_blk);
-      sd[buf][i] = w.act ? __ldg(segd + ((int64_t)b * pl.S + s) * pl.P + w.pa + ch) : 0.f;
+    for (int i = 0; i < CARRY_UB; ++i) {
+      const bool in = s0 + i < sB;
+      he[i] = in ? __ldg(hend + at0 + (s0 + i) * stride) : 0ull;
+      sd[i] = in && t.act ? __ldg(segd + ch0 + (int64_t)(s0 + i) * pl.P) : 0.f;
     }
   };
-  u64 hs = 0ull;
-  auto apply = [&](int s0, int buf) {
+  u64 v = 0ull;
+  float dsum = 0.f;
+  for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+    fetch(s0);
 #pragma unroll
-    for (int i = 0; i < UN; ++i) {
-      const int s = s0 + i;
-      if (s < pl.S) {
-        const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
-        hstart[sb * (TILE_FLOATS / 2) + in_blk] = hs;
-        hs = fma2(ex2_2(mul2(pk(sd[buf][i], sd[buf][i]), A2u)), hs, he[buf][i]);
-      }
-    }
-  };
-  fetch(0, 0);
-  for (int s0 = 0; s0 < pl.S; s0 += 2 * UN) {
-    if (s0 + UN < pl.S) fetch(s0 + UN, 1);
-    apply(s0, 0);
-    if (s0 + UN < pl.S) {
-      if (s0 + 2 * UN < pl.S) fetch(s0 + 2 * UN, 0);
-      apply(s0 + UN, 1);
+    for (int i = 0; i < CARRY_UB; ++i) { v = fma2(decay_of(t.A2, sd[i]), v, he[i]); dsum += sd[i]; }
+  }
+  sm.val[t.warp][t.lane] = v;
+  sm.dec[t.warp][t.lane] = decay_of(t.A2, dsum);
+  __syncthreads();
+  v = 0ull;
+  for (int w = 0; w < t.warp; ++w) v = fma2(sm.dec[w][t.lane], v, sm.val[w][t.lane]);
+  for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+    if (n > CARRY_UB) fetch(s0);   // a single batch is still in registers
+#pragma unroll
+    for (int i = 0; i < CARRY_UB; ++i) {
+      if (s0 + i < sB) hstart[at0 + (s0 + i) * stride] = v;
+      v = fma2(decay_of(t.A2, sd[i]), v, he[i]);
     }
   }
 }
 
-// carry[s] = abar_{e+1} * mu_{e+1} for e the last token of segment s: what the reverse recurrence inside
-// segment s starts from.  With mu_loc[s'] already carried to the token before segment s', this is
+// The reverse recurrence inside segment s starts from abar_{e+1} mu_{e+1}, e the last token of the segment.  With
+// mu_loc[s'] already carried to the token before segment s', this is
 //   mu_loc[s+1] + D[s+1] (mu_loc[s+2] + ... + D[s+m] mu_part[s+m+1]),   D[s'] = exp(A * sum of Delta over s'),
-// i.e. m whole segments plus the first r tokens of the next one (all later segments in the full form).
-// swin[s]: sum of Delta over the Tbar tokens after e (fp64), for the window-exit factor.
-__device__ __forceinline__ void fixup_mu_block(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws,
-                                               int tile, int sy, int b) {
-  const int P = pl.P, S = pl.S;
-  const Who w = who(tile, P);
-  A_log += (int64_t)(b / pl.Bg) * a_stride_dev(pl);
-  u64 A2[NU];
-  load_A2(A_log, w, A2, pl.scalar);
-  const float* muloc = reinterpret_cast<const float*>(ws + pl.off_muloc);
-  const float* mupart = reinterpret_cast<const float*>(ws + pl.off_mupart);
+// i.e. m whole segments plus the first r tokens of the next one (all later segments in the full form).  The segments are
+// cut into blocks of m; with suf[i] the sum from segment i to the end of its block and pre[j] the sum from the start of its
+// block to segment j, the window of m segments is suf[s+1] plus the decayed pre[s+m] (the main kernel puts them together).
+// Both are recurrences that start anew at block borders: the cost does not grow with m, and no term is ever subtracted.
+// total[s]: Delta sum of segments 0..s in fp64, for the decays between them and the window sum.
+template <bool SUF>
+__device__ __forceinline__ void carry_mu(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws, int tile,
+                                         int b, int sl, CarrySmem& sm) {
+  const Slot t = slot(pl, A_log, tile, b, sl);
+  const int S = pl.S, m = pl.full ? S : pl.m;
+  const u64* muloc = reinterpret_cast<const u64*>(ws + pl.off_muloc);
   const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd);
-  const float* partd = reinterpret_cast<const float*>(ws + pl.off_partd);
-  float* carry = reinterpret_cast<float*>(ws + pl.off_carry);
-  double* swin = reinterpret_cast<double*>(ws + pl.off_swin);
-  auto blk = [&](int s) -> int64_t { return (((int64_t)b * S + s) * pl.tiles + tile) * TILE_FLOATS; };
-  auto ld2 = [&](const float* arr, int s) -> ChV {
-    return (w.act && s < S) ? ldg_ch(arr + ((int64_t)b * S + s) * P + w.pa) : ch_zero();
-  };
-  auto step = [&](int sg, u64 (&val)[NU]) {   // val = mu_loc[sg] + D[sg] * val
-    const ChV sd = ld2(segd, sg);
-    u64 d2[NCH];
+  u64* out = reinterpret_cast<u64*>(ws + (SUF ? pl.off_suf : pl.off_pre));
+  double* total = reinterpret_cast<double*>(ws + pl.off_total);
+  const int n = (S + t.nw - 1) / t.nw, sA = min(S, t.warp * n), sB = min(S, sA + n);
+  const int64_t stride = (int64_t)pl.tiles * (TILE_FLOATS / 2);
+  const int64_t at0 = ((int64_t)b * S * pl.tiles + tile) * (TILE_FLOATS / 2) + t.iu, ch0 = (int64_t)b * S * pl.P + t.p;
+  u64 ml[CARRY_UB];
+  float sd[CARRY_UB];
+  auto fetch = [&](int s0) {   // slots past the range: decay 1, add 0
 #pragma unroll
-    for (int c = 0; c < NCH; ++c) d2[c] = pk(sd.v[c], sd.v[c]);
-    u64 ml[NU];
-    load_block_g(muloc + blk(sg), w.tid, ml);
-#pragma unroll
-    for (int u = 0; u < NU; ++u) val[u] = fma2(ex2_2(mul2(d2[u / 4], A2[u])), val[u], ml[u]);
-  };
-  if (pl.full) {
-    if (sy != 0) return;
-    u64 val[NU];
-#pragma unroll
-    for (int u = 0; u < NU; ++u) val[u] = 0ull;
-    for (int s = S - 1; s >= 0; --s) {
-      store_block(carry + blk(s), w.tid, val);
-      step(s, val);
-    }
-  } else {
-    const int s = sy;
-    const int s1 = s + 1;
-    u64 val[NU];
-#pragma unroll
-    for (int u = 0; u < NU; ++u) val[u] = 0ull;
-    if (s1 + pl.m < S) load_block_g(mupart + blk(s1 + pl.m), w.tid, val);
-    for (int k = pl.m - 1; k >= 0; --k) {
-      const int sg = s1 + k;
-      if (sg < S) step(sg, val);
-    }
-    store_block(carry + blk(s), w.tid, val);
-    if (w.half == 0 && w.act) {
-      double swv[NCH];
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) swv[c] = 0.0;
-      for (int k = 1; k <= pl.m; ++k) {
-        const ChV v = ld2(segd, s + k);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) swv[c] += (double)v.v[c];
-      }
-      const ChV pv = ld2(partd, s + pl.m + 1);
-      double* dst = swin + ((int64_t)b * S + s) * P + w.pa;
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) dst[c] = swv[c] + (double)pv.v[c];
-    }
-  }
-}
-
-// Both carry computations in one launch (they are independent and each is latency-bound): blockIdx.y < ny_h runs the
-// forward carry for unit u = blockIdx.y, the rest the reverse carry for segment blockIdx.y - ny_h.
-__global__ void __launch_bounds__(NTHR) fixup_kernel(Plan pl, const float* __restrict__ A_log, char* __restrict__ ws,
-                                                     int ny_h) {
-  const int tile = blockIdx.x, b = blockIdx.z;
-  if ((int)blockIdx.y < ny_h) fixup_h_block(pl, A_log, ws, tile, b, (int)blockIdx.y);
-  else fixup_mu_block(pl, A_log, ws, tile, (int)blockIdx.y - ny_h, b);
-}
-
-// abar for the NU units of a thread from the per-channel exponent scale e2[ch] = {e, e}: exp2(e * A2[u]).  With a
-// scalar rate the N states of a channel share one factor, so one pair of MUFU operations per channel is enough.
-template <bool SC>
-__device__ __forceinline__ void decay_units(const u64 (&e2)[NCH], const u64 (&A2)[NU], u64 (&a)[NU]) {
-  if (SC) {
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-      const u64 ac = ex2_2(mul2(e2[ch], A2[ch * 4]));
-#pragma unroll
-      for (int m = 0; m < 4; ++m) a[ch * 4 + m] = ac;
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < NU; ++u) a[u] = ex2_2(mul2(e2[u / 4], A2[u]));
-  }
-}
-
-// ---- tensor memory as a per-thread scratchpad ------------------------------------------------------
-// The main adjoint kernel runs no MMA, so the SM's tensor memory is free.  Each CTA allocates 128 of the 512
-// columns of its SM (three CTAs are resident) and every thread parks the chunk's eight states in its own TMEM lane:
-// warp w of the 4-warp CTA owns lanes [32w, 32w+32), a 32x32b access moves 16 registers of each lane to or
-// from 16 consecutive columns.
-constexpr int TM_TOK = 16;         // columns per token: the 16 state registers of a thread
-constexpr int TM_COLS = CK * TM_TOK;   // columns [16 j, 16 j + 16): state after token j of the current chunk
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const u64 (&v)[NU]) {
-  uint32_t r[16];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) asm("mov.b64 {%0, %1}, %2;" : "=r"(r[2 * u]), "=r"(r[2 * u + 1]) : "l"(v[u]));
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, u64 (&v)[NU]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int u = 0; u < 8; ++u) asm("mov.b64 %0, {%1, %2};" : "=l"(v[u]) : "r"(r[2 * u]), "r"(r[2 * u + 1]));
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// shared-memory stage of one chunk of the main adjoint kernel (the chunk checkpoint has a buffer of its own)
-template <int ESZ, bool WIN>
-struct StageM {
-  static constexpr int X = 0;
-  static constexpr int D = X + CK * CH * ESZ;
-  static constexpr int BC = D + CK * CH * 4;
-  static constexpr int G = BC + CK * NBC * 4;
-  static constexpr int CS = G + CK * CH * ESZ;
-  static constexpr int G2 = CS + CH * 4;
-  static constexpr int D2 = G2 + (WIN ? CK * CH * ESZ : 0);
-  static constexpr int BC2 = D2 + (WIN ? CK * CH * 4 : 0);
-  static constexpr int BYTES = BC2 + (WIN ? CK * NBC * 4 : 0);
-};
-template <int ESZ, bool WIN> struct MainCfg {
-  static constexpr int SMEM_DYN = NSTAGE_MAIN * StageM<ESZ, WIN>::BYTES + TILE_FLOATS * 4 + 128;
-};
-
-// ------------------------------------------------------------------------------------------------
-// main adjoint kernel: one CTA per (channel tile, segment, batch element), chunks walked last to first.
-// Per chunk: rebuild the states after its eight tokens from the chunk checkpoint and park them in tensor memory,
-// then walk the chunk's tokens backwards: mu recurrence (with the exact window exit), the per-token
-// vector-Jacobian products, the channel sums dB_t / dC_t, and the per-channel outputs du_t and dx_dir_t.
-// ------------------------------------------------------------------------------------------------
-template <typename IO, bool FULL, bool SC>
-__global__ void __launch_bounds__(NTHR, MAIN_CTAS)
-adjoint_main_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
-                    const __grid_constant__ CUtensorMap tmG, Plan pl, const float* __restrict__ A_log,
-                    char* __restrict__ ws, float* __restrict__ dA_log, float* __restrict__ db_delta) {
-  static_assert(NCH == 2 && NTHR == 128, "tensor-memory parking assumes 4 warps and 16 state registers per thread");
-  constexpr int ESZ = IoSz<IO>::v;
-  constexpr bool WIN = !FULL;
-  using St = StageM<ESZ, WIN>;
-  extern __shared__ __align__(128) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[NSTAGE_MAIN];
-  __shared__ __align__(8) uint64_t ckp_bar;          // the checkpoint tile of the current chunk has landed
-  __shared__ __align__(8) uint64_t ckp_free;         // all threads have read it (NTHR arrivals)
-  __shared__ uint32_t tmem_base_s;
-  __shared__ float red[2][NTHR / 32][CK][NBC];      // per-token [dB | dC] sums of each warp, two chunks in flight
-  __shared__ __align__(16) float wred[NTHR / 32][4 * WRED_Q];   // per-warp scratch of the channel reduction
-  __shared__ ulonglong2 hst_s[2 * NCH][NTHR];       // true segment-start state, read back once per chunk
-  uint8_t* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);   // stays a shared-space pointer
-  uint8_t* ckp_s = smem + NSTAGE_MAIN * St::BYTES;
-
-  const int tile = blockIdx.x, s = blockIdx.y, b = blockIdx.z;
-  const int P = pl.P;
-  const Who w = who(tile, P);
-  const int lane = w.tid & 31, warp = w.tid >> 5;
-  const int64_t T = pl.T, tbar = pl.tbar;
-  const int64_t t0 = (int64_t)s * pl.L;
-  const int64_t t1 = min(T, t0 + pl.L);
-  const int nchunk = (int)((t1 - t0 + CK - 1) / CK);
-  const float* bc = reinterpret_cast<const float*>(ws + pl.off_bc);
-  const float* ckpt = reinterpret_cast<const float*>(ws + pl.off_ckpt);
-  const float* cs = reinterpret_cast<const float*>(ws + pl.off_cs);
-  float* dbc = reinterpret_cast<float*>(ws + pl.off_dbc);
-  int* status = reinterpret_cast<int*>(ws + pl.off_status);
-  const int ncs = min(CH, P - tile * CH);   // channels of this tile that exist
-  const int64_t BT = (int64_t)pl.B * T;
-  {   // this layer's rates and parameter-gradient rows; dy is shared by the layers
-    const int lay = b / pl.Bg;
-    A_log += (int64_t)lay * a_stride_dev(pl);
-    dA_log += (int64_t)lay * a_stride_dev(pl);
-    db_delta += (int64_t)lay * P;
-  }
-  const int64_t grow0 = (int64_t)(b % pl.Bg) * T - (int64_t)b * T;   // added to an x / Delta row to get the dy row
-  const int du_ld = pl.du_ld;
-  // the two lanes of a pair end up with the same per-channel sums: lane `half` finalises channel `half`
-  const int chf = w.half;
-  const bool fin = w.act;
-  const int pmine = w.pa + chf;
-  IO* du = reinterpret_cast<IO*>(ws + pl.off_du) + pmine;
-  IO* dxdir = reinterpret_cast<IO*>(ws + pl.off_dxdir) + pmine;
-  // lanes whose channels do not exist (ragged last channel tile) store into a spare word of the status block, with
-  // zero strides, so that the per-token stores need no lane predicate
-  IO* const dummy = reinterpret_cast<IO*>(ws + pl.off_status + 128) + (w.tid & 15);
-  const int du_step = fin ? du_ld : 0, dx_step = fin ? P : 0;
-
-  if (w.tid == 0) {
-    for (int i = 0; i < NSTAGE_MAIN; ++i) mbar_init(&full_bar[i], 1);
-    mbar_init(&ckp_bar, 1);
-    mbar_init(&ckp_free, NTHR);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "n"(TM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tm = tmem_base_s + ((uint32_t)(32 * warp) << 16);   // this warp's lanes, column 0 of the allocation
-  // Window liveness of the whole segment, decided before anything is loaded for it.  For every token i of segment s
-  // the window (i, i + Tbar] contains the m - 1 whole segments s+1 .. s+m-1 (m = Tbar / L), so the sum of their Delta
-  // is a lower bound of every window sum of the segment.  If that bound already gives an exit factor below 2^-64 for
-  // every state of every channel of the tile, no exit term of the segment can matter (far below one rounding unit of
-  // mu): the rows Tbar ahead are then neither loaded nor looked at.
-  bool seg_dead = false;
-  if (WIN) {
-    float lb[NCH];
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) lb[c] = 0.f;
-    if (w.act) {
-      const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd);
-      for (int k2 = 1; k2 < pl.m && s + k2 < pl.S; ++k2) {
-        const ChV v = ldg_ch(segd + ((int64_t)b * pl.S + s + k2) * P + w.pa);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) lb[c] += v.v[c];
-      }
-    }
-    bool dead = true;   // channels that do not exist never veto
-    if (w.act) {
-      // least negative exponent scale of each channel over this thread's 8 states; the pair lane tests its own 8
-      const float* al = A_log + (pl.scalar ? (int64_t)w.pa : (int64_t)w.pa * NS + 8 * w.half);
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) {
-        float mn = 3.0e38f;   // smallest A_log = least negative A
-        if (pl.scalar) mn = __ldg(al + c);
-        else
-          for (int n = 0; n < 8; ++n) mn = fminf(mn, __ldg(al + c * NS + n));
-        dead = dead && (lb[c] * (-__expf(mn) * LOG2E) <= -64.f);
-      }
-      // a window that reaches past the sequence end has no exit term at all; tokens whose window ends inside it do
-    }
-    seg_dead = __syncthreads_and(dead ? 1 : 0) != 0;
-  }
-  const bool win_on = WIN && !seg_dead;
-  const uint32_t tx_base = (uint32_t)(CK * CH * ESZ * 2 + CK * CH * 4 + CK * NBC * 4 + ncs * 4 +
-                                      (win_on ? CK * CH * ESZ + CK * CH * 4 : 0));
-  // chunks are visited last to first: the i-th visited chunk is c = nchunk-1-i
-  auto issue = [&](int i) {
-    const int st = i % NSTAGE_MAIN;
-    const int c = nchunk - 1 - i;
-    uint8_t* sm = smem + st * St::BYTES;
-    const int64_t tc = t0 + (int64_t)c * CK;
-    const int64_t row = (int64_t)b * T + tc;
-    const int64_t cc = (int64_t)b * pl.NC + tc / CK;
-    const int64_t row2 = row + tbar;             // first token leaving the window of this chunk's tokens
-    const bool win_rows = win_on && row2 < BT;   // its B/C rows exist (else no token of the chunk has t + Tbar < T)
-    mbar_expect_tx(&full_bar[st], tx_base + (win_rows ? CK * NBC * 4 : 0));
-    tma_2d(sm + St::X, &tmX, tile * CH, row, &full_bar[st]);
-    tma_2d(sm + St::D, &tmD, tile * CH, row, &full_bar[st]);
-    tma_2d(sm + St::G, &tmG, tile * CH, row + grow0, &full_bar[st]);
-    bulk_1d(sm + St::BC, bc + row * NBC, CK * NBC * 4, &full_bar[st]);
-    bulk_1d(sm + St::CS, cs + cc * P + tile * CH, ncs * 4, &full_bar[st]);
-    if (win_on) {
-      // rows of the tokens leaving the window; past the end of the whole tensor TMA fills zeros, and rows
-      // that belong to the next batch element are masked out below (t + Tbar < T fails)
-      tma_2d(sm + St::G2, &tmG, tile * CH, row2 + grow0, &full_bar[st]);
-      tma_2d(sm + St::D2, &tmD, tile * CH, row2, &full_bar[st]);
-      if (win_rows) bulk_1d(sm + St::BC2, bc + row2 * NBC, CK * NBC * 4, &full_bar[st]);
+    for (int i = 0; i < CARRY_UB; ++i) {
+      const bool in = s0 + i < sB;
+      ml[i] = in ? __ldg(muloc + at0 + (s0 + i) * stride) : 0ull;
+      sd[i] = in && t.act ? __ldg(segd + ch0 + (int64_t)(s0 + i) * pl.P) : 0.f;
     }
   };
-  auto issue_ckp = [&](int i) {   // checkpoint tile of the i-th visited chunk (single buffer)
-    const int c = nchunk - 1 - i;
-    const int64_t cc = (int64_t)b * pl.NC + (t0 + (int64_t)c * CK) / CK;
-    mbar_expect_tx(&ckp_bar, TILE_FLOATS * 4);
-    bulk_1d(ckp_s, ckpt + (cc * pl.tiles + tile) * TILE_FLOATS, TILE_FLOATS * 4, &ckp_bar);
-  };
-  if (w.tid == 0) {
-    for (int i = 0; i < NSTAGE_MAIN && i < nchunk; ++i) issue(i);
-    issue_ckp(0);
+  const bool one = n <= CARRY_UB;
+  u64 v = 0ull;
+  float c = 0.f;
+  if (SUF) {   // downwards, starting anew below each block end
+    const int last = sA + max(0, sB - sA - 1) / CARRY_UB * CARRY_UB;
+    const int end0 = sB <= sA ? -1 : sB / m * m - 1;   // highest block end below sB
+    int be = end0;
+    for (int s0 = last; s0 >= sA && sA < sB; s0 -= CARRY_UB) {
+      fetch(s0);
+#pragma unroll
+      for (int i = CARRY_UB - 1; i >= 0; --i) {
+        if (s0 + i == be) { v = 0ull; c = 0.f; be -= m; }
+        v = fma2(decay_of(t.A2, sd[i]), v, ml[i]);
+        c += sd[i];
+      }
+    }
+    sm.val[t.warp][t.lane] = v;
+    sm.dec[t.warp][t.lane] = end0 >= sA ? 0ull : decay_of(t.A2, c);
+    __syncthreads();
+    v = 0ull;
+    for (int w = t.nw - 1; w > t.warp; --w) v = fma2(sm.dec[w][t.lane], v, sm.val[w][t.lane]);
+    be = end0;
+    for (int s0 = last; s0 >= sA && sA < sB; s0 -= CARRY_UB) {
+      if (!one) fetch(s0);
+#pragma unroll
+      for (int i = CARRY_UB - 1; i >= 0; --i) {
+        if (s0 + i == be) { v = 0ull; be -= m; }
+        v = fma2(decay_of(t.A2, sd[i]), v, ml[i]);
+        if (s0 + i < sB) out[at0 + (s0 + i) * stride] = v;
+      }
+    }
+  } else {   // upwards, starting anew at each block start: the decays count from there
+    const int start0 = (sA + m - 1) / m * m;   // lowest block start from sA on
+    double tot = 0.0;
+    int bs = start0;
+    for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+      fetch(s0);
+#pragma unroll
+      for (int i = 0; i < CARRY_UB; ++i) {
+        if (s0 + i == bs && bs < sB) { v = 0ull; c = 0.f; bs += m; }
+        v = fma2(decay_of(t.A2, c), ml[i], v);
+        c += sd[i];
+        if (t.first) tot += (double)sd[i];
+      }
+    }
+    const bool border = start0 < sB;
+    sm.val[t.warp][t.lane] = v;
+    sm.sum[t.warp][t.lane] = border ? -c : c;   // sign bit: the range holds a block start (sums are >= 0)
+    sm.tot[t.warp][t.lane] = tot;
+    __syncthreads();
+    v = 0ull; c = 0.f; tot = 0.0;
+    for (int w = 0; w < t.warp; ++w) {
+      const float x = sm.sum[w][t.lane];
+      if (__float_as_uint(x) >> 31) { v = sm.val[w][t.lane]; c = -x; }
+      else { v = fma2(decay_of(t.A2, c), sm.val[w][t.lane], v); c += x; }
+      tot += sm.tot[w][t.lane];
+    }
+    bs = start0;
+    for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+      if (!one) fetch(s0);
+#pragma unroll
+      for (int i = 0; i < CARRY_UB; ++i) {
+        if (s0 + i == bs && bs < sB) { v = 0ull; c = 0.f; bs += m; }
+        v = fma2(decay_of(t.A2, c), ml[i], v);
+        c += sd[i];
+        if (s0 + i < sB) {
+          out[at0 + (s0 + i) * stride] = v;
+          if (t.first) { tot += (double)sd[i]; total[ch0 + (int64_t)(s0 + i) * pl.P] = tot; }
+        }
+      }
+    }
   }
+}
 
-  u64 A2[NU], mu[NU], dAacc[NU];
-  load_A2(A_log, w, A2, pl.scalar);
-  const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
-  load_block_g(reinterpret_cast<const float*>(ws + pl.off_carry) + sb * TILE_FLOATS, w.tid, mu);
-  {   // true segment-start state: parked in shared memory
-    u64 hst[NU];
-    load_block_g(reinterpret_cast<const float*>(ws + pl.off_hstart) + sb * TILE_FLOATS, w.tid, hst);
+// Can any window-exit term of segment s matter?  If a lower bound of every window sum of Delta already gives an exit factor
+// below 2^-64 for every state of every channel of the tile, none can (far below one rounding unit of mu), and the main
+// kernel neither loads nor looks at the rows Tbar ahead.  The windows of the tokens of a group of LIVE_G chunks that starts
+// at tc contain all chunks between the group and token tc + Tbar.  (In the main kernel's own prologue the same test cost
+// 10 % of its time, 50 us per CTA waiting for the loads.)  One warp per segment and tile, a lane owns four channels.
+constexpr int LIVE_G = 8;
+__device__ __forceinline__ void mark_live(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws, int64_t item) {
+  const int tile = (int)(item % pl.tiles), P = pl.P, m = pl.m, pa = tile * CH + 4 * (threadIdx.x & 31);
+  const int s = (int)(item / pl.tiles % pl.S), b = (int)(item / pl.tiles / pl.S);
+  const int64_t T = pl.T, tbar = pl.tbar, t0 = (int64_t)s * pl.L;
+  const int nchunk = (int)((min(T, t0 + pl.L) - t0 + CK - 1) / CK);
+  // chunks with a token whose window ends inside the sequence
+  const int nexit = (int)max((int64_t)0, min((int64_t)nchunk, (T - tbar - t0 + CK - 1) / CK));
+  bool live = nexit > 0 && m < 1;
+  if (nexit > 0 && m >= 1 && pa < P) {   // channels that do not exist never veto
+    const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd) + (int64_t)b * pl.S * P + pa;
+    const float* cs = reinterpret_cast<const float*>(ws + pl.off_cs) + (int64_t)b * pl.NC * P + pa;
+    auto at4 = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
+    A_log += (int64_t)(b / pl.Bg) * a_stride_dev(pl);
+    float am[4];   // least negative rate over the 16 states
 #pragma unroll
-    for (int q = 0; q < 2 * NCH; ++q) hst_s[q][w.tid] = make_ulonglong2(hst[2 * q], hst[2 * q + 1]);
+    for (int c = 0; c < 4; ++c) {
+      float mn = 3.0e38f;
+      if (pl.scalar) mn = __ldg(A_log + pa + c);
+      else
+#pragma unroll
+        for (int n = 0; n < NS; n += 4) {
+          const float4 v = at4(A_log + (int64_t)(pa + c) * NS + n);
+          mn = fminf(fminf(mn, fminf(v.x, v.y)), fminf(v.z, v.w));
+        }
+      am[c] = -__expf(mn) * LOG2E;
+    }
+    auto alive = [&](const float4& w) {
+      return w.x * am[0] > -64.f || w.y * am[1] > -64.f || w.z * am[2] > -64.f || w.w * am[3] > -64.f;
+    };
+    auto sum = [](const float4& a, const float4& b2, float f) {
+      return make_float4(fmaf(f, b2.x, a.x), fmaf(f, b2.y, a.y), fmaf(f, b2.z, a.z), fmaf(f, b2.w, a.w));
+    };
+    float4 whole = make_float4(0.f, 0.f, 0.f, 0.f);   // Delta of segments s .. s+m-1
+#pragma unroll 4
+    for (int k = s; k < min(s + m, pl.S); ++k) whole = sum(whole, at4(segd + (int64_t)k * P), 1.f);
+    const float4 own = at4(segd + (int64_t)s * P);
+    if (alive(sum(whole, own, -1.f))) {   // the whole segments do not suffice
+      const float4 next = at4(segd + (int64_t)min(s + m, pl.S - 1) * P), last = at4(segd + (int64_t)min(s + m - 1, pl.S - 1) * P);
+      const int cps = pl.L / CK, q0 = s * cps;
+#pragma unroll 4
+      for (int c = 0; c < nexit; c += LIVE_G) {
+        const int q2 = (int)min((t0 + (int64_t)c * CK + tbar + 1) / CK, pl.NC - 1);   // chunks before q2 end at token tc + Tbar or sooner
+        const int d = q2 - q0 - m * cps;   // chunk of segment s + m; one segment further, or (at the very end) one less
+        const float4 hi = at4(cs + (int64_t)q2 * P);
+        const float4 lo = c + LIVE_G < nchunk ? at4(cs + (int64_t)(q0 + c + LIVE_G) * P) : own;
+        float4 w = sum(sum(whole, hi, 1.f), lo, -1.f);
+        if (d < 0) w = sum(w, last, -1.f);
+        if (d >= cps) w = sum(w, next, 1.f);
+        live = live || alive(w);
+      }
+    }
   }
-#pragma unroll
-  for (int u = 0; u < NU; ++u) dAacc[u] = 0ull;
-  // least negative exponent scale of each channel over all 16 states (for the window-term skip test)
-  float a2max[NCH];
-#pragma unroll
-  for (int ch = 0; ch < NCH; ++ch) {
-    float mx = -3.0e38f;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) { float lo, hi; upk(A2[ch * 4 + m], lo, hi); mx = fmaxf(mx, fmaxf(lo, hi)); }
-    a2max[ch] = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  }
-  double sw[NCH];
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) sw[c] = 0.0;
-  if (win_on && w.act) {
-    const double* swp = reinterpret_cast<const double*>(ws + pl.off_swin) + ((int64_t)b * pl.S + s) * P + w.pa;
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) sw[c] = swp[c];
-  }
-  float dbacc = 0.f;
-  bool failed = false;
-  int fail_i = 0, ckp_issued = 0;   // thread 0: where the walk stopped, last checkpoint copy issued
+  const bool any = __any_sync(0xffffffffu, live);
+  if ((threadIdx.x & 31) == 0) reinterpret_cast<int*>(ws + pl.off_live)[((int64_t)b * pl.S + s) * pl.tiles + tile] = any ? 1 : 0;
+}
 
-  // The walk over the segment's chunks, compiled twice: with the window-exit terms and without them (the full form,
-  // and every segment whose exit terms were ruled out above).
-  auto walk_segment = [&](auto winon_tag) {
-  constexpr bool WINON = decltype(winon_tag)::value;
-  for (int i = 0; i < nchunk; ++i) {
-    const int st = i % NSTAGE_MAIN;
-    const int c = nchunk - 1 - i;
-    uint8_t* sm = smem + st * St::BYTES;
-    bool ok = mbar_wait(&full_bar[st], (i / NSTAGE_MAIN) & 1);
-    ok = mbar_wait(&ckp_bar, i & 1) && ok;
-    ok = __all_sync(0xffffffffu, ok);   // warp-uniform: the tensor-memory accesses below are warp-collective
-    const int64_t tc = t0 + (int64_t)c * CK;
-    const int nt = (int)min((int64_t)CK, t1 - tc);
-    const int rb = i & 1;
-    const int nwin = WINON ? (int)max((int64_t)0, min((int64_t)CK, T - tbar - tc)) : 0;   // tokens j < nwin have t + Tbar < T
-    // window Delta sum: fp64 value at the chunk's last token + an fp32 running offset inside the chunk
-    float swc[NCH], swl[NCH], dsumc[NCH], sd2[NCH];
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) { swc[c] = (float)sw[c]; swl[c] = 0.f; dsumc[c] = 0.f; sd2[c] = 0.f; }
-    bool chunk_live = false;   // warp-uniform: does any exit factor W of this chunk reach 2^-64 ?
-    bool tfail = false;
-    if (nt < CK) {   // only the last chunk of a sequence: neutralise the slots past its end
-      if (ok) {
-        zero_rows(sm + St::D, CH * 4, nt, w.tid);
-        zero_rows(sm + St::G, CH * ESZ, nt, w.tid);
-        zero_rows(sm + St::BC, NBC * 4, nt, w.tid);
-      }
-      __syncthreads();
-    }
-    if (ok) {
-      // state at the chunk start: local checkpoint + decayed true segment-start state
-      u64 h[NU];
-      load_block(reinterpret_cast<const float*>(ckp_s), w.tid, h);
-      mbar_arrive(&ckp_free);   // this thread is done with the checkpoint buffer
-      {
-        u64 hst[NU], c2[NCH];
-#pragma unroll
-        for (int q = 0; q < 2 * NCH; ++q) {
-          const ulonglong2 hq = hst_s[q][w.tid];
-          hst[2 * q] = hq.x; hst[2 * q + 1] = hq.y;
-        }
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          float csv = *reinterpret_cast<const float*>(sm + St::CS + 4 * (NCH * w.k + c));
-          if (!w.act) csv = 0.f;   // the 1D copy only covers existing channels
-          c2[c] = pk(csv, csv);
-        }
-        u64 dec[NU];
-        decay_units<SC>(c2, A2, dec);
-#pragma unroll
-        for (int u = 0; u < NU; ++u) h[u] = fma2(dec[u], hst[u], h[u]);
-      }
-      if (WINON) {
-        // Delta of the tokens leaving the window during this chunk.  Inside the chunk the window sum never drops
-        // below (sum at the chunk's last token) - (their total), so if even that bound gives W < 2^-64 for every
-        // state of every lane, the exit terms of the whole chunk are skipped: they are far below one rounding unit
-        // of mu.  The decision is taken once per chunk and per warp.
-#pragma unroll
-        for (int j = 0; j < CK; ++j) {
-          const ChV d2v = lds_ch<float>(sm + St::D2, j, w.k);
-#pragma unroll
-          for (int c = 0; c < NCH; ++c) sd2[c] += j < nwin ? d2v.v[c] : 0.f;
-        }
-        bool live = false;
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) live = live || ((swc[c] - sd2[c]) * a2max[c] > -64.f);
-        chunk_live = __any_sync(0xffffffffu, live && w.act && nwin > 0);
-      }
-      // forward rebuild: the states after the chunk's eight tokens go to tensor memory
-      {
-        const float* bck = reinterpret_cast<const float*>(sm + St::BC) + 8 * w.half;
-#pragma unroll FW_UNROLL
-        for (int j = 0; j < CK; ++j) {
-          const ChV dv = lds_ch<float>(sm + St::D, j, w.k);
-          const ChV xv = lds_ch<IO>(sm + St::X, j, w.k);
-          const float* brow = bck + j * NBC;
-          const ulonglong2 b01 = *reinterpret_cast<const ulonglong2*>(brow);
-          const ulonglong2 b23 = *reinterpret_cast<const ulonglong2*>(brow + 4);
-          const u64 Bp[4] = {b01.x, b01.y, b23.x, b23.y};
-          u64 d2[NCH], dx2[NCH];
-#pragma unroll
-          for (int c = 0; c < NCH; ++c) {
-            const float dxc = dv.v[c] * xv.v[c];
-            d2[c] = pk(dv.v[c], dv.v[c]); dx2[c] = pk(dxc, dxc);
-          }
-          u64 af[NU];
-          decay_units<SC>(d2, A2, af);
-#pragma unroll
-          for (int u = 0; u < NU; ++u) h[u] = fma2(af[u], h[u], mul2(dx2[u / 4], Bp[u % 4]));
-          tmem_st16(tm + TM_TOK * j, h);
-        }
-        tmem_wait_st();
-      }
-      if (w.tid == 0 && i + 1 < nchunk) {
-        // every thread has copied the checkpoint into registers long ago: fetch the next chunk's
-        if (mbar_wait(&ckp_free, i & 1)) { issue_ckp(i + 1); ckp_issued = i + 1; }
-        else tfail = true;
-      }
-      // output rows of this chunk, walked from its last token down
-      IO* du_p = fin ? du + ((int64_t)b * T + tc + (CK - 1)) * du_ld : dummy;
-      IO* dx_p = fin ? dxdir + ((int64_t)b * T + tc + (CK - 1)) * P : dummy;
-      // backward walk: h_i comes back from tensor memory, abar_i h_{i-1} is formed as h_i - Delta_i x_i B_i.
-      // Row pointers walk down with the token.
-      const uint8_t* pD = sm + St::D + (CK - 1) * CH * 4 + 4 * NCH * w.k;       // Delta row (fp32)
-      const uint8_t* pX = sm + St::X + (CK - 1) * CH * ESZ + ESZ * NCH * w.k;   // x row; dy row at + (St::G - St::X)
-      const float* pB = reinterpret_cast<const float*>(sm + St::BC) + 8 * w.half + (CK - 1) * NBC;   // [B | C] row
-      float* pR = &red[rb][warp][CK - 1][((lane >> 1) & 8) * 2 + 8 * w.half + ((lane >> 1) & 7)];
-      uint32_t tmj = tm + TM_TOK * (CK - 1);
-#pragma unroll BW_UNROLL
-      for (int j = CK - 1; j >= 0; --j) {
-        u64 hT[NU];
-        tmem_ld16(tmj, hT);
-        tmj -= TM_TOK;
-        const ChV dv = lds_chp<float>(pD);
-        const ChV xv = lds_chp<IO>(pX);
-        const ChV gv = lds_chp<IO>(pX + (St::G - St::X));
-        const ulonglong2 b01 = *reinterpret_cast<const ulonglong2*>(pB);
-        const ulonglong2 b23 = *reinterpret_cast<const ulonglong2*>(pB + 4);
-        const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(pB + NS);
-        const ulonglong2 c23 = *reinterpret_cast<const ulonglong2*>(pB + NS + 4);
-        const u64 Bp[4] = {b01.x, b01.y, b23.x, b23.y};
-        const u64 Cp[4] = {c01.x, c01.y, c23.x, c23.y};
-        float dd[NCH], xs[NCH];
-        u64 d2[NCH], dx2[NCH], ndx2[NCH], g2[NCH];
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          dd[c] = dv.v[c]; xs[c] = xv.v[c];
-          const float dxc = dv.v[c] * xv.v[c];
-          d2[c] = pk(dd[c], dd[c]); dx2[c] = pk(dxc, dxc); ndx2[c] = pk(-dxc, -dxc); g2[c] = pk(gv.v[c], gv.v[c]);
-        }
-        // mu_i += g_i C_i   (mu already carries abar_{i+1} mu_{i+1})
-#pragma unroll
-        for (int u = 0; u < NU; ++u) mu[u] = fma2(g2[u / 4], Cp[u % 4], mu[u]);
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) dsumc[c] += dd[c];
-        if (WINON && chunk_live) {
-          // exact exit of token t2 = t + Tbar from the window: subtract W_i gC_{t2},
-          // W_i = exp(A * sum_{j=i+1..t2} Delta_j); masked out when t2 >= T
-          const float wm = j < nwin ? 1.f : 0.f;
-          const ChV d2v = lds_chp<float>(pD + (St::D2 - St::D));
-          const ChV g2v = lds_chp<IO>(pX + (St::G2 - St::X));
-          const float* crow = pB + (St::BC2 - St::BC) / 4 + NS;
-          const ulonglong2 e01 = *reinterpret_cast<const ulonglong2*>(crow);
-          const ulonglong2 e23 = *reinterpret_cast<const ulonglong2*>(crow + 4);
-          // rows of tokens past the sequence end are not staged: their C values must not be touched
-          const u64 C2p[4] = {wm != 0.f ? e01.x : 0ull, wm != 0.f ? e01.y : 0ull, wm != 0.f ? e23.x : 0ull,
-                              wm != 0.f ? e23.y : 0ull};
-          u64 ng2[NCH], sw2[NCH];
-#pragma unroll
-          for (int c = 0; c < NCH; ++c) {
-            const float swf = swc[c] + swl[c];
-            ng2[c] = pk(-g2v.v[c] * wm, -g2v.v[c] * wm);
-            sw2[c] = pk(swf, swf);
-            swl[c] += dd[c] - d2v.v[c] * wm;   // window of token t-1: (t-1, t-1+Tbar]
-          }
-          u64 wf[NU];
-          decay_units<SC>(sw2, A2, wf);
-#pragma unroll
-          for (int u = 0; u < NU; ++u) mu[u] = fma2(wf[u], mul2(ng2[u / 4], C2p[u % 4]), mu[u]);
-        }
-        u64 vB[4], vC[4];
-        float ssum[NCH], dsum[NCH];
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-          u64 sacc, dacc;
-          u64 ach = 0ull;
-          if (SC) ach = ex2_2(mul2(d2[ch], A2[ch * 4]));   // scalar rate: one factor for the channel's states
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int u = ch * 4 + m;
-            const u64 a = SC ? ach : ex2_2(mul2(d2[ch], A2[u]));
-            const u64 hn = hT[u];                                  // h_i
-            const u64 hb = fma2(ndx2[ch], Bp[m], hn);              // abar_i h_{i-1} = h_i - Delta_i x_i B_i
-            vB[m] = ch == 0 ? mul2(mu[u], dx2[ch]) : fma2(mu[u], dx2[ch], vB[m]);   // dB partial (two channels)
-            vC[m] = ch == 0 ? mul2(g2[ch], hn) : fma2(g2[ch], hn, vC[m]);           // dC partial
-            sacc = m == 0 ? mul2(mu[u], Bp[m]) : fma2(mu[u], Bp[m], sacc);
-            const u64 q = mul2(mu[u], hb);
-            dacc = m == 0 ? mul2(q, A2[u]) : fma2(q, A2[u], dacc);
-            dAacc[u] = fma2(q, d2[ch], dAacc[u]);
-            mu[u] = mul2(mu[u], a);                                                  // ready for token i-1
-          }
-          ssum[ch] = hsum(sacc);
-          dsum[ch] = hsum(dacc);
-        }
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-          ssum[ch] += __shfl_xor_sync(0xffffffffu, ssum[ch], 1);
-          dsum[ch] += __shfl_xor_sync(0xffffffffu, dsum[ch], 1);
-        }
-        {
-          const float d = chf ? dd[NCH - 1] : dd[0], xx = chf ? xs[NCH - 1] : xs[0];   // selects, not indexed local arrays
-          const float sv = chf ? ssum[NCH - 1] : ssum[0], dsv = chf ? dsum[NCH - 1] : dsum[0];
-          const float ddelta = fmaf(dsv, LN2, xx * sv);
-          // sigmoid(u) = 1 - exp(-Delta).  bf16 outputs: the direct form (absolute error 2e-7) above Delta = 1/32, three
-          // series terms below (relative error < 2e-6); fp32 outputs use the longer cancellation-free form
-          const float sg_small = d * fmaf(d, fmaf(d, 1.f / 6.f, -0.5f), 1.f);
-          const float sg = ESZ == 2 ? (d < 0.03125f ? sg_small : 1.f - ex2_approx(-d * LOG2E)) : sig_from_delta(d);
-          const float duv = ddelta * sg;
-          dbacc += duv;
-          if (j < nt) {
-            st_io<IO>(du_p, duv);
-            st_io<IO>(dx_p, d * sv);
-          }
-          du_p -= du_step;
-          dx_p -= dx_step;
-        }
-        // sum over the warp's 16 channel pairs: every lane parks its 16 partials (dB[8*half+0..7], dC[8*half+0..7])
-        // in shared memory, then lane l adds up value (l >> 1) over the 16 lanes of its parity.  Quarter-blocks
-        // of 4 values are 544 bytes apart so that both the 16-byte stores and the 4-byte loads are conflict-free.
-        {
-          float* wr = wred[warp];
-          __syncwarp();   // the previous token's loads from wr are done
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            *reinterpret_cast<u64*>(wr + (m >> 1) * WRED_Q + lane * 4 + 2 * (m & 1)) = vB[m];
-            *reinterpret_cast<u64*>(wr + (2 + (m >> 1)) * WRED_Q + lane * 4 + 2 * (m & 1)) = vC[m];
-          }
-          __syncwarp();
-          const int vi = lane >> 1;
-          const float* rd = wr + (vi >> 2) * WRED_Q + (lane & 1) * 4 + (vi & 3);
-          float part[16];
-#pragma unroll
-          for (int i2 = 0; i2 < 16; ++i2) part[i2] = rd[i2 * 8];
-#pragma unroll
-          for (int wdt = 8; wdt >= 1; wdt >>= 1)   // pairwise tree: 4 dependent adds instead of 16
-#pragma unroll
-            for (int i2 = 0; i2 < wdt; ++i2) part[i2] += part[i2 + wdt];
-          *pR = part[0];   // this warp's slot: plain store, the four warps are added up when the chunk is flushed
-        }
-        pD -= CH * 4; pX -= CH * ESZ; pB -= NBC; pR -= NBC;
-      }
-    }
-    if (WINON) {
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) sw[c] += (double)(dsumc[c] - sd2[c]);   // window sum at the previous chunk's last token
-    }
-    (void)swl;
-    const int bad = __syncthreads_or((ok && !tfail) ? 0 : 1);
-    if (bad) { failed = true; fail_i = i; break; }
-    if (w.tid == 0 && i + NSTAGE_MAIN < nchunk) issue(i + NSTAGE_MAIN);
-    for (int e = w.tid; e < CK * NBC; e += NTHR) {
-      const int j = e / NBC, q = e % NBC;
-      const float sum = (red[rb][0][j][q] + red[rb][1][j][q]) + (red[rb][2][j][q] + red[rb][3][j][q]);
-      if (j < nt) atomicAdd(dbc + ((int64_t)b * T + tc + j) * NBC + q, sum);
-    }
-  }
-  };
-  if (WIN && !seg_dead) walk_segment(std::integral_constant<bool, WIN>{});
-  else walk_segment(std::false_type{});
-  if (failed) {
-    if (w.tid == 0) {
-      // copies already issued still target this CTA's shared memory: one more bounded wait for each before leaving
-      for (int i2 = fail_i; i2 < nchunk && i2 < fail_i + NSTAGE_MAIN; ++i2)
-        mbar_wait(&full_bar[i2 % NSTAGE_MAIN], (i2 / NSTAGE_MAIN) & 1);
-      mbar_wait(&ckp_bar, ckp_issued & 1);
-      atomicExch(status, AS_ERR_TIMEOUT);
-    }
-  } else {
-    if (w.act && !pl.scalar) {
-#pragma unroll
-      for (int u = 0; u < NU; ++u) {
-        float alo, ahi, vlo, vhi;
-        upk(A2[u], alo, ahi);
-        upk(dAacc[u], vlo, vhi);
-        float* dst = dA_log + (int64_t)(w.pa + u / 4) * NS + 8 * w.half + 2 * (u % 4);
-        atomicAdd(dst, vlo * (alo * LN2));
-        atomicAdd(dst + 1, vhi * (ahi * LN2));
-      }
-    }
-    if (pl.scalar) {   // tied rate: the channel's gradient is the sum over its 16 states (8 here, 8 in the pair lane)
-      float tot[NCH];
-#pragma unroll
-      for (int ch = 0; ch < NCH; ++ch) {
-        tot[ch] = 0.f;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          float alo, ahi, vlo, vhi;
-          upk(A2[ch * 4 + m], alo, ahi);
-          upk(dAacc[ch * 4 + m], vlo, vhi);
-          tot[ch] += vlo * (alo * LN2) + vhi * (ahi * LN2);
-        }
-        tot[ch] += __shfl_xor_sync(0xffffffffu, tot[ch], 1);
-      }
-      if (fin) atomicAdd(dA_log + pmine, chf ? tot[NCH - 1] : tot[0]);
-    }
-    if (fin) atomicAdd(db_delta + pmine, dbacc);
-  }
-  // give the tensor memory back (every exit path comes through here)
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "n"(TM_COLS) : "memory");
-  }
+// All carries of a call in one launch (they are independent): blocks [0, nh) the forward carry, then the suffixes, then
+// (windows of more than four whole segments) the prefixes; shorter windows are summed by the main kernel; one CTA per
+// (slice, tile, batch element) each.  Then (truncated form) the liveness of the segments.
+__global__ void __launch_bounds__(32 * CARRY_WARPS, 1) fixup_kernel(Plan pl, const float* __restrict__ A_log,
+                                                                   char* __restrict__ ws, int nh, int roles) {
+  __shared__ CarrySmem sm;
+  const int role = min((int)blockIdx.x / nh, roles), blk = (int)blockIdx.x - role * nh;
+  const int tile = blk % pl.tiles, rest = blk / pl.tiles;
+  const int b = rest % pl.B, i = rest / pl.B;
+  if (role == roles) {
+    const int64_t item = (int64_t)blk * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (item < (int64_t)pl.tiles * pl.S * pl.B) mark_live(pl, A_log, ws, item);
+  } else if (role == 0) carry_h(pl, A_log, ws, tile, b, i, sm);
+  else if (role == 1) carry_mu<true>(pl, A_log, ws, tile, b, i, sm);
+  else carry_mu<false>(pl, A_log, ws, tile, b, i, sm);
 }
 
 // Self test of the bounded wait: one warp waits for a phase of an mbarrier that nothing will ever complete, with a
@@ -1175,44 +593,6 @@ __global__ void wait_selftest_kernel(int* status, uint32_t limit) {
   if (bad && threadIdx.x == 0) atomicExch(status, AS_ERR_TIMEOUT);
 }
 
-// ---- tensor maps for the [B*T, P] activation tiles (box = CK tokens x bw channels, no swizzle) --------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn get_encode() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-int act_map(CUtensorMap* tm, const void* base, const Plan& pl, int batches, int elem_bytes, bool is_bf16) {
-  EncodeTiledFn enc = get_encode();
-  if (!enc) return 1;
-  cuuint64_t dims[2] = {(cuuint64_t)pl.P, (cuuint64_t)batches * (cuuint64_t)pl.T};
-  cuuint64_t strides[1] = {(cuuint64_t)pl.P * elem_bytes};
-  cuuint32_t box[2] = {(cuuint32_t)CH, (cuuint32_t)CK};   // wider than P when P < CH: the rest is zero-filled
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(tm, is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                   const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? 0 : 1;
-}
-struct Maps { CUtensorMap x, d, g; };
-int make_maps(const Plan& pl, const ScanPtrs& sp, Maps* m) {
-  const bool bf = pl.io == AS_BF16;
-  const int e = bf ? 2 : 4;
-  if (act_map(&m->x, sp.x, pl, pl.B, e, bf)) return 1;
-  if (act_map(&m->d, sp.ws + pl.off_delta, pl, pl.B, 4, false)) return 1;
-  if (act_map(&m->g, sp.dy ? sp.dy : sp.x, pl, sp.dy ? pl.Bg : pl.B, e, bf)) return 1;   // dy: one copy for all layers
-  return 0;
-}
-
-
 template <typename IO, int MODE, bool SC>
 int launch_ascend_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
   Maps m;
@@ -1227,19 +607,6 @@ int launch_ascend_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st
   return (int)cudaGetLastError();
 }
 
-template <typename IO, bool FULL, bool SC>
-int launch_main_t(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
-  Maps m;
-  if (make_maps(pl, sp, &m)) return 1;
-  const int bytes = MainCfg<sizeof(IO), !FULL>::SMEM_DYN;
-  auto kern = adjoint_main_kernel<IO, FULL, SC>;
-  static bool done[AS_MAX_DEVICES] = {};
-  if (ensure_dynamic_smem(kern, bytes, done)) return 1;
-  kern<<<dim3(pl.tiles, pl.S, pl.B), NTHR, bytes, st>>>(m.x, m.d, m.g, pl, sp.A_log, sp.ws, dA_log, db_delta);
-  count_launch();
-  return (int)cudaGetLastError();
-}
-
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------
@@ -1249,12 +616,6 @@ template <typename IO, int MODE>
 int launch_ascend_s(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
   return pl.scalar ? launch_ascend_t<IO, MODE, true>(pl, sp, y, st) : launch_ascend_t<IO, MODE, false>(pl, sp, y, st);
 }
-template <typename IO, bool FULL>
-int launch_main_s(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
-  return pl.scalar ? launch_main_t<IO, FULL, true>(pl, sp, dA_log, db_delta, st)
-                   : launch_main_t<IO, FULL, false>(pl, sp, dA_log, db_delta, st);
-}
-
 int launch_prepass(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st) {
   if (pl.io == AS_BF16)
     return with_mu ? launch_ascend_s<__nv_bfloat16, PRE_ADJ>(pl, sp, nullptr, st)
@@ -1263,8 +624,19 @@ int launch_prepass(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_
 }
 
 int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st) {
-  const int ny_mu = with_mu ? (pl.full ? 1 : pl.S) : 0;
-  fixup_kernel<<<dim3(pl.tiles, NU + ny_mu, pl.B), NTHR, 0, st>>>(pl, sp.A_log, sp.ws, NU);
+  const int64_t nh = (int64_t)CARRY_SLICES * pl.tiles * pl.B;
+  const int roles = !with_mu || pl.direct ? 1 : (pl.full ? 2 : 3);
+  const int64_t nlive = with_mu && !pl.full ? (int64_t)pl.tiles * pl.B * pl.S : 0;
+  // Few CTAs: as many warps as the chip holds, four segments or more each.  Many: eight warps each (T = 65,536, P = 768,
+  // B = 2: 9.7 us; 4 warps 11.6, 16 warps 10.0, 32 warps 16.3).
+  // By one layer's CTAs: a layer's results do not depend on how many it is computed with.
+  int64_t warps = (int64_t)sm_count() * 32 / ((int64_t)CARRY_SLICES * pl.tiles * pl.Bg * roles);
+  if (warps < 8) warps = 8;
+  if (warps > (pl.S + 3) / 4) warps = (pl.S + 3) / 4;
+  if (warps > CARRY_WARPS) warps = CARRY_WARPS;
+  const int64_t blocks = nh * roles + (nlive + warps - 1) / warps;
+  if (blocks > 0x7fffffff) return 1;
+  fixup_kernel<<<(unsigned)blocks, (unsigned)warps * 32, 0, st>>>(pl, sp.A_log, sp.ws, (int)nh, roles);
   count_launch();
   return (int)cudaGetLastError();
 }
@@ -1272,14 +644,6 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
 int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
   if (pl.io == AS_BF16) return launch_ascend_s<__nv_bfloat16, PRE_Y>(pl, sp, y, st);
   return launch_ascend_s<float, PRE_Y>(pl, sp, y, st);
-}
-
-int launch_adjoint_main(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {
-  if (pl.io == AS_BF16)
-    return pl.full ? launch_main_s<__nv_bfloat16, true>(pl, sp, dA_log, db_delta, st)
-                   : launch_main_s<__nv_bfloat16, false>(pl, sp, dA_log, db_delta, st);
-  return pl.full ? launch_main_s<float, true>(pl, sp, dA_log, db_delta, st)
-                 : launch_main_s<float, false>(pl, sp, dA_log, db_delta, st);
 }
 
 int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st) {

@@ -1,0 +1,236 @@
+// Device helpers shared by the scan kernels (as_scan.cu, as_adjoint.cu): packed fp32 arithmetic, staged-copy and mbarrier
+// wrappers, the thread mapping and the tensor maps of the [tokens, d_model] tiles.
+#pragma once
+
+#include <cuda.h>
+
+#include "as_internal.cuh"
+
+namespace as {
+namespace {
+
+typedef unsigned long long u64;   // two packed fp32 values (lo = even state, hi = odd state)
+
+__device__ __forceinline__ int64_t a_stride_dev(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }
+
+__device__ __forceinline__ u64 pk(float lo, float hi) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void upk(u64 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+  u64 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ u64 ex2_2(u64 e) {
+  float lo, hi;
+  upk(e, lo, hi);
+  return pk(ex2_approx(lo), ex2_approx(hi));
+}
+__device__ __forceinline__ float hsum(u64 v) {
+  float lo, hi;
+  upk(v, lo, hi);
+  return lo + hi;
+}
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+constexpr uint32_t WAIT_LIMIT = 1u << 22;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = WAIT_LIMIT) {
+  const uint32_t addr = smem_u32(bar);
+  for (uint32_t it = 0; it < limit; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* tm, int c0, int64_t c1, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(smem_u32(dst)), "l"(tm), "r"(c0), "r"((int)c1), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+template <typename IO> struct IoSz { static constexpr int v = sizeof(IO); };
+
+// per-thread values of its NCH channels
+struct ChV { float v[NCH]; };
+__device__ __forceinline__ ChV ch_zero() { ChV r; for (int c = 0; c < NCH; ++c) r.v[c] = 0.f; return r; }
+
+// row j of a staged [CK x CH] tile, channels NCH*k .. NCH*k + NCH-1
+template <typename IO> __device__ __forceinline__ ChV lds_ch(const uint8_t* tile, int j, int k);
+template <> __device__ __forceinline__ ChV lds_ch<float>(const uint8_t* tile, int j, int k) {
+  ChV r;
+  if (NCH == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(tile + (j * CH + 2 * k) * 4);
+    r.v[0] = t.x; r.v[NCH - 1] = t.y;
+  } else {
+    r.v[0] = *reinterpret_cast<const float*>(tile + (j * CH + k) * 4);
+  }
+  return r;
+}
+template <> __device__ __forceinline__ ChV lds_ch<__nv_bfloat16>(const uint8_t* tile, int j, int k) {
+  ChV r;
+  if (NCH == 2) {
+    const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + (j * CH + 2 * k) * 2));
+    r.v[0] = t.x; r.v[NCH - 1] = t.y;
+  } else {
+    r.v[0] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + (j * CH + k) * 2));
+  }
+  return r;
+}
+// the same from a pointer that already addresses this thread's channels in the row
+template <typename IO> __device__ __forceinline__ ChV lds_chp(const uint8_t* p);
+template <> __device__ __forceinline__ ChV lds_chp<float>(const uint8_t* p) {
+  ChV r;
+  const float2 t = *reinterpret_cast<const float2*>(p);
+  r.v[0] = t.x; r.v[NCH - 1] = t.y;
+  return r;
+}
+template <> __device__ __forceinline__ ChV lds_chp<__nv_bfloat16>(const uint8_t* p) {
+  ChV r;
+  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
+  r.v[0] = t.x; r.v[NCH - 1] = t.y;
+  return r;
+}
+// NCH consecutive floats of a global per-channel array
+__device__ __forceinline__ ChV ldg_ch(const float* p) {
+  ChV r;
+#pragma unroll
+  for (int c = 0; c < NCH; ++c) r.v[c] = __ldg(p + c);
+  return r;
+}
+__device__ __forceinline__ void stg_ch(float* p, const float (&v)[NCH]) {
+#pragma unroll
+  for (int c = 0; c < NCH; ++c) p[c] = v[c];
+}
+
+struct Who {          // what this thread owns
+  int tid, k, half;   // pair index, state half
+  int pa;             // first of its NCH channels
+  bool act;           // the channels exist (P is a multiple of 8, so all or none)
+};
+__device__ __forceinline__ Who who(int tile, int P) {
+  Who w;
+  w.tid = threadIdx.x; w.k = w.tid >> 1; w.half = w.tid & 1;
+  w.pa = tile * CH + NCH * w.k;
+  w.act = w.pa < P;
+  return w;
+}
+// A2[u] = -exp(A_log) * log2(e) for unit u = ch*4 + m  ->  states (8*half + 2m, +1) of channel pa + ch
+// (scalar structure: the channel's single rate for every state)
+__device__ __forceinline__ void load_A2(const float* A_log, const Who& w, u64 (&A2)[NU], int scalar) {
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    float2 v = make_float2(0.f, 0.f);
+    if (w.act) {
+      if (scalar) { const float a = __ldg(A_log + w.pa + u / 4); v = make_float2(a, a); }
+      else v = __ldg(reinterpret_cast<const float2*>(A_log + (int64_t)(w.pa + u / 4) * NS + 8 * w.half + 2 * (u % 4)));
+    }
+    A2[u] = pk(-__expf(v.x) * LOG2E, -__expf(v.y) * LOG2E);
+  }
+}
+// 16 values of this thread inside a 2048-float tile block: float4 q of thread tid at (q*128 + tid)
+__device__ __forceinline__ void load_block(const float* blk, int tid, u64 (&v)[NU]) {
+  const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
+#pragma unroll
+  for (int q = 0; q < 2 * NCH; ++q) {
+    const ulonglong2 t = b2[q * NTHR + tid];
+    v[2 * q] = t.x; v[2 * q + 1] = t.y;
+  }
+}
+__device__ __forceinline__ void load_block_g(const float* blk, int tid, u64 (&v)[NU]) {
+  const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
+#pragma unroll
+  for (int q = 0; q < 2 * NCH; ++q) {
+    const ulonglong2 t = __ldg(b2 + q * NTHR + tid);
+    v[2 * q] = t.x; v[2 * q + 1] = t.y;
+  }
+}
+__device__ __forceinline__ void store_block(float* blk, int tid, const u64 (&v)[NU]) {
+  ulonglong2* b2 = reinterpret_cast<ulonglong2*>(blk);
+#pragma unroll
+  for (int q = 0; q < 2 * NCH; ++q) b2[q * NTHR + tid] = make_ulonglong2(v[2 * q], v[2 * q + 1]);
+}
+
+// sigmoid(u) from Delta = softplus(u): 1 - exp(-Delta), without cancellation for small Delta
+__device__ __forceinline__ float sig_from_delta(float d) {
+  const float big = 1.f - ex2_approx(-d * LOG2E);
+  float s = fmaf(-d, 1.f / 7.f, 1.f);
+  s = fmaf(-d * (1.f / 6.f), s, 1.f);
+  s = fmaf(-d * (1.f / 5.f), s, 1.f);
+  s = fmaf(-d * (1.f / 4.f), s, 1.f);
+  s = fmaf(-d * (1.f / 3.f), s, 1.f);
+  s = fmaf(-d * (1.f / 2.f), s, 1.f);
+  return d < 0.125f ? d * s : big;
+}
+
+// zero the staged rows [nt, CK) of a [CK x CH] tile (row_bytes per token) - all threads of the CTA
+__device__ __forceinline__ void zero_rows(uint8_t* tile, int row_bytes, int nt, int tid) {
+  uint4* p = reinterpret_cast<uint4*>(tile + nt * row_bytes);
+  const int n16 = (CK - nt) * row_bytes / 16;
+  for (int i = tid; i < n16; i += NTHR) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ---- tensor maps for the [B*T, P] activation tiles (box = CK tokens x bw channels, no swizzle) --------
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn get_encode() {
+  static EncodeTiledFn fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<EncodeTiledFn>(p);
+  }
+  return fn;
+}
+int act_map(CUtensorMap* tm, const void* base, const Plan& pl, int batches, int elem_bytes, bool is_bf16, int ld,
+            int width = CH) {
+  EncodeTiledFn enc = get_encode();
+  if (!enc) return 1;
+  cuuint64_t dims[2] = {(cuuint64_t)pl.P, (cuuint64_t)batches * (cuuint64_t)pl.T};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * elem_bytes};
+  cuuint32_t box[2] = {(cuuint32_t)width, (cuuint32_t)CK};   // wider than P when P < CH: the rest is zero-filled
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = enc(tm, is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                   const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? 0 : 1;
+}
+struct Maps { CUtensorMap x, d, g; };
+int make_maps(const Plan& pl, const ScanPtrs& sp, Maps* m) {
+  const bool bf = pl.io == AS_BF16;
+  const int e = bf ? 2 : 4;
+  if (act_map(&m->x, sp.x, pl, pl.B, e, bf, pl.P)) return 1;
+  if (act_map(&m->d, sp.ws + pl.off_delta, pl, pl.B, 4, false, pl.P)) return 1;
+  if (act_map(&m->g, sp.dy ? sp.dy : sp.x, pl, sp.dy ? pl.Bg : pl.B, e, bf, pl.P)) return 1;   // dy: one copy for all layers
+  return 0;
+}
+
+}  // namespace
+}  // namespace as
