@@ -196,6 +196,11 @@ int as_rmsnorm_fwd(const as_shape_t *shape, const void *y, void *yhat, float eps
 /* y_out = y_in + ytilde (the residual connection y_k = y_{k-1} + SSM_k(Norm(y_{k-1}))); y_out may alias y_in. */
 int as_residual_add(const as_shape_t *shape, const void *y_in, const void *ytilde, void *y_out, void *stream);
 
+/* as_residual_add followed by as_rmsnorm_fwd of its result, in one pass: y_out = y_in + ytilde, yhat = norm(y_out).
+ * y_out may alias y_in; yhat may alias ytilde. */
+int as_residual_add_rmsnorm(const as_shape_t *shape, const void *y_in, const void *ytilde, void *y_out, void *yhat,
+                            float eps, void *stream);
+
 /* Backward of the glue: G_inout += RMSNormVJP(y, dyhat) = (dyhat - yhat * mean_p(dyhat*yhat)) / rms(y).
  * G_inout [Bsz,T,P] io dtype is the upstream gradient of y (read and overwritten). */
 int as_rmsnorm_bwd_add(const as_shape_t *shape, const void *y, const void *dyhat, void *G_inout,

@@ -24,7 +24,7 @@ AS_ERR_WORKSPACE, AS_ERR_ALIGN, AS_ERR_CUDA, AS_ERR_TIMEOUT, AS_ERR_LIMIT = -5, 
 EXPORTS = ("as_version", "as_strerror", "as_workspace_bytes", "as_check_status", "as_ssm_forward",
            "as_adjoint_grad", "as_full_bptt_grad", "as_rmsnorm_fwd", "as_residual_add", "as_rmsnorm_bwd_add",
            "as_launch_count", "as_set_timing", "as_get_timing", "as_ssm_forward_static", "as_wait_selftest", "as_sm_count",
-           "as_adjoint_grad_layers", "as_workspace_bytes_layers", "as_wcat_bytes", "as_pack_weights")
+           "as_residual_add_rmsnorm", "as_adjoint_grad_layers", "as_workspace_bytes_layers", "as_wcat_bytes", "as_pack_weights")
 AS_STATIC_SCRATCH_BYTES = 32 << 20
 AS_NUM_PHASES = 6
 PHASES = ("projections", "prepass", "fixup", "adjoint_main", "weight_grads", "input_grad")
@@ -75,6 +75,8 @@ def lib() -> C.CDLL:
                                         C.c_uint32, C.POINTER(as_grads_t), C.c_void_p, C.c_size_t, C.c_void_p]
         L.as_rmsnorm_fwd.argtypes = [C.POINTER(as_shape_t), C.c_void_p, C.c_void_p, C.c_float, C.c_void_p]
         L.as_residual_add.argtypes = [C.POINTER(as_shape_t), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+        L.as_residual_add_rmsnorm.argtypes = [C.POINTER(as_shape_t), C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                              C.c_float, C.c_void_p]
         L.as_rmsnorm_bwd_add.argtypes = [C.POINTER(as_shape_t), C.c_void_p, C.c_void_p, C.c_void_p, C.c_float,
                                          C.c_void_p]
         L.as_ssm_forward_static.argtypes = [C.POINTER(as_shape_t), C.POINTER(as_params_t), C.c_void_p, C.c_void_p,
@@ -237,6 +239,12 @@ def as_rmsnorm_fwd(shape, y, yhat, eps=1e-6, stream=None):
 def as_residual_add(shape, y_in, ytilde, y_out, stream=None):
     _check(lib().as_residual_add(C.byref(shape), _ptr(y_in), _ptr(ytilde), _ptr(y_out), _stream(stream)),
            "as_residual_add")
+
+
+def as_residual_add_rmsnorm(shape, y_in, ytilde, y_out, yhat, eps=1e-6, stream=None):
+    """y_out = y_in + ytilde and yhat = norm(y_out) in one pass."""
+    _check(lib().as_residual_add_rmsnorm(C.byref(shape), _ptr(y_in), _ptr(ytilde), _ptr(y_out), _ptr(yhat), float(eps),
+                                         _stream(stream)), "as_residual_add_rmsnorm")
 
 
 def as_rmsnorm_bwd_add(shape, y, dyhat, G_inout, eps=1e-6, stream=None):

@@ -298,6 +298,7 @@ int as_rmsnorm_fwd(const as_shape_t* shape, const void* y, void* yhat, float eps
   int e = check_shape(shape);
   if (e) return e;
   if (!y || !yhat) return AS_ERR_NULL;
+  if (!aligned16(y) || !aligned16(yhat)) return AS_ERR_ALIGN;
   AS_TRY(launch_rmsnorm_fwd(shape, y, yhat, eps, reinterpret_cast<cudaStream_t>(stream)));
   return AS_OK;
 }
@@ -306,7 +307,18 @@ int as_residual_add(const as_shape_t* shape, const void* y_in, const void* ytild
   int e = check_shape(shape);
   if (e) return e;
   if (!y_in || !ytilde || !y_out) return AS_ERR_NULL;
+  if (!aligned16(y_in) || !aligned16(ytilde) || !aligned16(y_out)) return AS_ERR_ALIGN;
   AS_TRY(launch_residual_add(shape, y_in, ytilde, y_out, reinterpret_cast<cudaStream_t>(stream)));
+  return AS_OK;
+}
+
+int as_residual_add_rmsnorm(const as_shape_t* shape, const void* y_in, const void* ytilde, void* y_out, void* yhat,
+                            float eps, void* stream) {
+  int e = check_shape(shape);
+  if (e) return e;
+  if (!y_in || !ytilde || !y_out || !yhat) return AS_ERR_NULL;
+  if (!aligned16(y_in) || !aligned16(ytilde) || !aligned16(y_out) || !aligned16(yhat)) return AS_ERR_ALIGN;
+  AS_TRY(launch_residual_add_rmsnorm(shape, y_in, ytilde, y_out, yhat, eps, reinterpret_cast<cudaStream_t>(stream)));
   return AS_OK;
 }
 
@@ -315,6 +327,7 @@ int as_rmsnorm_bwd_add(const as_shape_t* shape, const void* y, const void* dyhat
   int e = check_shape(shape);
   if (e) return e;
   if (!y || !dyhat || !G_inout) return AS_ERR_NULL;
+  if (!aligned16(y) || !aligned16(dyhat) || !aligned16(G_inout)) return AS_ERR_ALIGN;
   AS_TRY(launch_rmsnorm_bwd_add(shape, y, dyhat, G_inout, eps, reinterpret_cast<cudaStream_t>(stream)));
   return AS_OK;
 }

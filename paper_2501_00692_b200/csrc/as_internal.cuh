@@ -146,6 +146,8 @@ int launch_zero_regions(const ZeroList& z, cudaStream_t st);
 
 int launch_rmsnorm_fwd(const as_shape_t* sh, const void* y, void* yhat, float eps, cudaStream_t st);
 int launch_residual_add(const as_shape_t* sh, const void* a, const void* b, void* out, cudaStream_t st);
+int launch_residual_add_rmsnorm(const as_shape_t* sh, const void* a, const void* b, void* out, void* yhat, float eps,
+                                cudaStream_t st);
 int launch_rmsnorm_bwd_add(const as_shape_t* sh, const void* y, const void* dyhat, void* G, float eps,
                            cudaStream_t st);
 

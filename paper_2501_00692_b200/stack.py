@@ -43,11 +43,14 @@ class Stack:
     def forward(self, y0: torch.Tensor):
         """Runs the stack, keeping y_0..y_K (the per-layer inputs are re-normalised in the backward)."""
         self.ys = [y0]
-        for th in self.thetas:
-            B.as_rmsnorm_fwd(self.shape, self.ys[-1], self.yhat, self.eps)
+        B.as_rmsnorm_fwd(self.shape, y0, self.yhat, self.eps)
+        for k, th in enumerate(self.thetas):
             B.as_ssm_forward(self.shape, th, self.yhat, self.ytilde, self.ws)
             yk = torch.empty_like(y0)
-            B.as_residual_add(self.shape, self.ys[-1], self.ytilde, yk)
+            if k + 1 < self.K:   # the next layer's input is the norm of the sum: both in one pass
+                B.as_residual_add_rmsnorm(self.shape, self.ys[-1], self.ytilde, yk, self.yhat, self.eps)
+            else:
+                B.as_residual_add(self.shape, self.ys[-1], self.ytilde, yk)
             self.ys.append(yk)
         return self.ys[-1]
 
