@@ -644,6 +644,7 @@ adjoint_main_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                     const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmDu,
                     const __grid_constant__ CUtensorMap tmDx, const __grid_constant__ Plan pl, const float* __restrict__ A_log,
                     char* __restrict__ ws, float* __restrict__ dA_log, float* __restrict__ db_delta) {
+  pdl_begin();
   const int lay = (int)blockIdx.z / pl.Bg;   // this layer's rates and parameter-gradient rows; dy is shared by the layers
   A_log += (int64_t)lay * a_stride_dev(pl);
   dA_log += (int64_t)lay * a_stride_dev(pl);
@@ -667,9 +668,8 @@ int launch_main_t(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_d
   auto kern = adjoint_main_kernel<IO, FULL, SC>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
-  kern<<<dim3(pl.tiles, pl.S, pl.B), NTHR, bytes, st>>>(m.x, m.d, m.g, mdu, mdx, pl, sp.A_log, sp.ws, dA_log, db_delta);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, mdu, mdx, pl, sp.A_log, sp.ws,
+                          dA_log, db_delta);
 }
 template <typename IO, bool SC>
 int launch_main_s(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st) {

@@ -51,25 +51,25 @@ int check_params(const as_params_t* pr) {
     if (e__ != 0) return AS_ERR_CUDA;     \
   } while (0)
 
-// Wcat of the call and how often it holds W_B and W_C: the caller's packed copy if it gave one, else packed here into the
-// scratch.  The gradient of a width that is not a multiple of 32 needs them once per term of the dB, dC split.
+// Wcat of the call and how often it holds W_B and W_C
 struct Wcat { const void* p; int reps; };
-int wcat_of(const Plan& pl, const as_params_t* pr, bool grad, char* ws, cudaStream_t st, Wcat* wcat) {
-  wcat->reps = grad ? pl.gsplit : 1;
-  if (pr->Wcat && wcat->reps == 1) { wcat->p = pr->Wcat; return AS_OK; }
-  char* at = ws + (grad ? pl.off_wcatx : pl.off_wcat);
-  AS_TRY(tc_pack_wcat(pl.P, pl.KL, wcat->reps, pr, at, st));
-  wcat->p = at;
-  return AS_OK;
-}
 
-// steps 1-3 of SSM(.): Delta = softplus(x W_delta^T + b), B = x W_B^T, C = x W_C^T  (every layer of the call)
-int projections(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const void* x, char* ws, cudaStream_t st) {
-  if (pl.tc) {
-    AS_TRY(tc_projections(pl, pr, wcat.p, wcat.reps, x, ws, st));
+// What every call begins with: the regions `z` are cleared, Wcat is the caller's packed copy if it gave one or else packed into
+// the scratch, and steps 1-3 of SSM(.) run: Delta = softplus(x W_delta^T + b), B = x W_B^T, C = x W_C^T (every layer of the
+// call).  The gradient of a width that is not a multiple of 32 needs W_B and W_C once per term of the dB, dC split.
+int begin(const Plan& pl, const as_params_t* pr, const ZeroList& z, bool grad, const void* x, char* ws, cudaStream_t st,
+          Wcat* wcat) {
+  if (!pl.tc) {
+    AS_TRY(simt_projections(pl, pr, x, z, ws, st));
     return AS_OK;
   }
-  AS_TRY(simt_projections(pl, pr, x, ws, st));
+  wcat->reps = grad ? pl.gsplit : 1;
+  const bool packed = pr->Wcat && wcat->reps == 1;
+  char* at = ws + (grad ? pl.off_wcatx : pl.off_wcat);
+  wcat->p = packed ? pr->Wcat : at;
+  // with packed weights the projections clear the regions themselves
+  if (!packed) AS_TRY(launch_prepare(z, pl.P, pl.KL, wcat->reps, pr, at, st));
+  AS_TRY(tc_projections(pl, pr, wcat->p, wcat->reps, x, packed ? z : ZeroList{}, ws, st));
   return AS_OK;
 }
 
@@ -103,21 +103,21 @@ int check_grad_args(const as_shape_t* sh, const as_params_t* pr, const void* x, 
   return AS_OK;
 }
 
-int zero_outputs(const Plan& pl, uint32_t flags, const as_grads_t* out, char* ws, cudaStream_t st) {
+// regions a call accumulates into (the status block is always the first)
+void add_region(ZeroList* z, void* p, size_t bytes) { z->ptr[z->n] = p; z->bytes[z->n] = (bytes + 15) / 16 * 16; ++z->n; }
+ZeroList grad_regions(const Plan& pl, uint32_t flags, const as_grads_t* out, char* ws) {
   const size_t P = pl.P, K = pl.KL;
   ZeroList z{};
-  auto add = [&](void* p, size_t bytes) { z.ptr[z.n] = p; z.bytes[z.n] = (bytes + 15) / 16 * 16; ++z.n; };
-  add(ws + pl.off_status, 256);
-  add(ws + pl.off_dbc, (size_t)pl.B * pl.T * NBC * 4);
+  add_region(&z, ws + pl.off_status, 256);
+  add_region(&z, ws + pl.off_dbc, (size_t)pl.B * pl.T * NBC * 4);
   if (!(flags & AS_ACCUMULATE)) {
-    add(out->dW_delta, K * P * P * 4);
-    add(out->db_delta, K * P * 4);
-    add(out->dW_B, K * NS * P * 4);
-    add(out->dW_C, K * NS * P * 4);
-    add(out->dA_log, K * (pl.scalar ? P : P * NS) * 4);
+    add_region(&z, out->dW_delta, K * P * P * 4);
+    add_region(&z, out->db_delta, K * P * 4);
+    add_region(&z, out->dW_B, K * NS * P * 4);
+    add_region(&z, out->dW_C, K * NS * P * 4);
+    add_region(&z, out->dA_log, K * (pl.scalar ? P : P * NS) * 4);
   }
-  AS_TRY(launch_zero_regions(z, st));
-  return AS_OK;
+  return z;
 }
 
 }  // namespace
@@ -187,10 +187,10 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
   if (ws_bytes < pl.total_fwd) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
-  AS_TRY((int)cudaMemsetAsync(w + pl.off_status, 0, 256, st));
   Wcat wcat{};
-  if (pl.tc) { e = wcat_of(pl, params, false, w, st, &wcat); if (e) return e; }
-  e = projections(pl, params, wcat, x, w, st);
+  ZeroList z{};
+  add_region(&z, w + pl.off_status, 256);
+  e = begin(pl, params, z, false, x, w, st, &wcat);
   if (e) return e;
   ScanPtrs sp{x, nullptr, params->A_log, w};
   const bool mm = forward_y_mm_applies(pl);
@@ -235,7 +235,7 @@ int as_pack_weights(const as_shape_t* shape, int32_t layers, const as_params_t* 
   if (!aligned16(wcat)) return AS_ERR_ALIGN;
   if (layers < 1) return AS_ERR_SHAPE;
   if (shape->io != AS_BF16) return AS_ERR_DTYPE;   // only the bf16 tensor-core contractions read a packed copy
-  AS_TRY(tc_pack_wcat(shape->d_model, layers, 1, params, wcat, reinterpret_cast<cudaStream_t>(stream)));
+  AS_TRY(launch_prepare(ZeroList{}, shape->d_model, layers, 1, params, wcat, reinterpret_cast<cudaStream_t>(stream)));
   return AS_OK;
 }
 
@@ -254,11 +254,8 @@ int as_adjoint_grad_layers(const as_shape_t* shape, int32_t layers, const as_par
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
   mark(0, st);
-  e = zero_outputs(pl, flags, out, w, st);
-  if (e) return e;
   Wcat wcat{};
-  if (pl.tc) { e = wcat_of(pl, params, true, w, st, &wcat); if (e) return e; }
-  e = projections(pl, params, wcat, x, w, st);
+  e = begin(pl, params, grad_regions(pl, flags, out, w), true, x, w, st, &wcat);
   if (e) return e;
   mark(1, st);
   ScanPtrs sp{x, dy, params->A_log, w};
@@ -283,11 +280,8 @@ int as_full_bptt_grad(const as_shape_t* shape, const as_params_t* params, const 
   if (ws_bytes < pl.total_grad) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
-  e = zero_outputs(pl, flags, out, w, st);
-  if (e) return e;
   Wcat wcat{};
-  if (pl.tc) { e = wcat_of(pl, params, true, w, st, &wcat); if (e) return e; }
-  e = projections(pl, params, wcat, x, w, st);
+  e = begin(pl, params, grad_regions(pl, flags, out, w), true, x, w, st, &wcat);
   if (e) return e;
   ScanPtrs sp{x, dy, params->A_log, w};
   AS_TRY(launch_bptt(pl, sp, out->dA_log, out->db_delta, st));

@@ -25,6 +25,7 @@ struct SimtArgs {
   float *dW_delta, *dW_B, *dW_C, *dx;
   int64_t M;                         // token rows per layer
   int P, layers, splitk;
+  ZeroList zero;                     // PROJ: regions to clear for the later kernels of the call
   int ndx;                           // gradient launch: number of DX blocks (they come first); 0 when dx is not wanted
 };
 
@@ -175,12 +176,15 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)
 __global__ void __launch_bounds__(NT) simt_proj_kernel(const __grid_constant__ SimtArgs a) {
   __shared__ __align__(16) float As[2][BK][PADM];
   __shared__ __align__(16) float Bs[2][BK][PADN];
+  pdl_begin();
+  clear_regions(a.zero, (int64_t)blockIdx.x * NT + threadIdx.x, (int64_t)gridDim.x * NT);
   tile<C_PROJ>(a, blockIdx.x, As, Bs);
 }
 // both gradient contractions: the first ndx blocks compute dx, the rest the weight gradients
 __global__ void __launch_bounds__(NT) simt_grad_kernel(const __grid_constant__ SimtArgs a) {
   __shared__ __align__(16) float As[2][BK][PADM];
   __shared__ __align__(16) float Bs[2][BK][PADN];
+  pdl_begin();
   if ((int)blockIdx.x < a.ndx) tile<C_DX>(a, blockIdx.x, As, Bs);
   else tile<C_DW>(a, (int64_t)blockIdx.x - a.ndx, As, Bs);
 }
@@ -194,14 +198,13 @@ SimtArgs base_args(const Plan& pl, const as_params_t* pr, const void* x) {
 }
 }  // namespace
 
-int simt_projections(const Plan& pl, const as_params_t* pr, const void* x, char* ws, cudaStream_t st) {
+int simt_projections(const Plan& pl, const as_params_t* pr, const void* x, const ZeroList& z, char* ws, cudaStream_t st) {
   SimtArgs a = base_args(pl, pr, x);
+  a.zero = z;
   a.delta = (float*)(ws + pl.off_delta); a.bc = (float*)(ws + pl.off_bc);
   const int64_t blocks = cdiv(a.M, BM) * cdiv(pl.P + NBC, BN) * a.layers;
   if (blocks > 0x7fffffff) return 1;
-  simt_proj_kernel<<<(unsigned)blocks, NT, 0, st>>>(a);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(simt_proj_kernel, dim3((unsigned)blocks), dim3(NT), 0, st, a);
 }
 
 int simt_gradients(const Plan& pl, const as_params_t* pr, const void* x, const as_grads_t* out, char* ws, cudaStream_t st) {
@@ -217,9 +220,7 @@ int simt_gradients(const Plan& pl, const as_params_t* pr, const void* x, const a
   a.ndx = (int)ndx;
   const int64_t blocks = ndx + tiles * a.splitk;
   if (blocks > 0x7fffffff) return 1;
-  simt_grad_kernel<<<(unsigned)blocks, NT, 0, st>>>(a);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(simt_grad_kernel, dim3((unsigned)blocks), dim3(NT), 0, st, a);
 }
 
 }  // namespace as

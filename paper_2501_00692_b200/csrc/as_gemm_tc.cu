@@ -48,6 +48,7 @@ struct TcArgs {
   const float* bias;    // PROJ: b_delta [layers, P]
   float* bc;            // PROJ: [B | C] rows, for the plain stores where P is not a multiple of 16
   int* status;
+  ZeroList zero;        // PROJ: regions to clear for the later kernels, where the call has no kernel before this one
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -197,6 +198,8 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  pdl_begin();
+  if (EPI == TC_PROJ && a.zero.n > 0) clear_regions(a.zero, (int64_t)blockIdx.x * NTHREADS + threadIdx.x, (int64_t)gridDim.x * NTHREADS);
   if (warp == 1) {   // TMEM allocation: two BN-column fp32 accumulators
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(Cfg<BN>::TMEM_COLS)
                  : "memory");
@@ -444,23 +447,11 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
 }
 
 // ---- small helpers -------------------------------------------------------------------------------
-// Wcat[l] = [W_delta[l]; W_B[l]; W_C[l]] for every layer l (blockIdx.y), W_B and W_C `reps` times over
-__global__ void pack_wcat_kernel(int P, int reps, const __nv_bfloat16* __restrict__ Wd, const __nv_bfloat16* __restrict__ WB,
-                                 const __nv_bfloat16* __restrict__ WC, __nv_bfloat16* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n = (int64_t)(P + reps * NBC) * P;
-  if (i >= n) return;
-  const int64_t l = blockIdx.y;
-  Wd += l * P * P; WB += l * NS * P; WC += l * NS * P; out += l * n;
-  const int64_t row = i / P, col = i % P;
-  const int64_t e = (row - P) & (NBC - 1);
-  out[i] = row < P ? Wd[i] : (e < NS ? WB[e * P + col] : WC[(e - NS) * P + col]);
-}
-
 // [dB | dC] fp32 sums -> the last bf16 columns of Gcat; eight values per thread (P and the row pitch are multiples of 8
 // elements, so every access is 16-byte aligned).  SPLIT: as three bf16 terms, 32 columns each, that add up to the fp32 value.
 template <int SPLIT>
 __global__ void cvt_dbc_kernel(int64_t rows, int ldg, int P, const float* __restrict__ dbc, __nv_bfloat16* __restrict__ gcat) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // one group of 8 columns
   if (i >= rows * (NBC / 8)) return;
   const int64_t row = i / (NBC / 8);
@@ -531,9 +522,7 @@ int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorM
   const int64_t ntiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * (EPI == TC_DW ? a.layers : 1);
   const int sms = sm_count();
   const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);   // one persistent CTA per SM
-  kern<<<grid, NTHREADS, Cfg<BN>::SMEM_DYN, st>>>(tmA, tmB, tmO[0], tmO[1], tmO[2], a);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(kern, dim3(grid), dim3(NTHREADS), Cfg<BN>::SMEM_DYN, st, tmA, tmB, tmO[0], tmO[1], tmO[2], a);
 }
 
 template <int AMAJ, int BMAJ, int EPI, int BN>
@@ -550,15 +539,6 @@ int launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap 
 constexpr int TBN = 256;   // tile width of the weight-gradient and input-gradient contractions
 constexpr int PBN = 208;   // projections: N = P + 32; for P = 768 four 208-wide tiles waste 4 % where 256 wastes 22 %
 
-int tc_pack_wcat(int P, int layers, int reps, const as_params_t* pr, void* wcat, cudaStream_t st) {
-  const int64_t n = (int64_t)(P + reps * NBC) * P;
-  pack_wcat_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)layers), 256, 0, st>>>(
-      P, reps, (const __nv_bfloat16*)pr->W_delta, (const __nv_bfloat16*)pr->W_B, (const __nv_bfloat16*)pr->W_C,
-      (__nv_bfloat16*)wcat);
-  count_launch();
-  return (int)cudaGetLastError();
-}
-
 // The layers of a call go out as one launch when no 128-row tile straddles two layers (token rows per layer a
 // multiple of BM); otherwise one launch per layer, on that layer's slab of every tensor.
 struct LayerLoop { int first, count; };
@@ -568,7 +548,8 @@ static inline int layer_groups(const Plan& pl, LayerLoop* g) {
   return 0;   // the caller loops over single layers
 }
 
-int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x, char* ws, cudaStream_t st) {
+int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x,
+                   const ZeroList& z, char* ws, cudaStream_t st) {
   const int64_t rows = (int64_t)pl.Bg * pl.T;
   const int P = pl.P, NW = P + wreps * NBC;
   LayerLoop one;
@@ -582,6 +563,7 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int 
     TcArgs a{};
     a.M = M; a.N = P + NBC; a.kblocks = (P + BK - 1) / BK; a.splitk = 1; a.P = P; a.wrows = NW; a.layers = nl; a.rows_layer = rows;
     a.bias = pr->b_delta + (size_t)l0 * P;
+    if (l0 == 0) a.zero = z;
     a.bc = (float*)(ws + pl.off_bc) + (size_t)l0 * rows * NBC;
     a.status = (int*)(ws + pl.off_status);
     CUtensorMap tmO[3];
@@ -599,10 +581,9 @@ int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* 
   const int64_t Mall = rows * pl.KL;
   const int P = pl.P, NW = pl.du_ld;
   auto cvt = pl.gsplit == 3 ? cvt_dbc_kernel<3> : cvt_dbc_kernel<1>;
-  cvt<<<(unsigned)((Mall * (NBC / 8) + 255) / 256), 256, 0, st>>>(Mall, NW, P, (const float*)(ws + pl.off_dbc),
-                                                                       (__nv_bfloat16*)(ws + pl.off_du));
-  count_launch();
-  if (cudaGetLastError() != cudaSuccess) return 1;
+  if (launch_dependent(cvt, dim3((unsigned)((Mall * (NBC / 8) + 255) / 256)), dim3(256), 0, st, Mall, NW, P,
+                       (const float*)(ws + pl.off_dbc), (__nv_bfloat16*)(ws + pl.off_du)))
+    return 1;
   LayerLoop one;
   const bool batched = layer_groups(pl, &one) == 1;
   for (int l0 = 0; l0 < pl.KL; l0 += batched ? pl.KL : 1) {

@@ -49,6 +49,7 @@ __device__ __forceinline__ float stored(float v, __nv_bfloat16) { return __bfloa
 template <typename IO, int NP, bool ADD>
 __global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* __restrict__ b, IO* sum, IO* __restrict__ yhat,
                                    float eps) {
+  pdl_begin();
   constexpr int N = Vec<IO>::N;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -106,6 +107,7 @@ __global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* _
 template <typename IO, int NP>
 __global__ void rmsnorm_bwd_add_kernel(int64_t rows, int P, const IO* __restrict__ y, const IO* __restrict__ dyhat,
                                        IO* __restrict__ G, float eps) {
+  pdl_begin();
   constexpr int N = Vec<IO>::N, NK = NP > 0 ? NP : 1;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -156,6 +158,7 @@ __global__ void rmsnorm_bwd_add_kernel(int64_t rows, int P, const IO* __restrict
 
 template <typename IO>
 __global__ void residual_add_kernel(int64_t n, const IO* a, const IO* __restrict__ b, IO* out) {
+  pdl_begin();
   constexpr int N = Vec<IO>::N;
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * N;
   if (i >= n) return;
@@ -185,29 +188,24 @@ template <typename IO, bool ADD>
 int norm_fwd(const as_shape_t* sh, const void* a, const void* b, void* sum, void* yhat, float eps, cudaStream_t st) {
   const int64_t rows = (int64_t)sh->batch * sh->seqlen;
   return with_pieces<IO>(sh->d_model, [&](auto np) {
-    rmsnorm_fwd_kernel<IO, decltype(np)::value, ADD><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
-        rows, sh->d_model, (const IO*)a, (const IO*)b, (IO*)sum, (IO*)yhat, eps);
-    count_launch();
-    return (int)cudaGetLastError();
+    return launch_dependent(rmsnorm_fwd_kernel<IO, decltype(np)::value, ADD>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st,
+                            rows, sh->d_model, (const IO*)a, (const IO*)b, (IO*)sum, (IO*)yhat, eps);
   });
 }
 template <typename IO>
 int norm_bwd(const as_shape_t* sh, const void* y, const void* dyhat, void* G, float eps, cudaStream_t st) {
   const int64_t rows = (int64_t)sh->batch * sh->seqlen;
   return with_pieces<IO>(sh->d_model, [&](auto np) {
-    rmsnorm_bwd_add_kernel<IO, decltype(np)::value><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
-        rows, sh->d_model, (const IO*)y, (const IO*)dyhat, (IO*)G, eps);
-    count_launch();
-    return (int)cudaGetLastError();
+    return launch_dependent(rmsnorm_bwd_add_kernel<IO, decltype(np)::value>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st,
+                            rows, sh->d_model, (const IO*)y, (const IO*)dyhat, (IO*)G, eps);
   });
 }
 template <typename IO>
 int add_rows(const as_shape_t* sh, const void* a, const void* b, void* out, cudaStream_t st) {
   const int64_t n = (int64_t)sh->batch * sh->seqlen * sh->d_model;
   const int64_t pieces = n / Vec<IO>::N;
-  residual_add_kernel<IO><<<(unsigned)((pieces + 255) / 256), 256, 0, st>>>(n, (const IO*)a, (const IO*)b, (IO*)out);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(residual_add_kernel<IO>, dim3((unsigned)((pieces + 255) / 256)), dim3(256), 0, st, n, (const IO*)a,
+                          (const IO*)b, (IO*)out);
 }
 }  // namespace
 
@@ -231,29 +229,40 @@ int launch_residual_add(const as_shape_t* sh, const void* a, const void* b, void
 }
 
 // One launch clears every buffer a gradient call accumulates into (status block, the [dB|dC] accumulator and, unless
-// the caller accumulates, the five parameter gradients): seven separate memsets cost more in launch gaps than in
-// bytes.  All regions are 16-byte aligned and a multiple of 16 bytes long.
+// the caller accumulates, the five parameter gradients) and packs the weights: separate memsets and kernels cost more in
+// launch gaps than in bytes.  All regions are 16-byte aligned and a multiple of 16 bytes long; rows of the weights are
+// copied in 16-byte pieces.
 namespace {
-__global__ void zero_regions_kernel(ZeroList z) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int r = 0; r < z.n; ++r) {
-    uint4* p = reinterpret_cast<uint4*>(z.ptr[r]);
-    const int64_t n16 = (int64_t)(z.bytes[r] / 16);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
+__global__ void prepare_kernel(ZeroList z, int zblocks, int P, int layers, int reps, const uint4* __restrict__ Wd,
+                               const uint4* __restrict__ WB, const uint4* __restrict__ WC, uint4* __restrict__ out) {
+  pdl_begin();
+  if ((int)blockIdx.x < zblocks) {
+    clear_regions(z, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)zblocks * blockDim.x);
+    return;
   }
+  const int q = P / 8;                                  // 16-byte pieces of a bf16 row
+  const int64_t n = (int64_t)(P + reps * NBC) * q;      // pieces of one layer's Wcat
+  const int64_t i = ((int64_t)blockIdx.x - zblocks) * blockDim.x + threadIdx.x;
+  if (i >= n * layers) return;
+  const int64_t l = i / n, row = (i - l * n) / q, col = i % q;
+  const int64_t e = (row - P) & (NBC - 1);
+  out[i] = row < P ? Wd[(l * P + row) * q + col] : (e < NS ? WB[(l * NS + e) * q + col] : WC[(l * NS + e - NS) * q + col]);
 }
 }  // namespace
 
-int launch_zero_regions(const ZeroList& z, cudaStream_t st) {
+int launch_prepare(const ZeroList& z, int P, int layers, int reps, const as_params_t* pr, void* wcat, cudaStream_t st) {
   size_t total = 0;
   for (int r = 0; r < z.n; ++r) total += z.bytes[r];
-  int64_t blocks = (int64_t)((total / 16 + 255) / 256);
+  int64_t zblocks = (int64_t)((total / 16 + 255) / 256);
   const int64_t cap = (int64_t)sm_count() * 8;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  zero_regions_kernel<<<(unsigned)blocks, 256, 0, st>>>(z);
-  count_launch();
-  return (int)cudaGetLastError();
+  if (zblocks > cap) zblocks = cap;
+  const int64_t pieces = pr ? (int64_t)layers * (P + reps * NBC) * (P / 8) : 0;
+  const int64_t blocks = zblocks + (pieces + 255) / 256;
+  if (blocks < 1) return 0;
+  if (blocks > 0x7fffffff) return 1;
+  return launch_dependent(prepare_kernel, dim3((unsigned)blocks), dim3(256), 0, st, z, (int)zblocks, P, layers, reps,
+                          (const uint4*)(pr ? pr->W_delta : nullptr), (const uint4*)(pr ? pr->W_B : nullptr),
+                          (const uint4*)(pr ? pr->W_C : nullptr), (uint4*)wcat);
 }
 
 }  // namespace as

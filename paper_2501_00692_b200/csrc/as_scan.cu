@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
   A_log += (int64_t)(b / pl.Bg) * a_stride_dev(pl);   // this layer's rates
   const int bg = b % pl.Bg;                            // dy is shared by the layers: its rows know only the batch element
 
+  pdl_begin();
   if (w.tid == 0) {
     for (int i = 0; i < NSTAGE; ++i) mbar_init(&full_bar[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -568,6 +569,7 @@ __device__ __forceinline__ void mark_live(const Plan& pl, const float* __restric
 __global__ void __launch_bounds__(32 * CARRY_WARPS, 1) fixup_kernel(Plan pl, const float* __restrict__ A_log,
                                                                    char* __restrict__ ws, int nh, int roles) {
   __shared__ CarrySmem sm;
+  pdl_begin();
   const int role = min((int)blockIdx.x / nh, roles), blk = (int)blockIdx.x - role * nh;
   const int tile = blk % pl.tiles, rest = blk / pl.tiles;
   const int b = rest % pl.B, i = rest / pl.B;
@@ -602,9 +604,7 @@ int launch_ascend_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st
   auto kern = ascend_kernel<IO, MODE, SC>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
-  kern<<<dim3(pl.tiles, pl.S, pl.B), NTHR, bytes, st>>>(m.x, m.d, m.g, pl, sp.A_log, sp.ws, (IO*)y);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, pl, sp.A_log, sp.ws, (IO*)y);
 }
 
 }  // namespace
@@ -636,9 +636,7 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
   if (warps > CARRY_WARPS) warps = CARRY_WARPS;
   const int64_t blocks = nh * roles + (nlive + warps - 1) / warps;
   if (blocks > 0x7fffffff) return 1;
-  fixup_kernel<<<(unsigned)blocks, (unsigned)warps * 32, 0, st>>>(pl, sp.A_log, sp.ws, (int)nh, roles);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(fixup_kernel, dim3((unsigned)blocks), dim3((unsigned)warps * 32), 0, st, pl, sp.A_log, sp.ws, (int)nh, roles);
 }
 
 int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {

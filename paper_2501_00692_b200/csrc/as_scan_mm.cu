@@ -175,6 +175,7 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   const float* bc = reinterpret_cast<const float*>(ws + pl.off_bc);
   int* status = reinterpret_cast<int*>(ws + pl.off_status);
   const int pch = tile * MCH + pc;                                   // this thread's channel
+  pdl_begin();
   const float a2 = -__expf(__ldg(A_log + (int64_t)(b / pl.Bg) * P + pch)) * LOG2E;   // a_p log2(e)
 
   if (tid == 0) {
@@ -550,9 +551,7 @@ int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_
   auto kern = scalar_mm_kernel<true>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
-  kern<<<dim3(pl.P / MCH, pl.S, pl.B), MT, SMEM_DYN, st>>>(mx, md, my, pl, sp.A_log, sp.ws, (__nv_bfloat16*)y);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, my, pl, sp.A_log, sp.ws, (__nv_bfloat16*)y);
 }
 
 int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st) {
@@ -562,9 +561,8 @@ int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st)
   auto kern = scalar_mm_kernel<false>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
-  kern<<<dim3(pl.P / MCH, pl.S, pl.B), MT, SMEM_DYN, st>>>(mx, md, mx, pl, sp.A_log, sp.ws, nullptr);
-  count_launch();
-  return (int)cudaGetLastError();
+  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, mx, pl, sp.A_log, sp.ws,
+                          (__nv_bfloat16*)nullptr);
 }
 
 }  // namespace as
