@@ -44,6 +44,13 @@ template <> __device__ __forceinline__ void st_vec<__nv_bfloat16>(__nv_bfloat16*
 __device__ __forceinline__ float stored(float v, float) { return v; }
 __device__ __forceinline__ float stored(float v, __nv_bfloat16) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
+// The sums over a row, in bf16: lane l adds elements l, l + 32, ... in that order, whatever the layout of the loads, through a
+// copy of the row in shared memory.  A deep stack of bf16 layers turns differences of one rounding unit of a norm into
+// differences of some per cent of its gradients (12 layers: 2 %), so a wider load should not change the order.
+// fp32 rows are added up as they lie.
+template <typename IO> constexpr bool kOrdered = sizeof(IO) == 2;
+constexpr int NORM_WARPS = 4;   // rows per CTA
+
 // One row per warp.  NP = 16-byte pieces of a row per lane, or 0: any width, the row read again for the second pass.
 // ADD: the row is a + b, stored to `sum` (which may alias a), and the norm is that of the stored row.
 template <typename IO, int NP, bool ADD>
@@ -51,8 +58,10 @@ __global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* _
                                    float eps) {
   pdl_begin();
   constexpr int N = Vec<IO>::N;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  extern __shared__ __align__(16) uint8_t row_s[];
+  const int64_t row = (int64_t)blockIdx.x * NORM_WARPS + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
+  IO* copy = reinterpret_cast<IO*>(row_s) + (threadIdx.x / 32) * P;
   if (row >= rows) return;
   auto get = [&](int c, float (&v)[N]) {
     ld_vec<IO>(a + row * P + c, v);
@@ -72,8 +81,16 @@ __global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* _
 #pragma unroll
       for (int e = 0; e < N; ++e) v[k][e] = 0.f;
       if (c < P) get(c, v[k]);
+      if (kOrdered<IO>) {
+        if (c < P) st_vec<IO>(copy + c, v[k]);
+      } else {
 #pragma unroll
-      for (int e = 0; e < N; ++e) ss = fmaf(v[k][e], v[k][e], ss);
+        for (int e = 0; e < N; ++e) ss = fmaf(v[k][e], v[k][e], ss);
+      }
+    }
+    if (kOrdered<IO>) {
+      __syncwarp();
+      for (int i = lane; i < P; i += 32) { const float t = (float)copy[i]; ss = fmaf(t, t, ss); }
     }
     const float rinv = 1.f / sqrtf(wsum(ss) / (float)P + eps);
 #pragma unroll
@@ -90,8 +107,13 @@ __global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* _
     for (int c = lane * N; c < P; c += 32 * N) {
       get(c, v);
 #pragma unroll
-      for (int e = 0; e < N; ++e) ss = fmaf(v[e], v[e], ss);
+      for (int e = 0; e < N; ++e)
+        if (!kOrdered<IO>) ss = fmaf(v[e], v[e], ss);
       if (ADD) st_vec<IO>(sum + row * P + c, v);
+    }
+    if (kOrdered<IO>) {
+      __syncwarp();   // the row as the warp wrote it (ADD) or as it came
+      for (int i = lane; i < P; i += 32) { const float t = (float)(ADD ? sum : a)[row * P + i]; ss = fmaf(t, t, ss); }
     }
     const float rinv = 1.f / sqrtf(wsum(ss) / (float)P + eps);
     for (int c = lane * N; c < P; c += 32 * N) {
@@ -109,8 +131,10 @@ __global__ void rmsnorm_bwd_add_kernel(int64_t rows, int P, const IO* __restrict
                                        IO* __restrict__ G, float eps) {
   pdl_begin();
   constexpr int N = Vec<IO>::N, NK = NP > 0 ? NP : 1;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  extern __shared__ __align__(16) uint8_t row_s[];
+  const int64_t row = (int64_t)blockIdx.x * NORM_WARPS + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
+  IO* copy = reinterpret_cast<IO*>(row_s) + (threadIdx.x / 32) * 2 * P;   // y, then dyhat
   if (row >= rows) return;
   const IO* yr = y + row * P;
   const IO* dr = dyhat + row * P;
@@ -140,7 +164,19 @@ __global__ void rmsnorm_bwd_add_kernel(int64_t rows, int P, const IO* __restrict
       if (c < P) { yq[k] = raw(yr + c); dq[k] = raw(dr + c); gq[k] = raw(gr + c); }
     }
 #pragma unroll
-    for (int k = 0; k < NP; ++k) sums(yq[k], dq[k]);
+    for (int k = 0; k < NP; ++k) {
+      const int c = (k * 32 + lane) * N;
+      if (!kOrdered<IO>) sums(yq[k], dq[k]);
+      else if (c < P) { *reinterpret_cast<uint4*>(copy + c) = yq[k]; *reinterpret_cast<uint4*>(copy + P + c) = dq[k]; }
+    }
+    if (kOrdered<IO>) {
+      __syncwarp();
+      for (int i = lane; i < P; i += 32) {
+        const float v = (float)copy[i];
+        ss = fmaf(v, v, ss);
+        dot = fmaf(v, (float)copy[P + i], dot);
+      }
+    }
     ss = wsum(ss); dot = wsum(dot);
     const float rinv = 1.f / sqrtf(ss / (float)P + eps), m = dot * rinv / (float)P;   // m = mean_p(dyhat * yhat)
 #pragma unroll
@@ -149,7 +185,15 @@ __global__ void rmsnorm_bwd_add_kernel(int64_t rows, int P, const IO* __restrict
       if (c < P) add(c, yq[k], dq[k], gq[k], rinv, m);
     }
   } else {
-    for (int c = lane * N; c < P; c += 32 * N) sums(raw(yr + c), raw(dr + c));
+    if (kOrdered<IO>) {
+      for (int i = lane; i < P; i += 32) {
+        const float v = (float)yr[i];
+        ss = fmaf(v, v, ss);
+        dot = fmaf(v, (float)dr[i], dot);
+      }
+    } else {
+      for (int c = lane * N; c < P; c += 32 * N) sums(raw(yr + c), raw(dr + c));
+    }
     ss = wsum(ss); dot = wsum(dot);
     const float rinv = 1.f / sqrtf(ss / (float)P + eps), m = dot * rinv / (float)P;
     for (int c = lane * N; c < P; c += 32 * N) add(c, raw(yr + c), raw(dr + c), raw(gr + c), rinv, m);
@@ -188,7 +232,8 @@ template <typename IO, bool ADD>
 int norm_fwd(const as_shape_t* sh, const void* a, const void* b, void* sum, void* yhat, float eps, cudaStream_t st) {
   const int64_t rows = (int64_t)sh->batch * sh->seqlen;
   return with_pieces<IO>(sh->d_model, [&](auto np) {
-    return launch_dependent(rmsnorm_fwd_kernel<IO, decltype(np)::value, ADD>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st,
+    return launch_dependent(rmsnorm_fwd_kernel<IO, decltype(np)::value, ADD>, dim3((unsigned)((rows + NORM_WARPS - 1) / NORM_WARPS)),
+                            dim3(32 * NORM_WARPS), kOrdered<IO> && decltype(np)::value > 0 ? NORM_WARPS * sh->d_model * sizeof(IO) : 0, st,
                             rows, sh->d_model, (const IO*)a, (const IO*)b, (IO*)sum, (IO*)yhat, eps);
   });
 }
@@ -196,7 +241,8 @@ template <typename IO>
 int norm_bwd(const as_shape_t* sh, const void* y, const void* dyhat, void* G, float eps, cudaStream_t st) {
   const int64_t rows = (int64_t)sh->batch * sh->seqlen;
   return with_pieces<IO>(sh->d_model, [&](auto np) {
-    return launch_dependent(rmsnorm_bwd_add_kernel<IO, decltype(np)::value>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st,
+    return launch_dependent(rmsnorm_bwd_add_kernel<IO, decltype(np)::value>, dim3((unsigned)((rows + NORM_WARPS - 1) / NORM_WARPS)),
+                            dim3(32 * NORM_WARPS), kOrdered<IO> && decltype(np)::value > 0 ? 2 * NORM_WARPS * sh->d_model * sizeof(IO) : 0, st,
                             rows, sh->d_model, (const IO*)y, (const IO*)dyhat, (IO*)G, eps);
   });
 }
