@@ -177,7 +177,8 @@ int as_full_bptt_grad(const as_shape_t *shape, const as_params_t *params, const 
  * budget, a latency-critical loop that cannot afford cudaMalloc's device-wide synchronisation).  Same result as
  * as_ssm_forward, but the scratch is a fixed AS_STATIC_SCRATCH_BYTES array inside the library's device image:
  *   - every GPU context that loads the library holds that much memory until exit;
- *   - a shape whose forward scratch (as_workspace_bytes, fwd_bytes) is larger returns AS_ERR_LIMIT, nothing runs;
+ *   - a shape whose forward scratch is larger (as_workspace_bytes, fwd_bytes; large fp32 shapes can do with less than that)
+ *     returns AS_ERR_LIMIT, nothing runs;
  *   - the first call on a device resolves the array's device address (a synchronous runtime query made with that
  *     device current): make it during set-up, before any stream capture;
  *   - all calls on a device share the array and it keeps the previous call's contents (what must start at zero is

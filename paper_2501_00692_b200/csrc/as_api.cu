@@ -60,7 +60,7 @@ struct Wcat { const void* p; int reps; };
 int begin(const Plan& pl, const as_params_t* pr, const ZeroList& z, bool grad, const void* x, char* ws, cudaStream_t st,
           Wcat* wcat) {
   if (!pl.tc) {
-    AS_TRY(simt_projections(pl, pr, x, z, ws, st));
+    AS_TRY(pl.split ? split_projections(pl, pr, x, z, ws, st) : simt_projections(pl, pr, x, z, ws, st));
     return AS_OK;
   }
   wcat->reps = grad ? pl.gsplit : 1;
@@ -83,7 +83,8 @@ int contractions(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const 
     mark(6, st);
     return AS_OK;
   }
-  AS_TRY(simt_gradients(pl, pr, x, out, ws, st));   // both contractions in one launch: the second phase reads zero
+  // both contractions count as the first phase: the second reads zero
+  AS_TRY(pl.split ? split_gradients(pl, out, ws, st) : simt_gradients(pl, pr, x, out, ws, st));
   mark(5, st);
   mark(6, st);
   return AS_OK;
@@ -149,7 +150,12 @@ int as_workspace_bytes(const as_shape_t* shape, int64_t tbar, size_t* fwd_bytes,
   Plan pl;
   e = make_plan(shape, tbar, 1, &pl);
   if (e) return e;
-  if (fwd_bytes) *fwd_bytes = pl.total_fwd;
+  if (fwd_bytes) {
+    Plan pf;
+    e = make_plan(shape, shape->seqlen, 1, &pf, PLAN_FWD);
+    if (e) return e;
+    *fwd_bytes = pf.total_fwd;
+  }
   if (grad_bytes) {
     *grad_bytes = pl.total_grad;
     e = make_plan(shape, shape->seqlen, 1, &pl);   // as_full_bptt_grad and the full form cut the time differently
@@ -182,8 +188,12 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
   if (!x || !y || !ws) return AS_ERR_NULL;
   if (!aligned16(x) || !aligned16(y) || !aligned16(ws)) return AS_ERR_ALIGN;
   Plan pl;
-  e = make_plan(shape, shape->seqlen, 1, &pl);
+  e = make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD);
   if (e) return e;
+  if (ws_bytes < pl.total_fwd && pl.split) {   // the fixed scratch of as_ssm_forward_static may only hold the smaller plan
+    e = make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD_SMALL);
+    if (e) return e;
+  }
   if (ws_bytes < pl.total_fwd) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);

@@ -1,0 +1,394 @@
+// fp32 contractions on the bf16 tensor cores, without giving up fp32 accuracy.
+//
+// An fp32 value is the exact sum of three bf16 terms (8 significant bits each), v = v1 + v2 + v3.  Of the nine products of two
+// such sums the six with i + j <= 4 are formed; the other three are below 2^-26 of |a||b|, a quarter of the rounding of one
+// fp32 multiply-add.  Products of bf16 values are exact in the tensor core.  What could lose accuracy is its accumulation,
+// whose error grows with the number of steps (measured: fp32's own at 256 terms, six times that at 8,192), so:
+//   - the leading products a1 b1 and the five small ones go into accumulators of their own,
+//   - every 128 terms of the contraction both are added to fp32 registers by ordinary additions.
+// Errors against fp64 then are those of an fp32 FMA kernel or smaller (tests/test_gpu_split.py checks it).
+//
+// Bound: the L2 -> shared-memory path (96 KB per 64-deep block of a 128 x 128 tile feed 24 MMAs of 64 cycles).  8,192 tokens
+// x 768: projections 294 us on the FP32 pipe.  The three terms are written once per call by split kernels (6 bytes per value).
+#include <cuda.h>
+
+#include "as_tc.cuh"
+
+namespace as {
+namespace {
+
+constexpr int BM = 128, BN = 128, BK = 64, UK = 16, EPI_WARPS = 8, NTHREADS = 64 + 32 * EPI_WARPS;
+constexpr int TILE = 128 * BK * 2;                   // one operand term: 128 rows (or columns) x 64 of the contraction
+constexpr int STAGE = 6 * TILE, STAGES = 2;
+constexpr int GROUP = 2;                             // blocks between two drains of the accumulators
+constexpr int STG = 32 * 64;                         // staging tile of an epilogue warp: 32 rows of 64 bytes
+constexpr int SMEM_DYN = STAGES * STAGE + 1024 + EPI_WARPS * STG;
+
+struct SplitArgs {
+  int64_t R;            // output rows per layer (PROJ, DX: tokens; DW: P + 32)
+  int N;                // output columns
+  int kblocks;          // BK-blocks of the contraction
+  int splitk, kper;     // DW: splits of the contraction, blocks per split (a multiple of GROUP)
+  int P, layers;
+  int64_t M;            // tokens per layer
+  const float* bias;    // PROJ: b_delta
+  float* bc;            // PROJ: [B | C] rows
+  const float* dxdir;   // DX
+  int* status;
+};
+
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(smem_u32(dst)), "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, const void* src, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+               ::"l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(src)) : "memory");
+}
+__device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* tm, const void* src, int c0, int c1, int c2) {
+  asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2, %3}], [%4];"
+               ::"l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(src)) : "memory");
+}
+__device__ __forceinline__ float softplus_exact(float u) { return fmaxf(u, 0.f) + log1pf(expf(-fabsf(u))); }
+
+// Persistent, warp-specialised, one CTA per SM, as the bf16 kernel: warp 0 loads (one lane), warp 1 issues the MMAs (one
+// lane), eight epilogue warps keep 64 columns of 32 rows each in registers and drain one pair of accumulators while the
+// other pair fills.
+template <int AMAJ, int BMAJ, int EPI>
+__global__ void __launch_bounds__(NTHREADS) gemm_split_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                              const __grid_constant__ CUtensorMap tmB,
+                                                              const __grid_constant__ CUtensorMap tmO0,
+                                                              const __grid_constant__ CUtensorMap tmO1,
+                                                              const __grid_constant__ CUtensorMap tmO2,
+                                                              const __grid_constant__ SplitArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tmem_full_bar[2], tmem_empty_bar[2];
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int abort_s;
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int mt = (int)((a.R + BM - 1) / BM), nt = (a.N + BN - 1) / BN;
+  const int ntiles = mt * nt * a.splitk * a.layers;
+  volatile int* abortp = &abort_s;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full_bar[b], 1); mbar_init(&tmem_empty_bar[b], EPI_WARPS); }
+    abort_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  pdl_begin();
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "n"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = tmem_base_s;
+
+  auto decode = [&](int t, int& m0, int& n0, int& kb0, int& nkb, int& lay) {
+    n0 = t % nt * BN;
+    t /= nt;
+    m0 = t % mt * BM;
+    t /= mt;
+    kb0 = t % a.splitk * a.kper;
+    lay = t / a.splitk;
+    nkb = max(0, min(a.kblocks, kb0 + a.kper) - kb0);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        int m0, n0, kb0, nkb, lay;
+        decode(t, m0, n0, kb0, nkb, lay);
+        for (int i = 0; i < nkb; ++i, ++it) {
+          const int s = it % STAGES, round = it / STAGES;
+          if (round > 0 && !mbar_wait(&empty_bar[s], (round - 1) & 1, abortp)) { ok = false; break; }
+          uint8_t* st = smem + s * STAGE;
+          mbar_expect_tx(&full_bar[s], STAGE);
+          const int k = (kb0 + i) * BK;
+#pragma unroll
+          for (int p = 0; p < 3; ++p) {
+            const int z = lay * 3 + p;
+            uint8_t* sa = st + p * TILE;
+            uint8_t* sb = st + (3 + p) * TILE;
+            if (AMAJ == MAJ_K) {
+              tma_load_3d(sa, &tmA, k, m0, z, &full_bar[s]);
+            } else {
+              tma_load_3d(sa, &tmA, m0, k, z, &full_bar[s]);
+              tma_load_3d(sa + TILE / 2, &tmA, m0 + 64, k, z, &full_bar[s]);
+            }
+            if (BMAJ == MAJ_K) {
+              tma_load_3d(sb, &tmB, k, n0, z, &full_bar[s]);
+            } else {
+              tma_load_3d(sb, &tmB, n0, k, z, &full_bar[s]);
+              tma_load_3d(sb + TILE / 2, &tmB, n0 + 64, k, z, &full_bar[s]);
+            }
+          }
+        }
+      }
+      if (!ok) { *abortp = 1; atomicExch(a.status, AS_ERR_TIMEOUT); }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)AMAJ << 15) | ((uint32_t)BMAJ << 16) |
+                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      int it = 0, gi = 0;   // blocks and drain groups so far
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        int m0, n0, kb0, nkb, lay;
+        decode(t, m0, n0, kb0, nkb, lay);
+        for (int i = 0; i < nkb; ++i, ++it) {
+          const int s = it % STAGES, round = it / STAGES, ab = gi & 1, around = gi >> 1;
+          const bool first = i % GROUP == 0;
+          if (first) {
+            if (around > 0 && !mbar_wait(&tmem_empty_bar[ab], (around - 1) & 1, abortp)) { ok = false; break; }
+          }
+          if (!mbar_wait(&full_bar[s], round & 1, abortp)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t base = smem_u32(smem + s * STAGE), acc = tmem_base + (uint32_t)(ab * 256);
+          auto term = [&](int pa, int pb, uint32_t d, bool fresh) {
+#pragma unroll
+            for (int k = 0; k < BK / UK; ++k) {
+              const uint32_t sa = base + pa * TILE, sb = base + (3 + pb) * TILE;
+              const uint64_t ad = AMAJ == MAJ_K ? make_desc(sa + k * UK * 2, 16, 1024) : make_desc(sa + k * UK * 128, TILE / 2, 1024);
+              const uint64_t bd = BMAJ == MAJ_K ? make_desc(sb + k * UK * 2, 16, 1024) : make_desc(sb + k * UK * 128, TILE / 2, 1024);
+              umma_bf16(d, ad, bd, idesc, fresh && k == 0 ? 0u : 1u);
+            }
+          };
+          term(2, 0, acc + BN, first);
+          term(0, 2, acc + BN, false);
+          term(1, 1, acc + BN, false);
+          term(1, 0, acc + BN, false);
+          term(0, 1, acc + BN, false);
+          term(0, 0, acc, first);
+          umma_commit(&empty_bar[s]);
+          if (i % GROUP == GROUP - 1 || i + 1 == nkb) { umma_commit(&tmem_full_bar[ab]); ++gi; }
+        }
+      }
+      if (!ok) { *abortp = 1; atomicExch(a.status, AS_ERR_TIMEOUT); }
+    }
+  } else {
+    // A warp owns TMEM lanes [32 quarter, 32 quarter + 32) = 32 output rows, one row per lane, and 64 of the tile's columns.
+    const int quarter = warp & 3, c_lo = (warp - 2) / 4 * 64;
+    uint8_t* stg = smem + STAGES * STAGE + (warp - 2) * STG;
+    int gi = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      int m0, n0, kb0, nkb, lay;
+      decode(t, m0, n0, kb0, nkb, lay);
+      float acc[64];
+#pragma unroll
+      for (int i = 0; i < 64; ++i) acc[i] = 0.f;
+      for (int g = 0; g < (nkb + GROUP - 1) / GROUP; ++g, ++gi) {
+        const int ab = gi & 1;
+        if (!mbar_wait(&tmem_full_bar[ab], (gi >> 1) & 1, abortp)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t at = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * 256 + c_lo);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          uint32_t r[16], q[16];
+          tmem_ld16(at + 16 * h, r);
+          tmem_ld16(at + BN + 16 * h, q);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[16 * h + i] += __uint_as_float(r[i]) + __uint_as_float(q[i]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tmem_empty_bar[ab]);
+      }
+      if (!ok) break;
+      const int mrow = m0 + quarter * 32, row = mrow + lane;   // first row of the warp, row of the lane (inside the layer)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int nb = n0 + c_lo + 16 * h;
+        if (nb >= a.N || nkb == 0) continue;   // warp-uniform
+        if (lane == 0) bulk_wait_read<0>();
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int col = nb + 4 * q;   // four columns: all inside one part (its border is a multiple of 8) or all outside
+          float4 v = make_float4(acc[16 * h + 4 * q], acc[16 * h + 4 * q + 1], acc[16 * h + 4 * q + 2], acc[16 * h + 4 * q + 3]);
+          if (EPI == TC_PROJ) {
+            if (col < a.P) {
+              const float4 bv = __ldg(reinterpret_cast<const float4*>(a.bias + (int64_t)lay * a.P + col));
+              v = make_float4(softplus_exact(v.x + bv.x), softplus_exact(v.y + bv.y), softplus_exact(v.z + bv.z), softplus_exact(v.w + bv.w));
+            } else if (col < a.P + NBC && row < a.M) {
+              *reinterpret_cast<float4*>(a.bc + ((int64_t)lay * a.M + row) * NBC + col - a.P) = v;
+            }
+          }
+          if (EPI == TC_DX && col < a.P && row < a.M) {
+            const float4 d = __ldg(reinterpret_cast<const float4*>(a.dxdir + ((int64_t)lay * a.M + row) * a.P + col));
+            v = make_float4(v.x + d.x, v.y + d.y, v.z + d.z, v.w + d.w);
+          }
+          *reinterpret_cast<float4*>(stg + swz64(lane, q)) = v;
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (EPI != TC_DW) {
+            if (nb < a.P) tma_store_3d(&tmO0, stg, nb, mrow, lay);   // clipped at the layer's rows and at column P
+          } else {
+            // rows of Gcat space: [0, P) dW_delta, then 16 rows dW_B and 16 rows dW_C; eight rows never straddle two outputs
+#pragma unroll
+            for (int r0 = 0; r0 < 32; r0 += 8) {
+              const int mr = mrow + r0, e = mr - a.P;
+              if (e < 0) tma_reduce_add_3d(&tmO0, stg + r0 * 64, nb, mr, lay);
+              else if (e < NS) tma_reduce_add_3d(&tmO1, stg + r0 * 64, nb, e, lay);
+              else if (e < NBC) tma_reduce_add_3d(&tmO2, stg + r0 * 64, nb, e - NS, lay);
+            }
+          }
+          bulk_commit();
+        }
+      }
+    }
+    if (lane == 0) bulk_wait_all();
+    if (!ok) { *abortp = 1; if (lane == 0) atomicExch(a.status, AS_ERR_TIMEOUT); }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(512) : "memory");
+}
+
+// ---- fp32 -> three bf16 terms, eight values per thread ----
+__device__ __forceinline__ void split8(const float* src, __nv_bfloat16* dst, int64_t plane) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(src)), b = __ldg(reinterpret_cast<const float4*>(src) + 1);
+  float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    uint4 o;
+    __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      o2[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+      const float2 f = __bfloat1622float2(o2[k]);
+      v[2 * k] -= f.x; v[2 * k + 1] -= f.y;   // exact
+    }
+    *reinterpret_cast<uint4*>(dst + p * plane) = o;
+  }
+}
+// clears the regions, splits x into [layer][term][M][P] and the weights into [layer][term][P + 32][P]
+__global__ void split_inputs_kernel(ZeroList z, int P, int64_t M, int layers, const float* __restrict__ x, const float* __restrict__ Wd,
+                                    const float* __restrict__ WB, const float* __restrict__ WC, __nv_bfloat16* __restrict__ xs,
+                                    __nv_bfloat16* __restrict__ wsp) {
+  pdl_begin();
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  clear_regions(z, first, stride);
+  const int q = P / 8;
+  const int64_t nx = M * q, nw = (int64_t)(P + NBC) * q, total = (nx + nw) * layers;
+  for (int64_t i = first; i < total; i += stride) {
+    if (i < nx * layers) {
+      const int64_t l = i / nx, e = i - l * nx;
+      split8(x + i * 8, xs + (l * 3 * nx + e) * 8, nx * 8);
+    } else {
+      const int64_t k = i - nx * layers, l = k / nw, e = k - l * nw, row = e / q, col = (e - row * q) * 8, r = row - P;
+      const float* src = row < P ? Wd + (l * P + row) * P + col : (r < NS ? WB + (l * NS + r) * P + col : WC + (l * NS + r - NS) * P + col);
+      split8(src, wsp + (l * 3 * nw + e) * 8, nw * 8);
+    }
+  }
+}
+// [du | dB | dC] -> [layer][term][M][P + 32]
+__global__ void split_g_kernel(int P, int64_t M, int layers, const float* __restrict__ du, const float* __restrict__ dbc,
+                               __nv_bfloat16* __restrict__ gs) {
+  pdl_begin();
+  const int q = (P + NBC) / 8;
+  const int64_t n = M * q, total = n * layers, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+    const int64_t l = i / n, e = i - l * n, m = e / q, row = l * M + m;
+    const int c = (int)(e - m * q) * 8;
+    split8(c < P ? du + row * P + c : dbc + row * NBC + c - P, gs + (l * 3 * n + e) * 8, n * 8);
+  }
+}
+
+// [planes, rows, cols] row-major; box {box_cols, box_rows, 1}
+int map3(CUtensorMap* tm, bool f32, const void* base, uint64_t planes, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
+  EncodeTiledFn enc = get_encode();
+  if (!enc) return 1;
+  const uint64_t e = f32 ? 4 : 2;
+  cuuint64_t dims[3] = {cols, rows, planes};
+  cuuint64_t strides[2] = {cols * e, rows * cols * e};
+  cuuint32_t box[3] = {box_cols, box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return enc(tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
+             box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, f32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS ? 0 : 1;
+}
+
+template <int AMAJ, int BMAJ, int EPI>
+int launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const SplitArgs& a, cudaStream_t st) {
+  auto kern = gemm_split_kernel<AMAJ, BMAJ, EPI>;
+  static bool done[AS_MAX_DEVICES] = {};
+  if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
+  const int64_t ntiles = ((a.R + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * a.layers;
+  if (ntiles > 0x7fffffff) return 1;
+  const int sms = sm_count();
+  return launch_dependent(kern, dim3((unsigned)(ntiles < sms ? ntiles : sms)), dim3(NTHREADS), SMEM_DYN, st, tmA, tmB, tmO[0], tmO[1],
+                          tmO[2], a);
+}
+SplitArgs base_args(const Plan& pl, char* ws) {
+  SplitArgs a{};
+  a.P = pl.P; a.layers = pl.KL; a.M = (int64_t)pl.Bg * pl.T; a.splitk = 1;
+  a.status = (int*)(ws + pl.off_status);
+  return a;
+}
+unsigned split_blocks(int64_t pieces) {
+  const int64_t b = (pieces + 255) / 256, cap = (int64_t)sm_count() * 16;
+  return (unsigned)(b < cap ? b : cap);
+}
+}  // namespace
+
+int split_projections(const Plan& pl, const as_params_t* pr, const void* x, const ZeroList& z, char* ws, cudaStream_t st) {
+  SplitArgs a = base_args(pl, ws);
+  __nv_bfloat16* xs = (__nv_bfloat16*)(ws + pl.off_xs);
+  __nv_bfloat16* wsp = (__nv_bfloat16*)(ws + pl.off_wsp);
+  const int64_t pieces = (a.M + pl.P + NBC) * (pl.P / 8) * pl.KL;
+  if (launch_dependent(split_inputs_kernel, dim3(split_blocks(pieces)), dim3(256), 0, st, z, pl.P, a.M, pl.KL, (const float*)x,
+                       (const float*)pr->W_delta, (const float*)pr->W_B, (const float*)pr->W_C, xs, wsp))
+    return 1;
+  CUtensorMap tmA, tmB, tmO[3];
+  if (map3(&tmA, false, xs, 3 * pl.KL, a.M, pl.P, 64, BM)) return 1;
+  if (map3(&tmB, false, wsp, 3 * pl.KL, pl.P + NBC, pl.P, 64, BN)) return 1;
+  if (map3(&tmO[0], true, ws + pl.off_delta, pl.KL, a.M, pl.P, 16, 32)) return 1;
+  tmO[1] = tmO[2] = tmO[0];
+  a.R = a.M; a.N = pl.P + NBC; a.kblocks = (pl.P + BK - 1) / BK; a.kper = a.kblocks;
+  a.bias = pr->b_delta; a.bc = (float*)(ws + pl.off_bc);
+  return launch_split<MAJ_K, MAJ_K, TC_PROJ>(tmA, tmB, tmO, a, st);
+}
+
+int split_gradients(const Plan& pl, const as_grads_t* out, char* ws, cudaStream_t st) {
+  SplitArgs a = base_args(pl, ws);
+  const int P = pl.P, NW = P + NBC;
+  const __nv_bfloat16* xs = (const __nv_bfloat16*)(ws + pl.off_xs);
+  const __nv_bfloat16* wsp = (const __nv_bfloat16*)(ws + pl.off_wsp);
+  __nv_bfloat16* gs = (__nv_bfloat16*)(ws + pl.off_gs);
+  if (launch_dependent(split_g_kernel, dim3(split_blocks(a.M * (NW / 8) * pl.KL)), dim3(256), 0, st, P, a.M, pl.KL,
+                       (const float*)(ws + pl.off_du), (const float*)(ws + pl.off_dbc), gs))
+    return 1;
+  CUtensorMap tmA, tmB, tmO[3];
+  if (map3(&tmA, false, gs, 3 * pl.KL, a.M, NW, 64, BK)) return 1;    // Gcat as [K = tokens, M = P + 32]
+  if (map3(&tmB, false, xs, 3 * pl.KL, a.M, P, 64, BK)) return 1;     // X as [K = tokens, N = P]
+  if (map3(&tmO[0], true, out->dW_delta, pl.KL, P, P, 16, 8)) return 1;
+  if (map3(&tmO[1], true, out->dW_B, pl.KL, NS, P, 16, 8)) return 1;
+  if (map3(&tmO[2], true, out->dW_C, pl.KL, NS, P, 16, 8)) return 1;
+  a.R = NW; a.N = P; a.kblocks = (int)((a.M + BK - 1) / BK);
+  const int64_t tiles = (int64_t)((NW + BM - 1) / BM) * ((P + BN - 1) / BN) * pl.KL;
+  int64_t sk = sm_count() / tiles;   // about one tile per persistent CTA
+  if (sk < 1) sk = 1;
+  a.kper = (int)(((a.kblocks + sk - 1) / sk + GROUP - 1) / GROUP * GROUP);
+  a.splitk = (a.kblocks + a.kper - 1) / a.kper;   // no empty split
+  int e = launch_split<MAJ_MN, MAJ_MN, TC_DW>(tmA, tmB, tmO, a, st);
+  if (e || !out->dx) return e;
+  if (map3(&tmA, false, gs, 3 * pl.KL, a.M, NW, 64, BM)) return 1;    // Gcat as [M = tokens, K = P + 32]
+  if (map3(&tmB, false, wsp, 3 * pl.KL, NW, P, 64, BK)) return 1;     // Wcat as [K = P + 32, N = P]
+  if (map3(&tmO[0], true, out->dx, pl.KL, a.M, P, 16, 32)) return 1;
+  tmO[1] = tmO[2] = tmO[0];
+  a.R = a.M; a.N = P; a.kblocks = (NW + BK - 1) / BK; a.kper = a.kblocks; a.splitk = 1;
+  a.dxdir = (const float*)(ws + pl.off_dxdir);
+  return launch_split<MAJ_K, MAJ_MN, TC_DX>(tmA, tmB, tmO, a, st);
+}
+
+}  // namespace as

@@ -118,15 +118,20 @@ struct Plan {
   int tiles;        // ceil(P / CH) channel tiles
   int bw;           // channels per staged row: min(CH, P)
   int tc;           // 1: bf16 tensor-core contractions (bf16 I/O), 0: FP32-pipe GEMMs
+  int one_order;    // bf16 forward: one segmentation and one order of the carries for all sizes
+  int split;        // fp32 I/O: contractions on the tensor cores, every operand as three bf16 terms (as_gemm_split.cu)
   int gsplit;       // bf16 terms per value of dB, dC in Gcat: 1, or 3 (exact) where d_model % 32 != 0
   int du_ld;        // row pitch (elements) of the du buffer: P, or P + 32 gsplit when it is the left part of Gcat = [du|dB|dC..]
   // byte offsets into the workspace
   size_t off_status, off_delta, off_bc, off_bcd, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
       off_partd, off_hstart, off_suf, off_pre, off_total, off_live, off_du, off_dxdir, off_dbc,
-      off_bptt_ckpt, off_wcat, off_wcatx, total_fwd, total_grad;
+      off_bptt_ckpt, off_wcat, off_wcatx, off_xs, off_wsp, off_gs, total_fwd, total_grad;
 };
 
-int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl);
+// PLAN_GRAD: gradient calls.  PLAN_FWD: as_ssm_forward.  PLAN_FWD_SMALL: an fp32 forward with less scratch (contractions on
+// the FP32 pipe).
+enum { PLAN_GRAD = 0, PLAN_FWD = 1, PLAN_FWD_SMALL = 2 };
+int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind = PLAN_GRAD);
 // elements of A_log (and dA_log) per layer
 inline int64_t a_stride(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }
 
@@ -168,6 +173,10 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int 
                    const ZeroList& z, char* ws, cudaStream_t st);
 int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* ws, cudaStream_t st);
 int tc_input_grad(const Plan& pl, const void* wcat, void* dx, char* ws, cudaStream_t st);
+
+// fp32 I/O on the tensor cores by exact three-term splits (as_gemm_split.cu), for large enough products
+int split_projections(const Plan& pl, const as_params_t* pr, const void* x, const ZeroList& z, char* ws, cudaStream_t st);
+int split_gradients(const Plan& pl, const as_grads_t* out, char* ws, cudaStream_t st);
 
 int launch_bptt(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st);
 

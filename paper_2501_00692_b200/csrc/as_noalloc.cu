@@ -56,10 +56,12 @@ int as::static_scratch_address(void** out) { return scratch_for_current_device(o
 
 extern "C" int as_ssm_forward_static(const as_shape_t* shape, const as_params_t* params, const void* x, void* y,
                                      void* stream) {
-  size_t need = 0;
-  int e = as_workspace_bytes(shape, shape ? shape->seqlen : 1, &need, nullptr);
+  int e = as_workspace_bytes(shape, shape ? shape->seqlen : 1, nullptr, nullptr);   // checks the shape
   if (e) return e;
-  if (need > (size_t)AS_STATIC_SCRATCH_BYTES) return AS_ERR_LIMIT;
+  as::Plan pl;
+  e = as::make_plan(shape, shape->seqlen, 1, &pl, as::PLAN_FWD_SMALL);   // the least scratch the forward can work with
+  if (e) return e;
+  if (pl.total_fwd > (size_t)AS_STATIC_SCRATCH_BYTES) return AS_ERR_LIMIT;
   void* scratch = nullptr;
   e = scratch_for_current_device(&scratch);
   if (e) return e;

@@ -20,13 +20,15 @@ namespace as {
 // ------------------------------------------------------------------------------------------------
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
+int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind) {
   Plan p{};
   p.KL = layers < 1 ? 1 : layers; p.Bg = sh->batch;
   p.B = p.KL * p.Bg; p.P = sh->d_model; p.T = sh->seqlen; p.io = sh->io;
   p.scalar = sh->a_structure == AS_A_SCALAR ? 1 : 0;
   p.tc = sh->io == AS_BF16 ? 1 : 0;
   p.gsplit = p.P % 32 == 0 ? 1 : 3;
+  // below that the splits and the fixed cost of the tensor-core kernels outweigh what they save (8,192 tokens x 256 has 6e8)
+  p.split = kind != PLAN_FWD_SMALL && !p.tc && p.P >= 64 && (int64_t)p.Bg * p.T * p.P * (p.P + NBC) >= ((int64_t)1 << 28);
   p.du_ld = p.tc ? p.P + p.gsplit * NBC : p.P;
   p.full = tbar >= p.T;
   p.tbar = p.full ? p.T : tbar;
@@ -52,7 +54,18 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   // a layer's results do not depend on how many it is computed with).
   int64_t L = segment((int64_t)p.tiles * p.B);
   if (L < 160) L = segment((int64_t)p.tiles * p.Bg);
-  const int64_t lmin = p.full && p.T <= 1024 ? CK : 2 * CK;
+  int64_t lmin = p.full && p.T <= 1024 ? CK : 2 * CK;
+  if (kind != PLAN_GRAD && p.tc && !(p.P <= 256 && (int64_t)p.Bg * p.T <= 1024)) {
+    p.one_order = 1;
+    // The bf16 forward keeps one segmentation (two waves, 64 tokens at least) whatever the size: a deep stack of bf16 layers
+    // turns fp32 rounding differences of one layer's y into differences of some per cent of its outputs, so its results
+    // should not move when the schedule of other sizes is tuned.  Short narrow runs, which are all latency (256 tokens x
+    // 256: 37 us with these segments, 23 with short ones), are left out.
+    int64_t s_target = 2 * slots / ((int64_t)p.tiles * p.B);
+    if (s_target < 1) s_target = 1;
+    L = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;
+    lmin = 64;
+  }
   if (L < lmin) L = lmin;
   if (L > 2048) L = 2048;
   p.L = (int)L;
@@ -75,6 +88,8 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.off_segd = take(BSP * 4);
   p.off_hstart = take(BSB * 4);
   p.off_wcat = take((size_t)p.KL * (p.P + NBC) * p.P * 2);
+  p.off_xs = take(p.split ? BTP * 6 : 0);
+  p.off_wsp = take(p.split ? (size_t)p.KL * (p.P + NBC) * p.P * 6 : 0);
   p.total_fwd = o;
   p.off_wcatx = p.tc && p.gsplit > 1 ? take((size_t)p.KL * p.du_ld * p.P * 2) : p.off_wcat;
   p.off_bcd = take((BT + CK) * 2 * NBC * 4);   // doubled B rows, then doubled C rows
@@ -90,6 +105,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl) {
   p.off_du = take(BT * (size_t)p.du_ld * e);
   p.off_dxdir = take(BTP * e);
   p.off_dbc = take(BT * NBC * 4);
+  p.off_gs = take(p.split ? BT * (size_t)(p.P + NBC) * 6 : 0);
   p.off_bptt_ckpt = take((size_t)p.B * ((p.T + 63) / 64) * p.P * NS * 4);
   p.total_grad = o;
   *pl = p;
@@ -118,7 +134,8 @@ struct Stage {
   static constexpr int G = BC + CK * NBC * 4;
   static constexpr int BYTES = G + (WITH_G ? CK * CH * ESZ : 0);
 };
-constexpr int NSTAGE = 3;        // ascending kernels
+
+constexpr int NSTAGE = 3;   // chunks of the staging ring
 
 enum { PRE_FWD = 0, PRE_ADJ = 1, PRE_Y = 2 };
 
@@ -365,35 +382,39 @@ __device__ __forceinline__ void carry_h(const Plan& pl, const float* __restrict_
   const int n = (pl.S + t.nw - 1) / t.nw, sA = min(pl.S, t.warp * n), sB = min(pl.S, sA + n);
   const int64_t stride = (int64_t)pl.tiles * (TILE_FLOATS / 2);
   const int64_t at0 = ((int64_t)b * pl.S * pl.tiles + tile) * (TILE_FLOATS / 2) + t.iu, ch0 = (int64_t)b * pl.S * pl.P + t.p;
-  u64 he[CARRY_UB];
-  float sd[CARRY_UB];
-  auto fetch = [&](int s0) {   // slots past the range: decay 1, add 0
+  struct Batch { u64 he[CARRY_UB]; float sd[CARRY_UB]; } cur, nxt;
+  auto fetch = [&](int s0, Batch& q) {   // slots past the range: decay 1, add 0
 #pragma unroll
     for (int i = 0; i < CARRY_UB; ++i) {
       const bool in = s0 + i < sB;
-      he[i] = in ? __ldg(hend + at0 + (s0 + i) * stride) : 0ull;
-      sd[i] = in && t.act ? __ldg(segd + ch0 + (int64_t)(s0 + i) * pl.P) : 0.f;
+      q.he[i] = in ? __ldg(hend + at0 + (s0 + i) * stride) : 0ull;
+      q.sd[i] = in && t.act ? __ldg(segd + ch0 + (int64_t)(s0 + i) * pl.P) : 0.f;
     }
   };
   u64 v = 0ull;
-  float dsum = 0.f;
-  for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
-    fetch(s0);
+  fetch(sA, cur);
+  if (t.nw > 1) {
+    float dsum = 0.f;
+    for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+      if (s0 != sA) fetch(s0, cur);
 #pragma unroll
-    for (int i = 0; i < CARRY_UB; ++i) { v = fma2(decay_of(t.A2, sd[i]), v, he[i]); dsum += sd[i]; }
+      for (int i = 0; i < CARRY_UB; ++i) { v = fma2(decay_of(t.A2, cur.sd[i]), v, cur.he[i]); dsum += cur.sd[i]; }
+    }
+    sm.val[t.warp][t.lane] = v;
+    sm.dec[t.warp][t.lane] = decay_of(t.A2, dsum);
+    __syncthreads();
+    v = 0ull;
+    for (int w = 0; w < t.warp; ++w) v = fma2(sm.dec[w][t.lane], v, sm.val[w][t.lane]);
+    if (n > CARRY_UB) fetch(sA, cur);   // a single batch is still in registers
   }
-  sm.val[t.warp][t.lane] = v;
-  sm.dec[t.warp][t.lane] = decay_of(t.A2, dsum);
-  __syncthreads();
-  v = 0ull;
-  for (int w = 0; w < t.warp; ++w) v = fma2(sm.dec[w][t.lane], v, sm.val[w][t.lane]);
   for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
-    if (n > CARRY_UB) fetch(s0);   // a single batch is still in registers
+    fetch(s0 + CARRY_UB, nxt);          // past the range: loads nothing
 #pragma unroll
     for (int i = 0; i < CARRY_UB; ++i) {
       if (s0 + i < sB) hstart[at0 + (s0 + i) * stride] = v;
-      v = fma2(decay_of(t.A2, sd[i]), v, he[i]);
+      v = fma2(decay_of(t.A2, cur.sd[i]), v, cur.he[i]);
     }
+    cur = nxt;
   }
 }
 
@@ -606,7 +627,6 @@ int launch_ascend_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
   return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, pl, sp.A_log, sp.ws, (IO*)y);
 }
-
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------
@@ -634,6 +654,7 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
   if (warps < 8) warps = 8;
   if (warps > (pl.S + 3) / 4) warps = (pl.S + 3) / 4;
   if (warps > CARRY_WARPS) warps = CARRY_WARPS;
+  if (pl.one_order) warps = 1;   // the bf16 forward adds its segments up in one order whatever their number (see make_plan)
   const int64_t blocks = nh * roles + (nlive + warps - 1) / warps;
   if (blocks > 0x7fffffff) return 1;
   return launch_dependent(fixup_kernel, dim3((unsigned)blocks), dim3((unsigned)warps * 32), 0, st, pl, sp.A_log, sp.ws, (int)nh, roles);
