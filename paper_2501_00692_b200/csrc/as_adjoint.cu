@@ -61,24 +61,12 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16], u64 (&v)[NSU]) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 // lo * lo + hi * hi: two scalar operations take as long as one packed one, and save the addition
 __device__ __forceinline__ float dot2(u64 a, u64 b) {
   float al, ah, bl, bh;
   upk(a, al, ah);
   upk(b, bl, bh);
   return fmaf(ah, bh, al * bl);
-}
-// the channel pair of a staged row, from a pointer that already addresses it
-template <typename IO> __device__ __forceinline__ u64 lds_pair(const uint8_t* p);
-template <> __device__ __forceinline__ u64 lds_pair<float>(const uint8_t* p) { return *reinterpret_cast<const u64*>(p); }
-template <> __device__ __forceinline__ u64 lds_pair<__nv_bfloat16>(const uint8_t* p) {
-  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-  return pk(t.x, t.y);
 }
 // The thread's 16 values inside a tile block of the scan kernels, regrouped: slot u is state u (of the thread's eight) of
 // both channels.  Block order: pair iu = 2 q + e of scan thread tid at ((q * NTHR + tid) * 2 + e), pair 4 ch + m holding
@@ -101,11 +89,6 @@ template <int ESZ> __device__ __forceinline__ float sigmoid_of(float d) {
   if (ESZ == 4) return sig_from_delta(d);
   const float small = d * fmaf(d, __fadd_rn(__fmul_rn(d, 1.f / 6.f), -0.5f), 1.f);
   return d < 0.03125f ? small : 1.f - ex2_approx(-d * LOG2E);
-}
-template <typename IO> __device__ __forceinline__ void st_pair(uint8_t* p, float a, float b);
-template <> __device__ __forceinline__ void st_pair<float>(uint8_t* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
-template <> __device__ __forceinline__ void st_pair<__nv_bfloat16>(uint8_t* p, float a, float b) {
-  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
 }
 // abar for the slots from the channel pair's exponent scales.  With a scalar rate the states of a channel share one factor.
 template <bool SC>

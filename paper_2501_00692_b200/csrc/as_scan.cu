@@ -117,11 +117,10 @@ namespace {
 
 // ------------------------------------------------------------------------------------------------
 // ascending pass over one segment.
-//   PRE_FWD : local scan from h = 0; writes the segment's end state and Delta sum.
-//   PRE_ADJ : PRE_FWD + the state at every chunk start (relative to a zero segment start) and the local
+//   forward (MU = false) : local scan from h = 0; writes the segment's end state and Delta sum.
+//   gradients (MU = true): the same + the state at every chunk start (relative to a zero segment start) and the local
 //             exclusive cumulative Delta there, + the segment-local cotangent sum carried to the token before
 //             the segment, mu_loc = sum_t gC_t prod_{j=start..t} abar_j, and its snapshot after r tokens.
-//   PRE_Y   : scan from the true segment-start state, writes y_t = sum_n C_t[n] h_t[n].
 // Tokens past the end of the sequence inside the last chunk are neutralised by zeroing their staged
 // Delta, dy and B/C rows (Delta = 0 gives abar = 1 and a zero input term), so the token code has no branches.
 // ------------------------------------------------------------------------------------------------
@@ -137,16 +136,12 @@ struct Stage {
 
 constexpr int NSTAGE = 3;   // chunks of the staging ring
 
-enum { PRE_FWD = 0, PRE_ADJ = 1, PRE_Y = 2 };
-
-template <typename IO, int MODE, bool SC>
-__global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__ CUtensorMap tmX,
+template <typename IO, bool MU, bool SC>
+__global__ void __launch_bounds__(NTHR, 4) prepass_kernel(const __grid_constant__ CUtensorMap tmX,
                                                     const __grid_constant__ CUtensorMap tmD,
                                                     const __grid_constant__ CUtensorMap tmG, Plan pl,
-                                                    const float* __restrict__ A_log, char* __restrict__ ws,
-                                                    IO* __restrict__ y) {
+                                                    const float* __restrict__ A_log, char* __restrict__ ws) {
   constexpr int ESZ = IoSz<IO>::v;
-  constexpr bool MU = MODE == PRE_ADJ;
   using St = Stage<ESZ, MU>;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[NSTAGE];
@@ -186,14 +181,8 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
   u64 A2[NU], h[NU], Pr[NU], acc[NU];
   load_A2(A_log, w, A2, pl.scalar);
   const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
-  if (MODE == PRE_Y) {
-    load_block_g(reinterpret_cast<const float*>(ws + pl.off_hstart) + sb * TILE_FLOATS, w.tid, h);
-  } else {
 #pragma unroll
-    for (int u = 0; u < NU; ++u) h[u] = 0ull;
-  }
-#pragma unroll
-  for (int u = 0; u < NU; ++u) { Pr[u] = pk(1.f, 1.f); acc[u] = 0ull; }
+  for (int u = 0; u < NU; ++u) { h[u] = acc[u] = 0ull; Pr[u] = pk(1.f, 1.f); }
   bool snapped = false;   // the r-token snapshot of acc and of the Delta sum goes straight to global memory when it is taken
   float cum[NCH];
 #pragma unroll
@@ -206,13 +195,13 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
     const int64_t tc = t0 + (int64_t)c * CK;
     const int nt = (int)min((int64_t)CK, t1 - tc);
     const int jr = MU ? (int)(t0 + pl.r - 1 - tc) : -1;   // slot of the r-th token of the segment, if in this chunk
-    if (MODE == PRE_ADJ) {
+    if (MU) {
       const int64_t cc = ((int64_t)b * pl.NC + tc / CK);
       store_block(reinterpret_cast<float*>(ws + pl.off_ckpt) + (cc * pl.tiles + tile) * TILE_FLOATS, w.tid, h);
       if (w.half == 0 && w.act)
         stg_ch(reinterpret_cast<float*>(ws + pl.off_cs) + cc * P + w.pa, cum);
     }
-    if (MODE == PRE_ADJ && tile == 0 && ok) {   // the rows once more, doubled, for the main kernel's packed channel pairs
+    if (MU && tile == 0 && ok) {   // the rows once more, doubled, for the main kernel's packed channel pairs
       const int j = w.tid >> 4, q = w.tid & 15;
       const float2 v = *reinterpret_cast<const float2*>(sm + St::BC + j * NBC * 4 + 8 * q);
       if (j < nt) {   // B rows, then C rows
@@ -239,18 +228,15 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
         const ulonglong2 b23 = *reinterpret_cast<const ulonglong2*>(brow + 4);
         const u64 Bp[4] = {b01.x, b01.y, b23.x, b23.y};
         u64 Cp[4] = {0ull, 0ull, 0ull, 0ull};
-        if (MODE != PRE_FWD) {
+        if (MU) {
           const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(brow + NS);
           const ulonglong2 c23 = *reinterpret_cast<const ulonglong2*>(brow + NS + 4);
           Cp[0] = c01.x; Cp[1] = c01.y; Cp[2] = c23.x; Cp[3] = c23.y;
         }
-        float yv[NCH];
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
           const float ddc = dv.v[ch], dxc = dv.v[ch] * xv.v[ch], gc = gv.v[ch];
           const u64 d2 = pk(ddc, ddc), dx2 = pk(dxc, dxc), g2 = pk(gc, gc);
-          yv[ch] = 0.f;
-          u64 yacc = 0ull;
           u64 ach = 0ull;
           if (SC) ach = ex2_2(mul2(d2, A2[ch * 4]));   // scalar rate: one factor for the channel's states
 #pragma unroll
@@ -262,18 +248,8 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
               Pr[u] = mul2(Pr[u], a);
               acc[u] = fma2(mul2(g2, Cp[m]), Pr[u], acc[u]);
             }
-            if (MODE == PRE_Y) yacc = fma2(Cp[m], h[u], yacc);
           }
-          if (MODE == PRE_Y) yv[ch] = hsum(yacc);
           cum[ch] += ddc;
-        }
-        if (MODE == PRE_Y) {
-#pragma unroll
-          for (int ch = 0; ch < NCH; ++ch) yv[ch] += __shfl_xor_sync(0xffffffffu, yv[ch], 1);
-          // the two lanes of a pair hold the same sums: lane `half` writes channel `half` (one channel per thread: lane 0)
-          const int chf = NCH == 2 ? w.half : 0;
-          if (w.act && j < nt && (NCH == 2 || w.half == 0))
-            st_io<IO>(y + ((int64_t)b * pl.T + tc + j) * P + w.pa + chf, chf ? yv[NCH - 1] : yv[0]);
         }
     };
     if (ok) {
@@ -307,7 +283,6 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
     }
     if (w.tid == 0 && c + NSTAGE < nchunk) issue(c + NSTAGE);
   }
-  if (MODE == PRE_Y) return;
   store_block(reinterpret_cast<float*>(ws + pl.off_hend) + sb * TILE_FLOATS, w.tid, h);
   const int64_t sp = ((int64_t)b * pl.S + s) * P + w.pa;
   if (w.half == 0 && w.act) stg_ch(reinterpret_cast<float*>(ws + pl.off_segd) + sp, cum);
@@ -330,6 +305,138 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
 }
 
 // ------------------------------------------------------------------------------------------------
+// The forward's second pass: scan a segment from its true start state, y_t = sum_n C_t[n] h_t[n].
+// Here the two CHANNELS of a state share a packed register pair: the sum over states needs no unpacking, one shuffle finishes
+// a token's two channels instead of two, and the staged Delta and x rows are packed operands as they lie.  B_t and C_t, which
+// all channels share, are needed twice over, (B_n, B_n): each chunk's rows are doubled in shared memory while the chunk before
+// is worked on.  Bound: MUFU.EX2, one per state-step (346 us at 2 x 65,536 tokens x 768); measured there, kernel alone,
+// 518 -> 470 us against packing a channel's states.  (The segment pass above has no sum over states: there reading doubled rows
+// costs more, 413 against 402 us, than the packed operands save.)
+// ------------------------------------------------------------------------------------------------
+template <typename IO, bool SC>
+__global__ void __launch_bounds__(NTHR, 4) forward_y_kernel(const __grid_constant__ CUtensorMap tmX,
+                                                    const __grid_constant__ CUtensorMap tmD, Plan pl,
+                                                    const float* __restrict__ A_log, char* __restrict__ ws,
+                                                    IO* __restrict__ y) {
+  constexpr int ESZ = IoSz<IO>::v;
+  using St = Stage<ESZ, false>;
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[NSTAGE];
+  __shared__ float4 dbl[2][CK][NBC / 2];   // the chunk's doubled [B | C] rows, by chunk parity
+  uint8_t* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);   // stays a shared-space pointer
+
+  const int tile = blockIdx.x, s = blockIdx.y, b = blockIdx.z;
+  const int P = pl.P;
+  const Who w = who(tile, P);
+  const int64_t t0 = (int64_t)s * pl.L;
+  const int64_t t1 = min(pl.T, t0 + pl.L);
+  const int nchunk = (int)((t1 - t0 + CK - 1) / CK);
+  const float* bc = reinterpret_cast<const float*>(ws + pl.off_bc);
+  int* status = reinterpret_cast<int*>(ws + pl.off_status);
+  A_log += (int64_t)(b / pl.Bg) * a_stride_dev(pl);   // this layer's rates
+
+  pdl_begin();
+  if (w.tid == 0) {
+    for (int i = 0; i < NSTAGE; ++i) mbar_init(&full_bar[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const uint32_t tx_bytes = (uint32_t)(CK * CH * ESZ + CK * CH * 4 + CK * NBC * 4);
+  auto issue = [&](int c) {   // thread 0: stage chunk c
+    const int st = c % NSTAGE;
+    uint8_t* sm = smem + st * St::BYTES;
+    const int64_t row = (int64_t)b * pl.T + t0 + (int64_t)c * CK;
+    mbar_expect_tx(&full_bar[st], tx_bytes);
+    tma_2d(sm + St::X, &tmX, tile * CH, row, &full_bar[st]);
+    tma_2d(sm + St::D, &tmD, tile * CH, row, &full_bar[st]);
+    bulk_1d(sm + St::BC, bc + row * NBC, CK * NBC * 4, &full_bar[st]);
+  };
+  if (w.tid == 0)
+    for (int c = 0; c < NSTAGE && c < nchunk; ++c) issue(c);
+  // all threads, before the barrier that starts chunk c: wait for its tiles, double its [B | C] rows, neutralise the slots past
+  // the sequence end
+  auto prepare = [&](int c) -> bool {
+    uint8_t* sm = smem + c % NSTAGE * St::BYTES;
+    if (!mbar_wait(&full_bar[c % NSTAGE], (c / NSTAGE) & 1)) return false;
+    const int64_t tc = t0 + (int64_t)c * CK;
+    const int nt = (int)min((int64_t)CK, t1 - tc);
+    const int j = w.tid >> 4, q = w.tid & 15;
+    float2 v = *reinterpret_cast<const float2*>(sm + St::BC + j * NBC * 4 + 8 * q);
+    if (j >= nt) v = make_float2(0.f, 0.f);
+    dbl[c & 1][j][q] = make_float4(v.x, v.x, v.y, v.y);
+    if (nt < CK) zero_rows(sm + St::D, CH * 4, nt, w.tid);   // only the last chunk of a sequence
+    return true;
+  };
+
+  u64 A2[NU], h[NU];
+  load_A2(A_log, w, A2, pl.scalar);
+  to_slots(A2);
+  const int64_t sb = ((int64_t)b * pl.S + s) * pl.tiles + tile;
+  load_block_g(reinterpret_cast<const float*>(ws + pl.off_hstart) + sb * TILE_FLOATS, w.tid, h);
+  to_slots(h);
+  bool ok = prepare(0);
+  int bad = __syncthreads_or(ok ? 0 : 1);
+
+  int c = 0;
+  for (; c < nchunk && !bad; ++c) {
+    uint8_t* sm = smem + c % NSTAGE * St::BYTES;
+    const int64_t tc = t0 + (int64_t)c * CK;
+    const int nt = (int)min((int64_t)CK, t1 - tc);
+    const uint8_t* pD = sm + St::D + 8 * w.k;
+    const uint8_t* pX = sm + St::X + 2 * ESZ * w.k;
+    const ulonglong2* pB = reinterpret_cast<const ulonglong2*>(&dbl[c & 1][0][4 * w.half]);
+    // channels past P read the zero fill of the TMA box: Delta = x = 0 keeps their slots at zero
+    auto token = [&](int j) -> u64 {   // returns this thread's part of y for both channels
+      const u64 d2 = lds_pair<float>(pD + j * CH * 4);
+      const u64 dx2 = mul2(d2, lds_pair<IO>(pX + j * CH * ESZ));
+      u64 af = 0ull, ye = 0ull, yo = 0ull;
+      if (SC) af = ex2_2(mul2(d2, A2[0]));   // scalar rate: one factor for the channel's states
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const ulonglong2 bq = pB[j * (NBC / 2) + m];
+        const ulonglong2 cq = pB[j * (NBC / 2) + NS / 2 + m];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int u = 2 * m + e;
+          const u64 Bn = e ? bq.y : bq.x, Cn = e ? cq.y : cq.x;
+          const u64 a = SC ? af : ex2_2(mul2(d2, A2[u]));
+          h[u] = fma2(a, h[u], mul2(dx2, Bn));
+          if (e) yo = fma2(Cn, h[u], yo); else ye = fma2(Cn, h[u], ye);   // even and odd states
+        }
+      }
+      return add2(ye, yo);
+    };
+    // two tokens at a time: the lanes of a channel pair trade their parts, lane `half` finishes token 2 jp + half
+    IO* py = y + ((int64_t)b * pl.T + tc + w.half) * P + w.pa;
+    const int left = w.act ? nt - w.half : 0;
+#pragma unroll
+    for (int jp = 0; jp < CK / 2; ++jp) {
+      const u64 y0 = token(2 * jp), y1 = token(2 * jp + 1);
+      float a0, a1, b0, b1;
+      upk(y0, a0, a1);
+      upk(y1, b0, b1);
+      const float r0 = (w.half ? b0 : a0) + __shfl_xor_sync(0xffffffffu, w.half ? a0 : b0, 1);
+      const float r1 = (w.half ? b1 : a1) + __shfl_xor_sync(0xffffffffu, w.half ? a1 : b1, 1);
+      if (2 * jp < left) st_pair<IO>(py, r0, r1);
+      py += 2 * P;
+    }
+    ok = c + 1 >= nchunk || prepare(c + 1);
+    bad = __syncthreads_or(ok ? 0 : 1);
+    if (!bad && w.tid == 0 && c + NSTAGE < nchunk) issue(c + NSTAGE);
+  }
+  if (bad) {
+    if (w.tid == 0) {
+      // copies issued for the chunk that did not arrive and the following ones still target this CTA's shared memory: give each
+      // one more bounded wait before the CTA (and its shared memory) goes away
+      for (int c2 = c; c2 < nchunk && c2 < c + NSTAGE; ++c2) mbar_wait(&full_bar[c2 % NSTAGE], (c2 / NSTAGE) & 1);
+      atomicExch(status, AS_ERR_TIMEOUT);
+    }
+    __syncthreads();
+    return;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
 // carries across segments.  The segment decays are exp(A * sum of Delta), so each carry is a linear recurrence over the
 // segments; a chain of S dependent steps would leave the kernel waiting for latency (full form, T = 50,000, P = 80,
 // S = 1250: 200 us).  So a CTA takes 32 state pairs (one per lane: 256 contiguous bytes of a tile block) and its warps cut
@@ -337,6 +444,7 @@ __global__ void __launch_bounds__(NTHR, 4) ascend_kernel(const __grid_constant__
 // again from the true start.  Every pass reads CARRY_UB segments' values at once.
 // ------------------------------------------------------------------------------------------------
 constexpr int CARRY_UB = 8;
+constexpr int ONE_UB = 12;                       // of fixup_one_kernel, which has the registers
 constexpr int CARRY_WARPS = 32;                  // most warps of a CTA
 constexpr int CARRY_SLICES = TILE_FLOATS / 64;   // CTAs per (tile, batch element): 64 floats each
 
@@ -372,20 +480,21 @@ struct CarrySmem {      // one entry per warp and lane
   double tot[CARRY_WARPS][32];
 };
 
-// hstart[s]: true state entering segment s
+// hstart[s]: true state entering segment s.  ONE: by a single warp, the segments added up in one order whatever their number.
+template <bool ONE, int UB>
 __device__ __forceinline__ void carry_h(const Plan& pl, const float* __restrict__ A_log, char* __restrict__ ws, int tile,
-                                        int b, int sl, CarrySmem& sm) {
+                                        int b, int sl, CarrySmem* sm) {
   const Slot t = slot(pl, A_log, tile, b, sl);
   const u64* hend = reinterpret_cast<const u64*>(ws + pl.off_hend);
   const float* segd = reinterpret_cast<const float*>(ws + pl.off_segd);
   u64* hstart = reinterpret_cast<u64*>(ws + pl.off_hstart);
-  const int n = (pl.S + t.nw - 1) / t.nw, sA = min(pl.S, t.warp * n), sB = min(pl.S, sA + n);
+  const int n = ONE ? pl.S : (pl.S + t.nw - 1) / t.nw, sA = ONE ? 0 : min(pl.S, t.warp * n), sB = min(pl.S, sA + n);
   const int64_t stride = (int64_t)pl.tiles * (TILE_FLOATS / 2);
   const int64_t at0 = ((int64_t)b * pl.S * pl.tiles + tile) * (TILE_FLOATS / 2) + t.iu, ch0 = (int64_t)b * pl.S * pl.P + t.p;
-  struct Batch { u64 he[CARRY_UB]; float sd[CARRY_UB]; } cur, nxt;
+  struct Batch { u64 he[UB]; float sd[UB]; } cur, nxt;
   auto fetch = [&](int s0, Batch& q) {   // slots past the range: decay 1, add 0
 #pragma unroll
-    for (int i = 0; i < CARRY_UB; ++i) {
+    for (int i = 0; i < UB; ++i) {
       const bool in = s0 + i < sB;
       q.he[i] = in ? __ldg(hend + at0 + (s0 + i) * stride) : 0ull;
       q.sd[i] = in && t.act ? __ldg(segd + ch0 + (int64_t)(s0 + i) * pl.P) : 0.f;
@@ -393,24 +502,24 @@ __device__ __forceinline__ void carry_h(const Plan& pl, const float* __restrict_
   };
   u64 v = 0ull;
   fetch(sA, cur);
-  if (t.nw > 1) {
+  if (!ONE && t.nw > 1) {
     float dsum = 0.f;
-    for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
+    for (int s0 = sA; s0 < sB; s0 += UB) {
       if (s0 != sA) fetch(s0, cur);
 #pragma unroll
-      for (int i = 0; i < CARRY_UB; ++i) { v = fma2(decay_of(t.A2, cur.sd[i]), v, cur.he[i]); dsum += cur.sd[i]; }
+      for (int i = 0; i < UB; ++i) { v = fma2(decay_of(t.A2, cur.sd[i]), v, cur.he[i]); dsum += cur.sd[i]; }
     }
-    sm.val[t.warp][t.lane] = v;
-    sm.dec[t.warp][t.lane] = decay_of(t.A2, dsum);
+    sm->val[t.warp][t.lane] = v;
+    sm->dec[t.warp][t.lane] = decay_of(t.A2, dsum);
     __syncthreads();
     v = 0ull;
-    for (int w = 0; w < t.warp; ++w) v = fma2(sm.dec[w][t.lane], v, sm.val[w][t.lane]);
-    if (n > CARRY_UB) fetch(sA, cur);   // a single batch is still in registers
+    for (int w = 0; w < t.warp; ++w) v = fma2(sm->dec[w][t.lane], v, sm->val[w][t.lane]);
+    if (n > UB) fetch(sA, cur);   // a single batch is still in registers
   }
-  for (int s0 = sA; s0 < sB; s0 += CARRY_UB) {
-    fetch(s0 + CARRY_UB, nxt);          // past the range: loads nothing
+  for (int s0 = sA; s0 < sB; s0 += UB) {
+    fetch(s0 + UB, nxt);          // past the range: loads nothing
 #pragma unroll
-    for (int i = 0; i < CARRY_UB; ++i) {
+    for (int i = 0; i < UB; ++i) {
       if (s0 + i < sB) hstart[at0 + (s0 + i) * stride] = v;
       v = fma2(decay_of(t.A2, cur.sd[i]), v, cur.he[i]);
     }
@@ -597,9 +706,18 @@ __global__ void __launch_bounds__(32 * CARRY_WARPS, 1) fixup_kernel(Plan pl, con
   if (role == roles) {
     const int64_t item = (int64_t)blk * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (item < (int64_t)pl.tiles * pl.S * pl.B) mark_live(pl, A_log, ws, item);
-  } else if (role == 0) carry_h(pl, A_log, ws, tile, b, i, sm);
+  } else if (role == 0) carry_h<false, CARRY_UB>(pl, A_log, ws, tile, b, i, &sm);
   else if (role == 1) carry_mu<true>(pl, A_log, ws, tile, b, i, sm);
   else carry_mu<false>(pl, A_log, ws, tile, b, i, sm);
+}
+
+// The bf16 forward's own carry kernel (see make_plan: one order of the segments): a slice per warp, whose loads run ONE_UB to
+// 2 ONE_UB segments ahead of the chain (T = 65,536, P = 768, B = 2: 14.4 -> 10.7 us against one warp of fixup_kernel).
+__global__ void __launch_bounds__(128) fixup_one_kernel(Plan pl, const float* __restrict__ A_log, char* __restrict__ ws) {
+  pdl_begin();
+  const int item = (int)blockIdx.x * 4 + (int)(threadIdx.x >> 5);
+  const int tile = item % pl.tiles, rest = item / pl.tiles, b = rest % pl.B, sl = rest / pl.B;
+  if (sl < CARRY_SLICES) carry_h<true, ONE_UB>(pl, A_log, ws, tile, b, sl, nullptr);
 }
 
 // Self test of the bounded wait: one warp waits for a phase of an mbarrier that nothing will ever complete, with a
@@ -616,37 +734,51 @@ __global__ void wait_selftest_kernel(int* status, uint32_t limit) {
   if (bad && threadIdx.x == 0) atomicExch(status, AS_ERR_TIMEOUT);
 }
 
-template <typename IO, int MODE, bool SC>
-int launch_ascend_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
+template <typename IO, bool MU, bool SC>
+int launch_prepass_t(const Plan& pl, const ScanPtrs& sp, cudaStream_t st) {
   Maps m;
   if (make_maps(pl, sp, &m)) return 1;
-  using St = Stage<sizeof(IO), MODE == PRE_ADJ>;
-  const int bytes = NSTAGE * St::BYTES + 128;
-  auto kern = ascend_kernel<IO, MODE, SC>;
+  const int bytes = NSTAGE * Stage<sizeof(IO), MU>::BYTES + 128;
+  auto kern = prepass_kernel<IO, MU, SC>;
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
-  return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, pl, sp.A_log, sp.ws, (IO*)y);
+  return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, pl, sp.A_log, sp.ws);
+}
+template <typename IO, bool MU>
+int launch_prepass_s(const Plan& pl, const ScanPtrs& sp, cudaStream_t st) {
+  return pl.scalar ? launch_prepass_t<IO, MU, true>(pl, sp, st) : launch_prepass_t<IO, MU, false>(pl, sp, st);
+}
+template <typename IO, bool SC>
+int launch_forward_y_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
+  Maps m;
+  if (make_maps(pl, sp, &m)) return 1;
+  const int bytes = NSTAGE * Stage<sizeof(IO), false>::BYTES + 128;
+  auto kern = forward_y_kernel<IO, SC>;
+  static bool done[AS_MAX_DEVICES] = {};
+  if (ensure_dynamic_smem(kern, bytes, done)) return 1;
+  return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, pl, sp.A_log, sp.ws, (IO*)y);
+}
+template <typename IO>
+int launch_forward_y_s(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
+  return pl.scalar ? launch_forward_y_t<IO, true>(pl, sp, y, st) : launch_forward_y_t<IO, false>(pl, sp, y, st);
 }
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------
 // launchers
 // ------------------------------------------------------------------------------------------------
-template <typename IO, int MODE>
-int launch_ascend_s(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
-  return pl.scalar ? launch_ascend_t<IO, MODE, true>(pl, sp, y, st) : launch_ascend_t<IO, MODE, false>(pl, sp, y, st);
-}
 int launch_prepass(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st) {
   if (pl.io == AS_BF16)
-    return with_mu ? launch_ascend_s<__nv_bfloat16, PRE_ADJ>(pl, sp, nullptr, st)
-                   : launch_ascend_s<__nv_bfloat16, PRE_FWD>(pl, sp, nullptr, st);
-  return with_mu ? launch_ascend_s<float, PRE_ADJ>(pl, sp, nullptr, st) : launch_ascend_s<float, PRE_FWD>(pl, sp, nullptr, st);
+    return with_mu ? launch_prepass_s<__nv_bfloat16, true>(pl, sp, st) : launch_prepass_s<__nv_bfloat16, false>(pl, sp, st);
+  return with_mu ? launch_prepass_s<float, true>(pl, sp, st) : launch_prepass_s<float, false>(pl, sp, st);
 }
 
 int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st) {
   const int64_t nh = (int64_t)CARRY_SLICES * pl.tiles * pl.B;
   const int roles = !with_mu || pl.direct ? 1 : (pl.full ? 2 : 3);
   const int64_t nlive = with_mu && !pl.full ? (int64_t)pl.tiles * pl.B * pl.S : 0;
+  if (pl.one_order)
+    return launch_dependent(fixup_one_kernel, dim3((unsigned)((nh + 3) / 4)), dim3(128), 0, st, pl, sp.A_log, sp.ws);
   // Few CTAs: as many warps as the chip holds, four segments or more each.  Many: eight warps each (T = 65,536, P = 768,
   // B = 2: 9.7 us; 4 warps 11.6, 16 warps 10.0, 32 warps 16.3).
   // By one layer's CTAs: a layer's results do not depend on how many it is computed with.
@@ -654,15 +786,13 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
   if (warps < 8) warps = 8;
   if (warps > (pl.S + 3) / 4) warps = (pl.S + 3) / 4;
   if (warps > CARRY_WARPS) warps = CARRY_WARPS;
-  if (pl.one_order) warps = 1;   // the bf16 forward adds its segments up in one order whatever their number (see make_plan)
   const int64_t blocks = nh * roles + (nlive + warps - 1) / warps;
   if (blocks > 0x7fffffff) return 1;
   return launch_dependent(fixup_kernel, dim3((unsigned)blocks), dim3((unsigned)warps * 32), 0, st, pl, sp.A_log, sp.ws, (int)nh, roles);
 }
 
 int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
-  if (pl.io == AS_BF16) return launch_ascend_s<__nv_bfloat16, PRE_Y>(pl, sp, y, st);
-  return launch_ascend_s<float, PRE_Y>(pl, sp, y, st);
+  return pl.io == AS_BF16 ? launch_forward_y_s<__nv_bfloat16>(pl, sp, y, st) : launch_forward_y_s<float>(pl, sp, y, st);
 }
 
 int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st) {

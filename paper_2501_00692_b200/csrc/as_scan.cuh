@@ -36,12 +36,6 @@ __device__ __forceinline__ u64 ex2_2(u64 e) {
   upk(e, lo, hi);
   return pk(ex2_approx(lo), ex2_approx(hi));
 }
-__device__ __forceinline__ float hsum(u64 v) {
-  float lo, hi;
-  upk(v, lo, hi);
-  return lo + hi;
-}
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -101,27 +95,6 @@ template <> __device__ __forceinline__ ChV lds_ch<__nv_bfloat16>(const uint8_t* 
   }
   return r;
 }
-// the same from a pointer that already addresses this thread's channels in the row
-template <typename IO> __device__ __forceinline__ ChV lds_chp(const uint8_t* p);
-template <> __device__ __forceinline__ ChV lds_chp<float>(const uint8_t* p) {
-  ChV r;
-  const float2 t = *reinterpret_cast<const float2*>(p);
-  r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  return r;
-}
-template <> __device__ __forceinline__ ChV lds_chp<__nv_bfloat16>(const uint8_t* p) {
-  ChV r;
-  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-  r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  return r;
-}
-// NCH consecutive floats of a global per-channel array
-__device__ __forceinline__ ChV ldg_ch(const float* p) {
-  ChV r;
-#pragma unroll
-  for (int c = 0; c < NCH; ++c) r.v[c] = __ldg(p + c);
-  return r;
-}
 __device__ __forceinline__ void stg_ch(float* p, const float (&v)[NCH]) {
 #pragma unroll
   for (int c = 0; c < NCH; ++c) p[c] = v[c];
@@ -173,6 +146,39 @@ __device__ __forceinline__ void store_block(float* blk, int tid, const u64 (&v)[
   ulonglong2* b2 = reinterpret_cast<ulonglong2*>(blk);
 #pragma unroll
   for (int q = 0; q < 2 * NCH; ++q) b2[q * NTHR + tid] = make_ulonglong2(v[2 * q], v[2 * q + 1]);
+}
+
+// ---- two channels of a state in one register pair: "slot" u is state 8 half + u of the thread's two channels ----
+// block order (state pairs of a channel) -> slots
+__device__ __forceinline__ void to_slots(u64 (&v)[NU]) {
+  u64 t[NU];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    float a0, a1, b0, b1;
+    upk(v[m], a0, a1);
+    upk(v[4 + m], b0, b1);
+    t[2 * m] = pk(a0, b0);
+    t[2 * m + 1] = pk(a1, b1);
+  }
+#pragma unroll
+  for (int u = 0; u < NU; ++u) v[u] = t[u];
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// the channel pair of a staged row, from a pointer that already addresses it
+template <typename IO> __device__ __forceinline__ u64 lds_pair(const uint8_t* p);
+template <> __device__ __forceinline__ u64 lds_pair<float>(const uint8_t* p) { return *reinterpret_cast<const u64*>(p); }
+template <> __device__ __forceinline__ u64 lds_pair<__nv_bfloat16>(const uint8_t* p) {
+  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
+  return pk(t.x, t.y);
+}
+template <typename IO> __device__ __forceinline__ void st_pair(void* p, float a, float b);
+template <> __device__ __forceinline__ void st_pair<float>(void* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+template <> __device__ __forceinline__ void st_pair<__nv_bfloat16>(void* p, float a, float b) {
+  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
 }
 
 // sigmoid(u) from Delta = softplus(u): 1 - exp(-Delta), without cancellation for small Delta
