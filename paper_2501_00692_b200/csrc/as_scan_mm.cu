@@ -13,6 +13,9 @@
 // the operands are rounded to bf16).  One CTA = 128 channels x one segment, 256 threads: thread (p, h) owns channel p in
 // half h of every chunk.  The exponents are bounded by |a_p| times a quarter chunk's Delta sum; a channel whose bound
 // exceeds 2^+-96 in a chunk takes the plain recurrence for that chunk in thread (p, 0) (its TMEM lane is then ignored).
+// The CTA waits for such a channel, so the recurrence loads and scales several tokens at once before it runs their chain (decay
+// rates up to 16 and step sizes around 0.05, where some channels of every tile do this: 2 x 32,768 x 768 both passes 250 -> 240 us,
+// 2,048 x 512 the whole forward 53 -> 44 us).
 // Every mbarrier wait is bounded; on a timeout the kernel records AS_ERR_TIMEOUT, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -397,12 +400,27 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     if (c + 1 < nchunk) fetch_bc(row0 + TCK, (int)min((int64_t)TCK, t1 - tc - TCK));
     if (!YPASS && hf == 0 && slow) {
       // this channel left the factorised form in this chunk: its state by the plain recurrence (B as the bf16 operand holds it)
-      for (int t = 0; t < nt; ++t) {
-        const float d = dcol[t * MCH];
-        const float ab = ex2_approx(a2 * d), dx = d * __bfloat162float(xcol[t * MCH]);
+      // Eight tokens at a time (one load brings eight of a state's B), the 16 states' chains side by side; the Delta rows
+      // past the segment's end are zero.
+#pragma unroll 1
+      for (int t0s = 0; t0s < nt; t0s += 8) {
+        float ab[8], dx[8];
 #pragma unroll
-        for (int n = 0; n < NS; ++n)
-          S[n] = fmaf(ab, S[n], dx * __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sm + SM_BTT + sw128(n, t >> 3) + (t & 7) * 2)));
+        for (int i = 0; i < 8; ++i) {
+          const float d = dcol[(t0s + i) * MCH];
+          ab[i] = ex2_approx(a2 * d);
+          dx[i] = d * __bfloat162float(xcol[(t0s + i) * MCH]);
+        }
+#pragma unroll
+        for (int n = 0; n < NS; ++n) {
+          const uint4 bq = *reinterpret_cast<const uint4*>(sm + SM_BTT + sw128(n, t0s >> 3));
+          const uint32_t bw[4] = {bq.x, bq.y, bq.z, bq.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            S[n] = fmaf(ab[2 * i], S[n], dx[2 * i] * __uint_as_float(bw[i] << 16));
+            S[n] = fmaf(ab[2 * i + 1], S[n], dx[2 * i + 1] * __uint_as_float(bw[i] & 0xffff0000u));
+          }
+        }
       }
     }
     const float c0r = xch[0][pc], c0t = xch[1][pc], c1r = xch[2][pc], c1t = xch[3][pc];
@@ -436,28 +454,41 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       } else if (hf == 0) {
         // this channel left the factorised form in this chunk: plain recurrence over all its tokens, from the true
         // state at the chunk start (B and C as the bf16 operands hold them); its TMEM lane is not used
-        for (int t = 0; t < nt; ++t) {
-          const float d = dcol[t * MCH];
-          const float xv = __bfloat162float(xcol[t * MCH]);
-          const float ab = ex2_approx(a2 * d), dx = d * xv;
-          float acc = 0.f;
+        // Four tokens at a time: their loads, exponentials and y sums do not wait for one another.  Rows past the segment's
+        // end have Delta = 0; what is written there is not sent out.
+#pragma unroll 1
+        for (int t0s = 0; t0s < nt; t0s += 4) {
+          float ab[4], dx[4], acc[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float d = dcol[(t0s + i) * MCH];
+            ab[i] = ex2_approx(a2 * d);
+            dx[i] = d * __bfloat162float(xcol[(t0s + i) * MCH]);
+            acc[i] = 0.f;
+          }
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const uint4 bq = *reinterpret_cast<const uint4*>(sm + SM_BT + sw128(t, q));
-            const uint4 cq = *reinterpret_cast<const uint4*>(sm + SM_CT + sw128(t, q));
-            const uint32_t bw[4] = {bq.x, bq.y, bq.z, bq.w}, cw[4] = {cq.x, cq.y, cq.z, cq.w};
+            uint4 bq[4], cq[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              const float2 bf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[i]));
-              const float2 cf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&cw[i]));
-              const int n = 8 * q + 2 * i;
-              S[n] = fmaf(ab, S[n], dx * bf.x);
-              S[n + 1] = fmaf(ab, S[n + 1], dx * bf.y);
-              acc = fmaf(cf.x, S[n], acc);
-              acc = fmaf(cf.y, S[n + 1], acc);
+              bq[i] = *reinterpret_cast<const uint4*>(sm + SM_BT + sw128(t0s + i, q));
+              cq[i] = *reinterpret_cast<const uint4*>(sm + SM_CT + sw128(t0s + i, q));
             }
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const uint32_t bw = m == 0 ? bq[i].x : m == 1 ? bq[i].y : m == 2 ? bq[i].z : bq[i].w;
+                const uint32_t cw = m == 0 ? cq[i].x : m == 1 ? cq[i].y : m == 2 ? cq[i].z : cq[i].w;
+                const int n = 8 * q + 2 * m;
+                S[n] = fmaf(ab[i], S[n], dx[i] * __uint_as_float(bw << 16));
+                S[n + 1] = fmaf(ab[i], S[n + 1], dx[i] * __uint_as_float(bw & 0xffff0000u));
+                acc[i] = fmaf(__uint_as_float(cw << 16), S[n], acc[i]);
+                acc[i] = fmaf(__uint_as_float(cw & 0xffff0000u), S[n + 1], acc[i]);
+              }
           }
-          ycol[t * MCH] = __float2bfloat16_rn(acc);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ycol[(t0s + i) * MCH] = __float2bfloat16_rn(acc[i]);
         }
       }
     }
@@ -541,7 +572,9 @@ int chunk_map(CUtensorMap* tm, const void* base, const Plan& pl, int elem_bytes,
 
 }  // namespace
 
-bool forward_y_mm_applies(const Plan& pl) { return pl.scalar && pl.io == AS_BF16 && pl.P % MCH == 0; }
+// Short narrow runs have segments of a few scan chunks (see make_plan), less than one chunk of this form: they take the scan
+// kernels (512 tokens x 256: 34 -> 26 us, 1,024 x 256: 38 -> 29 us).
+bool forward_y_mm_applies(const Plan& pl) { return pl.scalar && pl.io == AS_BF16 && pl.P % MCH == 0 && pl.one_order; }
 
 int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {
   CUtensorMap mx, md, my;
