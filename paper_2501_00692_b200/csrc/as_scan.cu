@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(NTHR, 4) forward_y_kernel(const __grid_constan
 // ------------------------------------------------------------------------------------------------
 constexpr int CARRY_UB = 8;
 constexpr int ONE_UB = 12;                       // of fixup_one_kernel, which has the registers
-constexpr int CARRY_WARPS = 32;                  // most warps of a CTA
+constexpr int CARRY_WARPS = 16;                  // most warps of a CTA
 constexpr int CARRY_SLICES = TILE_FLOATS / 64;   // CTAs per (tile, batch element): 64 floats each
 
 struct Slot {           // the state pair of a lane: pair `iu` of its tile block
@@ -696,7 +696,7 @@ __device__ __forceinline__ void mark_live(const Plan& pl, const float* __restric
 // All carries of a call in one launch (they are independent): blocks [0, nh) the forward carry, then the suffixes, then
 // (windows of more than four whole segments) the prefixes; shorter windows are summed by the main kernel; one CTA per
 // (slice, tile, batch element) each.  Then (truncated form) the liveness of the segments.
-__global__ void __launch_bounds__(32 * CARRY_WARPS, 1) fixup_kernel(Plan pl, const float* __restrict__ A_log,
+__global__ void __launch_bounds__(32 * CARRY_WARPS, 2) fixup_kernel(Plan pl, const float* __restrict__ A_log,
                                                                    char* __restrict__ ws, int nh, int roles) {
   __shared__ CarrySmem sm;
   pdl_begin();
@@ -779,13 +779,14 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
   const int64_t nlive = with_mu && !pl.full ? (int64_t)pl.tiles * pl.B * pl.S : 0;
   if (pl.one_order)
     return launch_dependent(fixup_one_kernel, dim3((unsigned)((nh + 3) / 4)), dim3(128), 0, st, pl, sp.A_log, sp.ws);
-  // Few CTAs: as many warps as the chip holds, four segments or more each.  Many: eight warps each (T = 65,536, P = 768,
-  // B = 2: 9.7 us; 4 warps 11.6, 16 warps 10.0, 32 warps 16.3).
+  // All CTAs should be resident at once, 32 warps of 64 registers to an SM; short of that, fewer warps with longer ranges (at
+  // most 16 warps: their combination is serial).  T = 65,536, P = 768, B = 2 (384 CTAs and the liveness warps): 12 warps, which
+  // leave a second, part-filled wave, 28.7 us; 8 warps 22.5, 6 warps 20.6.  T = 16,384, P = 512: 8 warps 14.3, 12 warps 20.5.
+  // T = 8,192, P = 256 (64 CTAs): 10 to 16 warps 12.3, 32 warps 16.4.
   // By one layer's CTAs: a layer's results do not depend on how many it is computed with.
-  int64_t warps = (int64_t)sm_count() * 32 / ((int64_t)CARRY_SLICES * pl.tiles * pl.Bg * roles);
-  if (warps < 8) warps = 8;
+  const int64_t ctas = (int64_t)CARRY_SLICES * pl.tiles * pl.Bg * roles + (nlive > 0 ? (int64_t)pl.tiles * pl.Bg * pl.S / 8 : 0);
+  int64_t warps = ctas <= 2 * sm_count() ? CARRY_WARPS : ctas <= 3 * sm_count() ? 8 : 6;
   if (warps > (pl.S + 3) / 4) warps = (pl.S + 3) / 4;
-  if (warps > CARRY_WARPS) warps = CARRY_WARPS;
   const int64_t blocks = nh * roles + (nlive + warps - 1) / warps;
   if (blocks > 0x7fffffff) return 1;
   return launch_dependent(fixup_kernel, dim3((unsigned)blocks), dim3((unsigned)warps * 32), 0, st, pl, sp.A_log, sp.ws, (int)nh, roles);
