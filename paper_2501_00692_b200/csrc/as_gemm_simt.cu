@@ -14,8 +14,13 @@
 namespace as {
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16, TM = 8, TN = 4, NT = 128;
-constexpr int PADM = BM + 4, PADN = BN + 4;
+constexpr int NT = 128;
+// Output tiles of BT x BT by 128 threads, TM x TN each; either way two 16-byte pieces of each operand per thread and K-tile.
+// Small: four times the CTAs and half the K-tiles, for shapes whose 64 x 64 tiles leave SMs without a CTA and whose time is
+// the K-tiles' latency (512 tokens x 64, the whole gradient: 44 -> 36 us; 1,024 x 64 x 12 layers, a training step: 487 -> 425 us).
+struct Large { static constexpr int BT = 64, BK = 16, TM = 8, TN = 4, PAD = BT + 4; };
+struct Small { static constexpr int BT = 32, BK = 32, TM = 4, TN = 2, PAD = BT + 4; };
+template <typename Cf> struct Smem { float a[2][Cf::BK][Cf::PAD], b[2][Cf::BK][Cf::PAD]; };
 enum { C_PROJ = 0, C_DW = 1, C_DX = 2 };
 
 struct SimtArgs {
@@ -46,9 +51,24 @@ __device__ __forceinline__ const float* gcat_at(const SimtArgs& a, int64_t l, in
   return c < a.P ? a.du + row * a.P + c : a.dbc + row * NBC + c - a.P;
 }
 
-// one BM x BN output tile of one contraction; blk: tile index inside this contraction's grid
-template <int KIND>
-__device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)[2][BK][PADM], float (&Bs)[2][BK][PADN]) {
+template <int N> struct VecOf { typedef float4 T; };
+template <> struct VecOf<2> { typedef float2 T; };
+// N floats at a time
+template <int N> __device__ __forceinline__ void ldg_n(const float* p, float (&v)[N]) {
+  *reinterpret_cast<typename VecOf<N>::T*>(v) = __ldg(reinterpret_cast<const typename VecOf<N>::T*>(p));
+}
+template <int N> __device__ __forceinline__ void stg_n(float* p, const float (&v)[N]) {
+  *reinterpret_cast<typename VecOf<N>::T*>(p) = *reinterpret_cast<const typename VecOf<N>::T*>(v);
+}
+
+// one BT x BT output tile of one contraction; blk: tile index inside this contraction's grid
+template <int KIND, typename Cf>
+__device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, Smem<Cf>& sm) {
+  constexpr int BM = Cf::BT, BN = Cf::BT, BK = Cf::BK, TM = Cf::TM, TN = Cf::TN;
+  constexpr int KQ = BK / 4, RQ = Cf::BT / 4;   // 16-byte pieces of a K-tile row, of an output-tile row
+  static_assert(BM * KQ == 2 * NT && (BM / TM) * (BN / TN) == NT, "two pieces and one block of outputs per thread");
+  auto& As = sm.a;
+  auto& Bs = sm.b;
   const int tid = threadIdx.x;
   const int P = a.P, NW = P + NBC;
   // output extent [R, N] and contraction length K of one layer
@@ -79,14 +99,14 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)
     for (int i = 0; i < 2; ++i) {
       const int idx = tid + i * NT;
       {
-        const int64_t m = m0 + (A_K ? idx >> 2 : (idx & 15) * 4), k = k0 + (A_K ? (idx & 3) * 4 : idx >> 4);
+        const int64_t m = m0 + (A_K ? idx / KQ : (idx % RQ) * 4), k = k0 + (A_K ? (idx % KQ) * 4 : idx / RQ);
         const float* p = KIND == C_PROJ ? a.x + (lay * a.M + m) * P + k
                                         : (KIND == C_DX ? gcat_at(a, lay, m, (int)k) : gcat_at(a, lay, k, (int)m));
         ra[i] = m < R && k < kend ? ldg4(p) : zero4;
       }
       {
-        const int n = n0 + (B_K ? idx >> 2 : (idx & 15) * 4);
-        const int64_t k = k0 + (B_K ? (idx & 3) * 4 : idx >> 4);
+        const int n = n0 + (B_K ? idx / KQ : (idx % RQ) * 4);
+        const int64_t k = k0 + (B_K ? (idx % KQ) * 4 : idx / RQ);
         const float* p = KIND == C_PROJ ? wcat_at(a, lay, n, (int)k)
                                         : (KIND == C_DX ? wcat_at(a, lay, (int)k, n) : a.x + (lay * a.M + k) * P + n);
         rb[i] = n < N && k < kend ? ldg4(p) : zero4;
@@ -98,21 +118,21 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)
     for (int i = 0; i < 2; ++i) {
       const int idx = tid + i * NT;
       if (A_K) {
-        const int m = idx >> 2, k = (idx & 3) * 4;
+        const int m = idx / KQ, k = (idx % KQ) * 4;
         As[buf][k][m] = ra[i].x; As[buf][k + 1][m] = ra[i].y; As[buf][k + 2][m] = ra[i].z; As[buf][k + 3][m] = ra[i].w;
       } else {
-        *reinterpret_cast<float4*>(&As[buf][idx >> 4][(idx & 15) * 4]) = ra[i];
+        *reinterpret_cast<float4*>(&As[buf][idx / RQ][(idx % RQ) * 4]) = ra[i];
       }
       if (B_K) {
-        const int n = idx >> 2, k = (idx & 3) * 4;
+        const int n = idx / KQ, k = (idx % KQ) * 4;
         Bs[buf][k][n] = rb[i].x; Bs[buf][k + 1][n] = rb[i].y; Bs[buf][k + 2][n] = rb[i].z; Bs[buf][k + 3][n] = rb[i].w;
       } else {
-        *reinterpret_cast<float4*>(&Bs[buf][idx >> 4][(idx & 15) * 4]) = rb[i];
+        *reinterpret_cast<float4*>(&Bs[buf][idx / RQ][(idx % RQ) * 4]) = rb[i];
       }
     }
   };
 
-  const int tx = tid & 15, ty = tid >> 4;   // this thread's rows ty*8 .. +7, columns tx*4 .. +3
+  const int tx = tid % (BN / TN), ty = tid / (BN / TN);   // this thread's rows ty*TM .. and columns tx*TN ..
   float acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -128,11 +148,10 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)
     if (more) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * TN]);
-      const float av[TM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[TN] = {b0.x, b0.y, b0.z, b0.w};
+      __align__(16) float av[TM], bv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; i += 4) *reinterpret_cast<float4*>(av + i) = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + i]);
+      *reinterpret_cast<typename VecOf<TN>::T*>(bv) = *reinterpret_cast<const typename VecOf<TN>::T*>(&Bs[buf][kk][tx * TN]);
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -144,49 +163,55 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, float (&As)
     }
   }
 
-  const int n = n0 + tx * TN;   // four columns: all inside one part (its border is a multiple of 8) or all outside
+  const int n = n0 + tx * TN;   // TN columns: all inside one part (its border is a multiple of 8) or all outside
   if (n >= N) return;
-  float4 bias = zero4;
-  if (KIND == C_PROJ && n < P) bias = ldg4(a.b_delta + lay * P + n);
+  __align__(16) float bias[TN] = {};
+  if (KIND == C_PROJ && n < P) ldg_n<TN>(a.b_delta + lay * P + n, bias);
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int64_t m = m0 + ty * TM + i;
     if (m >= R) break;
     const int64_t row = lay * a.M + m;
-    float4 v = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __align__(16) float v[TN];
+#pragma unroll
+    for (int j = 0; j < TN; ++j) v[j] = acc[i][j];
     if (KIND == C_PROJ) {
       if (n < P) {
-        v = make_float4(softplus_f(v.x + bias.x), softplus_f(v.y + bias.y), softplus_f(v.z + bias.z), softplus_f(v.w + bias.w));
-        *reinterpret_cast<float4*>(a.delta + row * P + n) = v;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) v[j] = softplus_f(v[j] + bias[j]);
+        stg_n<TN>(a.delta + row * P + n, v);
       } else {
-        *reinterpret_cast<float4*>(a.bc + row * NBC + n - P) = v;
+        stg_n<TN>(a.bc + row * NBC + n - P, v);
       }
     } else if (KIND == C_DX) {
-      const float4 d = ldg4(a.dxdir + row * P + n);
-      *reinterpret_cast<float4*>(a.dx + row * P + n) = make_float4(v.x + d.x, v.y + d.y, v.z + d.z, v.w + d.w);
+      __align__(16) float d[TN];
+      ldg_n<TN>(a.dxdir + row * P + n, d);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) v[j] += d[j];
+      stg_n<TN>(a.dx + row * P + n, v);
     } else {
       const int e = (int)m - P;
       float* dst = e < 0 ? a.dW_delta + (lay * P + m) * P + n
                          : (e < NS ? a.dW_B + (lay * NS + e) * P + n : a.dW_C + (lay * NS + e - NS) * P + n);
-      atomicAdd(reinterpret_cast<float4*>(dst), v);
+      atomicAdd(reinterpret_cast<typename VecOf<TN>::T*>(dst), *reinterpret_cast<typename VecOf<TN>::T*>(v));
     }
   }
 }
 
+template <typename Cf>
 __global__ void __launch_bounds__(NT) simt_proj_kernel(const __grid_constant__ SimtArgs a) {
-  __shared__ __align__(16) float As[2][BK][PADM];
-  __shared__ __align__(16) float Bs[2][BK][PADN];
+  __shared__ __align__(16) Smem<Cf> sm;
   pdl_begin();
   clear_regions(a.zero, (int64_t)blockIdx.x * NT + threadIdx.x, (int64_t)gridDim.x * NT);
-  tile<C_PROJ>(a, blockIdx.x, As, Bs);
+  tile<C_PROJ, Cf>(a, blockIdx.x, sm);
 }
 // both gradient contractions: the first ndx blocks compute dx, the rest the weight gradients
+template <typename Cf>
 __global__ void __launch_bounds__(NT) simt_grad_kernel(const __grid_constant__ SimtArgs a) {
-  __shared__ __align__(16) float As[2][BK][PADM];
-  __shared__ __align__(16) float Bs[2][BK][PADN];
+  __shared__ __align__(16) Smem<Cf> sm;
   pdl_begin();
-  if ((int)blockIdx.x < a.ndx) tile<C_DX>(a, blockIdx.x, As, Bs);
-  else tile<C_DW>(a, (int64_t)blockIdx.x - a.ndx, As, Bs);
+  if ((int)blockIdx.x < a.ndx) tile<C_DX, Cf>(a, blockIdx.x, sm);
+  else tile<C_DW, Cf>(a, (int64_t)blockIdx.x - a.ndx, sm);
 }
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -202,25 +227,34 @@ int simt_projections(const Plan& pl, const as_params_t* pr, const void* x, const
   SimtArgs a = base_args(pl, pr, x);
   a.zero = z;
   a.delta = (float*)(ws + pl.off_delta); a.bc = (float*)(ws + pl.off_bc);
-  const int64_t blocks = cdiv(a.M, BM) * cdiv(pl.P + NBC, BN) * a.layers;
-  if (blocks > 0x7fffffff) return 1;
-  return launch_dependent(simt_proj_kernel, dim3((unsigned)blocks), dim3(NT), 0, st, a);
+  auto blocks = [&](int bt) { return cdiv(a.M, bt) * cdiv(pl.P + NBC, bt) * a.layers; };
+  if (blocks(Large::BT) > 0x7fffffff) return 1;
+  if (blocks(Large::BT) < sm_count())
+    return launch_dependent(simt_proj_kernel<Small>, dim3((unsigned)blocks(Small::BT)), dim3(NT), 0, st, a);
+  return launch_dependent(simt_proj_kernel<Large>, dim3((unsigned)blocks(Large::BT)), dim3(NT), 0, st, a);
 }
 
 int simt_gradients(const Plan& pl, const as_params_t* pr, const void* x, const as_grads_t* out, char* ws, cudaStream_t st) {
   SimtArgs a = base_args(pl, pr, x);
   a.du = (const float*)(ws + pl.off_du); a.dbc = (const float*)(ws + pl.off_dbc); a.dxdir = (const float*)(ws + pl.off_dxdir);
   a.dW_delta = out->dW_delta; a.dW_B = out->dW_B; a.dW_C = out->dW_C; a.dx = (float*)out->dx;
-  const int64_t ndx = out->dx ? cdiv(a.M, BM) * cdiv(pl.P, BN) * a.layers : 0;
-  const int64_t tiles = cdiv(pl.P + NBC, BM) * cdiv(pl.P, BN) * a.layers;
-  // split over the tokens: about four CTAs per SM, 64 tokens or more each (below that the reductions outweigh the sums)
-  int64_t s = cdiv((int64_t)sm_count() * 4, tiles);
-  if (s > cdiv(a.M, 64)) s = cdiv(a.M, 64);
-  a.splitk = (int)(s < 1 ? 1 : s);
-  a.ndx = (int)ndx;
-  const int64_t blocks = ndx + tiles * a.splitk;
+  auto grid = [&](int bt) {   // number of blocks; sets a.ndx and a.splitk
+    const int64_t ndx = out->dx ? cdiv(a.M, bt) * cdiv(pl.P, bt) * a.layers : 0;
+    const int64_t tiles = cdiv(pl.P + NBC, bt) * cdiv(pl.P, bt) * a.layers;
+    // split over the tokens: about four CTAs per SM, 64 tokens or more each (below that the reductions outweigh the sums)
+    int64_t s = cdiv((int64_t)sm_count() * 4, tiles);
+    if (s > cdiv(a.M, 64)) s = cdiv(a.M, 64);
+    a.splitk = (int)(s < 1 ? 1 : s);
+    a.ndx = (int)ndx;
+    return ndx + tiles * a.splitk;
+  };
+  int64_t blocks = grid(Large::BT);
   if (blocks > 0x7fffffff) return 1;
-  return launch_dependent(simt_grad_kernel, dim3((unsigned)blocks), dim3(NT), 0, st, a);
+  if (blocks < sm_count()) {
+    blocks = grid(Small::BT);
+    return launch_dependent(simt_grad_kernel<Small>, dim3((unsigned)blocks), dim3(NT), 0, st, a);
+  }
+  return launch_dependent(simt_grad_kernel<Large>, dim3((unsigned)blocks), dim3(NT), 0, st, a);
 }
 
 }  // namespace as
