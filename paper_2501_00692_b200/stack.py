@@ -43,10 +43,14 @@ class Stack:
     def forward(self, y0: torch.Tensor):
         """Runs the stack, keeping y_0..y_K (the per-layer inputs are re-normalised in the backward)."""
         self.ys = [y0]
+        # y_1 .. y_{K-1} in one block (one allocation, and the paper mode normalises them in one launch); y_K, which the
+        # caller may keep, on its own
+        block = torch.empty(max(self.K - 1, 0), *y0.shape, dtype=y0.dtype, device=y0.device)
+        outs = [*block.unbind(0), torch.empty_like(y0)] if self.K else []
         B.as_rmsnorm_fwd(self.shape, y0, self.yhat, self.eps)
         for k, th in enumerate(self.thetas):
             B.as_ssm_forward(self.shape, th, self.yhat, self.ytilde, self.ws)
-            yk = torch.empty_like(y0)
+            yk = outs[k]
             if k + 1 < self.K:   # the next layer's input is the norm of the sum: both in one pass
                 B.as_residual_add_rmsnorm(self.shape, self.ys[-1], self.ytilde, yk, self.yhat, self.eps)
             else:
@@ -85,11 +89,24 @@ class Stack:
             self._stacked = {k: torch.stack([th[k] for th in self.thetas]).contiguous() for k in keys}
             self._ws_layers = B.alloc_workspace(B.as_workspace_bytes_layers(sh, K, self.tbar), self.device)
             self._xall = torch.empty(K, sh.batch, sh.seqlen, sh.d_model, dtype=self.yhat.dtype, device=self.device)
-        for k in range(K):
-            B.as_rmsnorm_fwd(sh, self.ys[k], self._xall[k], self.eps)
-            if record is not None and k in record:
-                record[k] = (self._xall[k].clone(), g.clone())
+            self._x = self._xall.unbind(0)
+        # norms row by row: layers whose inputs lie one behind the other (as forward() leaves y_1 .. y_{K-1}) take one launch
+        step = self._x[0].numel() * self._x[0].element_size()
+        at = [y.data_ptr() for y in self.ys[:K]]
+        k = 0
+        while k < K:
+            e = k + 1
+            while e < K and at[e] == at[e - 1] + step:
+                e += 1
+            run = B.make_shape(sh.batch * (e - k), sh.seqlen, sh.d_model, sh.d_state, sh.io)
+            B.as_rmsnorm_fwd(run, self.ys[k], self._x[k], self.eps)
+            k = e
+        if record is not None:
+            for k in record:
+                if 0 <= k < K:
+                    record[k] = (self._x[k].clone(), g.clone())
         gl = B.alloc_grads_layers(sh, K, g.device)
         B.as_adjoint_grad_layers(sh, K, self._stacked, self._xall, g, self.tbar, gl, self._ws_layers)
         self.ws_last = self._ws_layers
-        return [{k: (v[i] if v is not None else None) for k, v in gl.items()} for i in range(K)]
+        per_layer = {k: (v.unbind(0) if v is not None else [None] * K) for k, v in gl.items()}
+        return [{k: v[i] for k, v in per_layer.items()} for i in range(K)]
