@@ -122,6 +122,13 @@ int as_check_status(const void *ws, void *stream);
 int as_ssm_forward(const as_shape_t *shape, const as_params_t *params, const void *x, void *y,
                    void *ws, size_t ws_bytes, void *stream);
 
+/* as_ssm_forward for the layers of a stack with bf16 I/O: always the same order of additions, for every size (one segmentation,
+ * one order of the carries; at widths that are no multiple of 32 the projections run on the fp32 pipe).  A deep stack that rounds
+ * every layer's output to bf16 turns differences in the last fp32 bit of one layer into differences of some per cent of its
+ * outputs, so there the order is part of the result; a single layer does not need it. */
+int as_ssm_forward_ordered(const as_shape_t *shape, const as_params_t *params, const void *x, void *y,
+                           void *ws, size_t ws_bytes, void *stream);
+
 /* Adjoint-method gradient of L = sum_t l^t(y^t) w.r.t. the layer parameters and x, given dy = dl^t/dy^t
  * (Proposition 2; with tbar < T the truncated form, Eq. 7 of Section 4.3; Algorithms 2-4 for one layer).
  * Token t contributes A-net and B-net vector-Jacobian products only for source tokens i in

@@ -59,7 +59,7 @@ struct Wcat { const void* p; int reps; };
 // call).  The gradient of a width that is not a multiple of 32 needs W_B and W_C once per term of the dB, dC split.
 int begin(const Plan& pl, const as_params_t* pr, const ZeroList& z, bool grad, const void* x, char* ws, cudaStream_t st,
           Wcat* wcat) {
-  if (!pl.tc) {
+  if (!pl.tc || pl.ffma) {
     AS_TRY(pl.split ? split_projections(pl, pr, x, z, ws, st) : simt_projections(pl, pr, x, z, ws, st));
     return AS_OK;
   }
@@ -179,8 +179,8 @@ int as_check_status(const void* ws, void* stream) {
   return word;
 }
 
-int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,
-                   size_t ws_bytes, void* stream) {
+static int forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes,
+                   void* stream, int kind) {
   int e = check_shape(shape);
   if (e) return e;
   e = check_params(params);
@@ -188,7 +188,7 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
   if (!x || !y || !ws) return AS_ERR_NULL;
   if (!aligned16(x) || !aligned16(y) || !aligned16(ws)) return AS_ERR_ALIGN;
   Plan pl;
-  e = make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD);
+  e = make_plan(shape, shape->seqlen, 1, &pl, kind);
   if (e) return e;
   if (ws_bytes < pl.total_fwd && pl.split) {   // the fixed scratch of as_ssm_forward_static may only hold the smaller plan
     e = make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD_SMALL);
@@ -210,6 +210,16 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
   if (mm) AS_TRY(launch_forward_y_mm(pl, sp, y, st));
   else AS_TRY(launch_forward_y(pl, sp, y, st));
   return AS_OK;
+}
+
+int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,
+                   size_t ws_bytes, void* stream) {
+  return forward(shape, params, x, y, ws, ws_bytes, stream, PLAN_FWD);
+}
+
+int as_ssm_forward_ordered(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,
+                           size_t ws_bytes, void* stream) {
+  return forward(shape, params, x, y, ws, ws_bytes, stream, PLAN_FWD_ORDERED);
 }
 
 int as_adjoint_grad(const as_shape_t* shape, const as_params_t* params, const void* x, const void* dy, int64_t tbar,

@@ -1,7 +1,7 @@
 // FP32-pipe contractions of the layer for fp32 I/O, where the 1e-4 parity bar rules out TF32 or single bf16 tensor-core
 // inputs.  One kernel body covers the three contractions over the virtual matrices Wcat = [W_delta; W_B; W_C] ([P+32, P])
 // and Gcat = [du | dB | dC] ([tokens, P+32]), whose parts are read where they lie:
-//   PROJ : [Delta | B | C] = X Wcat^T            (softplus + bias on the Delta columns)
+//   PROJ : [Delta | B | C] = X Wcat^T            (softplus + bias on the Delta columns) (bf16 I/O too: as_ssm_forward_ordered)
 //   DW   : [dW_delta; dW_B; dW_C] += Gcat^T X    (split over the tokens, fp32 reductions)
 //   DX   : dx = dx_dir + Gcat Wcat
 // Bound: the FP32 pipe for large shapes (8 x 4 outputs per thread: 32 FFMA per three 16-byte shared-memory loads), latency
@@ -24,7 +24,8 @@ template <typename Cf> struct Smem { float a[2][Cf::BK][Cf::PAD], b[2][Cf::BK][C
 enum { C_PROJ = 0, C_DW = 1, C_DX = 2 };
 
 struct SimtArgs {
-  const float *x, *W_delta, *W_B, *W_C, *b_delta;
+  const void *x, *W_delta, *W_B, *W_C;   // in the I/O type
+  const float* b_delta;
   float *delta, *bc;                 // PROJ outputs
   const float *du, *dbc, *dxdir;     // gradient inputs
   float *dW_delta, *dW_B, *dW_C, *dx;
@@ -37,14 +38,22 @@ struct SimtArgs {
 __device__ __forceinline__ float softplus_f(float u) {
   return fmaxf(u, 0.f) + log1pf(expf(-fabsf(u)));
 }
+// four values in a row
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ldg4(const __nv_bfloat16* p) {
+  const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
 
-// a 16-byte piece of row r of Wcat (columns c..c+3), of row m of Gcat
-__device__ __forceinline__ const float* wcat_at(const SimtArgs& a, int64_t l, int r, int c) {
+// columns c..c+3 of row r of Wcat, of row m of X, of row m of Gcat
+template <typename IO> __device__ __forceinline__ const IO* wcat_at(const SimtArgs& a, int64_t l, int r, int c) {
   const int64_t P = a.P;
-  if (r < a.P) return a.W_delta + (l * P + r) * P + c;
+  if (r < a.P) return static_cast<const IO*>(a.W_delta) + (l * P + r) * P + c;
   r -= a.P;
-  return r < NS ? a.W_B + (l * NS + r) * P + c : a.W_C + (l * NS + r - NS) * P + c;
+  return r < NS ? static_cast<const IO*>(a.W_B) + (l * NS + r) * P + c : static_cast<const IO*>(a.W_C) + (l * NS + r - NS) * P + c;
+}
+template <typename IO> __device__ __forceinline__ const IO* x_at(const SimtArgs& a, int64_t l, int64_t m, int64_t c) {
+  return static_cast<const IO*>(a.x) + (l * a.M + m) * a.P + c;
 }
 __device__ __forceinline__ const float* gcat_at(const SimtArgs& a, int64_t l, int64_t m, int c) {
   const int64_t row = l * a.M + m;
@@ -62,7 +71,7 @@ template <int N> __device__ __forceinline__ void stg_n(float* p, const float (&v
 }
 
 // one BT x BT output tile of one contraction; blk: tile index inside this contraction's grid
-template <int KIND, typename Cf>
+template <int KIND, typename Cf, typename IO = float>
 __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, Smem<Cf>& sm) {
   constexpr int BM = Cf::BT, BN = Cf::BT, BK = Cf::BK, TM = Cf::TM, TN = Cf::TN;
   constexpr int KQ = BK / 4, RQ = Cf::BT / 4;   // 16-byte pieces of a K-tile row, of an output-tile row
@@ -100,16 +109,16 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, Smem<Cf>& s
       const int idx = tid + i * NT;
       {
         const int64_t m = m0 + (A_K ? idx / KQ : (idx % RQ) * 4), k = k0 + (A_K ? (idx % KQ) * 4 : idx / RQ);
-        const float* p = KIND == C_PROJ ? a.x + (lay * a.M + m) * P + k
-                                        : (KIND == C_DX ? gcat_at(a, lay, m, (int)k) : gcat_at(a, lay, k, (int)m));
-        ra[i] = m < R && k < kend ? ldg4(p) : zero4;
+        const bool in = m < R && k < kend;
+        if constexpr (KIND == C_PROJ) ra[i] = in ? ldg4(x_at<IO>(a, lay, m, k)) : zero4;
+        else ra[i] = in ? ldg4(KIND == C_DX ? gcat_at(a, lay, m, (int)k) : gcat_at(a, lay, k, (int)m)) : zero4;
       }
       {
         const int n = n0 + (B_K ? idx / KQ : (idx % RQ) * 4);
         const int64_t k = k0 + (B_K ? (idx % KQ) * 4 : idx / RQ);
-        const float* p = KIND == C_PROJ ? wcat_at(a, lay, n, (int)k)
-                                        : (KIND == C_DX ? wcat_at(a, lay, (int)k, n) : a.x + (lay * a.M + k) * P + n);
-        rb[i] = n < N && k < kend ? ldg4(p) : zero4;
+        const bool in = n < N && k < kend;
+        if constexpr (KIND == C_PROJ) rb[i] = in ? ldg4(wcat_at<IO>(a, lay, n, (int)k)) : zero4;
+        else rb[i] = in ? ldg4(KIND == C_DX ? wcat_at<IO>(a, lay, (int)k, n) : x_at<IO>(a, lay, k, n)) : zero4;
       }
     }
   };
@@ -198,12 +207,12 @@ __device__ __forceinline__ void tile(const SimtArgs& a, int64_t blk, Smem<Cf>& s
   }
 }
 
-template <typename Cf>
+template <typename Cf, typename IO>
 __global__ void __launch_bounds__(NT) simt_proj_kernel(const __grid_constant__ SimtArgs a) {
   __shared__ __align__(16) Smem<Cf> sm;
   pdl_begin();
   clear_regions(a.zero, (int64_t)blockIdx.x * NT + threadIdx.x, (int64_t)gridDim.x * NT);
-  tile<C_PROJ, Cf>(a, blockIdx.x, sm);
+  tile<C_PROJ, Cf, IO>(a, blockIdx.x, sm);
 }
 // both gradient contractions: the first ndx blocks compute dx, the rest the weight gradients
 template <typename Cf>
@@ -217,7 +226,7 @@ __global__ void __launch_bounds__(NT) simt_grad_kernel(const __grid_constant__ S
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 SimtArgs base_args(const Plan& pl, const as_params_t* pr, const void* x) {
   SimtArgs a{};
-  a.x = (const float*)x; a.W_delta = (const float*)pr->W_delta; a.W_B = (const float*)pr->W_B; a.W_C = (const float*)pr->W_C;
+  a.x = x; a.W_delta = pr->W_delta; a.W_B = pr->W_B; a.W_C = pr->W_C;
   a.b_delta = pr->b_delta; a.M = (int64_t)pl.Bg * pl.T; a.P = pl.P; a.layers = pl.KL; a.splitk = 1;
   return a;
 }
@@ -229,9 +238,11 @@ int simt_projections(const Plan& pl, const as_params_t* pr, const void* x, const
   a.delta = (float*)(ws + pl.off_delta); a.bc = (float*)(ws + pl.off_bc);
   auto blocks = [&](int bt) { return cdiv(a.M, bt) * cdiv(pl.P + NBC, bt) * a.layers; };
   if (blocks(Large::BT) > 0x7fffffff) return 1;
-  if (blocks(Large::BT) < sm_count())
-    return launch_dependent(simt_proj_kernel<Small>, dim3((unsigned)blocks(Small::BT)), dim3(NT), 0, st, a);
-  return launch_dependent(simt_proj_kernel<Large>, dim3((unsigned)blocks(Large::BT)), dim3(NT), 0, st, a);
+  const bool small = blocks(Large::BT) < sm_count();
+  const dim3 grid((unsigned)blocks(small ? Small::BT : Large::BT));
+  auto kern = pl.io == AS_BF16 ? (small ? simt_proj_kernel<Small, __nv_bfloat16> : simt_proj_kernel<Large, __nv_bfloat16>)
+                               : (small ? simt_proj_kernel<Small, float> : simt_proj_kernel<Large, float>);
+  return launch_dependent(kern, grid, dim3(NT), 0, st, a);
 }
 
 int simt_gradients(const Plan& pl, const as_params_t* pr, const void* x, const as_grads_t* out, char* ws, cudaStream_t st) {

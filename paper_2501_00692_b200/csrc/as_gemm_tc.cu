@@ -8,6 +8,8 @@
 //   DW   : dWcat = Gcat^T X  over all tokens     (A MN-major, B MN-major; split-K, fp32 reduction)
 //   DX   : dx = dx_dir + Gcat Wcat               (A K-major, B MN-major; add + bf16 store)
 // with Wcat = [W_delta; W_B; W_C] ([P+32, P]) and Gcat = [du | dB | dC] ([tokens, P+32]), both bf16.
+// Widths that are not a multiple of 32 take the fp32-accurate softplus: a deep bf16 stack turns rounding differences of one
+// layer's Delta into differences of some per cent of its outputs, and these widths never had the shorter one.
 // Widths that are not a multiple of 32 keep all 24 bits of dB and dC: Gcat then ends in three such pairs (the fp32 sums
 // split into three bf16 terms, which is exact) and the Wcat of the input gradient repeats W_B and W_C three times
 // (Plan.gsplit), so the contraction of the split equals the contraction of the fp32 values.
@@ -55,7 +57,7 @@ struct TcArgs {
 //                      buffer a while the issuer already fills buffer a^1 for the next tile
 // Tile order: n fastest, then m, then the K split, so concurrently running CTAs share A rows through L2.
 // ML: several layers stacked along the leading dimension of every tensor (false compiles the single-layer code).
-// OFF: P is not a multiple of 16 (the code for it costs the projections 10 % wherever it is compiled in).
+// OFF: P is not a multiple of 16 (projections: of 32; the code for it costs them 10 % wherever it is compiled in).
 template <int AMAJ, int BMAJ, int EPI, int BN, bool ML, bool OFF>
 __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA,
                                                            const __grid_constant__ CUtensorMap tmB,
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
                                        __uint_as_float(r[4 * q + 3]));
                 if (col < a.P) {
                   const float4 bv = __ldg(reinterpret_cast<const float4*>(bias_l + col));
-                  v = make_float4(softplus_f(v.x + bv.x), softplus_f(v.y + bv.y), softplus_f(v.z + bv.z), softplus_f(v.w + bv.w));
+                  v = make_float4(softplus_fine(v.x + bv.x), softplus_fine(v.y + bv.y), softplus_fine(v.z + bv.z), softplus_fine(v.w + bv.w));
                 } else if (col < a.P + NBC && row < a.M) {
                   *reinterpret_cast<float4*>(a.bc + row * NBC + col - a.P) = v;
                 }
@@ -286,8 +288,8 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
               for (int q = 0; q < 4; ++q) {
                 const float4 bv = __ldg(b4 + q);
                 *reinterpret_cast<float4*>(buf + swz64(lane, q)) =
-                    make_float4(softplus_f(__uint_as_float(r[4 * q]) + bv.x), softplus_f(__uint_as_float(r[4 * q + 1]) + bv.y),
-                                softplus_f(__uint_as_float(r[4 * q + 2]) + bv.z), softplus_f(__uint_as_float(r[4 * q + 3]) + bv.w));
+                    make_float4(softplus<OFF>(__uint_as_float(r[4 * q]) + bv.x), softplus<OFF>(__uint_as_float(r[4 * q + 1]) + bv.y),
+                                softplus<OFF>(__uint_as_float(r[4 * q + 2]) + bv.z), softplus<OFF>(__uint_as_float(r[4 * q + 3]) + bv.w));
               }
             } else {
 #pragma unroll
@@ -400,7 +402,7 @@ int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorM
 
 template <int AMAJ, int BMAJ, int EPI, int BN>
 int launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const TcArgs& a, cudaStream_t st) {
-  if (EPI != TC_DX && a.P % 16)   // the input gradient has no border inside a chunk
+  if ((EPI == TC_DW && a.P % 16) || (EPI == TC_PROJ && a.P % 32))   // the input gradient has no border inside a chunk
     return a.layers > 1 ? launch_tc_ml<AMAJ, BMAJ, EPI, BN, true, EPI != TC_DX>(tmA, tmB, tmO, a, st)
                         : launch_tc_ml<AMAJ, BMAJ, EPI, BN, false, EPI != TC_DX>(tmA, tmB, tmO, a, st);
   return a.layers > 1 ? launch_tc_ml<AMAJ, BMAJ, EPI, BN, true, false>(tmA, tmB, tmO, a, st)

@@ -118,6 +118,7 @@ struct Plan {
   int tiles;        // ceil(P / CH) channel tiles
   int bw;           // channels per staged row: min(CH, P)
   int tc;           // 1: bf16 tensor-core contractions (bf16 I/O), 0: FP32-pipe GEMMs
+  int ffma;         // projections of bf16 I/O on the fp32 pipe (as_ssm_forward_ordered, widths off the 32-element grid)
   int one_order;    // bf16 forward: one segmentation and one order of the carries for all sizes
   int split;        // fp32 I/O: contractions on the tensor cores, every operand as three bf16 terms (as_gemm_split.cu)
   int gsplit;       // bf16 terms per value of dB, dC in Gcat: 1, or 3 (exact) where d_model % 32 != 0
@@ -130,7 +131,8 @@ struct Plan {
 
 // PLAN_GRAD: gradient calls.  PLAN_FWD: as_ssm_forward.  PLAN_FWD_SMALL: an fp32 forward with less scratch (contractions on
 // the FP32 pipe).
-enum { PLAN_GRAD = 0, PLAN_FWD = 1, PLAN_FWD_SMALL = 2 };
+// PLAN_FWD_ORDERED: as_ssm_forward_ordered.
+enum { PLAN_GRAD = 0, PLAN_FWD = 1, PLAN_FWD_SMALL = 2, PLAN_FWD_ORDERED = 3 };
 int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind = PLAN_GRAD);
 // elements of A_log (and dA_log) per layer
 inline int64_t a_stride(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }

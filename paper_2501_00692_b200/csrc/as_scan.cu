@@ -55,12 +55,14 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   int64_t L = segment((int64_t)p.tiles * p.B);
   if (L < 160) L = segment((int64_t)p.tiles * p.Bg);
   int64_t lmin = p.full && p.T <= 1024 ? CK : 2 * CK;
-  if (kind != PLAN_GRAD && p.tc && !(p.P <= 256 && (int64_t)p.Bg * p.T <= 1024)) {
+  const bool ordered = kind == PLAN_FWD_ORDERED;
+  p.ffma = ordered && p.tc && p.gsplit > 1;
+  if (kind != PLAN_GRAD && p.tc && (ordered || !(p.P <= 256 && (int64_t)p.Bg * p.T <= 1024))) {
     p.one_order = 1;
     // The bf16 forward keeps one segmentation (two waves, 64 tokens at least) whatever the size: a deep stack of bf16 layers
     // turns fp32 rounding differences of one layer's y into differences of some per cent of its outputs, so its results
     // should not move when the schedule of other sizes is tuned.  Short narrow runs, which are all latency (256 tokens x
-    // 256: 37 us with these segments, 23 with short ones), are left out.
+    // 256: 37 us with these segments, 23 with short ones), are left out unless the caller asks for the order.
     int64_t s_target = 2 * slots / ((int64_t)p.tiles * p.B);
     if (s_target < 1) s_target = 1;
     L = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;

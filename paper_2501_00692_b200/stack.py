@@ -49,7 +49,7 @@ class Stack:
         outs = [*block.unbind(0), torch.empty_like(y0)] if self.K else []
         B.as_rmsnorm_fwd(self.shape, y0, self.yhat, self.eps)
         for k, th in enumerate(self.thetas):
-            B.as_ssm_forward(self.shape, th, self.yhat, self.ytilde, self.ws)
+            B.as_ssm_forward_ordered(self.shape, th, self.yhat, self.ytilde, self.ws)
             yk = outs[k]
             if k + 1 < self.K:   # the next layer's input is the norm of the sum: both in one pass
                 B.as_residual_add_rmsnorm(self.shape, self.ys[-1], self.ytilde, yk, self.yhat, self.eps)

@@ -16,10 +16,11 @@ DEV = "cuda:0"
 CASES = [(1, 1, 8), (2, 15, 72), (3, 66, 136), (1, 769, 264), (1, 4099, 520), (2, 1543, 384)]
 
 
+@pytest.mark.parametrize("entry", [B.as_ssm_forward, B.as_ssm_forward_ordered], ids=["plain", "ordered"])
 @pytest.mark.parametrize("scalar", [False, True], ids=["diagonal", "scalar"])
 @pytest.mark.parametrize("io", ["f32", "bf16"])
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "B%d-T%d-P%d" % c)
-def test_forward_edges(case, io, scalar):
+def test_forward_edges(case, io, scalar, entry):
     build_library()
     batch, T, P = case
     w = synth.custom_workload("forward", 59, batch, T, P, tbar=T, io=io)
@@ -30,7 +31,7 @@ def test_forward_edges(case, io, scalar):
     sh = B.shape_of(x, w.d_state, a_scalar=scalar)
     ws = B.alloc_workspace(B.as_workspace_bytes(sh, T)[0], DEV)
     y = torch.full_like(x, float("nan"))
-    B.as_ssm_forward(sh, theta, x, y, ws)
+    entry(sh, theta, x, y, ws)
     assert B.as_check_status(ws) == 0
     ref = theta_f64(theta)
     if scalar:
