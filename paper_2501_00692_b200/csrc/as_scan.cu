@@ -36,7 +36,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   p.bw = p.P < CH ? p.P : CH;
   // Full waves of the main kernel's resident CTAs (SMs x CTAs per SM).  A partly filled wave costs as much as a full one
   // (T = 30,000, P = 256: 147 us at two waves, 155 at one and a half), and a CTA has a fixed cost of some 20 tokens' time.
-  // So: three waves (two in the full form) while segments stay at 160 tokens or more, which balances the tail of long
+  // So: three waves (two in the full form) while segments stay at 160 tokens (truncated: two waves at 112) or more, for the tail of long
   // runs; else two, else one; and where not even one wave can be filled, segments as short as two chunks (one chunk for
   // short sequences, whose full-form carries are cheap): latency counts there, and it is the tokens of a segment.
   const int64_t slots = (int64_t)sm_count() * 3;   // resident CTAs of the main kernel
@@ -46,7 +46,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
       int64_t s_target = waves * slots / ctas;
       if (s_target < 1) s_target = 1;
       l = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;
-      if (l >= 160) break;
+      if (l >= (waves == 2 && !p.full ? 112 : 160)) break;   // 2 x 8,192 x 1,024, two waves of 120 tokens: 598 -> 581 us
     }
     return l;
   };
