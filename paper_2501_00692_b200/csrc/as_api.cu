@@ -123,6 +123,36 @@ ZeroList grad_regions(const Plan& pl, uint32_t flags, const as_grads_t* out, cha
 
 }  // namespace
 
+// The layer forward; `kind` (a forward kind of make_plan) alone decides which kernels run and how much scratch they need.
+int as::forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes,
+                void* stream, int kind) {
+  int e = check_shape(shape);
+  if (e) return e;
+  e = check_params(params);
+  if (e) return e;
+  if (!x || !y || !ws) return AS_ERR_NULL;
+  if (!aligned16(x) || !aligned16(y) || !aligned16(ws)) return AS_ERR_ALIGN;
+  Plan pl;
+  e = make_plan(shape, shape->seqlen, 1, &pl, kind);
+  if (e) return e;
+  if (ws_bytes < pl.total_fwd) return AS_ERR_WORKSPACE;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  char* w = reinterpret_cast<char*>(ws);
+  Wcat wcat{};
+  ZeroList z{};
+  add_region(&z, w + pl.off_status, 256);
+  e = begin(pl, params, z, false, x, w, st, &wcat);
+  if (e) return e;
+  ScanPtrs sp{x, nullptr, params->A_log, w};
+  const bool mm = forward_y_mm_applies(pl);
+  if (mm) AS_TRY(launch_forward_state_mm(pl, sp, st));
+  else AS_TRY(launch_prepass(pl, sp, false, st));
+  AS_TRY(launch_fixup(pl, sp, false, st));
+  if (mm) AS_TRY(launch_forward_y_mm(pl, sp, y, st));
+  else AS_TRY(launch_forward_y(pl, sp, y, st));
+  return AS_OK;
+}
+
 extern "C" {
 
 int as_version(void) { return AS_VERSION; }
@@ -177,39 +207,6 @@ int as_check_status(const void* ws, void* stream) {
   if (cudaMemcpyAsync(&word, ws, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return AS_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return AS_ERR_CUDA;
   return word;
-}
-
-static int forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes,
-                   void* stream, int kind) {
-  int e = check_shape(shape);
-  if (e) return e;
-  e = check_params(params);
-  if (e) return e;
-  if (!x || !y || !ws) return AS_ERR_NULL;
-  if (!aligned16(x) || !aligned16(y) || !aligned16(ws)) return AS_ERR_ALIGN;
-  Plan pl;
-  e = make_plan(shape, shape->seqlen, 1, &pl, kind);
-  if (e) return e;
-  if (ws_bytes < pl.total_fwd && pl.split) {   // the fixed scratch of as_ssm_forward_static may only hold the smaller plan
-    e = make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD_SMALL);
-    if (e) return e;
-  }
-  if (ws_bytes < pl.total_fwd) return AS_ERR_WORKSPACE;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  char* w = reinterpret_cast<char*>(ws);
-  Wcat wcat{};
-  ZeroList z{};
-  add_region(&z, w + pl.off_status, 256);
-  e = begin(pl, params, z, false, x, w, st, &wcat);
-  if (e) return e;
-  ScanPtrs sp{x, nullptr, params->A_log, w};
-  const bool mm = forward_y_mm_applies(pl);
-  if (mm) AS_TRY(launch_forward_state_mm(pl, sp, st));
-  else AS_TRY(launch_prepass(pl, sp, false, st));
-  AS_TRY(launch_fixup(pl, sp, false, st));
-  if (mm) AS_TRY(launch_forward_y_mm(pl, sp, y, st));
-  else AS_TRY(launch_forward_y(pl, sp, y, st));
-  return AS_OK;
 }
 
 int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,

@@ -129,8 +129,8 @@ struct Plan {
       off_bptt_ckpt, off_wcat, off_wcatx, off_xs, off_wsp, off_gs, total_fwd, total_grad;
 };
 
-// PLAN_GRAD: gradient calls.  PLAN_FWD: as_ssm_forward.  PLAN_FWD_SMALL: an fp32 forward with less scratch (contractions on
-// the FP32 pipe).
+// PLAN_GRAD: gradient calls.  PLAN_FWD: as_ssm_forward.  PLAN_FWD_SMALL: as_ssm_forward_static where its array cannot hold
+// PLAN_FWD (fp32 I/O; projections on the FP32 pipe, which need no room for split operands).
 // PLAN_FWD_ORDERED: as_ssm_forward_ordered.
 enum { PLAN_GRAD = 0, PLAN_FWD = 1, PLAN_FWD_SMALL = 2, PLAN_FWD_ORDERED = 3 };
 int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind = PLAN_GRAD);
@@ -182,9 +182,12 @@ int split_gradients(const Plan& pl, const as_grads_t* out, char* ws, cudaStream_
 
 int launch_bptt(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st);
 
+// the layer forward behind as_ssm_forward, as_ssm_forward_ordered and as_ssm_forward_static; an AS_* code (as_api.cu)
+int forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes, void* stream,
+            int kind);
+
 // device address of the library's built-in scratch array on the current device (as_noalloc.cu); AS_OK or an error code
 int static_scratch_address(void** out);
-
 
 int launch_rmsnorm_fwd(const as_shape_t* sh, const void* y, void* yhat, float eps, cudaStream_t st);
 int launch_residual_add(const as_shape_t* sh, const void* a, const void* b, void* out, cudaStream_t st);

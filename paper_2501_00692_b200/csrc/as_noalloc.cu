@@ -11,7 +11,9 @@
 //   * Every GPU context that loads this library holds AS_STATIC_SCRATCH_BYTES of device memory for the
 //     array until the process exits, whether or not this entry point is ever called.
 //   * Shapes whose forward scratch (as_workspace_bytes, fwd_bytes) exceeds the array are rejected with
-//     AS_ERR_LIMIT; nothing is launched.
+//     AS_ERR_LIMIT; nothing is launched.  Large fp32 shapes, whose scratch holds the operands a second time, split for
+//     the tensor cores (6 of some 10 bytes per token and channel), are taken as long as the rest fits: their projections
+//     then run on the FP32 pipe.
 //   * The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that
 //     device current).  That is a synchronous runtime call: make the first call per device during set-up,
 //     before any stream capture begins.  Later calls only enqueue work.
@@ -59,12 +61,18 @@ extern "C" int as_ssm_forward_static(const as_shape_t* shape, const as_params_t*
   int e = as_workspace_bytes(shape, shape ? shape->seqlen : 1, nullptr, nullptr);   // checks the shape
   if (e) return e;
   as::Plan pl;
-  e = as::make_plan(shape, shape->seqlen, 1, &pl, as::PLAN_FWD_SMALL);   // the least scratch the forward can work with
+  int kind = as::PLAN_FWD;
+  e = as::make_plan(shape, shape->seqlen, 1, &pl, kind);
   if (e) return e;
-  if (pl.total_fwd > (size_t)AS_STATIC_SCRATCH_BYTES) return AS_ERR_LIMIT;
+  if (pl.total_fwd > (size_t)AS_STATIC_SCRATCH_BYTES) {   // large fp32 shapes: the plan that keeps no split operands
+    kind = as::PLAN_FWD_SMALL;
+    e = as::make_plan(shape, shape->seqlen, 1, &pl, kind);
+    if (e) return e;
+    if (pl.total_fwd > (size_t)AS_STATIC_SCRATCH_BYTES) return AS_ERR_LIMIT;
+  }
   void* scratch = nullptr;
   e = scratch_for_current_device(&scratch);
   if (e) return e;
-  // as_ssm_forward zeroes the status word at the head of the scratch and overwrites every other region it reads
-  return as_ssm_forward(shape, params, x, y, scratch, (size_t)AS_STATIC_SCRATCH_BYTES, stream);
+  // the forward zeroes the status word at the head of the scratch and overwrites every other region it reads
+  return as::forward(shape, params, x, y, scratch, (size_t)AS_STATIC_SCRATCH_BYTES, stream, kind);
 }

@@ -100,6 +100,19 @@ def test_workspace_query_and_argument_errors(L):
     assert L.as_adjoint_grad(C.byref(sh), C.byref(pw), ok, ok, 4, 0, C.byref(g), ok, 1 << 40, None) == B.AS_ERR_ALIGN
 
 
+@pytest.mark.parametrize("shape", [(1, 4100, 248, B.AS_F32), (2, 9000, 512, B.AS_F32), (1, 300, 64, B.AS_F32), (2, 5000, 256, B.AS_BF16)])
+def test_forward_refuses_less_scratch_than_reported(L, shape):
+    """Neither the kernels nor the result depend on the size of the scratch: one byte short of fwd_bytes is an error, also
+    where another form of the contractions could do with less."""
+    sh = B.make_shape(*shape[:3], 16, shape[3])
+    fwd = B.as_workspace_bytes(sh, shape[1])[0]
+    ok = C.c_void_p(0x1000)   # never dereferenced: the size check comes first
+    p = B.as_params_t(ok, ok, ok, ok, ok)
+    for entry in (L.as_ssm_forward, L.as_ssm_forward_ordered):
+        assert entry(C.byref(sh), C.byref(p), ok, ok, ok, 256, None) == B.AS_ERR_WORKSPACE
+    assert L.as_ssm_forward(C.byref(sh), C.byref(p), ok, ok, ok, fwd - 1, None) == B.AS_ERR_WORKSPACE
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libadjoint_ssm.so")

@@ -12,9 +12,12 @@ import ctypes as C
 import pytest
 import torch
 
+from oracle import ssm_oracle as O
 from paper_2501_00692_b200 import binding as B
 from paper_2501_00692_b200 import synth
 from paper_2501_00692_b200.build import build_library
+
+from gpu_util import TOL, assert_close, theta_f64
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -53,3 +56,25 @@ def test_static_scratch_forward_matches_regular_forward_twice(io):
     with pytest.raises(B.AsError) as ei:
         B.as_ssm_forward_static(big, theta, x, y)
     assert ei.value.code == B.AS_ERR_LIMIT
+
+
+@pytest.mark.parametrize("T,P", [(2500, 648), (7000, 648)])
+def test_static_scratch_with_and_without_room_for_split_operands(T, P):
+    """fp32 shapes whose projections as_ssm_forward runs on split operands (tokens * P * (P + 32) >= 2^28): with room for
+    them in the built-in array the results are as_ssm_forward's; without, the projections take the FP32 pipe."""
+    build_library()
+    w = synth.custom_workload("noalloc-split", 23, 1, T, P, io="f32")
+    theta = synth.layer_params(w, 0, DEV)
+    x, _ = synth.activations(w, DEV)
+    sh = B.shape_of(x)
+    fwd_bytes = B.as_workspace_bytes(sh, T)[0]
+    fits = fwd_bytes <= B.AS_STATIC_SCRATCH_BYTES
+    assert fits == (T == 2500)
+    y_ref, y = torch.empty_like(x), torch.full_like(x, float("nan"))
+    B.as_ssm_forward(sh, theta, x, y_ref, B.alloc_workspace(fwd_bytes, DEV))
+    B.as_ssm_forward_static(sh, theta, x, y)
+    assert B.as_check_status(None) == B.AS_OK
+    assert not fits or torch.equal(y, y_ref)
+    want = O.ssm_forward(theta_f64(theta), synth.to_f64(x[0]))
+    for got in (y, y_ref):
+        assert_close(synth.to_f64(got[0]), want, TOL["f32"], "y")
