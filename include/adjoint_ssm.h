@@ -111,7 +111,7 @@ const char *as_strerror(int code);
  * as_full_bptt_grad (the larger of the two).  Either output pointer may be NULL.  `tbar` as for as_adjoint_grad. */
 int as_workspace_bytes(const as_shape_t *shape, int64_t tbar, size_t *fwd_bytes, size_t *grad_bytes);
 
-/* Synchronises `stream` and returns the status word the kernels keep at the start of `ws`
+/* Synchronises `stream` and returns what the kernels report in the status block, the first 256 bytes of `ws`
  * (AS_OK, or AS_ERR_TIMEOUT if a bounded device-side wait ran out).  ws == NULL selects the built-in scratch
  * array of as_ssm_forward_static on the current device. */
 int as_check_status(const void *ws, void *stream);
@@ -191,7 +191,7 @@ int as_full_bptt_grad(const as_shape_t *shape, const as_params_t *params, const 
  *     device current): make it during set-up, before any stream capture;
  *   - all calls on a device share the array and it keeps the previous call's contents (what must start at zero is
  *     cleared by the call); calls whose kernels may overlap on the GPU race on it - order them on one stream;
- *   - the status word of the call's kernels sits at the head of the array: read it with as_check_status(NULL, stream);
+ *   - the status block of the call's kernels sits at the head of the array: read it with as_check_status(NULL, stream);
  *   - the array belongs to the device's primary context (the one the CUDA runtime API uses);
  *   - neither this call nor anything it launches calls cudaMalloc, cudaFree or another allocating routine.
  * x, y: [Bsz,T,P] io dtype device buffers supplied by the caller, as for as_ssm_forward. */
@@ -218,7 +218,7 @@ int as_rmsnorm_bwd_add(const as_shape_t *shape, const void *y, const void *dyhat
 /* ---- diagnostics ------------------------------------------------------------------------------------ */
 
 /* Self test of the failure-reporting path.  Every device-side wait of this library (mbarrier waits on staged
- * tiles) is bounded: after a fixed number of polls the kernel stops, writes AS_ERR_TIMEOUT into the status word at
+ * tiles) is bounded: after a fixed number of polls the kernel stops, reports AS_ERR_TIMEOUT in the status block at
  * the head of `ws` and returns, leaving the context usable.  This call enqueues a one-warp kernel that waits, with
  * `poll_limit` polls (1 .. 2^20), for an mbarrier phase that nothing completes; as_check_status(ws, stream) must
  * then return AS_ERR_TIMEOUT.  `ws` needs 256 bytes.  Nothing faults, traps or spins without bound. */

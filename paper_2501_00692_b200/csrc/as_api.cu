@@ -1,4 +1,6 @@
 // extern "C" entry points: argument checks, scratch layout, and the launch sequence of each call.
+#include <string.h>
+
 #include <atomic>
 
 #include "as_internal.cuh"
@@ -67,9 +69,12 @@ int begin(const Plan& pl, const as_params_t* pr, const ZeroList& z, bool grad, c
   const bool packed = pr->Wcat && wcat->reps == 1;
   char* at = ws + (grad ? pl.off_wcatx : pl.off_wcat);
   wcat->p = packed ? pr->Wcat : at;
-  // with packed weights the projections clear the regions themselves
-  if (!packed) AS_TRY(launch_prepare(z, pl.P, pl.KL, wcat->reps, pr, at, st));
-  AS_TRY(tc_projections(pl, pr, wcat->p, wcat->reps, x, packed ? z : ZeroList{}, ws, st));
+  ZeroList own{};
+  if (packed) {   // the projections clear the regions themselves, of the status block the word only
+    own = z;
+    own.bytes[0] = STATUS_CTA;
+  } else AS_TRY(launch_prepare(z, pl.P, pl.KL, wcat->reps, pr, at, st));
+  AS_TRY(tc_projections(pl, pr, wcat->p, wcat->reps, x, own, ws, st));
   return AS_OK;
 }
 
@@ -109,7 +114,7 @@ void add_region(ZeroList* z, void* p, size_t bytes) { z->ptr[z->n] = p; z->bytes
 ZeroList grad_regions(const Plan& pl, uint32_t flags, const as_grads_t* out, char* ws) {
   const size_t P = pl.P, K = pl.KL;
   ZeroList z{};
-  add_region(&z, ws + pl.off_status, 256);
+  add_region(&z, ws + pl.off_status, STATUS_BYTES);
   add_region(&z, ws + pl.off_dbc, (size_t)pl.B * pl.T * NBC * 4);
   if (!(flags & AS_ACCUMULATE)) {
     add_region(&z, out->dW_delta, K * P * P * 4);
@@ -140,7 +145,7 @@ int as::forward(const as_shape_t* shape, const as_params_t* params, const void* 
   char* w = reinterpret_cast<char*>(ws);
   Wcat wcat{};
   ZeroList z{};
-  add_region(&z, w + pl.off_status, 256);
+  add_region(&z, w + pl.off_status, STATUS_BYTES);
   e = begin(pl, params, z, false, x, w, st, &wcat);
   if (e) return e;
   ScanPtrs sp{x, nullptr, params->A_log, w};
@@ -203,10 +208,15 @@ int as_check_status(const void* ws, void* stream) {
     ws = p;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  int word = 0;
-  if (cudaMemcpyAsync(&word, ws, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return AS_ERR_CUDA;
+  alignas(int) unsigned char block[STATUS_BYTES];
+  if (cudaMemcpyAsync(block, ws, STATUS_BYTES, cudaMemcpyDeviceToHost, st) != cudaSuccess) return AS_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return AS_ERR_CUDA;
-  return word;
+  int word = 0;
+  memcpy(&word, block, sizeof word);
+  if (word != AS_OK) return word;
+  for (int i = STATUS_CTA; i < STATUS_BYTES; ++i)
+    if (block[i]) return AS_ERR_TIMEOUT;
+  return AS_OK;
 }
 
 int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,
@@ -345,11 +355,11 @@ int as_rmsnorm_bwd_add(const as_shape_t* shape, const void* y, const void* dyhat
 
 int as_wait_selftest(void* ws, size_t ws_bytes, uint32_t poll_limit, void* stream) {
   if (!ws) return AS_ERR_NULL;
-  if (ws_bytes < 256) return AS_ERR_WORKSPACE;
+  if (ws_bytes < STATUS_BYTES) return AS_ERR_WORKSPACE;
   if (!aligned16(ws)) return AS_ERR_ALIGN;
   if (poll_limit == 0 || poll_limit > (1u << 20)) return AS_ERR_LIMIT;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  AS_TRY((int)cudaMemsetAsync(ws, 0, 256, st));
+  AS_TRY((int)cudaMemsetAsync(ws, 0, STATUS_BYTES, st));
   AS_TRY(launch_wait_selftest(reinterpret_cast<int*>(ws), poll_limit, st));
   return AS_OK;
 }

@@ -14,7 +14,7 @@
 // split into three bf16 terms, which is exact) and the Wcat of the input gradient repeats W_B and W_C three times
 // (Plan.gsplit), so the contraction of the split equals the contraction of the fp32 values.
 // No cluster multicast is used anywhere.  Every mbarrier wait is bounded; on timeout the kernel records
-// AS_ERR_TIMEOUT in the status word, stops issuing work, frees its TMEM and returns.
+// AS_ERR_TIMEOUT in the status block, stops issuing work, frees its TMEM and returns.
 #include <cuda.h>
 
 #include "as_tc.cuh"
@@ -47,7 +47,8 @@ struct TcArgs {
   const float* bias;    // PROJ: b_delta [layers, P]
   float* bc;            // PROJ: [B | C] rows, for the plain stores where P is not a multiple of 16
   int* status;
-  ZeroList zero;        // PROJ: regions to clear for the later kernels, where the call has no kernel before this one
+  ZeroList zero;        // PROJ: regions to clear for the later kernels, where the call has no kernel before this one; the
+                        // status word is among them, which is why the CTAs report through bytes of their own
 };
 
 // Persistent, warp-specialised kernel: one CTA per SM walks tiles t = blockIdx.x, + gridDim.x, ...
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
   const int kper = (a.kblocks + a.splitk - 1) / a.splitk;
   const int NWc = a.wrows;                         // rows of one layer's Wcat
   volatile int* abortp = &abort_s;
+  uint8_t* const cta_bytes = reinterpret_cast<uint8_t*>(a.status) + STATUS_CTA;   // PROJ: where its CTAs report
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -90,7 +92,12 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_begin();
-  if (EPI == TC_PROJ && a.zero.n > 0) clear_regions(a.zero, (int64_t)blockIdx.x * NTHREADS + threadIdx.x, (int64_t)gridDim.x * NTHREADS);
+  if (EPI == TC_PROJ && a.zero.n > 0) {
+    static_assert(NTHREADS >= STATUS_CTAS, "one CTA alone clears all bytes");
+    const unsigned i = blockIdx.x + gridDim.x * threadIdx.x;   // this CTA's byte, and its share of those without a CTA
+    if (i < STATUS_CTAS) cta_bytes[i] = 0;
+    clear_regions(a.zero, (int64_t)blockIdx.x * NTHREADS + threadIdx.x, (int64_t)gridDim.x * NTHREADS);
+  }
   if (warp == 1) {   // TMEM allocation: two BN-column fp32 accumulators
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(Cfg<BN>::TMEM_COLS)
                  : "memory");
@@ -151,7 +158,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
           }
         }
       }
-      if (!ok) { *abortp = 1; atomicExch(a.status, AS_ERR_TIMEOUT); }
+      if (!ok) { *abortp = 1; if (EPI != TC_PROJ) atomicExch(a.status, AS_ERR_TIMEOUT); }
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -189,7 +196,7 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
         }
         if (ok) umma_commit(&tmem_full_bar[ab]);   // accumulator of this tile complete
       }
-      if (!ok) { *abortp = 1; atomicExch(a.status, AS_ERR_TIMEOUT); }
+      if (!ok) { *abortp = 1; if (EPI != TC_PROJ) atomicExch(a.status, AS_ERR_TIMEOUT); }
     }
   } else {
     // ---------------- epilogue warps ----------------
@@ -328,13 +335,16 @@ __global__ void __launch_bounds__(NTHREADS) gemm_tc_kernel(const __grid_constant
       }
     }
     if (lane == 0) bulk_wait_all();            // staging tiles must outlive the bulk operations that read them
-    if (!ok) { *abortp = 1; if (lane == 0) atomicExch(a.status, AS_ERR_TIMEOUT); }
+    if (!ok) { *abortp = 1; if (EPI != TC_PROJ && lane == 0) atomicExch(a.status, AS_ERR_TIMEOUT); }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Cfg<BN>::TMEM_COLS) : "memory");
   }
+  // the projections report here and not where a role gives up: a choice of the place inside the roles cost a forward of
+  // 2,048 x 512 3 us of 45
+  if (EPI == TC_PROJ && threadIdx.x == 0 && *abortp) cta_bytes[blockIdx.x] = 1;
 }
 
 // ---- small helpers -------------------------------------------------------------------------------
@@ -395,7 +405,7 @@ int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorM
   static bool done[AS_MAX_DEVICES] = {};
   if (ensure_dynamic_smem(kern, Cfg<BN>::SMEM_DYN, done)) return 1;
   const int64_t ntiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * (EPI == TC_DW ? a.layers : 1);
-  const int sms = sm_count();
+  const int sms = EPI == TC_PROJ && sm_count() > STATUS_CTAS ? STATUS_CTAS : sm_count();
   const unsigned grid = (unsigned)(ntiles < sms ? ntiles : sms);   // one persistent CTA per SM
   return launch_dependent(kern, dim3(grid), dim3(NTHREADS), Cfg<BN>::SMEM_DYN, st, tmA, tmB, tmO[0], tmO[1], tmO[2], a);
 }

@@ -94,6 +94,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// ---- status block: the first STATUS_BYTES of the scratch ------------------------------------
+// Word 0 is AS_OK or the code a kernel reported.  It is cleared by a kernel that reports nothing there, so a kernel that runs
+// later may simply set it.  The bf16 projections clear it themselves where the weights are packed (there is no kernel before
+// them), and a CTA that starts late would erase what another one has set: so they never set it.  Each of their CTAs owns one
+// byte behind the word's 16-byte piece, which it (or the kernel before) zeroes when it starts and sets to 1 if a wait gives up.
+// as_check_status looks at the whole block.  Ordered forward with packed weights, 256 x 256: 32.4 us with the race, 32.6 so,
+// 33.9 with a clearing kernel in front; 2,048 x 512: 45.3, 45.4, 47.3.
+constexpr int STATUS_BYTES = 256;
+constexpr int STATUS_CTA = 16;                          // offset of the CTAs' bytes
+constexpr int STATUS_CTAS = STATUS_BYTES - STATUS_CTA;  // as many CTAs can report
+
 // ---- time segmentation and scratch layout ---------------------------------------------------
 // Time is cut into S segments of L tokens (L a multiple of CK); a CTA owns (segment, batch element,
 // CH channels).  Per-(segment, channel, state) and per-(chunk, channel, state) arrays are stored as
@@ -170,7 +181,8 @@ int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st)
 int launch_adjoint_main(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st);
 int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st);
 
-// bf16 tensor-core path (as_gemm_tc.cu)
+// bf16 tensor-core path (as_gemm_tc.cu).  The projections clear the regions `z` (and the CTAs' bytes of the status block)
+// where the call has no kernel before them.
 int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x,
                    const ZeroList& z, char* ws, cudaStream_t st);
 int tc_weight_grads(const Plan& pl, const void* x, const as_grads_t* out, char* ws, cudaStream_t st);

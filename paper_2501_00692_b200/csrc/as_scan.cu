@@ -83,7 +83,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   const size_t BSP = (size_t)p.B * p.S * p.P;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
-  p.off_status = take(256);
+  p.off_status = take(STATUS_BYTES);
   p.off_delta = take(BTP * 4);
   p.off_bc = take((BT + CK) * NBC * 4);   // CK spare rows: a chunk's 1D copy may run past the last token
   p.off_hend = take(BSB * 4);

@@ -100,3 +100,29 @@ def test_bounded_wait_reports_timeout_and_context_survives():
     B.as_ssm_forward(sh, theta, x, y, ws2)
     assert B.as_check_status(ws2) == B.AS_OK
     assert torch.isfinite(y).all()
+
+
+@pytest.mark.parametrize("T,P", [(100, 64), (9000, 256)])   # fewer CTAs than bytes in the status block; one per SM
+def test_status_block_of_packed_weights_calls(T, P):
+    """With packed weights the projections both clear the status word and may report, each CTA through a byte of its own:
+    every byte of a stale block has to be written, and any byte set counts."""
+    build_library()
+    w = synth.custom_workload("status", 20, 1, T, P, tbar=T, io="bf16")
+    theta = dict(synth.layer_params(w, 0, DEV))
+    x, dy = synth.activations(w, DEV)
+    sh = B.shape_of(x)
+    theta["Wcat"] = torch.empty(B.as_wcat_bytes(sh), dtype=torch.uint8, device=DEV)
+    B.as_pack_weights(sh, 1, theta, theta["Wcat"])
+    fb, gb = B.as_workspace_bytes(sh, T)
+    ws = B.alloc_workspace(max(fb, gb), DEV)
+    y, grads = torch.empty_like(x), B.alloc_grads(sh, DEV)
+    for call in (lambda: B.as_ssm_forward(sh, theta, x, y, ws), lambda: B.as_ssm_forward_ordered(sh, theta, x, y, ws),
+                 lambda: B.as_adjoint_grad(sh, theta, x, dy, T, grads, ws)):
+        ws[:256] = 0xFF
+        call()
+        assert B.as_check_status(ws) == B.AS_OK
+        for cta in (0, 1, 147, 239):
+            ws[16 + cta] = 1
+            assert B.as_check_status(ws) == B.AS_ERR_TIMEOUT, cta
+            ws[16 + cta] = 0
+        assert B.as_check_status(ws) == B.AS_OK
