@@ -52,10 +52,11 @@ template <typename IO> constexpr bool kOrdered = sizeof(IO) == 2;
 constexpr int NORM_WARPS = 4;   // rows per CTA
 
 // One row per warp.  NP = 16-byte pieces of a row per lane, or 0: any width, the row read again for the second pass.
-// ADD: the row is a + b, stored to `sum` (which may alias a), and the norm is that of the stored row.
+// ADD: the row is a + b, stored to `sum` (which may alias a), and the norm, which may alias b, is that of the stored row.
+// None of the four is __restrict__: a lane has read all its pieces of a and b before it stores to sum or yhat (NP > 0), or has
+// read its pieces of b before the second pass stores yhat (NP = 0).
 template <typename IO, int NP, bool ADD>
-__global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* __restrict__ b, IO* sum, IO* __restrict__ yhat,
-                                   float eps) {
+__global__ void rmsnorm_fwd_kernel(int64_t rows, int P, const IO* a, const IO* b, IO* sum, IO* yhat, float eps) {
   pdl_begin();
   constexpr int N = Vec<IO>::N;
   extern __shared__ __align__(16) uint8_t row_s[];
