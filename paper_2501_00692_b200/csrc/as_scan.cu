@@ -27,8 +27,15 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   p.scalar = sh->a_structure == AS_A_SCALAR ? 1 : 0;
   p.tc = sh->io == AS_BF16 ? 1 : 0;
   p.gsplit = p.P % 32 == 0 ? 1 : 3;
-  // below that the splits and the fixed cost of the tensor-core kernels outweigh what they save (8,192 tokens x 256 has 6e8)
-  p.split = kind != PLAN_FWD_SMALL && !p.tc && p.P >= 64 && (int64_t)p.Bg * p.T * p.P * (p.P + NBC) >= ((int64_t)1 << 28);
+  // fp32 I/O: the splits and the fixed cost of the tensor-core kernels have to be outweighed.  Whole calls, us, split | FP32
+  // pipe.  Gradients at 2^28 multiply-adds: 43,691 x 64 247 | 247, 29,960 x 80 199 | 223, 3,640 x 256 111 | 143; at 2^27:
+  // 21,845 x 64 169 | 159, 6,553 x 128 126 | 132, 1,820 x 256 95 | 107, 481 x 512 96 | 132.  So the line lies where the
+  // narrowest width breaks even; wide calls would gain below it too and keep the pipe's order of additions.
+  // Forwards have only the projections to gain by, and lose where these are a single column tile (P + 32 <= 128): 43,691 x 64
+  // 121 | 111, 29,960 x 80 94 | 88, 21,846 x 96 84 | 77; with two tiles 33,289 x 112 117 | 117, 37,073 x 128 123 | 132,
+  // 24,967 x 192 132 | 168.
+  const bool wide = kind == PLAN_GRAD ? p.P >= 64 : p.P + NBC > 128;
+  p.split = kind != PLAN_FWD_SMALL && !p.tc && wide && (int64_t)p.Bg * p.T * p.P * (p.P + NBC) >= ((int64_t)1 << 28);
   p.du_ld = p.tc ? p.P + p.gsplit * NBC : p.P;
   p.full = tbar >= p.T;
   p.tbar = p.full ? p.T : tbar;

@@ -1,14 +1,16 @@
 """fp32 contractions on the tensor cores (exact three-term bf16 splits) against the FP32-pipe kernels' accuracy: projections
 and all dense gradients, measured against fp64 products of the same operands; shapes with ragged tiles and K blocks, several
-layers, and the forward with too little scratch for the splits (needs a B200)."""
+layers, and forwards on both sides of the width from which they take them (needs a B200).  The fixed scratch that has no room
+for the splits: tests/test_zz_no_alloc.py."""
 import pytest
 import torch
 
+from oracle import ssm_oracle as O
 from paper_2501_00692_b200 import binding as B
 from paper_2501_00692_b200 import synth
 from paper_2501_00692_b200.build import build_library
 
-from gpu_util import TOL, assert_close, compare_grads, oracle_adjoint
+from gpu_util import TOL, assert_close, compare_grads, oracle_adjoint, theta_f64
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -36,3 +38,19 @@ def test_split_contractions(layers, batch, T, P):
     y = torch.empty_like(x)
     B.as_ssm_forward(sh, thetas[0], x, y, ws)
     assert_close(synth.to_f64(y), refs[0]["y"], 1e-5, "y")
+
+
+# forwards take the tensor cores from two column tiles on (P + 32 > 128)
+@pytest.mark.parametrize("T,P", [(21900, 96), (19000, 104)])
+def test_forward_on_both_sides_of_the_width_rule(T, P):
+    build_library()
+    w = synth.custom_workload("split-width", 46, 1, T, P, io="f32")
+    theta = synth.layer_params(w, 0, DEV)
+    x, _ = synth.activations(w, DEV)
+    sh = B.shape_of(x, w.d_state)
+    fwd = B.as_workspace_bytes(sh, T)[0]
+    assert (fwd > 10 * T * P) == (P > 96)      # the split operands are part of the scratch
+    ws, y = B.alloc_workspace(fwd, DEV), torch.full_like(x, float("nan"))
+    B.as_ssm_forward(sh, theta, x, y, ws)
+    assert B.as_check_status(ws) == B.AS_OK
+    assert_close(synth.to_f64(y[0]), O.ssm_forward(theta_f64(theta), synth.to_f64(x[0])), 1e-5, "y")
