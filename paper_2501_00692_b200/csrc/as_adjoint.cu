@@ -649,7 +649,7 @@ int launch_main_t(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_d
   if (act_map(&mdx, sp.ws + pl.off_dxdir, pl, pl.B, sizeof(IO), BF, pl.P, 32)) return 1;
   constexpr int bytes = MainCfg<sizeof(IO), !FULL>::SMEM_DYN;
   auto kern = adjoint_main_kernel<IO, FULL, SC>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
   return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, mdu, mdx, pl, sp.A_log, sp.ws,
                           dA_log, db_delta);

@@ -9,7 +9,21 @@ using namespace as;
 
 namespace as {
 std::atomic<int64_t> g_launches{0};
+
+EncodeTiledFn encode_tiled() {
+  static std::atomic<EncodeTiledFn> found{nullptr};   // host threads that come first at once look it up more than once
+  EncodeTiledFn fn = found.load(std::memory_order_relaxed);
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<EncodeTiledFn>(p);
+    found.store(fn, std::memory_order_relaxed);
+  }
+  return fn;
 }
+}  // namespace as
 
 namespace {
 

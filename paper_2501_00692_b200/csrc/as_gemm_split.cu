@@ -306,7 +306,7 @@ __global__ void split_g_kernel(int P, int64_t M, int layers, const float* __rest
 
 // [planes, rows, cols] row-major; box {box_cols, box_rows, 1}
 int map3(CUtensorMap* tm, bool f32, const void* base, uint64_t planes, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
-  EncodeTiledFn enc = get_encode();
+  EncodeTiledFn enc = encode_tiled();
   if (!enc) return 1;
   const uint64_t e = f32 ? 4 : 2;
   cuuint64_t dims[3] = {cols, rows, planes};
@@ -321,7 +321,7 @@ int map3(CUtensorMap* tm, bool f32, const void* base, uint64_t planes, uint64_t 
 template <int AMAJ, int BMAJ, int EPI>
 int launch_split(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const SplitArgs& a, cudaStream_t st) {
   auto kern = gemm_split_kernel<AMAJ, BMAJ, EPI>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
   const int64_t ntiles = ((a.R + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * a.layers;
   if (ntiles > 0x7fffffff) return 1;

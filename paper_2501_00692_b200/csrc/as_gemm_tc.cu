@@ -377,7 +377,7 @@ __global__ void cvt_dbc_kernel(int64_t rows, int ldg, int P, const float* __rest
 // row-major [rows, cols] tensor with row pitch `ld` elements; box = {box_cols, box_rows}; OOB reads give 0, OOB writes are dropped
 int make_map_t(CUtensorMap* tm, CUtensorMapDataType dt, int esz, CUtensorMapSwizzle swz, const void* base, uint64_t rows,
                uint64_t cols, uint64_t ld, uint32_t box_cols, uint32_t box_rows) {
-  EncodeTiledFn enc = get_encode();
+  EncodeTiledFn enc = encode_tiled();
   if (!enc) return 1;
   cuuint64_t dims[2] = {cols, rows};
   cuuint64_t strides[1] = {ld * (uint64_t)esz};
@@ -402,7 +402,7 @@ int make_map_out_bf16(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t
 template <int AMAJ, int BMAJ, int EPI, int BN, bool ML, bool OFF>
 int launch_tc_ml(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap (&tmO)[3], const TcArgs& a, cudaStream_t st) {
   auto kern = gemm_tc_kernel<AMAJ, BMAJ, EPI, BN, ML, OFF>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, Cfg<BN>::SMEM_DYN, done)) return 1;
   const int64_t ntiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) * a.splitk * (EPI == TC_DW ? a.layers : 1);
   const int sms = EPI == TC_PROJ && sm_count() > STATUS_CTAS ? STATUS_CTAS : sm_count();

@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libadjoint_ssm (not part of the C ABI).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -38,18 +39,26 @@ __device__ __forceinline__ void pdl_begin() {
 }
 
 // Function attributes (the dynamic shared-memory limit) belong to a device: remember per device, per kernel
-// instantiation, whether the limit has been raised.  `done` is a static array of the launcher, one flag per device.
+// instantiation, whether the limit has been raised.  `done` is a static array of the launcher, one flag per device; host
+// threads that make their first calls at once at worst repeat the (idempotent) setting.
 constexpr int AS_MAX_DEVICES = 64;
+typedef std::atomic<bool> DeviceFlags[AS_MAX_DEVICES];
 template <typename K>
-inline int ensure_dynamic_smem(K kern, int bytes, bool (&done)[AS_MAX_DEVICES]) {   // idempotent: a race between host threads only repeats the call
+inline int ensure_dynamic_smem(K kern, int bytes, DeviceFlags& done) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= AS_MAX_DEVICES) return 1;
-  if (!done[dev]) {
+  if (!done[dev].load(std::memory_order_acquire)) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return 1;
-    done[dev] = true;
+    done[dev].store(true, std::memory_order_release);
   }
   return 0;
 }
+
+// cuTensorMapEncodeTiled, looked up through the runtime once per process (as_api.cu); null if the driver does not have it
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_tiled();
 
 // Number of SMs of the current device (grids are sized in multiples of it); queried once per device.  The cache is
 // a plain array of atomics: concurrent first calls from several host threads at worst query twice.
@@ -67,7 +76,7 @@ inline int sm_count() {
 
 constexpr int NS = 16;        // d_state handled by the scan kernels
 constexpr int CK = 8;         // tokens per checkpoint chunk (h of one chunk lives in registers)
-constexpr int NCH = 2;        // channels per thread of the scan kernels (1 or 2)
+constexpr int NCH = 2;        // channels per thread of the scan kernels
 constexpr int NTHR = 128;     // threads per CTA of the scan kernels; two threads share a channel set, 8 states each
 constexpr int CH = NTHR / 2 * NCH;   // channels per CTA
 constexpr int NU = 4 * NCH;   // packed state pairs (f32x2) a thread owns
@@ -127,7 +136,6 @@ struct Plan {
   int io;           // as_dtype_t
   int scalar;       // 1: one decay rate per channel (A_log is [P]), 0: one per (channel, state)
   int tiles;        // ceil(P / CH) channel tiles
-  int bw;           // channels per staged row: min(CH, P)
   int tc;           // 1: bf16 tensor-core contractions (bf16 I/O), 0: FP32-pipe GEMMs
   int ffma;         // projections of bf16 I/O on the fp32 pipe (as_ssm_forward_ordered, widths off the 32-element grid)
   int one_order;    // bf16 forward: one segmentation and one order of the carries for all sizes
@@ -145,8 +153,6 @@ struct Plan {
 // PLAN_FWD_ORDERED: as_ssm_forward_ordered.
 enum { PLAN_GRAD = 0, PLAN_FWD = 1, PLAN_FWD_SMALL = 2, PLAN_FWD_ORDERED = 3 };
 int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind = PLAN_GRAD);
-// elements of A_log (and dA_log) per layer
-inline int64_t a_stride(const Plan& pl) { return pl.scalar ? (int64_t)pl.P : (int64_t)pl.P * NS; }
 
 // ---- launchers (each returns a cudaError_t as int) ------------------------------------------
 

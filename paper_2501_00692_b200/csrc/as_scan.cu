@@ -40,7 +40,6 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   p.full = tbar >= p.T;
   p.tbar = p.full ? p.T : tbar;
   p.tiles = (p.P + CH - 1) / CH;
-  p.bw = p.P < CH ? p.P : CH;
   // Full waves of the main kernel's resident CTAs (SMs x CTAs per SM).  A partly filled wave costs as much as a full one
   // (T = 30,000, P = 256: 147 us at two waves, 155 at one and a half), and a CTA has a fixed cost of some 20 tokens' time.
   // So: three waves (two in the full form) while segments stay at 160 tokens (truncated: two waves at 112) or more, for the tail of long
@@ -749,7 +748,7 @@ int launch_prepass_t(const Plan& pl, const ScanPtrs& sp, cudaStream_t st) {
   if (make_maps(pl, sp, &m)) return 1;
   const int bytes = NSTAGE * Stage<sizeof(IO), MU>::BYTES + 128;
   auto kern = prepass_kernel<IO, MU, SC>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
   return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, m.g, pl, sp.A_log, sp.ws);
 }
@@ -763,7 +762,7 @@ int launch_forward_y_t(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t
   if (make_maps(pl, sp, &m)) return 1;
   const int bytes = NSTAGE * Stage<sizeof(IO), false>::BYTES + 128;
   auto kern = forward_y_kernel<IO, SC>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, bytes, done)) return 1;
   return launch_dependent(kern, dim3(pl.tiles, pl.S, pl.B), dim3(NTHR), bytes, st, m.x, m.d, pl, sp.A_log, sp.ws, (IO*)y);
 }

@@ -69,31 +69,20 @@ __device__ __forceinline__ void bulk_1d(void* dst, const void* src, uint32_t byt
 
 template <typename IO> struct IoSz { static constexpr int v = sizeof(IO); };
 
-// per-thread values of its NCH channels
+// per-thread values of its two channels
+static_assert(NCH == 2, "the loads below fetch a channel pair");
 struct ChV { float v[NCH]; };
 __device__ __forceinline__ ChV ch_zero() { ChV r; for (int c = 0; c < NCH; ++c) r.v[c] = 0.f; return r; }
 
 // row j of a staged [CK x CH] tile, channels NCH*k .. NCH*k + NCH-1
 template <typename IO> __device__ __forceinline__ ChV lds_ch(const uint8_t* tile, int j, int k);
 template <> __device__ __forceinline__ ChV lds_ch<float>(const uint8_t* tile, int j, int k) {
-  ChV r;
-  if (NCH == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(tile + (j * CH + 2 * k) * 4);
-    r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  } else {
-    r.v[0] = *reinterpret_cast<const float*>(tile + (j * CH + k) * 4);
-  }
-  return r;
+  const float2 t = *reinterpret_cast<const float2*>(tile + (j * CH + 2 * k) * 4);
+  return ChV{{t.x, t.y}};
 }
 template <> __device__ __forceinline__ ChV lds_ch<__nv_bfloat16>(const uint8_t* tile, int j, int k) {
-  ChV r;
-  if (NCH == 2) {
-    const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + (j * CH + 2 * k) * 2));
-    r.v[0] = t.x; r.v[NCH - 1] = t.y;
-  } else {
-    r.v[0] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + (j * CH + k) * 2));
-  }
-  return r;
+  const float2 t = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + (j * CH + 2 * k) * 2));
+  return ChV{{t.x, t.y}};
 }
 __device__ __forceinline__ void stg_ch(float* p, const float (&v)[NCH]) {
 #pragma unroll
@@ -126,14 +115,6 @@ __device__ __forceinline__ void load_A2(const float* A_log, const Who& w, u64 (&
   }
 }
 // 16 values of this thread inside a 2048-float tile block: float4 q of thread tid at (q*128 + tid)
-__device__ __forceinline__ void load_block(const float* blk, int tid, u64 (&v)[NU]) {
-  const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
-#pragma unroll
-  for (int q = 0; q < 2 * NCH; ++q) {
-    const ulonglong2 t = b2[q * NTHR + tid];
-    v[2 * q] = t.x; v[2 * q + 1] = t.y;
-  }
-}
 __device__ __forceinline__ void load_block_g(const float* blk, int tid, u64 (&v)[NU]) {
   const ulonglong2* b2 = reinterpret_cast<const ulonglong2*>(blk);
 #pragma unroll
@@ -200,24 +181,10 @@ __device__ __forceinline__ void zero_rows(uint8_t* tile, int row_bytes, int nt, 
   for (int i = tid; i < n16; i += NTHR) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// ---- tensor maps for the [B*T, P] activation tiles (box = CK tokens x bw channels, no swizzle) --------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn get_encode() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
+// ---- tensor maps for the [B*T, P] activation tiles (box = CK tokens x `width` channels, no swizzle) --------
 int act_map(CUtensorMap* tm, const void* base, const Plan& pl, int batches, int elem_bytes, bool is_bf16, int ld,
             int width = CH) {
-  EncodeTiledFn enc = get_encode();
+  EncodeTiledFn enc = encode_tiled();
   if (!enc) return 1;
   cuuint64_t dims[2] = {(cuuint64_t)pl.P, (cuuint64_t)batches * (cuuint64_t)pl.T};
   cuuint64_t strides[1] = {(cuuint64_t)ld * elem_bytes};

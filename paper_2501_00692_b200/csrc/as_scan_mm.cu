@@ -541,23 +541,9 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn get_encode() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
 // [rows = batches * T, cols = P] row-major, boxes of `bw` channels x TCK tokens
 int chunk_map(CUtensorMap* tm, const void* base, const Plan& pl, int elem_bytes, bool is_bf16, int bw, bool swz) {
-  EncodeTiledFn enc = get_encode();
+  EncodeTiledFn enc = encode_tiled();
   if (!enc) return 1;
   cuuint64_t dims[2] = {(cuuint64_t)pl.P, (cuuint64_t)pl.B * (cuuint64_t)pl.T};
   cuuint64_t strides[1] = {(cuuint64_t)pl.P * elem_bytes};
@@ -582,7 +568,7 @@ int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_
   if (chunk_map(&md, sp.ws + pl.off_delta, pl, 4, false, MCH, false)) return 1;
   if (chunk_map(&my, y, pl, 2, true, MCH, false)) return 1;
   auto kern = scalar_mm_kernel<true>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
   return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, my, pl, sp.A_log, sp.ws, (__nv_bfloat16*)y);
 }
@@ -592,7 +578,7 @@ int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st)
   if (chunk_map(&mx, sp.x, pl, 2, true, MCH, false)) return 1;
   if (chunk_map(&md, sp.ws + pl.off_delta, pl, 4, false, MCH, false)) return 1;
   auto kern = scalar_mm_kernel<false>;
-  static bool done[AS_MAX_DEVICES] = {};
+  static DeviceFlags done = {};
   if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
   return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, mx, pl, sp.A_log, sp.ws,
                           (__nv_bfloat16*)nullptr);

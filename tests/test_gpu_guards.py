@@ -126,3 +126,49 @@ def test_status_block_of_packed_weights_calls(T, P):
             assert B.as_check_status(ws) == B.AS_ERR_TIMEOUT, cta
             ws[16 + cta] = 0
         assert B.as_check_status(ws) == B.AS_OK
+
+
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+def test_host_threads_on_their_own_streams(io):
+    """Several host threads may call at once, each with its own stream and scratch; what the launchers remember per process
+    is shared between them.  Sequential calls before and after give the same outputs, to the rounding of the atomics."""
+    import threading
+    build_library()
+    w = synth.custom_workload("threads", 24, 1, 700, 136, tbar=90, io=io)
+    theta = synth.layer_params(w, 0, DEV)
+    x, dy = synth.activations(w, DEV)
+    sh = B.shape_of(x)
+    _, gb = B.as_workspace_bytes(sh, w.tbar)
+    n = 4
+    ws = [B.alloc_workspace(gb, DEV) for _ in range(n)]
+    ys = [torch.empty_like(x) for _ in range(n)]
+    grads = [B.alloc_grads(sh, DEV) for _ in range(n)]
+    streams = [torch.cuda.Stream() for _ in range(n)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(i):
+        try:
+            for _ in range(5):
+                B.as_ssm_forward(sh, theta, x, ys[i], ws[i], stream=streams[i])
+                B.as_adjoint_grad(sh, theta, x, dy, w.tbar, grads[i], ws[i], stream=streams[i])
+        except Exception as e:   # an assertion in a thread would be lost
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    assert all(B.as_check_status(ws[i], streams[i]) == B.AS_OK for i in range(n))
+    y, ref = torch.empty_like(x), B.alloc_grads(sh, DEV)
+    B.as_ssm_forward(sh, theta, x, y, ws[0])
+    B.as_adjoint_grad(sh, theta, x, dy, w.tbar, ref, ws[0])
+    rtol = 1e-5 if io == "f32" else 1e-2
+    for i in range(n):
+        assert torch.equal(ys[i], y)
+        for k, v in ref.items():
+            a, b = grads[i][k].double(), v.double()
+            assert float((a - b).abs().max()) <= rtol * float(b.abs().max()) + 1e-30, k
