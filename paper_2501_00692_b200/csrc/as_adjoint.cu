@@ -6,7 +6,7 @@
 // packed operands as they lie, sums over states end with both channels' sums in one pair, and only B_t and C_t, which all
 // channels share, are needed twice: the pre-pass leaves them doubled, (B_n, B_n), in a buffer of their own.
 //
-// Bound: dispatch of the arithmetic pipes, with MUFU.EX2 next (3 warps per scheduler; each token costs a warp about 320
+// Bound: dispatch of the arithmetic pipes, with MUFU.EX2 next (3 warps per scheduler; each token costs a warp 314
 // instructions for 512 state-steps).  Measured at C3 sizes (2 x 65,536 tokens, 768 channels): full form 1.50 -> 1.39 ms
 // against packing the states of a channel, whose (Delta, Delta), (x, x), (dy, dy) pairs, finalisation of every token by
 // both lanes and separate abar h product cost more.  Tried on the way and slower: sums over channels by a shuffle

@@ -45,6 +45,15 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
   // So: three waves (two in the full form) while segments stay at 160 tokens (truncated: two waves at 112) or more, for the tail of long
   // runs; else two, else one; and where not even one wave can be filled, segments as short as two chunks (one chunk for
   // short sequences, whose full-form carries are cheap): latency counts there, and it is the tokens of a segment.
+  // Both choices on both sides of the lines, whole bf16 gradient calls in us (tokens of the longer count's segments in brackets):
+  //   truncated, two waves | one, line at 112: 1 x 28,416 x 256 [64] 245 | 239, 1 x 42,624 x 256 [96] 335 | 336, 1 x 49,728 x 256
+  //     [112] 377 | 380, 1 x 9,472 x 768 [64] 284 | 283, 1 x 16,576 x 768 [112] 372 | 384, 2 x 6,160 x 1,024 [112] 456 | 470: the
+  //     crossover moves with the width, at most 96 tokens; from 112 on two waves are the faster ones everywhere;
+  //   truncated, three | two, line at 160: 2 x 15,984 x 768 [144] 663 | 654, 2 x 17,760 x 768 [160] 727 | 719, 2 x 28,416 x 768 [256]
+  //     1,138 | 1,143, 2 x 11,952 x 1,024 [144] 779 | 782, 2 x 13,280 x 1,024 [160] 758 | 775: within 2 % either way from 112 to
+  //     256 tokens, the crossover depends on the width;
+  //   full, two | one, line at 160: 1 x 35,520 x 512 [160] 471 | 491, 1 x 21,312 x 512 [96] 312 | 320, 2 x 5,280 x 1,024 [96] 331 | 347:
+  //     not a crossover, two waves would still be the faster ones at 96 tokens.
   const int64_t slots = (int64_t)sm_count() * 3;   // resident CTAs of the main kernel
   auto segment = [&](int64_t ctas) {
     int64_t l = 0;
@@ -52,7 +61,7 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
       int64_t s_target = waves * slots / ctas;
       if (s_target < 1) s_target = 1;
       l = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;
-      if (l >= (waves == 2 && !p.full ? 112 : 160)) break;   // 2 x 8,192 x 1,024, two waves of 120 tokens: 598 -> 581 us
+      if (l >= (waves == 2 && !p.full ? 112 : 160)) break;
     }
     return l;
   };
@@ -67,8 +76,10 @@ int make_plan(const as_shape_t* sh, int64_t tbar, int layers, Plan* pl, int kind
     p.one_order = 1;
     // The bf16 forward keeps one segmentation (two waves, 64 tokens at least) whatever the size: a deep stack of bf16 layers
     // turns fp32 rounding differences of one layer's y into differences of some per cent of its outputs, so its results
-    // should not move when the schedule of other sizes is tuned.  Short narrow runs, which are all latency (256 tokens x
-    // 256: 37 us with these segments, 23 with short ones), are left out unless the caller asks for the order.
+    // should not move when the schedule of other sizes is tuned.  Short narrow runs, which are all latency, are left out
+    // unless the caller asks for the order: short segments | these, 256 x 256 22.5 | 34.3 us, 1,024 x 256 27.2 | 35.2.  The
+    // line is not a crossover (1,032 x 256 28.6 | 35.3, 256 x 264 24.1 | 35.9, 4,096 x 256 40.9 | 49.6, 1,024 x 512
+    // 34.1 | 36.5): it bounds the sizes whose results differ in the last bits from as_ssm_forward_ordered's.
     int64_t s_target = 2 * slots / ((int64_t)p.tiles * p.B);
     if (s_target < 1) s_target = 1;
     L = ((p.T + s_target - 1) / s_target + CK - 1) / CK * CK;

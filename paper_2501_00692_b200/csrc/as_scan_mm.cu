@@ -13,9 +13,10 @@
 // the operands are rounded to bf16).  One CTA = 128 channels x one segment, 256 threads: thread (p, h) owns channel p in
 // half h of every chunk.  The exponents are bounded by |a_p| times a quarter chunk's Delta sum; a channel whose bound
 // exceeds 2^+-96 in a chunk takes the plain recurrence for that chunk in thread (p, 0) (its TMEM lane is then ignored).
-// The CTA waits for such a channel, so the recurrence loads and scales several tokens at once before it runs their chain (decay
-// rates up to 16 and step sizes around 0.05, where some channels of every tile do this: 2 x 32,768 x 768 both passes 250 -> 240 us,
-// 2,048 x 512 the whole forward 53 -> 44 us).
+// The CTA waits for such a channel, so the recurrence loads and scales several tokens at once before it runs their chain: 2 x
+// 32,768 x 768 both passes 250 -> 240 us, 2,048 x 512 the whole forward 53 -> 44 us.  With decay rates up to 16 and step sizes
+// around 0.08 one (channel, chunk) in 4,000 is such a case, which is one chunk of a CTA in 33; all of them together cost a
+// forward of 2 x 32,768 x 768 about 8 % (349 us against 323 with rates up to 4, where no channel leaves the form).
 // Every mbarrier wait is bounded; on a timeout the kernel records AS_ERR_TIMEOUT, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -559,7 +560,7 @@ int chunk_map(CUtensorMap* tm, const void* base, const Plan& pl, int elem_bytes,
 }  // namespace
 
 // Short narrow runs have segments of a few scan chunks (see make_plan), less than one chunk of this form: they take the scan
-// kernels (512 tokens x 256: 34 -> 26 us, 1,024 x 256: 38 -> 29 us).
+// kernels (512 tokens x 256: 34 -> 26 us, 1,024 x 256: 38 -> 29 us; the line is make_plan's, which says why it lies there).
 bool forward_y_mm_applies(const Plan& pl) { return pl.scalar && pl.io == AS_BF16 && pl.P % MCH == 0 && pl.one_order; }
 
 int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st) {

@@ -105,12 +105,13 @@ def compare_all(g, ref, tol):
 
 
 def assert_dalog_rows(got, ref, tol, what="dA_log"):
-    """dA_log channel by channel.  The library forms abar_i h_{i-1} as h_i - Delta_i x_i B_i (one fused operation);
-    h_i carries its own fp32 rounding, so each term mu_i (abar_i h_{i-1}) Delta_i A of the sum has an absolute error of
-    up to a few units of eps_fp32 |Delta_i A mu_i h_i|, whatever the size of abar_i h_{i-1} itself.  Per channel p:
+    """dA_log channel by channel.  The library forms abar_i h_{i-1} as the product, from the state before the token; a
+    build may also form it as h_i - Delta_i x_i B_i, whose error is a few units of eps_fp32 |Delta_i A mu_i h_i| in each term
+    mu_i (abar_i h_{i-1}) Delta_i A of the sum (h_i carries its own fp32 rounding), whatever the size of abar_i h_{i-1} itself.
+    Per channel p:
         max_n |got - oracle|  <=  tol * max_n |oracle[p, :]|  +  DALOG_C * eps_fp32 * max_n absq[p, :]
-    with absq from the oracle.  The second term is what the difference form may add; it is reported so that a run shows
-    how much of it was used."""
+    with absq from the oracle.  The second term is what the difference form may add and the product form does not need; it
+    is reported so that a run shows how much of it was used."""
     got = np.asarray(got, dtype=np.float64)
     want = ref["dA_log"]
     if want.ndim == 1:

@@ -151,9 +151,9 @@ def test_degenerate_and_tiny_shapes(batch, T, P, tbar, io):
 @pytest.mark.parametrize("T", [2, 3, 8, 64, 300])
 def test_dalog_row_by_row(T, law, io):
     """dA_log channel by channel where abar_i h_{i-1} is small against h_i: very short sequences (h_{i-1} is zero or
-    one step old) and the fast-decay corner b_delta ~ U(-1, 1) (abar << 1).  The library forms abar_i h_{i-1} as
-    h_i - Delta_i x_i B_i; the bound allows DALOG_C rounding units of h_i per term beyond the tolerance and the test
-    reports how much of that allowance was used."""
+    one step old) and the fast-decay corner b_delta ~ U(-1, 1) (abar << 1).  The bound allows what forming
+    abar_i h_{i-1} as h_i - Delta_i x_i B_i would cost, DALOG_C rounding units of h_i per term beyond the tolerance, and
+    the test reports how much of that allowance was used."""
     w = synth.custom_workload("dalog", 18, 2, T, 72, tbar=max(1, T // 2), io=io)
     rng = {"fast": (-1.0, 1.0), "standard": None, "slow": (-9.0, -7.0)}[law]
     theta = synth.layer_params(w, 0, DEV, b_delta_range=rng)
