@@ -1,5 +1,5 @@
 """Times `as_ssm_forward` on one workload for the diagonal structure (scan kernels) and the scalar structure (bf16 I/O,
-d_model % 128 == 0: y pass in the matmul form), CUDA events, median over the calls.
+d_model % 128 == 0: both passes in the matmul form), CUDA events, median over the calls.
 
     python -m paper_2501_00692_b200.examples.forward_bench [--workload C3] [--batch B --seq-len T --d-model P] [--calls 20]
 """
