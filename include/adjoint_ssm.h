@@ -142,7 +142,8 @@ int as_ssm_forward_ordered(const as_shape_t *shape, const as_params_t *params, c
  * [max(1, t+1-tbar), t]; the C-net term is never truncated.  tbar >= seqlen selects the full form.
  * The adjoint states lambda^{t,i} are never materialised: the cotangents of all tokens t whose window
  * contains i are summed on chip (a reverse-time recurrence with the exact removal of the term that
- * leaves the window) and each source token's three VJPs are evaluated once.
+ * leaves the window) and each source token's three VJPs are evaluated once.  The removal is exact up to fp32 rounding: a term is
+ * left in where it has decayed below 2^-64 of the cotangent that it is made of, or below 2^-30 of the sum that it would be taken from.
  * Self-contained: recomputes the forward quantities it needs from x; no prior as_ssm_forward call needed.
  * dx also uses the windowed sum for the A/B paths and the exact C path. */
 int as_adjoint_grad(const as_shape_t *shape, const as_params_t *params, const void *x, const void *dy,
