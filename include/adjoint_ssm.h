@@ -245,8 +245,10 @@ int64_t as_launch_count(int reset);
  * events on its stream between its phases (this creates the events once; timing mode is opt-in and is the one
  * place where the library creates CUDA objects).  as_get_timing synchronises on the last event of the most
  * recent call and writes elapsed milliseconds into ms[0..AS_NUM_PHASES): projections (S1, incl. zeroing),
- * segment pre-pass, carry fix-up, main adjoint kernel, gradient contractions (weights and input), and 0 (the contractions
- * share launches).  Returns AS_OK, or AS_ERR_NULL if timing is off or no call was recorded. */
+ * segment pre-pass, carry fix-up, main adjoint kernel, weight-gradient contractions, input-gradient contractions.  With bf16
+ * I/O a timed call makes a launch of each of the last two, where an untimed one mostly makes one launch of both (the same sums, in
+ * another order); with fp32 I/O they share a launch either way, which counts as the first of them.
+ * Returns AS_OK, or AS_ERR_NULL if timing is off or no call was recorded. */
 #define AS_NUM_PHASES 6
 int as_set_timing(int enable);
 int as_get_timing(float *ms, int n);

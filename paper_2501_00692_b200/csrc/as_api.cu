@@ -100,10 +100,12 @@ int begin(const Plan& pl, const as_params_t* pr, const ZeroList& z, bool grad, c
 // the net-VJPs: weight gradients (contractions over all tokens) and the input gradient, for every layer of the call
 int contractions(const Plan& pl, const as_params_t* pr, const Wcat& wcat, const void* x, const as_grads_t* out, char* ws,
                  cudaStream_t st) {
-  // most calls compute both in one launch: the first phase counts them, the second reads zero
-  AS_TRY(pl.tc ? tc_gradients(pl, pr, wcat.p, x, out, ws, st)
-               : pl.split ? split_gradients(pl, out, ws, st) : simt_gradients(pl, pr, x, out, ws, st));
-  mark(5, st);
+  if (pl.tc) {
+    AS_TRY(tc_gradients(pl, pr, wcat.p, x, out, ws, st, g_timing ? g_ev[5] : nullptr));
+  } else {   // fp32: one launch for both, the first phase counts them, the second reads zero
+    AS_TRY(pl.split ? split_gradients(pl, out, ws, st) : simt_gradients(pl, pr, x, out, ws, st));
+    mark(5, st);
+  }
   mark(6, st);
   return AS_OK;
 }

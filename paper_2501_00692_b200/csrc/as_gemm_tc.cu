@@ -583,7 +583,8 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int 
   return pl.alone ? launch_tc<false, SP_POLY>(t, a, st) : launch_tc<false, SP_LOG>(t, a, st);
 }
 
-int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws, cudaStream_t st) {
+int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws, cudaStream_t st,
+                 cudaEvent_t between) {
   const int64_t rows = (int64_t)pl.Bg * pl.T, all = rows * pl.KL;
   const int P = pl.P, NW = pl.gcols;   // columns of Gcat, rows of Wcat
   auto cvt = pl.gsplit == 3 ? cvt_dbc_kernel<3> : cvt_dbc_kernel<1>;
@@ -600,7 +601,7 @@ int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const 
     dx.M = rows; dx.N = P; dx.kblocks = (NW + BK - 1) / BK;
     const int64_t cdx = cut_columns(CUT_DX, &dx, pl.KL, pairs);
     const int rest = pairs - dx.ntiles;
-    if (dx.ntiles > 0 && rest > 0) {   // short runs: side by side, if DW on the other pairs takes no longer than both in turn
+    if (dx.ntiles > 0 && rest > 0 && !between) {   // short runs: side by side, if DW on the other pairs takes no longer than both in turn
       Job side = dw;
       if (cut_columns(CUT_DW, &side, pl.KL, rest) < cdw + cdx) dw = side;
     }
@@ -628,11 +629,14 @@ int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const 
   // One launch for both where dx is a few waves of tiles: it saves a launch and its ramp, and DX fills DW's last wave (us, two
   // launches | one: 588 x 128 52 | 46, 3,447 x 64 71 | 66, 3 x 5,003 x 1,000 554 | 546, 131,072 x 768 273 | 269).  Long runs have nothing
   // to gain, and the two pairs without a tile of DW that then run ahead cost them (262,144 x 2,048 3,250 | 3,390).
-  if (dw.ntiles < 0 || dx.ntiles <= 8 * pairs) return launch_tc<true, SP_LOG>(t, a, st);
+  // With phase timing always two launches, so that the phases can be told apart.
+  if (dw.ntiles < 0 || (dx.ntiles <= 8 * pairs && !between)) return launch_tc<true, SP_LOG>(t, a, st);
   TcArgs first = a;
   first.job[1].ntiles = 0;
   dw.ntiles = 0;
-  return launch_tc<true, SP_LOG>(t, first, st) || launch_tc<true, SP_LOG>(t, a, st);
+  if (dx.ntiles < 0 || launch_tc<true, SP_LOG>(t, first, st)) return 1;
+  if (between && cudaEventRecord(between, st) != cudaSuccess) return 1;
+  return out->dx ? launch_tc<true, SP_LOG>(t, a, st) : 0;
 }
 
 }  // namespace as

@@ -230,7 +230,9 @@ int launch_wait_selftest(int* status, unsigned limit, cudaStream_t st);
 // where the call has no kernel before them.  wcat: the packed weights, or null: W_delta, W_B, W_C are read where they lie.
 int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int wreps, const void* x,
                    const ZeroList& z, char* ws, cudaStream_t st);
-int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws, cudaStream_t st);
+// between: phase timing's event between weight and input gradient, which then are two launches at every size; or null.
+int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws, cudaStream_t st,
+                 cudaEvent_t between);
 
 // fp32 I/O on the tensor cores by exact three-term splits (as_gemm_split.cu), for large enough products
 int split_projections(const Plan& pl, const as_params_t* pr, const void* x, const ZeroList& z, char* ws, cudaStream_t st);
