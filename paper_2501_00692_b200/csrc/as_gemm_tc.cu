@@ -519,6 +519,7 @@ int pair_count() { return sm_count() / 2 < STATUS_CTAS / 2 ? sm_count() / 2 : ST
 // Returns that time in cycles.
 constexpr int64_t EPI_CYCLES = 1500;
 enum { CUT_PROJ, CUT_DW, CUT_DX };
+constexpr int64_t ONE_LAUNCH_BLOCKS = 400;   // see tc_gradients
 int64_t cut_columns(int what, Job* j, int layers, int pairs) {
   const int u = unit(what == CUT_DX), units = (int)cdiv(j->N, u);
   const bool split = what == CUT_DW;
@@ -626,11 +627,15 @@ int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const 
   } else {
     t.m[GM_GK] = t.m[GM_W] = t.m[GM_DX] = t.m[GM_DIR] = t.m[GM_W1] = t.m[GM_WB] = t.m[GM_WC] = t.m[GM_X];
   }
-  // One launch for both where dx is a few waves of tiles: it saves a launch and its ramp, and DX fills DW's last wave (us, two
-  // launches | one: 588 x 128 52 | 46, 3,447 x 64 71 | 66, 3 x 5,003 x 1,000 554 | 546, 131,072 x 768 273 | 269).  Long runs have nothing
-  // to gain, and the two pairs without a tile of DW that then run ahead cost them (262,144 x 2,048 3,250 | 3,390).
+  // One launch for both up to ONE_LAUNCH_BLOCKS blocks of the input gradient a pair: it saves a launch and its ramp, and DX fills DW's
+  // last wave.  Longer runs have nothing to gain, and the two pairs without a tile of DW that then run ahead cost them.  Both
+  // gradients, us, two launches | one, by blocks a pair: 588 x 128 (whole call) 52 | 46, 3,447 x 64 71 | 66, 3 x 5,003 x 1,000 554 | 546;
+  // 40,000 x 512 [38] 68 | 60; 2 x 32,768 x 768 [135] 146 | 142; 262,144 x 384 [194] 249 | 243, x 512 [249] 310 | 304; 131,072 x 768
+  // [270] 278 | 277; 43,690 x 1,536 [347] 314 | 310; 98,304 x 1,024 [354] 343 | 340; 400,000 x 512 [380] 473 | 472; 200,000 x 768 [412]
+  // 429 | 432; 32,768 x 2,048 [457] 388 | 390; 131,072 x 1,024 [470] 460 | 460; 65,536 x 1,536 [520] 466 | 468; 49,152 x 2,048 [686]
+  // 589 | 605; 262,144 x 2,048 [3,650] 3,258 | 3,400.
   // With phase timing always two launches, so that the phases can be told apart.
-  if (dw.ntiles < 0 || (dx.ntiles <= 8 * pairs && !between)) return launch_tc<true, SP_LOG>(t, a, st);
+  if (dw.ntiles < 0 || ((int64_t)dx.ntiles * dx.kblocks <= ONE_LAUNCH_BLOCKS * pairs && !between)) return launch_tc<true, SP_LOG>(t, a, st);
   TcArgs first = a;
   first.job[1].ntiles = 0;
   dw.ntiles = 0;

@@ -54,3 +54,24 @@ def test_phases_tell_the_contractions_apart(with_dx):
     assert all(v > 0 for v in best.values())
     assert best["weight_grads"] > 0.01
     assert (best["input_grad"] > 0.01) == with_dx, best
+
+
+def test_large_layers_take_two_launches():
+    """3 x 10,001 x 2,048: 960 tiles of 33 blocks for the input gradient, past the line of 400 blocks a pair of CTAs; rows that end inside
+    a tile.  Every layer against a call of its own, which makes one launch: the same sums in another order, rounded to bf16 on the way
+    (dx, and du as the operand of both contractions)."""
+    build_library()
+    w = synth.custom_workload("large", 61, 1, 10001, 2048, tbar=300, io="bf16")
+    B.as_launch_count(reset=True)
+    thetas, xs, dy, g, _ = stacked_call(w, 3, True, False)
+    two = B.as_launch_count() // 3
+    sh = B.shape_of(dy, w.d_state)
+    ws = B.alloc_workspace(B.as_workspace_bytes(sh, w.tbar)[1], DEV)
+    one = B.alloc_grads(sh, DEV, with_dx=True)
+    for k in range(3):
+        B.as_launch_count(reset=True)
+        B.as_adjoint_grad(sh, thetas[k], xs[k], dy, w.tbar, one, ws)
+        assert B.as_check_status(ws) == B.AS_OK
+        assert two == B.as_launch_count() + 1
+        for name, v in one.items():
+            assert float((g[name][k].float() - v.float()).norm() / v.float().norm()) <= 2.0 ** -8, name
