@@ -113,6 +113,17 @@ def test_forward_refuses_less_scratch_than_reported(L, shape):
     assert L.as_ssm_forward(C.byref(sh), C.byref(p), ok, ok, ok, fwd - 1, None) == B.AS_ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("P,split", [(8, False), (32, False), (56, False), (64, True), (88, True)])
+def test_narrow_fp32_gradients_keep_no_split_operands(P, split):
+    """From 2^30 multiply-adds on fp32 gradients keep x and the cotangents as three bf16 terms, 12 bytes a value, but not below a width
+    of 64, where the tensor-core form is no faster (bytes a token, by a short run that never does, and a long one)."""
+    def per_token(T):
+        return B.as_workspace_bytes(B.make_shape(1, T, P), 256)[1] / T
+    T = (1 << 31) // (P * (P + 32))
+    grown = (per_token(T) - per_token(T // 4)) / P
+    assert (grown > 4) == split, grown   # the arrays by the segment take less a token in the longer run
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libadjoint_ssm.so")
