@@ -71,6 +71,9 @@ enum {
 
 /* flags */
 #define AS_ACCUMULATE 1u  /* add into the parameter-gradient buffers instead of overwriting them */
+#define AS_ORDERED 2u     /* bf16 io: the layer's forward was as_ssm_forward_ordered (a layer of a stack).  Both forwards have a softplus of
+                             their own, which differ by up to 2e-5; with the flag that fits, and d_model % 32 == 0, a gradient call
+                             forms the very Delta that the forward formed, bit for bit.  fp32 io: no effect */
 
 typedef struct {
   int32_t batch;      /* Bsz >= 1 */
@@ -130,8 +133,8 @@ int as_ssm_forward(const as_shape_t *shape, const as_params_t *params, const voi
 /* as_ssm_forward for the layers of a stack with bf16 I/O: always the same order of additions, for every size (one segmentation,
  * one order of the carries; at widths that are no multiple of 32 the projections run on the fp32 pipe).  A deep stack that rounds
  * every layer's output to bf16 turns differences in the last fp32 bit of one layer into differences of some per cent of its
- * outputs, so there the order is part of the result; a single layer does not need it.  It is the order of the forward alone:
- * the gradient calls form Delta, B, C and the states again in an order of their own (on the tensor cores at every width).  At
+ * outputs, so there the order is part of the result; a single layer does not need it.  The gradient of such a layer takes AS_ORDERED;
+ * it forms the states in segments of its own, and at widths that are no multiple of 32 Delta, B and C on the tensor cores.  At
  * widths that are no multiple of 32 it has its price: 3 x 5,003 x 1,000 1,190 us against 198. */
 int as_ssm_forward_ordered(const as_shape_t *shape, const as_params_t *params, const void *x, void *y,
                            void *ws, size_t ws_bytes, void *stream);

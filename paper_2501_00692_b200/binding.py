@@ -17,6 +17,7 @@ LIB_PATH = os.path.join(_HERE, "libadjoint_ssm.so")
 AS_F32, AS_BF16 = 0, 1
 AS_A_DIAGONAL, AS_A_SCALAR = 0, 1
 AS_ACCUMULATE = 1
+AS_ORDERED = 2
 AS_OK = 0
 AS_ERR_NULL, AS_ERR_SHAPE, AS_ERR_DTYPE, AS_ERR_TBAR = -1, -2, -3, -4
 AS_ERR_WORKSPACE, AS_ERR_ALIGN, AS_ERR_CUDA, AS_ERR_TIMEOUT, AS_ERR_LIMIT = -5, -6, -7, -8, -9

@@ -295,6 +295,7 @@ int as_adjoint_grad_layers(const as_shape_t* shape, int32_t layers, const as_par
   Plan pl;
   e = make_plan(shape, tbar, layers, &pl);
   if (e) return e;
+  pl.ordered = (flags & AS_ORDERED) != 0;
   if (ws_bytes < pl.total_grad) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
@@ -322,6 +323,7 @@ int as_full_bptt_grad(const as_shape_t* shape, const as_params_t* params, const 
   Plan pl;
   e = make_plan(shape, shape->seqlen, 1, &pl);
   if (e) return e;
+  pl.ordered = (flags & AS_ORDERED) != 0;
   if (ws_bytes < pl.total_grad) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);

@@ -581,7 +581,7 @@ int tc_projections(const Plan& pl, const as_params_t* pr, const void* wcat, int 
   if (output(&t.m[PM_DELTA], true, CU_TENSOR_MAP_SWIZZLE_128B, ws + pl.off_delta, pl.KL, j.M, P, 32, 32)) return 1;
   if (output(&t.m[PM_BC], true, CU_TENSOR_MAP_SWIZZLE_128B, ws + pl.off_bc, pl.KL, j.M, NBC, 32, 32)) return 1;
   if (P % 32) return launch_tc<false, SP_FINE>(t, a, st);
-  return pl.alone ? launch_tc<false, SP_POLY>(t, a, st) : launch_tc<false, SP_LOG>(t, a, st);
+  return pl.ordered ? launch_tc<false, SP_LOG>(t, a, st) : launch_tc<false, SP_POLY>(t, a, st);
 }
 
 int tc_gradients(const Plan& pl, const as_params_t* pr, const void* wcat, const void* x, const as_grads_t* out, char* ws, cudaStream_t st,

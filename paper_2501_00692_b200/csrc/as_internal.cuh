@@ -174,7 +174,7 @@ struct Plan {
   int scalar;       // 1: one decay rate per channel (A_log is [P]), 0: one per (channel, state)
   int tiles;        // ceil(P / CH) channel tiles
   int tc;           // 1: bf16 tensor-core contractions (bf16 I/O), 0: FP32-pipe GEMMs
-  int alone;        // the forward of a single layer (as_ssm_forward, as_ssm_forward_static), no part of a stack's step
+  int ordered;      // a call of a bf16 stack's step: as_ssm_forward_ordered, or a gradient with AS_ORDERED
   int ffma;         // projections of bf16 I/O on the fp32 pipe (as_ssm_forward_ordered, widths off the 32-element grid)
   int one_order;    // bf16 forwards of stacks and of the matmul form: one segmentation and one order of the carries for all sizes
   int split;        // fp32 I/O: contractions on the tensor cores, every operand as three bf16 terms (as_gemm_split.cu)

@@ -73,7 +73,7 @@ class Stack:
             if record is not None and k in record:
                 record[k] = (self.yhat.clone(), G.clone())
             gk = B.alloc_grads(self.shape, dev, with_dx=(mode == "chained"))
-            B.as_adjoint_grad(self.shape, self.thetas[k], self.yhat, G, self.tbar, gk, self.ws)
+            B.as_adjoint_grad(self.shape, self.thetas[k], self.yhat, G, self.tbar, gk, self.ws, B.AS_ORDERED)
             if mode == "chained":
                 B.as_rmsnorm_bwd_add(self.shape, self.ys[k], gk["dx"], G, self.eps)
                 gk["dx"] = None
@@ -106,7 +106,7 @@ class Stack:
                 if 0 <= k < K:
                     record[k] = (self._x[k].clone(), g.clone())
         gl = B.alloc_grads_layers(sh, K, g.device)
-        B.as_adjoint_grad_layers(sh, K, self._stacked, self._xall, g, self.tbar, gl, self._ws_layers)
+        B.as_adjoint_grad_layers(sh, K, self._stacked, self._xall, g, self.tbar, gl, self._ws_layers, B.AS_ORDERED)
         self.ws_last = self._ws_layers
         per_layer = {k: (v.unbind(0) if v is not None else [None] * K) for k, v in gl.items()}
         return [{k: v[i] for k, v in per_layer.items()} for i in range(K)]
