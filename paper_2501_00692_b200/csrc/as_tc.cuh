@@ -84,7 +84,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 
 // softplus(u) = max(u, 0) + log(1 + z), z = exp(-|u|) in (0, 1].  SP_LOG: two MUFU ops (ex2, lg2) and a short series for small z,
 // where forming 1 + z would lose z's low bits (relative error of the result < 1e-5 from Delta = 0.02 on, 2e-5 below); kept for
-// the calls that make up a step of a bf16 stack, which turns a change of Delta's last bits into some per cent of its outputs.
+// the calls that make up a step of a bf16 stack (Plan.ordered), which turns a change of Delta's last bits into some per cent of its outputs.
 __device__ __forceinline__ float softplus_log(float u) {
   const float z = ex2_approx(-fabsf(u) * LOG2E);
   float l;
@@ -93,8 +93,11 @@ __device__ __forceinline__ float softplus_log(float u) {
   const float small = z * fmaf(z, fmaf(z, 1.f / 3.f, -0.5f), 1.f);   // z - z^2/2 + z^3/3
   return fmaxf(u, 0.f) + (z < 0.0078125f ? small : big);
 }
-// SP_POLY, SP_FINE, of a packed pair: log(1 + z) is z Q(z) with the polynomial Q of least relative error on [0, 1] (Remez exchange; degree 7: 1.9e-7, with fp32 rounding 3.4e-7; degree 9: 4.7e-9 and 1.6e-7): packed
-// multiply-adds, where the logarithm takes a second MUFU operation and the series beside it.  SP_FINE: degree 9, and the rounding of the product -|u| log2 e is put back as a factor of z (relative error < 5e-7 for all u).
+// SP_POLY, SP_FINE, of a packed pair: log(1 + z) is z Q(z) with the polynomial Q of least relative error on [0, 1] (Remez exchange;
+// degree 7: 1.9e-7, degree 9: 4.7e-9): packed multiply-adds, where the logarithm takes a second MUFU operation and the series beside it.
+// SP_POLY, degree 7: with fp32 rounding and an exact exp2 the relative error is 3.9e-7 for u in [-2, 10], 5.4e-7 in [-10, -2], 8.1e-7 in
+// [-20, -10] and 3.6e-6 in [-80, -60], for the product -|u| log2 e is rounded.  SP_FINE, degree 9, puts that rounding back as a factor of z:
+// 2.1e-7 for all u.  ex2.approx adds up to 2.4e-7 to either.
 // The projections of 131,072 x 768: 174 us with SP_LOG, 166 with SP_POLY.
 enum { SP_LOG = 0, SP_POLY = 1, SP_FINE = 2 };
 template <int SP> __device__ __forceinline__ u64 softplus2(u64 u) {
