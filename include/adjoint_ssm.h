@@ -27,9 +27,11 @@
  *   - Device-side waits: every wait on staged data (mbarrier waits on TMA / bulk copies and on tensor-core commits)
  *     is bounded and ends in AS_ERR_TIMEOUT.  The one wait that has no software bound is the hardware allocation of
  *     tensor memory (tcgen05.alloc) at the start of the contraction, adjoint and matmul-form forward kernels: it blocks until enough of
- *     the SM's 512 columns are free, which happens when CTAs that hold them finish; a kernel of this library frees
- *     its columns on every exit path and never waits for another CTA while holding them, so the allocation of a
- *     later CTA always completes.
+ *     the SM's 512 columns are free, which happens when CTAs that hold them finish, and a kernel of this library frees
+ *     its columns on every exit path.  The only CTAs that wait for another CTA while holding columns are the two of a pair in the
+ *     bf16 contractions: a cluster, which the hardware starts together, each with 225 of the 227 KB of shared memory of its SM.  No
+ *     other CTA that holds columns fits beside one (they use 50 KB and more), a pair waits for nobody else, and so the allocation
+ *     of a later CTA always completes.
  *   - Results are deterministic up to floating-point summation order (fp32 atomics are used for the
  *     sums over channels, segments and the batch).
  */
@@ -94,7 +96,7 @@ typedef struct {          /* parameters of one layer (device pointers) */
                              by as_pack_weights.  Only the bf16 tensor-core contractions read it (bf16 io; the
                              gradient calls only where P % 32 == 0); when NULL, or in a gradient call at another width,
                              they pack a copy into the scratch on every call (one more small kernel) or, up to 1,024
-                             tokens a layer and with P % 16 == 0, read W_delta, W_B and W_C where they lie. */
+                             tokens in all layers and with P % 16 == 0, read W_delta, W_B and W_C where they lie. */
 } as_params_t;
 
 typedef struct {          /* gradient outputs (device pointers); parameter gradients are fp32, summed over the batch */
