@@ -390,7 +390,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps<GRAD> maps, const __grid_constant_
               for (int p = 0; p < 4; ++p) {
                 // four columns: all inside one part (its border is a multiple of 8) or all outside
                 if (!border || col + 4 * p < a.P) {
-                  const ulonglong2 bv = __ldg(reinterpret_cast<const ulonglong2*>(bias_l + 4 * p));
+                  const f2x2 bv = split4(__ldg(reinterpret_cast<const float4*>(bias_l + 4 * p)));
                   float v[4];
                   upk(softplus2<SP>(add2(pk(__uint_as_float(r[4 * p]), __uint_as_float(r[4 * p + 1])), bv.x)), v[0], v[1]);
                   upk(softplus2<SP>(add2(pk(__uint_as_float(r[4 * p + 2]), __uint_as_float(r[4 * p + 3])), bv.y)), v[2], v[3]);

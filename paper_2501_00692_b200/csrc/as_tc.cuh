@@ -100,7 +100,7 @@ __device__ __forceinline__ float softplus_log(float u) {
 // 2.1e-7 for all u.  ex2.approx adds up to 2.4e-7 to either.
 // The projections of 131,072 x 768: 174 us with SP_LOG, 166 with SP_POLY.
 enum { SP_LOG = 0, SP_POLY = 1, SP_FINE = 2 };
-template <int SP> __device__ __forceinline__ u64 softplus2(u64 u) {
+template <int SP> __device__ __forceinline__ f2 softplus2(f2 u) {
   constexpr bool FINE = SP == SP_FINE;
   float u0, u1;
   upk(u, u0, u1);
@@ -111,14 +111,14 @@ template <int SP> __device__ __forceinline__ u64 softplus2(u64 u) {
     const float back = fmaf(a, 1.925963e-8f, fmaf(a, LOG2E, -t));   // log2 e = LOG2E + 1.925963e-8
     return fmaf(z, back * LN2, z);
   };
-  const u64 z = pk(expm(u0), expm(u1));
+  const f2 z = pk(expm(u0), expm(u1));
   constexpr int N = FINE ? 10 : 8;
   constexpr float c7[8] = {9.999998212e-01f, -4.999740422e-01f, 3.327547908e-01f, -2.449546307e-01f,
                            1.774524152e-01f, -1.076817140e-01f, 4.408963397e-02f, -8.539208211e-03f};
   constexpr float c9[10] = {1.0f, -4.999990165e-01f, 3.332996368e-01f, -2.495413423e-01f, 1.967593879e-01f,
                             -1.530559212e-01f, 1.060365513e-01f, -5.695953593e-02f, 1.985146292e-02f, -3.244025167e-03f};
   auto coef = [&](int i) { const float c = FINE ? c9[i] : c7[i < 8 ? i : 7]; return pk(c, c); };
-  u64 q = coef(N - 1);
+  f2 q = coef(N - 1);
 #pragma unroll
   for (int i = N - 2; i >= 0; --i) q = fma2(q, z, coef(i));
   return fma2(z, q, pk(fmaxf(u0, 0.f), fmaxf(u1, 0.f)));
