@@ -184,7 +184,7 @@ struct Plan {
   int gcols;        // columns of Gcat = [du|dB|dC..]: P + 32 gsplit
   int du_ld;        // row pitch (elements) of the du buffer: P, or that of Gcat where it is the left part of it
   // byte offsets into the workspace
-  size_t off_status, off_delta, off_bc, off_bcd, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
+  size_t off_status, off_delta, off_bc, off_ckpt, off_cs, off_hend, off_muloc, off_mupart, off_segd,
       off_partd, off_hstart, off_suf, off_pre, off_total, off_live, off_du, off_dxdir, off_dbc,
       off_bptt_ckpt, off_wcat, off_wcatx, off_xs, off_wsp, off_gs, total_fwd, total_grad;
 };
