@@ -158,7 +158,8 @@ constexpr int STATUS_CTAS = STATUS_BYTES - STATUS_CTA;  // as many CTAs can repo
 // CH channels).  Per-(segment, channel, state) and per-(chunk, channel, state) arrays are stored as
 // blocks of TILE_FLOATS floats per channel tile, in the order the owning thread keeps them in registers
 // (float4 q of thread tid at float offset (q*NTHR + tid)*4), so one bulk copy moves a CTA's block and
-// every thread's access is a contiguous 16 bytes.
+// every thread's access is a contiguous 16 bytes.  A thread's values are the state pairs of its channels, in the chunk
+// checkpoints the channel pairs of its states.
 struct Plan {
   int KL;           // layers handled by one call (independent problems that share dy); 1 for the single-layer entry points
   int Bg;           // batch elements per layer
