@@ -39,8 +39,11 @@ constexpr int SM_CT = SM_SP + 16384;     // C   [64 tokens][16 states] bf16 (fir
 constexpr int SM_BT = SM_CT + 8192;      // B   [64 tokens][16 states] bf16
 constexpr int SM_GM = SM_BT + 8192;      // tril(G) [64 tokens t][64 tokens j] bf16
 constexpr int SM_BTT = SM_GM + 8192;     // B^T [16 states][64 tokens] bf16
-constexpr int SM_TOTAL = SM_BTT + 2048;
-constexpr int SMEM_DYN = SM_TOTAL + 1024;   // + alignment slack
+// The segment pass needs x, Delta, V and B^T alone, 67 of the 107 KB, and 80 registers with V written eight tokens at a time: three CTAs to an SM,
+// which wait for their loads at different times (2 x 32,768 x 768, whole forward: 331 us with two, 326 with three).
+template <bool YPASS> constexpr int sm_btt() { return YPASS ? SM_BTT : SM_SP; }
+template <bool YPASS> constexpr int smem_dyn() { return sm_btt<YPASS>() + 2048 + 1024; }   // + alignment slack
+template <bool YPASS> constexpr int mm_ctas() { return YPASS ? 2 : 3; }
 // tensor-memory columns (lane = channel): G [t][j] lives in lanes 0..63 of columns 0..63 until it has been masked
 constexpr int TM_D = 0;       // [0,32): half 0, [32,64): half 1 (own half), [64,96): half 1 (what reaches it from half 0 and before)
 constexpr int TM_S0 = 96;     // S' + V0^T B0
@@ -157,7 +160,7 @@ __device__ __forceinline__ uint64_t desc_at(uint32_t tile, int row, int kstep) {
 // YPASS: the y pass from the true segment-start state.  !YPASS: the segment pass of the forward (local scan from a zero
 // state: only V and the state products), which writes the segment's end state and Delta sum for the carry kernel.
 template <bool YPASS>
-__global__ void __launch_bounds__(MT, 2)
+__global__ void __launch_bounds__(MT, mm_ctas<YPASS>())
 scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
                    const __grid_constant__ CUtensorMap tmY, Plan pl, const float* __restrict__ A_log,
                    char* __restrict__ ws, __nv_bfloat16* __restrict__ y) {
@@ -250,7 +253,7 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       if (bpart < 2) {
 #pragma unroll
         for (int n = 0; n < 8; ++n)
-          *reinterpret_cast<__nv_bfloat16*>(sm + SM_BTT + sw128(8 * bpart + n, bt >> 3) + (bt & 7) * 2) = __float2bfloat16_rn(v[n]);
+          *reinterpret_cast<__nv_bfloat16*>(sm + sm_btt<YPASS>() + sw128(8 * bpart + n, bt >> 3) + (bt & 7) * 2) = __float2bfloat16_rn(v[n]);
       }
       fence_async_smem();
     }
@@ -276,27 +279,27 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     float cs_r, cs_t;
     {
       constexpr int R = HCK / 2 - 1;
-      float fv[HCK];
-      float up = 0.f, dn = 0.f;
+      float up = 0.f, dn = 0.f, fv[8];
+      auto piece = [&](int q) {
+        *reinterpret_cast<uint4*>(sm + SM_V + sw128(pc, (HCK * hf) / 8 + q)) =
+            make_uint4(pack_bf16(fv[0], fv[1]), pack_bf16(fv[2], fv[3]), pack_bf16(fv[4], fv[5]), pack_bf16(fv[6], fv[7]));
+      };
 #pragma unroll
       for (int t = R + 1; t < HCK; ++t) {
         const float d = dcol[t * MCH];
         up += d;
-        fv[t] = ex2_approx(-a2 * up) * d * __bfloat162float(xcol[t * MCH]);
+        fv[t & 7] = ex2_approx(-a2 * up) * d * __bfloat162float(xcol[t * MCH]);
+        if ((t & 7) == 7) piece(t >> 3);
       }
 #pragma unroll
       for (int t = R; t >= 0; --t) {
         const float d = dcol[t * MCH];
-        fv[t] = ex2_approx(a2 * dn) * d * __bfloat162float(xcol[t * MCH]);
+        fv[t & 7] = ex2_approx(a2 * dn) * d * __bfloat162float(xcol[t * MCH]);
         dn += d;
+        if ((t & 7) == 0) piece(t >> 3);
       }
       cs_r = dn;            // sum over tokens 0..r
       cs_t = dn + up;       // sum over the half
-#pragma unroll
-      for (int q = 0; q < HCK / 8; ++q)
-        *reinterpret_cast<uint4*>(sm + SM_V + sw128(pc, (HCK * hf) / 8 + q)) =
-            make_uint4(pack_bf16(fv[8 * q], fv[8 * q + 1]), pack_bf16(fv[8 * q + 2], fv[8 * q + 3]),
-                       pack_bf16(fv[8 * q + 4], fv[8 * q + 5]), pack_bf16(fv[8 * q + 6], fv[8 * q + 7]));
     }
     // a channel whose exponents pass the bound writes whatever it has (possibly infinities): its operand row only
     // reaches its own TMEM lane, which is ignored for this chunk
@@ -376,7 +379,7 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     }
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t V = sm_b + SM_V, GM = sm_b + SM_GM, CT = sm_b + SM_CT, SP = sm_b + SM_SP, BTT = sm_b + SM_BTT;
+      const uint32_t V = sm_b + SM_V, GM = sm_b + SM_GM, CT = sm_b + SM_CT, SP = sm_b + SM_SP, BTT = sm_b + sm_btt<YPASS>();
       if (YPASS) {
       // half 0:  V0 G00^T + S' C0^T
       umma_bf16(tm + TM_D, desc_at(V, 0, 0), desc_at(GM, 0, 0), idesc_n(32), 0u);
@@ -414,7 +417,7 @@ scalar_mm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
         }
 #pragma unroll
         for (int n = 0; n < NS; ++n) {
-          const uint4 bq = *reinterpret_cast<const uint4*>(sm + SM_BTT + sw128(n, t0s >> 3));
+          const uint4 bq = *reinterpret_cast<const uint4*>(sm + sm_btt<YPASS>() + sw128(n, t0s >> 3));
           const uint32_t bw[4] = {bq.x, bq.y, bq.z, bq.w};
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -568,20 +571,22 @@ int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_
   if (chunk_map(&mx, sp.x, pl, 2, true, MCH, false)) return 1;
   if (chunk_map(&md, sp.ws + pl.off_delta, pl, 4, false, MCH, false)) return 1;
   if (chunk_map(&my, y, pl, 2, true, MCH, false)) return 1;
-  auto kern = scalar_mm_kernel<true>;
+  constexpr bool YP = true;
+  auto kern = scalar_mm_kernel<YP>;
   static DeviceFlags done = {};
-  if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
-  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, my, pl, sp.A_log, sp.ws, (__nv_bfloat16*)y);
+  if (ensure_dynamic_smem(kern, smem_dyn<YP>(), done)) return 1;
+  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), smem_dyn<YP>(), st, mx, md, my, pl, sp.A_log, sp.ws, (__nv_bfloat16*)y);
 }
 
 int launch_forward_state_mm(const Plan& pl, const ScanPtrs& sp, cudaStream_t st) {
   CUtensorMap mx, md;
   if (chunk_map(&mx, sp.x, pl, 2, true, MCH, false)) return 1;
   if (chunk_map(&md, sp.ws + pl.off_delta, pl, 4, false, MCH, false)) return 1;
-  auto kern = scalar_mm_kernel<false>;
+  constexpr bool YP = false;
+  auto kern = scalar_mm_kernel<YP>;
   static DeviceFlags done = {};
-  if (ensure_dynamic_smem(kern, SMEM_DYN, done)) return 1;
-  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), SMEM_DYN, st, mx, md, mx, pl, sp.A_log, sp.ws,
+  if (ensure_dynamic_smem(kern, smem_dyn<YP>(), done)) return 1;
+  return launch_dependent(kern, dim3(pl.P / MCH, pl.S, pl.B), dim3(MT), smem_dyn<YP>(), st, mx, md, mx, pl, sp.A_log, sp.ws,
                           (__nv_bfloat16*)nullptr);
 }
 
