@@ -141,6 +141,12 @@ int as_ssm_forward(const as_shape_t *shape, const as_params_t *params, const voi
 int as_ssm_forward_ordered(const as_shape_t *shape, const as_params_t *params, const void *x, void *y,
                            void *ws, size_t ws_bytes, void *stream);
 
+/* One layer of a residual stack with fp32 I/O and d_model <= 128 (and one rate per state) in one call: y_out = y_in + SSM(x), where the SSM is
+ * as_ssm_forward_ordered, and yhat = norm(y_out) as as_residual_add_rmsnorm has it, or no norm where yhat is NULL; the same
+ * bits as those two calls.  y_out may alias y_in, yhat may alias x.  Other shapes: AS_ERR_LIMIT. */
+int as_ssm_forward_residual(const as_shape_t *shape, const as_params_t *params, const void *x, const void *y_in,
+                            void *y_out, void *yhat, float eps, void *ws, size_t ws_bytes, void *stream);
+
 /* Adjoint-method gradient of L = sum_t l^t(y^t) w.r.t. the layer parameters and x, given dy = dl^t/dy^t
  * (Proposition 2; with tbar < T the truncated form, Eq. 7 of Section 4.3; Algorithms 2-4 for one layer).
  * Token t contributes A-net and B-net vector-Jacobian products only for source tokens i in

@@ -145,16 +145,18 @@ ZeroList grad_regions(const Plan& pl, uint32_t flags, const as_grads_t* out, cha
 
 // The layer forward; `kind` (a forward kind of make_plan) alone decides which kernels run and how much scratch they need.
 int as::forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes,
-                void* stream, int kind) {
+                void* stream, int kind, const Residual* res) {
   int e = check_shape(shape);
   if (e) return e;
   e = check_params(params);
   if (e) return e;
-  if (!x || !y || !ws) return AS_ERR_NULL;
+  if (!x || !(res ? res->y_out : y) || !ws || (res && !res->y_in)) return AS_ERR_NULL;
   if (!aligned16(x) || !aligned16(y) || !aligned16(ws)) return AS_ERR_ALIGN;
+  if (res && (!aligned16(res->y_in) || !aligned16(res->y_out) || !aligned16(res->yhat))) return AS_ERR_ALIGN;
   Plan pl;
   e = make_plan(shape, shape->seqlen, 1, &pl, kind);
   if (e) return e;
+  if (res && !residual_applies(pl)) return AS_ERR_LIMIT;
   if (ws_bytes < pl.total_fwd) return AS_ERR_WORKSPACE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = reinterpret_cast<char*>(ws);
@@ -169,7 +171,7 @@ int as::forward(const as_shape_t* shape, const as_params_t* params, const void* 
   else AS_TRY(launch_prepass(pl, sp, false, st));
   AS_TRY(launch_fixup(pl, sp, false, st));
   if (mm) AS_TRY(launch_forward_y_mm(pl, sp, y, st));
-  else AS_TRY(launch_forward_y(pl, sp, y, st));
+  else AS_TRY(launch_forward_y(pl, sp, y, res, st));
   return AS_OK;
 }
 
@@ -245,6 +247,12 @@ int as_ssm_forward(const as_shape_t* shape, const as_params_t* params, const voi
 int as_ssm_forward_ordered(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws,
                            size_t ws_bytes, void* stream) {
   return forward(shape, params, x, y, ws, ws_bytes, stream, PLAN_FWD_ORDERED);
+}
+
+int as_ssm_forward_residual(const as_shape_t* shape, const as_params_t* params, const void* x, const void* y_in, void* y_out, void* yhat,
+                            float eps, void* ws, size_t ws_bytes, void* stream) {
+  const Residual res{y_in, y_out, yhat, eps};
+  return forward(shape, params, x, nullptr, ws, ws_bytes, stream, PLAN_FWD_ORDERED, &res);
 }
 
 int as_adjoint_grad(const as_shape_t* shape, const as_params_t* params, const void* x, const void* dy, int64_t tbar,

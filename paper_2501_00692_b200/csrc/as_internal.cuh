@@ -221,7 +221,10 @@ struct ScanPtrs {
 };
 int launch_prepass(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st);
 int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t st);
-int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st);
+// res: a layer of a residual stack of one channel tile, y_out = y_in + y and yhat = norm(y_out) in place of y (yhat may be null)
+struct Residual { const void* y_in; void* y_out; void* yhat; float eps; };
+bool residual_applies(const Plan& pl);
+int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, const Residual* res, cudaStream_t st);
 // matmul form of the y pass (as_scan_mm.cu): scalar structure with bf16 I/O and d_model % 128 == 0
 bool forward_y_mm_applies(const Plan& pl);
 int launch_forward_y_mm(const Plan& pl, const ScanPtrs& sp, void* y, cudaStream_t st);
@@ -243,9 +246,9 @@ int split_gradients(const Plan& pl, const as_grads_t* out, char* ws, cudaStream_
 
 int launch_bptt(const Plan& pl, const ScanPtrs& sp, float* dA_log, float* db_delta, cudaStream_t st);
 
-// the layer forward behind as_ssm_forward, as_ssm_forward_ordered and as_ssm_forward_static; an AS_* code (as_api.cu)
+// the layer forward behind as_ssm_forward, as_ssm_forward_ordered, as_ssm_forward_residual and as_ssm_forward_static; an AS_* code (as_api.cu)
 int forward(const as_shape_t* shape, const as_params_t* params, const void* x, void* y, void* ws, size_t ws_bytes, void* stream,
-            int kind);
+            int kind, const Residual* res = nullptr);
 
 // device address of the library's built-in scratch array on the current device (as_noalloc.cu); AS_OK or an error code
 int static_scratch_address(void** out);

@@ -49,6 +49,11 @@ class Stack:
         outs = [*block.unbind(0), torch.empty_like(y0)] if self.K else []
         B.as_rmsnorm_fwd(self.shape, y0, self.yhat, self.eps)
         for k, th in enumerate(self.thetas):
+            if self.shape.d_model <= 128 and self.shape.io == B.AS_F32:   # the layer's last kernel holds whole rows: it ends in the sum and the norm
+                B.as_ssm_forward_residual(self.shape, th, self.yhat, self.ys[-1], outs[k], self.yhat if k + 1 < self.K else None, self.ws,
+                                          self.eps)
+                self.ys.append(outs[k])
+                continue
             B.as_ssm_forward_ordered(self.shape, th, self.yhat, self.ytilde, self.ws)
             yk = outs[k]
             if k + 1 < self.K:   # the next layer's input is the norm of the sum: both in one pass

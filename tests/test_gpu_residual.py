@@ -1,0 +1,48 @@
+"""A layer of a residual stack in one call against its parts, bit for bit, at ragged lengths and widths, in place and without the norm
+(needs a B200)."""
+import pytest
+import torch
+
+from paper_2501_00692_b200 import binding as B
+from paper_2501_00692_b200 import synth
+from paper_2501_00692_b200.build import build_library
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("T,P", [(1, 8), (7, 128), (8, 64), (129, 72), (600, 120), (5000, 96)])
+def test_one_call_and_its_parts(T, P):
+    build_library()
+    w = synth.custom_workload("residual", 59, 2, T, P, io="f32")
+    theta = synth.layer_params(w, 0, DEV)
+    x, acc = synth.activations(w, DEV)
+    sh = B.shape_of(x)
+    ws = B.alloc_workspace(B.as_workspace_bytes(sh, T)[0], DEV)
+    tilde, total, norm = (torch.empty_like(x) for _ in range(3))
+    B.as_ssm_forward_ordered(sh, theta, x, tilde, ws)
+    B.as_residual_add_rmsnorm(sh, acc, tilde, total, norm)
+    out, yhat = torch.empty_like(x), torch.empty_like(x)
+    B.as_ssm_forward_residual(sh, theta, x, acc, out, yhat, ws)
+    assert B.as_check_status(ws) == B.AS_OK
+    assert torch.equal(out, total) and torch.equal(yhat, norm)
+    out.zero_()
+    B.as_ssm_forward_residual(sh, theta, x, acc, out, None, ws)
+    assert torch.equal(out, total)
+    B.as_ssm_forward_residual(sh, theta, x, acc, acc, x, ws)   # the sum over y_in, the norm over the layer's input
+    assert torch.equal(acc, total) and torch.equal(x, norm)
+
+
+@pytest.mark.parametrize("P,scalar,io", [(136, False, "f32"), (64, True, "f32"), (64, False, "bf16")])
+def test_other_shapes_are_refused(P, scalar, io):
+    build_library()
+    w = synth.custom_workload("residual", 59, 1, 40, P, io=io)
+    theta = synth.layer_params(w, 0, DEV)
+    if scalar:
+        theta["A_log"] = theta["A_log"][:, 0].contiguous()
+    x, acc = synth.activations(w, DEV)
+    sh = B.shape_of(x, 16, a_scalar=scalar)
+    ws = B.alloc_workspace(B.as_workspace_bytes(sh, 40)[0], DEV)
+    with pytest.raises(B.AsError) as e:
+        B.as_ssm_forward_residual(sh, theta, x, acc, torch.empty_like(x), None, ws)
+    assert e.value.code == B.AS_ERR_LIMIT
