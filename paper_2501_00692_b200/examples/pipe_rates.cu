@@ -2,8 +2,8 @@
 // dependent LDS chain, alone and in the mixes the scan kernels use, at 128..1024 threads per SM (one CTA per SM).
 // The benchmark's ALU roofline takes its MUFU and FP32 rates from this program's output.
 // A second table mixes two instruction kinds with independent operands and prints the cycles one scheduler spends per
-// warp on a group of them: it shows which pipes overlap (FP32 with MUFU, shared-memory loads, shuffles) and which share
-// the dispatch path (FP32 with the integer/logic pipe: LOP3 and IMAD each cost two cycles that FFMA cannot hide).
+// warp on a group of them, a third what one instruction of a kind adds to a stream of packed FMAs, and a fourth what a packed FMA costs by
+// the registers it reads.  Packed values are float2 throughout: as 64-bit integers the loops move both halves of each on every trip.
 //   nvcc -gencode arch=compute_100a,code=sm_100a -O3 -o pipe_rates pipe_rates.cu && ./pipe_rates
 #include <cstdio>
 #include <cuda_runtime.h>
@@ -12,31 +12,30 @@
 template <int MODE>
 __global__ void k(float* out, long long* cyc, float a, float b) {
   float x[8];
-  unsigned long long p[8];
+  float2 p[8];
   __shared__ float sm[4096];
-  for (int i = 0; i < 8; ++i) { x[i] = threadIdx.x * 0.001f + i; p[i] = (unsigned long long)__float_as_uint(x[i]) | ((unsigned long long)__float_as_uint(x[i]+1.f) << 32); }
+  for (int i = 0; i < 8; ++i) { x[i] = threadIdx.x * 0.001f + i; p[i] = make_float2(x[i], x[i] + 1.f); }
   for (int i = threadIdx.x; i < 4096; i += blockDim.x) sm[i] = i;
-  unsigned long long aa = (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(a) << 32);
-  unsigned long long bb = (unsigned long long)__float_as_uint(b) | ((unsigned long long)__float_as_uint(b) << 32);
+  const float2 aa = make_float2(a, a), bb = make_float2(b, b);
   __syncthreads();
   long long t0 = clock64();
   for (int it = 0; it < ITERS; ++it) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       if (MODE == 0) x[i] = fmaf(x[i], a, b);
-      if (MODE == 1) asm volatile("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(p[i]) : "l"(aa), "l"(bb));
+      if (MODE == 1) p[i] = __ffma2_rn(p[i], aa, bb);
       if (MODE == 2) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[i]));
       if (MODE == 3) x[i] = __shfl_xor_sync(0xffffffffu, x[i], 1 + (i & 15));
       if (MODE == 4) { x[i] = fmaf(x[i], a, b); if ((i & 7) == 0) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[i])); }
       if (MODE == 5) x[i] = sm[(threadIdx.x + (int)x[i]) & 4095];
-      if (MODE == 6) { asm volatile("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(p[i]) : "l"(aa), "l"(bb)); if ((i & 3) == 0) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[i])); }
-      if (MODE == 7) { asm volatile("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(p[i]) : "l"(aa), "l"(bb)); if ((i & 3) == 0) x[i] = __shfl_xor_sync(0xffffffffu, x[i], 1); }
+      if (MODE == 6) { p[i] = __ffma2_rn(p[i], aa, bb); if ((i & 3) == 0) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[i])); }
+      if (MODE == 7) { p[i] = __ffma2_rn(p[i], aa, bb); if ((i & 3) == 0) x[i] = __shfl_xor_sync(0xffffffffu, x[i], 1); }
       if (MODE == 8) { x[i] = fmaf(x[i], a, b); if ((i & 3) == 0) x[(i+1)&7] = __shfl_xor_sync(0xffffffffu, x[(i+1)&7], 1); }
       if (MODE == 9) { x[i] = fmaf(x[i], a, b); if ((i & 3) == 0) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[(i+1)&7])); }
     }
   }
   long long t1 = clock64();
-  float s = 0; for (int i = 0; i < 8; ++i) s += x[i] + (float)(p[i] & 0xff);
+  float s = 0; for (int i = 0; i < 8; ++i) s += x[i] + p[i].x + p[i].y;
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
   if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
 }
@@ -51,35 +50,41 @@ template <int MODE> void run(const char* name, double ops_per_iter_per_thread, i
 }
 
 // ---- mixes: NA operations of kind KA interleaved with NB of kind KB, all on independent registers ----
-// kinds: 0 FFMA, 1 FFMA2, 2 LOP3, 3 EX2, 5 SHFL, 6 IMAD
-template <int K> __device__ __forceinline__ void op(float& x, unsigned long long& p, int& q, float& e, float a, float b,
-                                                    unsigned long long aa, unsigned long long bb, int ia) {
+// kinds: 0 FFMA, 1 FFMA2, 2 LOP3, 3 EX2, 5 SHFL, 6 IMAD, 7 SEL, 8 FMNMX, 9 PRMT, 10 IADD, 11 FADD, 12 FMUL2
+template <int K> __device__ __forceinline__ void op(float& x, float2& p, int& q, float& e, float a, float b, float2 aa, float2 bb, int ia,
+                                                    bool c) {
   if (K == 0) x = fmaf(x, a, b);
-  if (K == 1) asm volatile("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(p) : "l"(aa), "l"(bb));
+  if (K == 1) p = __ffma2_rn(p, aa, bb);
   if (K == 2) asm volatile("lop3.b32 %0, %0, %1, %2, 0x96;" : "+r"(q) : "r"(ia), "r"(ia));
   if (K == 3) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(e));
   if (K == 5) e = __shfl_xor_sync(0xffffffffu, e, 1);
   if (K == 6) asm volatile("mad.lo.s32 %0, %0, %1, %2;" : "+r"(q) : "r"(ia), "r"(ia));
+  if (K == 7) { q = c ? q : ia; asm volatile("" : "+r"(q)); }
+  if (K == 8) asm volatile("max.f32 %0, %0, %1;" : "+f"(x) : "f"(a));
+  if (K == 9) asm volatile("prmt.b32 %0, %0, %1, 0x5410;" : "+r"(q) : "r"(ia));
+  if (K == 10) asm volatile("add.s32 %0, %0, %1;" : "+r"(q) : "r"(ia));
+  if (K == 11) asm volatile("add.f32 %0, %0, %1;" : "+f"(x) : "f"(a));
+  if (K == 12) p = __fmul2_rn(p, aa);
 }
 template <int KA, int NA, int KB, int NB>
-__global__ void mixk(float* out, long long* cyc, float a, float b, int ia) {
-  float x[16]; unsigned long long p[16]; int q[16]; float e[16];
+__global__ void __launch_bounds__(1024) mixk(float* out, long long* cyc, float a, float b, int ia) {
+  float x[16]; float2 p[16]; int q[16]; float e[16];
+  const bool c = (threadIdx.x * ia) & 4;
   for (int i = 0; i < 16; ++i) { x[i] = threadIdx.x * 0.001f + i; q[i] = threadIdx.x + i; e[i] = -0.001f * threadIdx.x - i;
-    p[i] = (unsigned long long)__float_as_uint(x[i]) | ((unsigned long long)__float_as_uint(x[i] + 1.f) << 32); }
-  unsigned long long aa = (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(a) << 32);
-  unsigned long long bb = (unsigned long long)__float_as_uint(b) | ((unsigned long long)__float_as_uint(b) << 32);
+    p[i] = make_float2(x[i], x[i] + 1.f); }
+  const float2 aa = make_float2(a, a), bb = make_float2(b, b);
   __syncthreads();
   long long t0 = clock64();
   for (int it = 0; it < ITERS; ++it) {
     constexpr int N = NA > NB ? NA : NB;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      if (i < NA) op<KA>(x[i & 15], p[i & 15], q[i & 15], e[i & 15], a, b, aa, bb, ia);
-      if (i < NB) op<KB>(x[(i + 8) & 15], p[(i + 8) & 15], q[(i + 8) & 15], e[(i + 8) & 15], a, b, aa, bb, ia);
+      if (i < NA) op<KA>(x[i & 15], p[i & 15], q[i & 15], e[i & 15], a, b, aa, bb, ia, c);
+      if (i < NB) op<KB>(x[(i + 8) & 15], p[(i + 8) & 15], q[(i + 8) & 15], e[(i + 8) & 15], a, b, aa, bb, ia, c);
     }
   }
   long long t1 = clock64();
-  float s = 0; for (int i = 0; i < 16; ++i) s += x[i] + (float)(p[i] & 0xff) + q[i] + e[i];
+  float s = 0; for (int i = 0; i < 16; ++i) s += x[i] + p[i].x + p[i].y + q[i] + e[i];
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
   if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
 }
@@ -90,6 +95,67 @@ template <int KA, int NA, int KB, int NB> void runmix(const char* name, int thre
   double c = 0; for (int i = 0; i < 148; ++i) c += h[i]; c /= 148;
   printf("%-28s threads/SM %4d: %6.2f cycles per warp and group on one scheduler\n", name, threads, c / ITERS / (threads / 128.0));
   cudaFree(out); cudaFree(cyc);
+}
+// ---- 64 operations of kind K spread over 128 packed FMAs: what one adds ----
+template <int K, int NK>
+__global__ void addk(float* out, long long* cyc, float a, float b, int ia) {
+  float x[16]; float2 p[16], p2[8]; int q[16]; float e[16];
+  const bool c = (threadIdx.x * ia) & 4;
+  for (int i = 0; i < 16; ++i) { x[i] = threadIdx.x * 0.001f + i; q[i] = threadIdx.x + i; e[i] = -0.001f * threadIdx.x - i;
+    p[i] = make_float2(x[i], x[i] + 1.f); p2[i & 7] = p[i]; }
+  const float2 aa = make_float2(a, a), bb = make_float2(b, b);
+  __syncthreads();
+  long long t0 = clock64();
+#pragma unroll 1
+  for (int it = 0; it < ITERS; ++it) {
+#pragma unroll
+    for (int i = 0; i < 128; ++i) {
+      p[i & 15] = __ffma2_rn(p[i & 15], aa, bb);
+      if ((i & 1) && (i >> 1) < NK) op<K>(x[(i >> 1) & 15], p2[(i >> 1) & 7], q[(i >> 1) & 15], e[(i >> 1) & 15], a, b, aa, bb, ia, c);
+    }
+  }
+  long long t1 = clock64();
+  float s = 0; for (int i = 0; i < 16; ++i) s += x[i] + p[i].x + p[i].y + p2[i & 7].x + q[i] + e[i];
+  out[blockIdx.x * blockDim.x + threadIdx.x] = s;
+  if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
+}
+// ---- 128 packed operations by what they read ----
+// W: an FMA of 0 one pair of its own, 1 two, 2 three, 4 two and a single register for both halves; 3 a product of two
+template <int W>
+__global__ void readk(float* out, long long* cyc, float a, float b, int ia) {
+  float2 p[8], u[8], v[8];
+  for (int i = 0; i < 8; ++i) { p[i] = make_float2(threadIdx.x, i); u[i] = make_float2(a * i + threadIdx.x, b); v[i] = make_float2(b * i + ia, a * threadIdx.x); }
+  __syncthreads();
+  long long t0 = clock64();
+#pragma unroll 1
+  for (int it = 0; it < ITERS; ++it) {
+#pragma unroll
+    for (int i = 0; i < 128; ++i) {
+      const int j = i & 7, r = (i >> 3) & 7;
+      if (W == 0) p[j] = __ffma2_rn(p[j], u[0], v[0]);
+      if (W == 1) p[j] = __ffma2_rn(u[j], v[0], p[j]);
+      if (W == 2) p[j] = __ffma2_rn(u[j], v[(j + r) & 7], p[j]);
+      if (W == 3) p[j] = __fmul2_rn(p[j], u[j]);
+      if (W == 4) p[j] = __ffma2_rn(u[j], make_float2(v[r].x, v[r].x), p[j]);
+    }
+  }
+  long long t1 = clock64();
+  float s = 0; for (int i = 0; i < 8; ++i) s += p[i].x + p[i].y;
+  out[blockIdx.x * blockDim.x + threadIdx.x] = s;
+  if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
+}
+typedef void (*Kern)(float*, long long*, float, float, int);
+double cycles(Kern kern, int threads) {   // of a scheduler, per warp and group
+  float* out; long long* cyc; cudaMalloc(&out, 148 * 1024 * 4); cudaMalloc(&cyc, 148 * 8);
+  for (int r = 0; r < 2; ++r) { kern<<<148, threads>>>(out, cyc, 0.999f, 0.001f, 12345); cudaDeviceSynchronize(); }
+  long long h[148]; cudaMemcpy(h, cyc, sizeof(h), cudaMemcpyDeviceToHost);
+  double c = 0; for (int i = 0; i < 148; ++i) c += h[i];
+  cudaFree(out); cudaFree(cyc);
+  return c / 148 / ITERS / (threads / 128.0);
+}
+template <int K> void runadd(const char* name) {
+  const double base = cycles(addk<K, 0>, 384), with = cycles(addk<K, 64>, 384);
+  printf("%-28s adds %5.2f cycles beside packed FMAs (128 of them: %.0f)\n", name, (with - base) / 64, base);
 }
 int main() {
   for (int th : {128, 256, 512, 1024}) {
@@ -120,5 +186,10 @@ int main() {
     runmix<1, 16, 6, 16>("16 FFMA2 + 16 IMAD", th);
     runmix<1, 16, 0, 16>("16 FFMA2 + 16 FFMA", th);
   }
+  runadd<7>("SEL"); runadd<8>("FMNMX"); runadd<5>("SHFL"); runadd<10>("IADD"); runadd<3>("EX2"); runadd<11>("FADD"); runadd<0>("FFMA");
+  runadd<9>("PRMT"); runadd<6>("IMAD"); runadd<12>("FMUL2"); runadd<2>("LOP3");
+  printf("packed FMA of one pair of its own %.2f cycles, two %.2f, three %.2f, two and a register %.2f; packed product %.2f\n",
+         cycles(readk<0>, 384) / 128, cycles(readk<1>, 384) / 128, cycles(readk<2>, 384) / 128, cycles(readk<4>, 384) / 128,
+         cycles(readk<3>, 384) / 128);
   return 0;
 }
