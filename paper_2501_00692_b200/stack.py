@@ -11,12 +11,22 @@ Two gradient modes:
 """
 from __future__ import annotations
 
+from operator import is_
+
 import torch
 
 from . import binding as B
 
 
+WEIGHTS = ("W_delta", "W_B", "W_C")   # what a packed copy is made of
+
+
 class Stack:
+    """The parameters stay the caller's tensors and may be updated in place between two calls.  The copies of them that this object
+    keeps, packed weights (bf16) and, for the batched "paper" gradients, all parameters stacked, are made again by the next call
+    after a write that PyTorch counts; after any other (through `.data`, by a kernel of one's own, by replaying a graph that does not hold
+    the stack's calls) call parameters_changed()."""
+
     def __init__(self, thetas, batch, seqlen, d_model, d_state=16, dtype=torch.float32, device="cuda:0", tbar=None,
                  eps=1e-6):
         self.thetas = [dict(t) for t in thetas]   # own dicts: a packed copy of the weights is added below
@@ -31,17 +41,51 @@ class Stack:
         self.ys = None       # y_0 .. y_K
         self.yhat = torch.empty(batch, seqlen, d_model, dtype=dtype, device=device)
         self.ytilde = torch.empty_like(self.yhat)
-        # the bf16 tensor-core contractions read [W_delta; W_B; W_C] as one matrix: packed once here, per layer
-        if io == B.AS_BF16:
-            for th in self.thetas:
-                if th.get("Wcat") is None:
-                    th["Wcat"] = torch.empty(B.as_wcat_bytes(self.shape), dtype=torch.uint8, device=device)
-                    B.as_pack_weights(self.shape, 1, th, th["Wcat"])
+        # the bf16 tensor-core contractions read [W_delta; W_B; W_C] as one matrix: packed per layer, but for the layers whose
+        # packed copy is the caller's
+        self._own = [th for th in self.thetas if th.get("Wcat") is None] if io == B.AS_BF16 else []
+        for th in self._own:
+            th["Wcat"] = torch.empty(B.as_wcat_bytes(self.shape), dtype=torch.uint8, device=device)
         self._stacked = None   # parameters with a leading [K] dimension, built on first use of the batched call
         self._ws_layers = None
+        self._captured = False
+        self.parameters_changed()
+        self._pack()
+
+    def parameters_changed(self):
+        """The copies of the parameters are made again before their next use."""
+        self._packed_of = self._stacked_of = None
+
+    def _contents(self, thetas, keys):
+        """The parameters `keys` and how often each has been written; None where that cannot be told: inference tensors do not count
+        writes, and a graph's replays write without a count, to the stack's parameters or before its captured calls."""
+        self._captured = self._captured or torch.cuda.is_current_stream_capturing()
+        if self._captured:
+            return None
+        ts = [th[k] for th in thetas for k in keys]
+        try:
+            return ts, [t._version for t in ts]
+        except RuntimeError:
+            return None
+
+    @staticmethod
+    def _same(a, b):
+        return a is not None and b is not None and a[1] == b[1] and all(map(is_, a[0], b[0]))
+
+    def _pack(self):
+        """Brings the packed weights in line with the parameters."""
+        if not self._own:
+            return
+        now = self._contents(self._own, WEIGHTS)
+        if self._same(now, self._packed_of):
+            return
+        for th in self._own:
+            B.as_pack_weights(self.shape, 1, th, th["Wcat"])
+        self._packed_of = now
 
     def forward(self, y0: torch.Tensor):
         """Runs the stack, keeping y_0..y_K (the per-layer inputs are re-normalised in the backward)."""
+        self._pack()
         self.ys = [y0]
         # y_1 .. y_{K-1} in one block (one allocation, and the paper mode normalises them in one launch); y_K, which the
         # caller may keep, on its own
@@ -71,6 +115,7 @@ class Stack:
         dev = g.device
         if mode == "paper" and batched:
             return self._paper_grad_batched(g, record), None
+        self._pack()
         grads = [None] * self.K
         G = g.clone() if mode == "chained" else g
         for k in range(self.K - 1, -1, -1):
@@ -89,12 +134,22 @@ class Stack:
         """Proposition 3: all K layers in one as_adjoint_grad_layers call (stacked parameters, stacked layer inputs,
         the one upstream gradient shared)."""
         K, sh = self.K, self.shape
+        keys = ("W_delta", "b_delta", "W_B", "W_C", "A_log")
         if self._stacked is None:
-            keys = ["W_delta", "b_delta", "W_B", "W_C", "A_log"] + (["Wcat"] if self.thetas[0].get("Wcat") is not None else [])
-            self._stacked = {k: torch.stack([th[k] for th in self.thetas]).contiguous() for k in keys}
+            self._stacked = {k: torch.empty(K, *self.thetas[0][k].shape, dtype=self.thetas[0][k].dtype, device=self.device) for k in keys}
+            if sh.io == B.AS_BF16:
+                self._stacked["Wcat"] = torch.empty(B.as_wcat_bytes(sh, K), dtype=torch.uint8, device=self.device)
             self._ws_layers = B.alloc_workspace(B.as_workspace_bytes_layers(sh, K, self.tbar), self.device)
             self._xall = torch.empty(K, sh.batch, sh.seqlen, sh.d_model, dtype=self.yhat.dtype, device=self.device)
             self._x = self._xall.unbind(0)
+        now = self._contents(self.thetas, keys)
+        if not self._same(now, self._stacked_of):
+            with torch.no_grad():
+                for k in keys:
+                    torch.stack([th[k] for th in self.thetas], out=self._stacked[k])
+            if sh.io == B.AS_BF16:
+                B.as_pack_weights(sh, K, self._stacked, self._stacked["Wcat"])
+            self._stacked_of = now
         # norms row by row: layers whose inputs lie one behind the other (as forward() leaves y_1 .. y_{K-1}) take one launch
         step = self._x[0].numel() * self._x[0].element_size()
         at = [y.data_ptr() for y in self.ys[:K]]
