@@ -85,20 +85,6 @@ inline int sm_count() {
   return n;
 }
 
-// Dynamic shared memory with which no SM takes more than its even share of a launch that does not fill the chip (`least` CTAs, if the
-// share is smaller).  The CTAs of a dependent launch come in while the kernel before drains and crowd on the SMs that are free
-// first, four to one beside two to another, and a scan kernel is as slow as its fullest SM.  us, without | with: gradients of
-// 3,000 x 512 90.3 | 87.0, 10,506 x 128 85.3 | 80.6, 6,000 x 1,024 197 | 188, 1,500 x 640 scalar 57.7 | 54.9; forwards of 3 x 1,177 x 256
-// 30.8 | 28.2, 4 x 970 x 128 fp32 28.4 | 25.6, 571 x 512 fp32 34.1 | 31.6; step of 5 layers of 799 x 704 494 | 469.  least: 1 in the forward's
-// kernels (2: 485 in the last), 2 in the gradient's (1: 4 x 218 x 64 fp32 29.0, 26.7 with 2 and without).
-constexpr int SM_SMEM = 228 * 1024, CTA_SMEM = 1024;   // of an SM; what the system takes of it for a CTA
-constexpr int SPREAD_SMEM = SM_SMEM / 2 - CTA_SMEM + 128;   // the most that spread_smem adds up to
-inline int spread_smem(int bytes, int64_t ctas, int least) {
-  const int64_t share = (ctas + sm_count() - 1) / sm_count(), per = share > least ? share : least;
-  const int64_t need = SM_SMEM / (per + 1) / 128 * 128 - CTA_SMEM + 128;   // one CTA more than `per` does not fit
-  return need > bytes ? (int)need : bytes;
-}
-
 constexpr int NS = 16;        // d_state handled by the scan kernels
 constexpr int CK = 8;         // tokens per checkpoint chunk (h of one chunk lives in registers)
 constexpr int NCH = 2;        // channels per thread of the scan kernels
