@@ -114,7 +114,7 @@ int as_version(void);
 /* Static description of a status code. */
 const char *as_strerror(int code);
 
-/* Scratch sizes in bytes for a shape: *fwd_bytes for as_ssm_forward and as_ssm_forward_ordered, *grad_bytes for as_adjoint_grad
+/* Scratch sizes in bytes for a shape: *fwd_bytes for as_ssm_forward, as_ssm_forward_ordered and as_ssm_forward_residual, *grad_bytes for as_adjoint_grad
  * and as_full_bptt_grad (the larger of the two; never less than *fwd_bytes).  Either output pointer may be NULL.  `tbar` as for
  * as_adjoint_grad.  Long sequences need some 4 bytes per token and channel for a forward and 19 (bf16) or 26 (fp32) for a
  * gradient; large fp32 products also keep their operands split for the tensor cores, 6 bytes more in a forward and 12 in a
@@ -143,9 +143,12 @@ int as_ssm_forward_ordered(const as_shape_t *shape, const as_params_t *params, c
 
 /* One layer of a residual stack with fp32 I/O and d_model <= 128 (and one rate per state) in one call: y_out = y_in + SSM(x), where the SSM is
  * as_ssm_forward_ordered, and yhat = norm(y_out) as as_residual_add_rmsnorm has it, or no norm where yhat is NULL; the same
- * bits as those two calls.  y_out may alias y_in, yhat may alias x.  Other shapes: AS_ERR_LIMIT. */
+ * bits as those two calls.  y_out may alias y_in, yhat may alias x.  Scratch: fwd_bytes of as_workspace_bytes.  Other shapes: AS_ERR_LIMIT. */
 int as_ssm_forward_residual(const as_shape_t *shape, const as_params_t *params, const void *x, const void *y_in,
                             void *y_out, void *yhat, float eps, void *ws, size_t ws_bytes, void *stream);
+
+/* 1 where as_ssm_forward_residual takes the shape and is no slower than the two calls (not the case for long runs at d_model <= 64), else 0. */
+int as_ssm_forward_residual_applies(const as_shape_t *shape);
 
 /* Adjoint-method gradient of L = sum_t l^t(y^t) w.r.t. the layer parameters and x, given dy = dl^t/dy^t
  * (Proposition 2; with tbar < T the truncated form, Eq. 7 of Section 4.3; Algorithms 2-4 for one layer).

@@ -25,7 +25,8 @@ AS_ERR_WORKSPACE, AS_ERR_ALIGN, AS_ERR_CUDA, AS_ERR_TIMEOUT, AS_ERR_LIMIT = -5, 
 EXPORTS = ("as_version", "as_strerror", "as_workspace_bytes", "as_check_status", "as_ssm_forward",
            "as_adjoint_grad", "as_full_bptt_grad", "as_rmsnorm_fwd", "as_residual_add", "as_rmsnorm_bwd_add",
            "as_launch_count", "as_set_timing", "as_get_timing", "as_ssm_forward_static", "as_wait_selftest", "as_sm_count",
-           "as_residual_add_rmsnorm", "as_ssm_forward_ordered", "as_adjoint_grad_layers", "as_workspace_bytes_layers", "as_wcat_bytes", "as_pack_weights", "as_ssm_forward_residual")
+           "as_residual_add_rmsnorm", "as_ssm_forward_ordered", "as_adjoint_grad_layers", "as_workspace_bytes_layers", "as_wcat_bytes", "as_pack_weights", "as_ssm_forward_residual",
+           "as_ssm_forward_residual_applies")
 AS_STATIC_SCRATCH_BYTES = 32 << 20
 AS_NUM_PHASES = 6
 PHASES = ("projections", "prepass", "fixup", "adjoint_main", "weight_grads", "input_grad")
@@ -73,6 +74,7 @@ def lib() -> C.CDLL:
         L.as_ssm_forward_ordered.argtypes = L.as_ssm_forward.argtypes
         L.as_ssm_forward_residual.argtypes = [C.POINTER(as_shape_t), C.POINTER(as_params_t), C.c_void_p, C.c_void_p, C.c_void_p,
                                               C.c_void_p, C.c_float, C.c_void_p, C.c_size_t, C.c_void_p]
+        L.as_ssm_forward_residual_applies.argtypes = [C.POINTER(as_shape_t)]
         L.as_adjoint_grad.argtypes = [C.POINTER(as_shape_t), C.POINTER(as_params_t), C.c_void_p, C.c_void_p,
                                       C.c_int64, C.c_uint32, C.POINTER(as_grads_t), C.c_void_p, C.c_size_t, C.c_void_p]
         L.as_full_bptt_grad.argtypes = [C.POINTER(as_shape_t), C.POINTER(as_params_t), C.c_void_p, C.c_void_p,
@@ -202,6 +204,11 @@ def as_ssm_forward_residual(shape, theta, x, y_in, y_out, yhat, ws, eps=1e-6, st
     p = make_params(theta)
     _check(lib().as_ssm_forward_residual(C.byref(shape), C.byref(p), _ptr(x), _ptr(y_in), _ptr(y_out), _ptr(yhat), float(eps), _ptr(ws),
                                          ws.numel(), _stream(stream)), "as_ssm_forward_residual")
+
+
+def as_ssm_forward_residual_applies(shape) -> bool:
+    """Whether a layer of this shape is to be one as_ssm_forward_residual call, or as_ssm_forward_ordered and as_residual_add_rmsnorm."""
+    return bool(lib().as_ssm_forward_residual_applies(C.byref(shape)))
 
 
 def as_adjoint_grad(shape, theta, x, dy, tbar, grads, ws, flags=0, stream=None):

@@ -249,6 +249,11 @@ int as_ssm_forward_ordered(const as_shape_t* shape, const as_params_t* params, c
   return forward(shape, params, x, y, ws, ws_bytes, stream, PLAN_FWD_ORDERED);
 }
 
+int as_ssm_forward_residual_applies(const as_shape_t* shape) {
+  Plan pl;
+  return check_shape(shape) == AS_OK && make_plan(shape, shape->seqlen, 1, &pl, PLAN_FWD_ORDERED) == AS_OK && residual_pays(pl) ? 1 : 0;
+}
+
 int as_ssm_forward_residual(const as_shape_t* shape, const as_params_t* params, const void* x, const void* y_in, void* y_out, void* yhat,
                             float eps, void* ws, size_t ws_bytes, void* stream) {
   const Residual res{y_in, y_out, yhat, eps};

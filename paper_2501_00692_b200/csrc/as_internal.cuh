@@ -210,6 +210,7 @@ int launch_fixup(const Plan& pl, const ScanPtrs& sp, bool with_mu, cudaStream_t 
 // res: a layer of a residual stack of one channel tile, y_out = y_in + y and yhat = norm(y_out) in place of y (yhat may be null)
 struct Residual { const void* y_in; void* y_out; void* yhat; float eps; };
 bool residual_applies(const Plan& pl);
+bool residual_pays(const Plan& pl);
 int launch_forward_y(const Plan& pl, const ScanPtrs& sp, void* y, const Residual* res, cudaStream_t st);
 // matmul form of the y pass (as_scan_mm.cu): scalar structure with bf16 I/O and d_model % 128 == 0
 bool forward_y_mm_applies(const Plan& pl);

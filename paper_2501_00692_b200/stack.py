@@ -40,7 +40,8 @@ class Stack:
         self.ws = B.alloc_workspace(gbytes, device)
         self.ys = None       # y_0 .. y_K
         self.yhat = torch.empty(batch, seqlen, d_model, dtype=dtype, device=device)
-        self.ytilde = torch.empty_like(self.yhat)
+        self._residual = B.as_ssm_forward_residual_applies(self.shape)   # a layer's last kernel ends in the sum and the norm
+        self.ytilde = None if self._residual else torch.empty_like(self.yhat)
         # the bf16 tensor-core contractions read [W_delta; W_B; W_C] as one matrix: packed per layer, but for the layers whose
         # packed copy is the caller's
         self._own = [th for th in self.thetas if th.get("Wcat") is None] if io == B.AS_BF16 else []
@@ -93,7 +94,7 @@ class Stack:
         outs = [*block.unbind(0), torch.empty_like(y0)] if self.K else []
         B.as_rmsnorm_fwd(self.shape, y0, self.yhat, self.eps)
         for k, th in enumerate(self.thetas):
-            if self.shape.d_model <= 128 and self.shape.io == B.AS_F32:   # the layer's last kernel holds whole rows: it ends in the sum and the norm
+            if self._residual:
                 B.as_ssm_forward_residual(self.shape, th, self.yhat, self.ys[-1], outs[k], self.yhat if k + 1 < self.K else None, self.ws,
                                           self.eps)
                 self.ys.append(outs[k])

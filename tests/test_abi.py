@@ -113,6 +113,15 @@ def test_forward_refuses_less_scratch_than_reported(L, shape):
     assert L.as_ssm_forward(C.byref(sh), C.byref(p), ok, ok, ok, fwd - 1, None) == B.AS_ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("shape,applies", [((1, 1, 8), 1), ((2, 4096, 64), 1), ((3, 2731, 64), 0), ((1, 65536, 32), 0), ((1, 65536, 72), 1),
+                                           ((4, 65536, 128), 1), ((1, 100, 136), 0), ((1, 100, 60), 0), ((0, 100, 64), 0)])
+def test_where_a_stack_takes_the_residual_call(L, shape, applies):
+    """Narrow fp32 layers, long runs at widths up to 64 apart, which two calls are faster for; bf16 and scalar rates never."""
+    assert B.as_ssm_forward_residual_applies(B.make_shape(*shape)) == applies
+    assert not B.as_ssm_forward_residual_applies(B.make_shape(*shape, io=B.AS_BF16))
+    assert not B.as_ssm_forward_residual_applies(B.make_shape(*shape, a_structure=B.AS_A_SCALAR))
+
+
 @pytest.mark.parametrize("P,split", [(8, False), (32, False), (56, False), (64, True), (88, True)])
 def test_narrow_fp32_gradients_keep_no_split_operands(P, split):
     """From 2^30 multiply-adds on fp32 gradients keep x and the cotangents as three bf16 terms, 12 bytes a value, but not below a width

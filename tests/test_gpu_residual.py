@@ -6,6 +6,7 @@ import torch
 from paper_2501_00692_b200 import binding as B
 from paper_2501_00692_b200 import synth
 from paper_2501_00692_b200.build import build_library
+from paper_2501_00692_b200.stack import Stack
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -31,6 +32,23 @@ def test_one_call_and_its_parts(T, P):
     assert torch.equal(out, total)
     B.as_ssm_forward_residual(sh, theta, x, acc, acc, x, ws)   # the sum over y_in, the norm over the layer's input
     assert torch.equal(acc, total) and torch.equal(x, norm)
+
+
+@pytest.mark.parametrize("T,P", [(8192, 64), (8193, 64), (9000, 72)])   # both sides of the line from which a stack makes two calls
+def test_stack_forward_by_either_form(T, P):
+    build_library()
+    w = synth.custom_workload("residual", 59, 1, T, P, layers=3, io="f32")
+    thetas = [synth.layer_params(w, k, DEV) for k in range(3)]
+    y0, _ = synth.activations(w, DEV)
+    st = Stack(thetas, 1, T, P, dtype=torch.float32, device=DEV)
+    assert st._residual == (T <= 8192 or P > 64)
+    got = st.forward(y0)
+    yhat, tilde, cur = torch.empty_like(y0), torch.empty_like(y0), y0.clone()
+    B.as_rmsnorm_fwd(st.shape, cur, yhat)
+    for th in thetas:
+        B.as_ssm_forward_ordered(st.shape, th, yhat, tilde, st.ws)
+        B.as_residual_add_rmsnorm(st.shape, cur, tilde, cur, yhat)
+    assert B.as_check_status(st.ws) == B.AS_OK and torch.equal(got, cur)
 
 
 @pytest.mark.parametrize("P,scalar,io", [(136, False, "f32"), (64, True, "f32"), (64, False, "bf16")])
