@@ -138,3 +138,21 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libadjoint_ssm.so")
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         B.lib()
+
+
+def test_residual_forward_argument_errors(L):
+    sh = B.make_shape(1, 300, 64)
+    fwd = B.as_workspace_bytes(sh, 300)[0]
+    ok, off = C.c_void_p(0x1000), C.c_void_p(0x1008)   # never dereferenced: the checks come first
+    p = B.as_params_t(ok, ok, ok, ok, ok)
+
+    def rc(x=ok, y_in=ok, y_out=ok, yhat=None, ws=ok, ws_bytes=fwd - 1, shape=sh):
+        return L.as_ssm_forward_residual(C.byref(shape), C.byref(p), x, y_in, y_out, yhat, 1e-6, ws, ws_bytes, None)
+
+    for one in ("x", "y_in", "y_out", "ws"):
+        assert rc(**{one: None}) == B.AS_ERR_NULL, one
+    for one in ("x", "y_in", "y_out", "yhat", "ws"):
+        assert rc(**{one: off}) == B.AS_ERR_ALIGN, one
+    assert rc() == rc(yhat=ok) == B.AS_ERR_WORKSPACE
+    for other in (B.make_shape(1, 300, 136), B.make_shape(1, 300, 64, io=B.AS_BF16), B.make_shape(1, 300, 64, a_structure=B.AS_A_SCALAR)):
+        assert rc(shape=other, ws_bytes=1 << 40) == B.AS_ERR_LIMIT

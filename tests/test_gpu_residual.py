@@ -64,3 +64,22 @@ def test_other_shapes_are_refused(P, scalar, io):
     with pytest.raises(B.AsError) as e:
         B.as_ssm_forward_residual(sh, theta, x, acc, torch.empty_like(x), None, ws)
     assert e.value.code == B.AS_ERR_LIMIT
+
+
+# two batch elements whose projections take the tensor cores (split operands are part of the scratch), in place too
+@pytest.mark.parametrize("T,P", [(4003, 128), (9603, 104)])
+def test_one_call_and_its_parts_with_split_projections(T, P):
+    assert B.as_workspace_bytes(B.make_shape(2, T, P), T)[0] > 14 * 2 * T * P
+    test_one_call_and_its_parts(T, P)
+
+
+def test_residual_call_clears_a_stale_status():
+    build_library()
+    w = synth.custom_workload("residual", 59, 1, 100, 64, io="f32")
+    theta = synth.layer_params(w, 0, DEV)
+    x, acc = synth.activations(w, DEV)
+    sh = B.shape_of(x)
+    ws = B.alloc_workspace(B.as_workspace_bytes(sh, 100)[0], DEV)
+    ws[:256] = 0xFF
+    B.as_ssm_forward_residual(sh, theta, x, acc, torch.empty_like(x), None, ws)
+    assert B.as_check_status(ws) == B.AS_OK
