@@ -2,13 +2,15 @@
 whose factors the segment pass forms on the FP32 pipe (needs a B200)."""
 import math
 
+import numpy as np
 import pytest
 import torch
 
+from oracle import ssm_oracle as O
 from paper_2501_00692_b200 import synth
 from paper_2501_00692_b200.build import build_library
 
-from gpu_util import TOL, assert_close, gpu_forward, oracle_adjoint
+from gpu_util import TOL, assert_close, gpu_forward, oracle_adjoint, theta_f64
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -54,3 +56,20 @@ def test_nothing_is_left_of_a_large_state(io):
     ref = oracle_adjoint(theta, x, torch.zeros_like(x), T)["y"][..., 0]
     assert abs(ref).max() < 1e-6
     assert abs(y - ref).max() < 1e-6, abs(y - ref).max()
+
+
+# 41,428 tokens of one channel tile: on 148 SMs segments of 96 (fp32) and 40 (bf16) tokens, more chunks than the staging ring holds, so the
+# two states go from chunk to chunk and from segment to segment through the polynomial factors; a ragged last chunk
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+@pytest.mark.parametrize("b_range", [(-9, -7), (-4, -2), (-1, 1)])
+def test_factors_of_two_states_over_many_chunks(b_range, io):
+    build_library()
+    w = synth.custom_workload("factors", 54, 4, 10357, 72, io=io)
+    theta = synth.layer_params(w, 0, DEV, b_delta_range=b_range)
+    for n in range(16):
+        if n not in (7, 15):
+            theta["W_B"][n].zero_()
+    x, _ = synth.activations(w, DEV)
+    y = synth.to_f64(gpu_forward(w, theta, x))
+    th = theta_f64(theta)
+    assert_close(y, np.stack([O.ssm_forward(th, one) for one in synth.to_f64(x)]), TOL[io], "y")
