@@ -6,11 +6,13 @@
 // the registers it reads.  Packed values are float2 throughout: as 64-bit integers the loops move both halves of each on every trip.
 //   nvcc -gencode arch=compute_100a,code=sm_100a -O3 -o pipe_rates pipe_rates.cu && ./pipe_rates
 #include <cstdio>
+#include <cstdlib>
+#include <vector>
 #include <cuda_runtime.h>
 #include <cstdint>
 #define ITERS 4096
 template <int MODE>
-__global__ void k(float* out, long long* cyc, float a, float b) {
+__global__ void __launch_bounds__(1024) k(float* out, long long* cyc, float a, float b, int) {
   float x[8];
   float2 p[8];
   __shared__ float sm[4096];
@@ -39,14 +41,33 @@ __global__ void k(float* out, long long* cyc, float a, float b) {
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
   if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
 }
+void check(cudaError_t e) {
+  if (e != cudaSuccess) { fprintf(stderr, "%s\n", cudaGetErrorString(e)); exit(1); }
+}
+typedef void (*Kern)(float*, long long*, float, float, int);
+double cycles(Kern kern, int threads) {   // of a CTA's run, mean over the SMs, second launch
+  int dev, sms;
+  check(cudaGetDevice(&dev));
+  check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  float* out; long long* cyc;
+  check(cudaMalloc(&out, sizeof(float) * sms * threads));
+  check(cudaMalloc(&cyc, sizeof(long long) * sms));
+  for (int r = 0; r < 2; ++r) {
+    kern<<<sms, threads>>>(out, cyc, 0.999f, 0.001f, 12345);
+    check(cudaGetLastError());
+    check(cudaDeviceSynchronize());
+  }
+  std::vector<long long> h(sms);
+  check(cudaMemcpy(h.data(), cyc, sizeof(long long) * sms, cudaMemcpyDeviceToHost));
+  check(cudaFree(out)); check(cudaFree(cyc));
+  double c = 0;
+  for (long long v : h) c += v;
+  return c / sms;
+}
+double per_group(Kern kern, int threads) { return cycles(kern, threads) / ITERS / (threads / 128.0); }   // of a scheduler, per warp and group
 template <int MODE> void run(const char* name, double ops_per_iter_per_thread, int threads) {
-  float* out; long long* cyc; cudaMalloc(&out, 148 * 1024 * 4); cudaMalloc(&cyc, 148 * 8);
-  k<MODE><<<148, threads>>>(out, cyc, 0.999f, 0.001f); cudaDeviceSynchronize();
-  k<MODE><<<148, threads>>>(out, cyc, 0.999f, 0.001f); cudaDeviceSynchronize();
-  long long h[148]; cudaMemcpy(h, cyc, sizeof(h), cudaMemcpyDeviceToHost);
-  double c = 0; for (int i = 0; i < 148; ++i) c += h[i]; c /= 148;
+  const double c = cycles(k<MODE>, threads);
   printf("%-28s threads/SM %4d: %7.2f lane-ops/clk/SM (%.0f cycles)\n", name, threads, ops_per_iter_per_thread * ITERS * threads / c, c);
-  cudaFree(out); cudaFree(cyc);
 }
 
 // ---- mixes: NA operations of kind KA interleaved with NB of kind KB, all on independent registers ----
@@ -89,12 +110,8 @@ __global__ void __launch_bounds__(1024) mixk(float* out, long long* cyc, float a
   if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
 }
 template <int KA, int NA, int KB, int NB> void runmix(const char* name, int threads) {
-  float* out; long long* cyc; cudaMalloc(&out, 148 * 1024 * 4); cudaMalloc(&cyc, 148 * 8);
-  for (int r = 0; r < 2; ++r) { mixk<KA, NA, KB, NB><<<148, threads>>>(out, cyc, 0.999f, 0.001f, 12345); cudaDeviceSynchronize(); }
-  long long h[148]; cudaMemcpy(h, cyc, sizeof(h), cudaMemcpyDeviceToHost);
-  double c = 0; for (int i = 0; i < 148; ++i) c += h[i]; c /= 148;
-  printf("%-28s threads/SM %4d: %6.2f cycles per warp and group on one scheduler\n", name, threads, c / ITERS / (threads / 128.0));
-  cudaFree(out); cudaFree(cyc);
+  printf("%-28s threads/SM %4d: %6.2f cycles per warp and group on one scheduler\n", name, threads,
+         per_group(mixk<KA, NA, KB, NB>, threads));
 }
 // ---- 64 operations of kind K spread over 128 packed FMAs: what one adds ----
 template <int K, int NK>
@@ -144,17 +161,8 @@ __global__ void readk(float* out, long long* cyc, float a, float b, int ia) {
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
   if (threadIdx.x == 0) cyc[blockIdx.x] = t1 - t0;
 }
-typedef void (*Kern)(float*, long long*, float, float, int);
-double cycles(Kern kern, int threads) {   // of a scheduler, per warp and group
-  float* out; long long* cyc; cudaMalloc(&out, 148 * 1024 * 4); cudaMalloc(&cyc, 148 * 8);
-  for (int r = 0; r < 2; ++r) { kern<<<148, threads>>>(out, cyc, 0.999f, 0.001f, 12345); cudaDeviceSynchronize(); }
-  long long h[148]; cudaMemcpy(h, cyc, sizeof(h), cudaMemcpyDeviceToHost);
-  double c = 0; for (int i = 0; i < 148; ++i) c += h[i];
-  cudaFree(out); cudaFree(cyc);
-  return c / 148 / ITERS / (threads / 128.0);
-}
 template <int K> void runadd(const char* name) {
-  const double base = cycles(addk<K, 0>, 384), with = cycles(addk<K, 64>, 384);
+  const double base = per_group(addk<K, 0>, 384), with = per_group(addk<K, 64>, 384);
   printf("%-28s adds %5.2f cycles beside packed FMAs (128 of them: %.0f)\n", name, (with - base) / 64, base);
 }
 int main() {
@@ -189,7 +197,7 @@ int main() {
   runadd<7>("SEL"); runadd<8>("FMNMX"); runadd<5>("SHFL"); runadd<10>("IADD"); runadd<3>("EX2"); runadd<11>("FADD"); runadd<0>("FFMA");
   runadd<9>("PRMT"); runadd<6>("IMAD"); runadd<12>("FMUL2"); runadd<2>("LOP3");
   printf("packed FMA of one pair of its own %.2f cycles, two %.2f, three %.2f, two and a register %.2f; packed product %.2f\n",
-         cycles(readk<0>, 384) / 128, cycles(readk<1>, 384) / 128, cycles(readk<2>, 384) / 128, cycles(readk<4>, 384) / 128,
-         cycles(readk<3>, 384) / 128);
+         per_group(readk<0>, 384) / 128, per_group(readk<1>, 384) / 128, per_group(readk<2>, 384) / 128, per_group(readk<4>, 384) / 128,
+         per_group(readk<3>, 384) / 128);
   return 0;
 }
