@@ -315,7 +315,7 @@ METHOD_EX2_PER_STATE_STEP = 1.0
 METHOD_FMA_PER_STATE_STEP = 12.0
 KERNEL_EX2_PER_STATE_STEP = {"forward rebuild of the chunk (abar)": 1.0, "backward walk (abar again)": 1.0,
                              "chunk-start fix-up": 1.0 / 8}
-# measured pipe rates per clock per SM (profiles/pipe_rates_microbenchmark.md)
+# pipe rates per clock per SM, measured by paper_2501_00692_b200/examples/pipe_rates.cu
 MUFU_PER_CLK_SM = 16.0
 FMA_PER_CLK_SM = 128.0
 
@@ -343,7 +343,7 @@ def report(args, B, w, world, rank, tokens, ms, ms_e2e, h2d, d2h, launches, phas
         sec = k_ms * 1e-3
         alu = {"kernel": "adjoint_main_kernel", "bound": "alu", "sm_mhz": sm_mhz, "launch_ms": k_ms,
                "peak_source": f"{MUFU_PER_CLK_SM:g} ex2 and {FMA_PER_CLK_SM:g} FP32 FMA lanes per clock per SM (measured, "
-                              f"profiles/pipe_rates_microbenchmark.md) x {sms} SMs x sampled SM clock",
+                              f"paper_2501_00692_b200/examples/pipe_rates.cu) x {sms} SMs x sampled SM clock",
                "method_ops": {"ex2_per_state_step": METHOD_EX2_PER_STATE_STEP + live, "fma_per_state_step": METHOD_FMA_PER_STATE_STEP},
                "mufu": {"achieved": ex2_method / sec, "peak": mufu_peak, "unit": "ex2/s", "frac": ex2_method / sec / mufu_peak},
                "fma": {"achieved": fma_method / sec, "peak": fma_peak, "unit": "FP32 op/s", "frac": fma_method / sec / fma_peak},

@@ -40,7 +40,7 @@ constexpr int SM_BT = SM_CT + 8192;      // B   [64 tokens][16 states] bf16
 constexpr int SM_GM = SM_BT + 8192;      // tril(G) [64 tokens t][64 tokens j] bf16
 constexpr int SM_BTT = SM_GM + 8192;     // B^T [16 states][64 tokens] bf16
 // The segment pass needs x, Delta, V and B^T alone, 67 of the 107 KB, and 80 registers with V written eight tokens at a time: three CTAs to an SM,
-// which wait for their loads at different times (2 x 32,768 x 768, whole forward: 331 us with two, 326 with three).
+// which wait for their loads at different times (2 x 32,768 x 768, whole forward in two sessions: 342 and 329 us with two, 332 and 322 with three).
 template <bool YPASS> constexpr int sm_btt() { return YPASS ? SM_BTT : SM_SP; }
 template <bool YPASS> constexpr int smem_dyn() { return sm_btt<YPASS>() + 2048 + 1024; }   // + alignment slack
 template <bool YPASS> constexpr int mm_ctas() { return YPASS ? 2 : 3; }
