@@ -14,9 +14,20 @@ from __future__ import annotations
 from operator import is_
 
 import torch
+from torch.optim.optimizer import register_optimizer_step_post_hook
 
 from . import binding as B
 
+
+_optimizer_steps = 0   # of any optimizer: fused ones write parameters without PyTorch counting it
+
+
+def _after_optimizer_step(*_):
+    global _optimizer_steps
+    _optimizer_steps += 1
+
+
+register_optimizer_step_post_hook(_after_optimizer_step)
 
 WEIGHTS = ("W_delta", "W_B", "W_C")   # what a packed copy is made of
 
@@ -24,8 +35,8 @@ WEIGHTS = ("W_delta", "W_B", "W_C")   # what a packed copy is made of
 class Stack:
     """The parameters stay the caller's tensors and may be updated in place between two calls.  The copies of them that this object
     keeps, packed weights (bf16) and, for the batched "paper" gradients, all parameters stacked, are made again by the next call
-    after a write that PyTorch counts; after any other (through `.data`, by a kernel of one's own, by replaying a graph that does not hold
-    the stack's calls) call parameters_changed()."""
+    after a write that PyTorch counts and after the step of any torch.optim optimizer; after any other write (through `.data`, by
+    a kernel of one's own, by replaying a graph that does not hold the stack's calls) call parameters_changed()."""
 
     def __init__(self, thetas, batch, seqlen, d_model, d_state=16, dtype=torch.float32, device="cuda:0", tbar=None,
                  eps=1e-6):
@@ -58,14 +69,15 @@ class Stack:
         self._packed_of = self._stacked_of = None
 
     def _contents(self, thetas, keys):
-        """The parameters `keys` and how often each has been written; None where that cannot be told: inference tensors do not count
-        writes, and a graph's replays write without a count, to the stack's parameters or before its captured calls."""
+        """The parameters `keys`, how often each has been written, and the optimizers' steps so far; None where that cannot be told:
+        inference tensors do not count writes, and a graph's replays write without a count, to the stack's parameters or
+        before its captured calls."""
         self._captured = self._captured or torch.cuda.is_current_stream_capturing()
         if self._captured:
             return None
         ts = [th[k] for th in thetas for k in keys]
         try:
-            return ts, [t._version for t in ts]
+            return ts, [t._version for t in ts] + [_optimizer_steps]
         except RuntimeError:
             return None
 

@@ -92,3 +92,17 @@ def test_update_between_replays(mode):
     check(out, step(build(w, thetas), x, g, mode), "bf16")
     update(thetas)
     check(step(st, x, g, mode), step(build(w, thetas), x, g, mode), "bf16")
+
+
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+@pytest.mark.parametrize("mode", ["chained", "paper"])
+def test_step_of_a_fused_optimizer(io, mode):
+    """Fused optimizers write the parameters without counting it."""
+    w, thetas, x, g = setting(io)
+    st = build(w, thetas)
+    step(st, x, g, mode)
+    params = [v for th in thetas for v in th.values()]
+    for v in params:
+        v.grad = -v   # p - 0.5 * -p
+    torch.optim.SGD(params, lr=0.5, fused=True).step()
+    check(step(st, x, g, mode), step(build(w, thetas), x, g, mode), io)
